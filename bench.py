@@ -56,9 +56,6 @@ MEASURED_TRAFFIC_PER_KEY = {
     "L1.classify": 9.50,       # 0.5473 + 0.0897 GB (k_classify_ids, ids included)
     "L2.scatter": 25.35,       # 0.9512 + 0.7498 GB (k_scatter_units<512,12,1,0>)
     "L2.classify": 9.39,       # 0.5517 + 0.0787 GB (k_classify_count<2>)
-    "local_sort_mid": 23.15,   # 0.6691 + 0.6138 GB over 55.4 M keys of the class
-    "local_sort_medium": 18.42,  # 0.1037 + 0.0548 GB over 8.6 M keys (writes left in L2)
-    "local_sort": 13.08,       # 0.0379 + 0.0025 GB over 3.1 M keys (writes left in L2)
 }
 
 
@@ -603,9 +600,9 @@ def run_rsort(args):
     torch.cuda.synchronize(dev)
     elems = {"L1": n, "L2": st.level_elems[1] if len(st.level_elems) > 1 else n,
              "L3": st.level_elems[2] if len(st.level_elems) > 2 else 0,
-             "local_copy": st.class_elems[0], "local_sort": st.class_elems[1],
-             "local_sort_mid": st.class_elems[2], "local_sort_medium": st.class_elems[3],
-             "local_big": st.class_elems[4]}
+             "local_sort": st.class_elems[1], "local_sort_mid": st.class_elems[2],
+             "local_sort_medium": st.class_elems[3],
+             "local_rest": st.class_elems[0] + st.class_elems[4]}
     peak, peak_kind = _peaks()
     kernels = {}
     for name, (ms, cnt) in phases.items():

@@ -4,17 +4,22 @@
 //
 //   size 1 or equality bucket  copy through (a stable scatter already left
 //   of a stable level          the elements in position order)
-//   size <= kBucketCap         cta_sort_pairs (cta_sort.cuh): rank-by-counting
-//                              for tiny buckets, equal-width bins + rank-by-
-//                              counting for the rest, bitonic when keys cluster
+//   size <= kBucketCap         rank-by-counting for tiny buckets, equal-width
+//                              bins for the rest; where keys cluster, refined
+//                              bins, then the bitonic network (cta_sort.cuh)
 //   larger (only after the     merge sort through global memory by one CTA:
 //   last partition level)      bitonic-sorted runs, then pairwise merges
 //
-// The sorted buckets come in three size classes, each its own kernel with a
-// CTA shape that fits it: <= 1024 keys (128 threads, 10 CTAs per SM),
-// <= 2048 keys (128 threads, 5 per SM), <= 4096 keys (256 threads, 2 per SM).
-// Buckets are taken from a device work list with an atomic cursor by a
-// persistent grid.  The final store restores float64 bit patterns.
+// Kernels:
+//   k_direct_sort  a whole sort of at most kBucketCap keys, in one launch
+//   k_local_sort   one instantiation per size class with a CTA shape that fits
+//                  it: <= 1024 keys (128 threads, 8 CTAs per SM), <= 2048 keys
+//                  (128 threads, 5 per SM), <= 4096 keys (256 threads, 2 per
+//                  SM)
+//   k_local_rest   what the classes leave (crowded, copied and oversize
+//                  buckets), or every bucket of a call that has few
+// Buckets are taken from device work lists with atomic cursors by persistent
+// grids.  The final store restores float64 bit patterns.
 #include "cta_quicksort.cuh"
 #include "cta_sort.cuh"
 #include "rsort_internal.cuh"
@@ -47,7 +52,7 @@ __device__ __forceinline__ void load_elem(const Bufs& B, const FinalItem& f, uin
   if (f.where == kWhereInput) {
     const uint64_t raw = B.in_key[pos];
     k = B.f64 ? f64_to_ordered(raw) : raw;
-    i = (uint32_t)(pos - f.idx_base);
+    i = (uint32_t)(pos - f.aux);
   } else {
     const Dst& s = f.where == kWhereOut ? B.out : B.tmp;
     k = s.key[pos];
@@ -80,8 +85,11 @@ __device__ __forceinline__ uint64_t merge_split(const uint64_t* ak, const uint32
 // kBucketCap in shared memory, then merges runs pairwise through the two
 // global buffers.  The bucket's range in the other buffer is free: other
 // levels only write ranges of segments that are still being partitioned.
+// Threads of k_local_rest: its buckets are few or its tail is one bucket long,
+// so latency counts (10^5 keys: 256 threads 17.5 us, 512 15.2, 1024 16.7).
+constexpr int kRestThreads = 512;
 __device__ void sort_big(const Bufs& B, const FinalItem& f, uint64_t* sk, uint32_t* si) {
-  constexpr int NT = kLocalThreads;
+  constexpr int NT = kRestThreads;
   const uint64_t m = f.size;
   Dst A = f.where == kWhereOut ? B.out : B.tmp;
   Dst C = f.where == kWhereOut ? B.tmp : B.out;
@@ -159,81 +167,318 @@ __device__ __forceinline__ int64_t next_item(DevState* st, int cls, uint64_t cap
   return it < umin64(st->nfinal_c[cls], cap) ? (int64_t)it : -1;
 }
 
-// The same in two steps: claim_item() sends the atomic (thread 0 keeps its
-// result in a register, so nothing waits for it), take_item() publishes the
-// claimed item to the CTA later, after the atomic's round trip has passed in
-// other work.
-__device__ __forceinline__ uint32_t claim_item(DevState* st, int cls) {
-  return threadIdx.x == 0 ? atomicAdd(&st->cursor_c[cls], 1u) : 0u;
-}
-__device__ __forceinline__ int64_t take_item(const DevState* st, int cls, uint64_t cap,
-                                             uint32_t claimed, uint32_t* s_item) {
-  if (threadIdx.x == 0) *s_item = claimed;
-  __syncthreads();
-  const uint32_t it = *s_item;
-  __syncthreads();
-  return it < umin64(st->nfinal_c[cls], cap) ? (int64_t)it : -1;
+// ---------------------------------------------------------------------------
+// The common in-SM sort of a size class: equal-width bins, one CTA per bucket.
+//
+// A bucket of a partition level brings the range of its keys along (its two
+// splitters); an input bucket's is reduced here.  Its pairs sit in registers,
+// IT a thread; every pair takes its rank inside its bin from one shared-memory
+// atomic on the bin's 16-bit counter, the counters are scanned, the pairs go
+// to their slots, and the few bins that hold several are ordered by insertion.
+// A bucket with a crowded bin is handed to k_local_rest instead (a list of its
+// own), so that no register of this kernel serves that case: with the refined
+// bins and the bitonic network in this kernel the compiler spilled, and the
+// 1025..2048-key class of a 2^28-key sort took 2.63 to 3.40 ms.
+//   2^28 uniform keys, before / after: 1025..2048 keys 2.12 / 1.50 ms (3.5
+//   TB/s of keys and positions read and written), 2049..4096 0.53 / 0.38,
+//   up to 1024 0.12 / 0.087.
+//
+// The kernel is bound by its instructions and by the latency between its
+// barriers, not by memory, hence
+//   - the counters of a thread's run (IT words, two bins each) are cleared,
+//     summed and replaced by 16-byte accesses, runs 4 words apart so that
+//     eight lanes' accesses cover all banks; a word is added to the running
+//     sum by one dp2a; whether a bin is crowded falls out of the OR of the
+//     words;
+//   - slots beyond the bucket's size are skipped four at a time by uniform
+//     branches (a bucket of 1536 keys uses 12 of 16 slots);
+//   - six block barriers per bucket; the claim of the next bucket and its item
+//     travel while this one is sorted, and its loads go out as soon as this
+//     one's pairs have left the registers.
+// ---------------------------------------------------------------------------
+template <int NT, int IT>
+struct BinSort {
+  static constexpr int kCap = NT * IT;
+  static constexpr int kLogIt = IT == 8 ? 3 : 4;
+  static_assert((1 << kLogIt) == IT, "8 or 16 slots a thread");
+  static constexpr int kRun = IT + 4;                       // counter words between two runs
+  static constexpr int kLogBins = kLogIt + 1 + (NT == 128 ? 7 : 8);
+  static_assert((1 << kLogBins) == 2 * kCap, "two bins per slot");
+  // counters, the end of the last bin, and the list of bins to order
+  static constexpr size_t kSmem =
+      (size_t)kCap * 12 + (size_t)NT * kRun * 4 + 16 + (size_t)kCap;
+  // halfword of bin b's counter
+  static __device__ __forceinline__ uint32_t half_of(uint32_t b) {
+    return b + ((b >> (kLogIt + 1)) << 3);
+  }
+  // halfword of the bin after the one at halfword h
+  static __device__ __forceinline__ uint32_t next_half(uint32_t h) {
+    return h % (2 * kRun) == 2 * IT - 1 ? h + 9 : h + 1;
+  }
+};
+
+// Runs fn(r) for every slot r of a thread that some thread of the CTA fills
+// (m pairs, slot r holding element r*NT + tid), four slots per uniform branch.
+template <int NT, int IT, typename Fn>
+__device__ __forceinline__ void for_slots(uint32_t m, Fn fn) {
+#pragma unroll
+  for (int q = 0; q < IT; q += 4) {
+    if (q == 0 || m > (uint32_t)(q * NT)) {
+#pragma unroll
+      for (int r = q; r < q + 4; ++r)
+        if (r * NT + threadIdx.x < m) fn(r);
+    }
+  }
 }
 
-// Resident CTAs per SM of the small class: the sort is latency-bound per
-// bucket, so more buckets in flight per SM pay more than registers (10 CTAs
-// of 128 threads measured 17% faster than 6 at 2^28 keys).
-constexpr int kSmallPerSm = 10;
-
-// Buckets of up to NT*IT keys, sorted by one CTA each (cta_sort_pairs),
-// MINB CTAs resident per SM.
-template <int NT, int IT, int CLS, int MINB>
+// REFINE: crowded bins are refined once (as in cta_sort_crowded) before the
+// bucket is given up; the instantiations for a batch's float64 buckets that
+// span many octaves (a separate kernel for the same reason of registers).
+//   100,000 normal float64 segments of 1 to 2^15 keys, all in-SM kernels:
+//   9.0 ms with the bitonic network for such buckets, 3.3 ms with these.
+template <int NT, int IT, int CLS, int MINB, bool REFINE>
 __global__ void __launch_bounds__(NT, MINB)
-k_local_sort(DevState* st, const FinalItem* items, uint64_t cap, Bufs B) {
-  constexpr int kCap = NT * IT;
+k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
+  using BS = BinSort<NT, IT>;
+  constexpr int NW = NT / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  CtaSortSmem s;
-  s.k = (uint64_t*)smem_raw;          // [kCap]
-  s.i = (uint32_t*)(s.k + kCap);      // [kCap]
-  s.hist = s.i + kCap;                // [kCap]
-  __shared__ uint64_t red[2 * NT / 32];
-  __shared__ uint64_t scan_sm[NT / 32];
-  __shared__ uint32_t s_item;
-  const FinalItem* list = items + (uint64_t)CLS * cap;
-  const uint32_t rank_max = st->local.rank_max;
-  const bool bitonic = st->local.algo[CLS - kClassSmall] == kLocalBitonic;
+  uint64_t* sk = (uint64_t*)smem_raw;                  // [kCap]
+  uint32_t* si = (uint32_t*)(sk + BS::kCap);           // [kCap]
+  uint32_t* hist = si + BS::kCap;                      // [NT * kRun + 4]
+  uint16_t* half = (uint16_t*)hist;
+  uint16_t* multi = (uint16_t*)(hist + NT * BS::kRun + 4);  // [kCap / 2]
+  __shared__ __align__(16) uint32_t s_sum[NW];
+  __shared__ uint64_t s_red[2 * NW];
+  __shared__ FinalItem s_f;
+  __shared__ uint32_t s_nmulti;
+  constexpr int kList = REFINE ? kListRefine + (CLS - kClassSmall) : CLS;
+  const FinalItem* list = items + (uint64_t)kList * cap;
+  const uint32_t nitems = (uint32_t)umin64(st->nfinal_c[kList], cap);
+  const uint32_t rank_max = min(st->local.rank_max, (uint32_t)NT);
+  const uint32_t tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
   uint64_t key[IT];
   uint32_t idx[IT];
-  int64_t it = next_item(st, CLS, cap, &s_item);
-  FinalItem f{};
-  if (it >= 0) {
-    f = list[it];
-    load_bucket<NT, IT>(B, f, key, idx);
-  }
-  while (it >= 0) {
-    // the next bucket is claimed now (the atomic's round trip passes during
-    // this sort) and loaded into the registers as soon as this one's pairs
-    // sit in shared memory (the classes above the small one, whose buckets
-    // take long enough to finish), else after sorting, so its loads are in
-    // flight while this one is finished and stored (the small class has too
-    // few registers to hold the claim across the sort)
-    const uint32_t claimed = claim_item(st, CLS);
-    int64_t it2 = -1;
-    FinalItem f2{};
-    auto claim_next = [&] {
-      it2 = take_item(st, CLS, cap, claimed, &s_item);
-      if (it2 >= 0) {
-        f2 = list[it2];
-        load_bucket<NT, IT>(B, f2, key, idx);
-      }
-    };
-    if constexpr (CLS == kClassSmall) {
-      cta_sort_pairs<NT, IT>(key, idx, f.size, [&] { return list[it].kind == kKindSort; }, s,
-                             red, scan_sm, st->algo_elems, rank_max, bitonic);
-      claim_next();
+  auto load = [&](const FinalItem& f) {
+    if (f.where == kWhereInput) {
+      const uint64_t* kp = B.in_key + f.start + tid;
+      const uint32_t i0 = (uint32_t)(f.start - f.aux) + tid;
+      for_slots<NT, IT>(f.size, [&](int r) {
+        const uint64_t raw = kp[r * NT];
+        key[r] = B.f64 ? f64_to_ordered(raw) : raw;
+        idx[r] = i0 + r * NT;
+      });
     } else {
-      cta_sort_pairs<NT, IT>(key, idx, f.size, [&] { return list[it].kind == kKindSort; }, s,
-                             red, scan_sm, st->algo_elems, rank_max, bitonic, claim_next);
+      const Dst& d = f.where == kWhereOut ? B.out : B.tmp;
+      const uint64_t* kp = d.key + f.start + tid;
+      const uint32_t* ip = d.idx + f.start + tid;
+      for_slots<NT, IT>(f.size, [&](int r) {
+        key[r] = kp[r * NT];
+        idx[r] = ip[r * NT];
+      });
     }
-    for (uint32_t t = threadIdx.x; t < f.size; t += NT) store_out(B, f.start + t, s.k[t], s.i[t]);
-    __syncthreads();
-    it = it2;
-    f = f2;
+  };
+  // the CTA's first bucket by its number, the others by the work counter
+  // (which starts at the grid's size)
+  FinalItem f{};
+  if (blockIdx.x < nitems) {
+    f = list[blockIdx.x];
+    load(f);
+  }
+  while (f.size) {
+    const uint32_t m = f.size;
+    // the next bucket: thread 0 claims it now, reads its item below and
+    // publishes it before the registers free
+    uint32_t claim = 0;
+    if (tid == 0) claim = gridDim.x + atomicAdd(&st->cursor_c[kList], 1u);
+    FinalItem fn{};
+    bool sorted = true;
+    if (m <= rank_max) {
+      // rank-by-counting (Appendix "Fast Work-Inefficient Ranking")
+      __syncthreads();  // the previous bucket has been written out
+      if (tid < m) {
+        sk[tid] = key[0];
+        si[tid] = idx[0];
+      }
+      if (tid == 0) {
+        if (claim < nitems) fn = list[claim];
+        s_f = fn;
+        count_algo(st->algo_elems, kAlgoRank, m);
+      }
+      __syncthreads();
+      uint32_t rank = 0;
+      if (tid < m)
+        for (uint32_t q = 0; q < m; ++q) rank += pair_less(sk[q], si[q], key[0], idx[0]) ? 1u : 0u;
+      __syncthreads();
+      if (tid < m) {
+        sk[rank] = key[0];
+        si[rank] = idx[0];
+      }
+      fn = s_f;
+      load(fn);
+    } else {
+      // smallest key and width of the key range in bits
+      uint64_t mn;
+      int bits;
+      if (f.where == kWhereInput || f.bits == kBitsUnknown) {
+        uint64_t mx = 0;
+        mn = ~0ULL;
+        for_slots<NT, IT>(m, [&](int r) {
+          mn = key[r] < mn ? key[r] : mn;
+          mx = key[r] > mx ? key[r] : mx;
+        });
+        block_minmax_u64<NT>(mn, mx, s_red);
+        bits = mx != mn ? 64 - __clzll((long long)(mx - mn)) : 0;
+      } else {
+        mn = f.aux;
+        bits = f.bits;
+      }
+      const int shift = bits > BS::kLogBins ? bits - BS::kLogBins : 0;
+      uint32_t hr[IT];  // counter halfword, then that << 16 | rank inside the bin
+      for_slots<NT, IT>(m, [&](int r) {
+        hr[r] = BS::half_of((uint32_t)((key[r] - mn) >> shift));
+      });
+      if (tid == 0) s_nmulti = 0;
+#pragma unroll 1
+      for (int pass = 0;; ++pass) {
+        uint4* run = (uint4*)(hist + tid * BS::kRun);
+#pragma unroll
+        for (int q = 0; q < IT / 4; ++q) run[q] = make_uint4(0, 0, 0, 0);
+        __syncthreads();  // (1) counters clear; the previous bucket written out
+        for_slots<NT, IT>(m, [&](int r) {
+          const uint32_t h = hr[r];
+          const uint32_t sh = (h & 1) << 4;
+          const uint32_t old = atomicAdd(&hist[h >> 1], 1u << sh);
+          hr[r] = (h << 16) | ((old >> sh) & 0xffffu);
+        });
+        if (tid == 0 && pass == 0 && claim < nitems) fn = list[claim];
+        __syncthreads();  // (2) counts complete
+        uint32_t sum = 0, any = 0;
+#pragma unroll
+        for (int q = 0; q < IT / 4; ++q) {
+          const uint4 v = run[q];
+          sum = __dp2a_lo(v.x, 0x0101u, sum);
+          sum = __dp2a_lo(v.y, 0x0101u, sum);
+          sum = __dp2a_lo(v.z, 0x0101u, sum);
+          sum = __dp2a_lo(v.w, 0x0101u, sum);
+          any |= v.x | v.y | v.z | v.w;
+        }
+        uint32_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += y;
+        }
+        // a bin of kBinLimit or more pairs sets one of the high bits
+        static_assert((kBinLimit & (kBinLimit - 1)) == 0, "the crowd test reads high bits");
+        constexpr uint32_t kHigh = 0xffffu & ~(uint32_t)(kBinLimit - 1);
+        const bool crowd = __any_sync(0xffffffffu, (any & (kHigh | (kHigh << 16))) != 0);
+        if (lane == 31) s_sum[warp] = inc | (crowd ? 0x80000000u : 0u);
+        __syncthreads();  // (3) warp sums
+        uint32_t pre = 0, all = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+          const uint32_t v = s_sum[w];
+          pre += w < warp ? v : 0u;
+          all |= v;
+        }
+        sorted = (all >> 31) == 0;
+        const bool again = REFINE && pass == 0 && !sorted && shift > 0;
+        if (sorted || again) {
+          // (the crowd flags of the sums before, if any, shift out of at)
+          uint32_t at = (pre & 0xffffu) + inc - sum;
+#pragma unroll
+          for (int q = 0; q < IT / 4; ++q) {
+            uint4 v = run[q];
+            auto step = [&](uint32_t& w) {
+              const uint32_t c = w;
+              w = at * 0x10001u + (c << 16);
+              at = __dp2a_lo(c, 0x0101u, at);
+            };
+            step(v.x);
+            step(v.y);
+            step(v.z);
+            step(v.w);
+            run[q] = v;
+          }
+          if (tid == NT - 1) half[NT * BS::kRun * 2] = (uint16_t)m;
+        }
+        if (!again) break;
+        __syncthreads();
+        // bin b, whose c pairs start at slot lo, becomes 2c parts from 2 lo
+        for_slots<NT, IT>(m, [&](int r) {
+          const uint32_t h = hr[r] >> 16;
+          const uint32_t lo = half[h], c = half[BS::next_half(h)] - lo;
+          const uint64_t off = (key[r] - mn) << (64 - shift);
+          hr[r] = BS::half_of(2 * lo + (uint32_t)__umul64hi(off, (uint64_t)(2 * c)));
+        });
+        __syncthreads();
+      }
+      if (tid == 0) s_f = fn;
+      if (!sorted) {
+        // crowded: the bucket goes to k_local_rest's list
+        if (tid == 0) {
+          const uint32_t slot = atomicAdd(&st->nfinal_c[kListCrowd], 1u);
+          if (slot < cap) items[(uint64_t)kListCrowd * cap + slot] = f;
+          else atomicOr(&st->error, kErrFinalCap);
+        }
+        __syncthreads();
+        f = s_f;
+        load(f);
+        continue;
+      }
+      __syncthreads();  // (4) bin starts in place
+      for_slots<NT, IT>(m, [&](int r) {
+        const uint32_t h = hr[r] >> 16, o = hr[r] & 0xffffu;
+        const uint32_t p = half[h] + o;
+        sk[p] = key[r];
+        si[p] = idx[r];
+        if (o == 1) multi[atomicAdd(&s_nmulti, 1u)] = (uint16_t)h;
+      });
+      if (tid == 0) count_algo(st->algo_elems, kAlgoBins, m);
+      __syncthreads();  // (5) pairs in place, the registers are free
+      fn = s_f;
+      load(fn);
+      // order every listed bin by insertion (an element alone in its bin is
+      // already in its final slot)
+      const uint32_t nmulti = s_nmulti;
+      for (uint32_t j = tid; j < nmulti; j += NT) {
+        const uint32_t h = multi[j];
+        const uint32_t lo = half[h], cnt = half[BS::next_half(h)] - lo;
+        uint64_t* bk = sk + lo;
+        uint32_t* bi = si + lo;
+        for (uint32_t a = 1; a < cnt; ++a) {
+          const uint64_t ka = bk[a];
+          const uint32_t ia = bi[a];
+          uint32_t q = a;
+          while (q > 0 && pair_less(ka, ia, bk[q - 1], bi[q - 1])) {
+            bk[q] = bk[q - 1];
+            bi[q] = bi[q - 1];
+            --q;
+          }
+          bk[q] = ka;
+          bi[q] = ia;
+        }
+      }
+    }
+    __syncthreads();  // (6) sorted
+    {
+      uint64_t* ko = B.out.key + f.start;
+      uint32_t* io = B.out.idx + f.start;
+      if (B.f64) {
+        for (uint32_t t = tid; t < m; t += NT) {
+          ko[t] = ordered_to_f64(sk[t]);
+          io[t] = si[t];
+        }
+      } else {
+#pragma unroll 4
+        for (uint32_t t = tid; t < m; t += NT) {
+          ko[t] = sk[t];
+          io[t] = si[t];
+        }
+      }
+    }
+    f = fn;
   }
 }
 
@@ -269,42 +514,133 @@ k_local_quicksort(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, ui
   }
 }
 
-// Copy-through buckets (size 1, or equality buckets already in position
-// order): a coalesced copy that restores float64 bit patterns.
-__global__ void __launch_bounds__(256)
-k_local_copy(DevState* st, const FinalItem* items, uint64_t cap, Bufs B) {
-  __shared__ uint32_t s_item;
-  const FinalItem* list = items + (uint64_t)kClassCopy * cap;
-  for (;;) {
-    const int64_t it = next_item(st, kClassCopy, cap, &s_item);
-    if (it < 0) break;
-    const FinalItem f = list[it];
-    if (f.where == kWhereOut && !B.f64) continue;  // already in place
-    for (uint32_t t = threadIdx.x; t < f.size; t += blockDim.x) {
-      uint64_t k;
-      uint32_t i;
-      load_elem(B, f, t, k, i);
-      store_out(B, f.start + t, k, i);
-    }
-  }
-}
-
-// Oversize buckets (after the last partition level; vanishingly rare).
-__global__ void __launch_bounds__(kLocalThreads)
-k_local_big(DevState* st, const FinalItem* items, uint64_t cap, Bufs B) {
+// Everything the class kernels leave, by 512-thread CTAs of 8 slots: the
+// copy-through buckets (size 1, or equality buckets already in position order:
+// a coalesced copy that restores float64 bit patterns), the buckets with
+// crowded bins (cta_sort_pairs: refined bins, the bitonic network), and the
+// oversize ones (after the last partition level; rare).  With `classes` the
+// size classes' own lists too (bit c: list c): a call of few buckets finishes
+// in this one launch, whose slowest bucket bounds it, instead of one launch
+// per class, each as long as its slowest bucket.  bitonic: bit c sorts class
+// c's buckets by bitonic sort.
+__global__ void __launch_bounds__(kRestThreads, 2)
+k_local_rest(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, uint32_t lists,
+             uint32_t bitonic) {
+  constexpr int NT = kRestThreads, IT = kBucketCap / kRestThreads;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  uint64_t* sk = (uint64_t*)smem_raw;
-  uint32_t* si = (uint32_t*)(sk + kBucketCap);
-  __shared__ uint32_t s_item;
-  const FinalItem* list = items + (uint64_t)kClassBig * cap;
-  for (;;) {
-    const int64_t it = next_item(st, kClassBig, cap, &s_item);
-    if (it < 0) break;
-    count_algo(st->algo_elems, kAlgoMerge, list[it].size);
-    sort_big(B, list[it], sk, si);
+  CtaSortSmem s;
+  s.k = (uint64_t*)smem_raw;
+  s.i = (uint32_t*)(s.k + NT * IT);
+  s.hist = s.i + NT * IT;
+  __shared__ uint64_t red[2 * NT / 32];
+  __shared__ uint64_t scan_sm[NT / 32];
+  __shared__ uint32_t s_next;
+  const uint32_t rank_max = st->local.rank_max;
+  // lists in turn, the longest work first (an oversize bucket's merges run
+  // longest)
+  auto list_of = [](int q) {
+    constexpr int order[kNumLists] = {kClassBig,       kListCrowd,      kListRefine + 2,
+                                      kClassMedium,    kListRefine + 1, kClassMid,
+                                      kListRefine + 0, kClassSmall,     kClassCopy};
+    return order[q];
+  };
+  uint32_t end[kNumLists], total = 0;
+#pragma unroll
+  for (int q = 0; q < kNumLists; ++q) {
+    const int l = list_of(q);
+    total += (lists >> l) & 1u ? (uint32_t)umin64(st->nfinal_c[l], cap) : 0u;
+    end[q] = total;
+  }
+  uint32_t at = blockIdx.x;
+  while (at < total) {
+    int l = list_of(0);
+    uint32_t from = 0;
+#pragma unroll
+    for (int q = 0; q + 1 < kNumLists; ++q) {
+      if (at >= end[q]) {
+        l = list_of(q + 1);
+        from = end[q];
+      }
+    }
+    const FinalItem f = items[(uint64_t)l * cap + (at - from)];
+    if (threadIdx.x == 0) s_next = gridDim.x + atomicAdd(&st->cursor_rest, 1u);
+    if (l == kClassCopy) {
+      if (f.where != kWhereOut || B.f64) {  // else already in place
+        for (uint32_t t = threadIdx.x; t < f.size; t += NT) {
+          uint64_t k;
+          uint32_t i;
+          load_elem(B, f, t, k, i);
+          store_out(B, f.start + t, k, i);
+        }
+      }
+    } else if (l == kClassBig) {
+      count_algo(st->algo_elems, kAlgoMerge, f.size);
+      sort_big(B, f, s.k, s.i);
+    } else {
+      uint64_t key[IT];
+      uint32_t idx[IT];
+      load_bucket<NT, IT>(B, f, key, idx);
+      cta_sort_pairs<NT, IT>(key, idx, f.size, [&] { return f.kind == kKindSort; }, s, red,
+                             scan_sm, st->algo_elems, rank_max,
+                             (bitonic >> l) & 1u);
+      for (uint32_t t = threadIdx.x; t < f.size; t += NT)
+        store_out(B, f.start + t, s.k[t], s.i[t]);
+    }
+    __syncthreads();
+    at = s_next;
+    __syncthreads();
   }
 }
 
+// A whole sort of n <= kBucketCap keys by one CTA, which also resets the
+// control block (statistics and the error word are read from it): one launch
+// instead of six.  One bucket alone is bound by the latency of its steps, so
+// it takes 512 threads, eight slots each (1024 of four measured 1 to 2 us slower).
+constexpr int kDirectThreads = 512;
+__global__ void __launch_bounds__(kDirectThreads, 1)
+k_direct_sort(DevState* st, Bufs B, uint32_t n, LocalPlan local) {
+  constexpr int NT = kDirectThreads, IT = kBucketCap / kDirectThreads;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  CtaSortSmem s;
+  s.k = (uint64_t*)smem_raw;
+  s.i = (uint32_t*)(s.k + NT * IT);
+  s.hist = s.i + NT * IT;
+  __shared__ uint64_t red[2 * NT / 32];
+  __shared__ uint64_t scan_sm[NT / 32];
+  FinalItem f;
+  f.start = f.aux = 0;
+  f.size = n;
+  f.where = kWhereInput;
+  f.kind = kKindSort;
+  f.bits = kBitsUnknown;
+  uint64_t key[IT];
+  uint32_t idx[IT];
+  load_bucket<NT, IT>(B, f, key, idx);
+  static_assert(sizeof(DevState) % 4 == 0 && sizeof(DevState) / 4 <= NT, "one word a thread");
+  if (threadIdx.x < sizeof(DevState) / 4) reinterpret_cast<uint32_t*>(st)[threadIdx.x] = 0;
+  __syncthreads();
+  const int c = n == 1 ? kClassCopy
+                       : (n <= local.small_cap ? kClassSmall
+                                               : (n <= local.mid_cap ? kClassMid : kClassMedium));
+  if (threadIdx.x == 0) {
+    st->local = local;
+    st->nfinal_c[c] = 1;
+    st->class_elems[c] = n;
+  }
+  if (n > 1)
+    cta_sort_pairs<NT, IT>(key, idx, n, [&] { return true; }, s, red, scan_sm, st->algo_elems,
+                           local.rank_max, local.algo[c - kClassSmall] == kLocalBitonic);
+  if (n == 1) {
+    if (threadIdx.x == 0) store_out(B, 0, key[0], idx[0]);
+  } else {
+    for (uint32_t t = threadIdx.x; t < n; t += NT) store_out(B, t, s.k[t], s.i[t]);
+  }
+}
+
+// Resident CTAs per SM of the small class: the sort is latency-bound per
+// bucket, so more buckets in flight per SM pay more than registers.
+constexpr int kSmallPerSm = 8;
+constexpr int kSmallRefinePerSm = 6;
 constexpr int kSmallThreads = 128;
 constexpr int kSmallItems = kSmallCap / kSmallThreads;  // 8
 static_assert(kSmallThreads * kSmallItems == (int)kSmallCap, "small class fits one CTA");
@@ -314,73 +650,131 @@ static_assert(kSmallThreads * kSmallItems == (int)kSmallCap, "small class fits o
 constexpr int kMidThreads = 128;
 constexpr int kMidItems = (int)kMidCap / kMidThreads;  // 16
 constexpr int kMidPerSm = 5;
+constexpr int kMidRefinePerSm = 4;
 static_assert(kMidThreads * kMidItems == (int)kMidCap, "mid class fits one CTA");
 // The medium class (2049..4096 keys): 256 threads of 16 slots, two CTAs per
 // SM (with the next bucket claimed and loaded early, this measured 2 %
 // faster than 512 threads of 8 slots, which had spread every bucket's fixed
 // work over half the keys per thread).
 constexpr int kMediumThreads = 256;
+constexpr int kMediumPerSm = 2;
 constexpr int kMediumItems = kBucketCap / kMediumThreads;  // 16
 static_assert(kMediumThreads * kMediumItems == kBucketCap, "medium class fits one CTA");
+
+
+// Calls whose buckets cannot outnumber this many per SM finish in one launch
+// of k_local_rest: 66 buckets (10^5 keys) 54 -> 15 us, 714 buckets (2^20 keys)
+// 43 -> 29 us against a launch per class; the class kernels sort a bucket in
+// less SM time and win above.
+constexpr uint64_t kOneLaunchPerSm = 8;
+
+template <int NT, int IT, int CLS, int MINB, bool REFINE>
+void launch_class(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t cap, const Bufs& B,
+                  const char* name) {
+  Scope sc(e, name);
+  k_local_sort<NT, IT, CLS, MINB, REFINE>
+      <<<e.num_sms * MINB, NT, BinSort<NT, IT>::kSmem, e.stream>>>(st, items, cap, B);
+}
+
+template <int NT, int IT, int CLS, int MINB, int MINBR>
+void set_class_attributes() {
+  cudaFuncSetAttribute(k_local_sort<NT, IT, CLS, MINB, false>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BinSort<NT, IT>::kSmem);
+  cudaFuncSetAttribute(k_local_sort<NT, IT, CLS, MINBR, true>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BinSort<NT, IT>::kSmem);
+}
 
 }  // namespace
 
 void set_local_kernel_attributes() {
-  cudaFuncSetAttribute(k_local_sort<kSmallThreads, kSmallItems, kClassSmall, kSmallPerSm>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallCap * kCtaSortBytesPerElem);
-  cudaFuncSetAttribute(k_local_sort<kMidThreads, kMidItems, kClassMid, kMidPerSm>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMidCap * kCtaSortBytesPerElem);
+  set_class_attributes<kSmallThreads, kSmallItems, kClassSmall, kSmallPerSm, kSmallRefinePerSm>();
+  set_class_attributes<kMidThreads, kMidItems, kClassMid, kMidPerSm, kMidRefinePerSm>();
+  set_class_attributes<kMediumThreads, kMediumItems, kClassMedium, kMediumPerSm,
+                       kMediumPerSm>();
+  cudaFuncSetAttribute(k_direct_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       kBucketCap * kCtaSortBytesPerElem);
   cudaFuncSetAttribute(k_local_quicksort<kLocalThreads, (int)kMidCap, kClassMid>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs_smem_bytes(kMidCap));
-  cudaFuncSetAttribute(k_local_sort<kMediumThreads, kMediumItems, kClassMedium, 2>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, kBucketCap * kCtaSortBytesPerElem);
   cudaFuncSetAttribute(k_local_quicksort<kLocalThreads, kBucketCap, kClassMedium>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs_smem_bytes(kBucketCap));
-  cudaFuncSetAttribute(k_local_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kBucketCap * 12);
+  cudaFuncSetAttribute(k_local_rest, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       kBucketCap * kCtaSortBytesPerElem);
 }
 
-void launch_local_sort(const LaunchEnv& e, DevState* st, const FinalItem* items,
-                       uint64_t item_cap, const uint64_t* in_key, Dst out, Dst tmp, int f64) {
+bool direct_sort_takes(const LocalPlan& local, uint64_t n) {
+  const int c = n <= local.small_cap ? 0 : (n <= local.mid_cap ? 1 : 2);
+  return n <= (uint64_t)kBucketCap && local.algo[c] != kLocalQuick;
+}
+
+void launch_direct_sort(const LaunchEnv& e, DevState* st, const uint64_t* in_key, Dst out,
+                        uint32_t n, int f64) {
+  Bufs B;
+  B.in_key = in_key;
+  B.out = out;
+  B.tmp = out;
+  B.f64 = f64;
+  Scope sc(e, "direct_sort");
+  k_direct_sort<<<1, kDirectThreads, kBucketCap * kCtaSortBytesPerElem, e.stream>>>(st, B, n,
+                                                                                    e.local);
+}
+
+void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t item_cap,
+                       uint64_t max_items, const uint64_t* in_key, Dst out, Dst tmp, int f64,
+                       bool segmented) {
   Bufs B;
   B.in_key = in_key;
   B.out = out;
   B.tmp = tmp;
   B.f64 = f64;
-  {
-    Scope sc(e, "local_copy");
-    k_local_copy<<<e.num_sms * 4, 256, 0, e.stream>>>(st, items, item_cap, B);
+  // k_local_rest takes a class whose algorithm is bitonic, and every class of
+  // a call with few buckets
+  const uint8_t* algo = e.local.algo;
+  const bool one = max_items <= kOneLaunchPerSm * (uint64_t)e.num_sms;
+  const bool refine = segmented && f64;
+  uint32_t lists = (1u << kClassCopy) | (1u << kClassBig) | (1u << kListCrowd), bitonic = 0;
+  for (int c = kClassSmall; c <= kClassMedium; ++c) {
+    const uint8_t a = algo[c - kClassSmall];
+    if (a == kLocalBitonic) bitonic |= 1u << c;
+    if (a == kLocalBitonic || (one && a == kLocalBins)) lists |= 1u << c;
+    if (one && a == kLocalBins) lists |= 1u << (kListRefine + c - kClassSmall);
   }
-  {
-    Scope sc(e, "local_sort");
-    k_local_sort<kSmallThreads, kSmallItems, kClassSmall, kSmallPerSm>
-        <<<e.num_sms * kSmallPerSm, kSmallThreads, kSmallCap * kCtaSortBytesPerElem, e.stream>>>(st, items, item_cap, B);
+  auto own = [&](int c) { return algo[c - kClassSmall] == kLocalBins && !((lists >> c) & 1u); };
+  if (own(kClassSmall)) {
+    launch_class<kSmallThreads, kSmallItems, kClassSmall, kSmallPerSm, false>(
+        e, st, items, item_cap, B, "local_sort");
+    if (refine)
+      launch_class<kSmallThreads, kSmallItems, kClassSmall, kSmallRefinePerSm, true>(
+          e, st, items, item_cap, B, "local_sort_refine");
   }
-  {
+  if (algo[kClassMid - kClassSmall] == kLocalQuick) {
     Scope sc(e, "local_sort_mid");
-    if (e.local.algo[kClassMid - kClassSmall] == kLocalQuick)
-      k_local_quicksort<kLocalThreads, (int)kMidCap, kClassMid>
-          <<<e.num_sms * 2, kLocalThreads, qs_smem_bytes(kMidCap), e.stream>>>(
-              st, items, item_cap, B, 0x243f6a8885a308d3ULL);
-    else
-      k_local_sort<kMidThreads, kMidItems, kClassMid, kMidPerSm>
-          <<<e.num_sms * kMidPerSm, kMidThreads, kMidCap * kCtaSortBytesPerElem, e.stream>>>(
-              st, items, item_cap, B);
+    k_local_quicksort<kLocalThreads, (int)kMidCap, kClassMid>
+        <<<e.num_sms * 2, kLocalThreads, qs_smem_bytes(kMidCap), e.stream>>>(
+            st, items, item_cap, B, 0x243f6a8885a308d3ULL);
+  } else if (own(kClassMid)) {
+    launch_class<kMidThreads, kMidItems, kClassMid, kMidPerSm, false>(e, st, items, item_cap, B,
+                                                                      "local_sort_mid");
+    if (refine)
+      launch_class<kMidThreads, kMidItems, kClassMid, kMidRefinePerSm, true>(
+          e, st, items, item_cap, B, "local_sort_mid_refine");
   }
-  {
+  if (algo[kClassMedium - kClassSmall] == kLocalQuick) {
     Scope sc(e, "local_sort_medium");
-    if (e.local.algo[kClassMedium - kClassSmall] == kLocalQuick)
-      k_local_quicksort<kLocalThreads, kBucketCap, kClassMedium>
-          <<<e.num_sms * 2, kLocalThreads, qs_smem_bytes(kBucketCap), e.stream>>>(
-              st, items, item_cap, B, 0x9e3779b97f4a7c15ULL);
-    else
-      k_local_sort<kMediumThreads, kMediumItems, kClassMedium, 2>
-          <<<e.num_sms * 2, kMediumThreads, kBucketCap * kCtaSortBytesPerElem, e.stream>>>(
-              st, items, item_cap, B);
+    k_local_quicksort<kLocalThreads, kBucketCap, kClassMedium>
+        <<<e.num_sms * 2, kLocalThreads, qs_smem_bytes(kBucketCap), e.stream>>>(
+            st, items, item_cap, B, 0x9e3779b97f4a7c15ULL);
+  } else if (own(kClassMedium)) {
+    launch_class<kMediumThreads, kMediumItems, kClassMedium, kMediumPerSm, false>(
+        e, st, items, item_cap, B, "local_sort_medium");
+    if (refine)
+      launch_class<kMediumThreads, kMediumItems, kClassMedium, kMediumPerSm, true>(
+          e, st, items, item_cap, B, "local_sort_medium_refine");
   }
   {
-    Scope sc(e, "local_big");
-    k_local_big<<<e.num_sms, kLocalThreads, kBucketCap * 12, e.stream>>>(st, items, item_cap, B);
+    Scope sc(e, "local_rest");
+    const uint64_t grid = umin64(umax64(max_items, 1), (uint64_t)e.num_sms * 2);
+    k_local_rest<<<(int)grid, kRestThreads, kBucketCap * kCtaSortBytesPerElem, e.stream>>>(
+        st, items, item_cap, B, lists, bitonic);
   }
 }
 

@@ -46,11 +46,12 @@ __global__ void k_init_plain(DevState* st, SegIn* list_l1, FinalItem* items, uin
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   st->local = local;
   st->nseg[0] = st->nseg[1] = 0;
-  for (int c = 0; c < kNumClasses; ++c) {
+  for (int c = 0; c < kNumLists; ++c) {
     st->nfinal_c[c] = 0;
     st->cursor_c[c] = 0;
-    st->class_elems[c] = 0;
   }
+  for (int c = 0; c < kNumClasses; ++c) st->class_elems[c] = 0;
+  st->cursor_rest = 0;
   for (int a = 0; a < kNumAlgos; ++a) st->algo_elems[a] = 0;
   st->error = 0;
   st->max_bucket_l1 = 0;
@@ -64,16 +65,18 @@ __global__ void k_init_plain(DevState* st, SegIn* list_l1, FinalItem* items, uin
   if (direct) {
     FinalItem f;
     f.start = 0;
-    f.idx_base = 0;
+    f.aux = 0;
     f.size = (uint32_t)n;
     f.where = kWhereInput;
     f.kind = n == 1 ? kKindCopy : kKindSort;
+    f.bits = kBitsUnknown;
     push_final(st, items, final_cap, f, kErrFinalCap);
   } else {
     SegIn s;
     s.start = 0;
     s.m = (uint32_t)n;
     s.k_hint = k1;
+    s.range = KeyRange{0, ~0ULL, 0, 0};
     list_l1[0] = s;
     st->nseg[1] = 1;  // level 1 reads list parity 1
   }
@@ -155,6 +158,7 @@ k_level_plan(DevState* st, const SegIn* list_in, LevelSeg* segs, LevelParams P, 
       // equal chunks inside the segment (the level's W bounds their size)
       s.W = nch ? (uint32_t)(((uint64_t)in.m + nch - 1) / nch) : P.W;
       s.pad = 0;
+      s.range = in.range;
       segs[g] = s;
     }
     __syncthreads();
@@ -1111,16 +1115,24 @@ k_collect(DevState* st, const LevelSeg* segs, const uint64_t* ssk, const uint32_
     }
     if (P.level == 1) atomicMax(&st->max_bucket_l1, size);
     if (!emit_final || size == 0) continue;
-    bool eq = false;
-    if (ordered && b >= 1 && b + 1 < sg.k) {
-      const uint64_t klo = ssk[sg.samp_off + ((uint64_t)b * sg.S) / sg.k];
-      const uint64_t khi = ssk[sg.samp_off + ((uint64_t)(b + 1) * sg.S) / sg.k];
-      eq = klo == khi;
+    // its keys lie between its splitters (the segment's bounds at the ends)
+    KeyRange kr = sg.range;
+    if (b >= 1) {
+      kr.lo = ssk[sg.samp_off + ((uint64_t)b * sg.S) / sg.k];
+      kr.known |= 1u;
     }
+    if (b + 1 < sg.k) {
+      kr.hi = ssk[sg.samp_off + ((uint64_t)(b + 1) * sg.S) / sg.k];
+      kr.known |= 2u;
+    }
+    const bool eq = ordered && b >= 1 && b + 1 < sg.k && kr.lo == kr.hi;
     if (eq || size <= kBucketCap || last_level) {
       FinalItem it;
       it.start = start;
-      it.idx_base = 0;
+      it.aux = kr.lo;
+      it.bits = kr.known != 3u       ? kBitsUnknown
+                : kr.hi == kr.lo     ? (uint8_t)0
+                                     : (uint8_t)(64 - __clzll((long long)(kr.hi - kr.lo)));
       it.size = size;
       it.where = where;
       it.kind = (eq || size == 1)      ? kKindCopy
@@ -1128,12 +1140,15 @@ k_collect(DevState* st, const LevelSeg* segs, const uint64_t* ssk, const uint32_
                 : ordered              ? kKindSort
                                        : kKindSortAny;
       if (it.kind == kKindBig) atomicAdd((unsigned long long*)&st->big_items, 1ull);
-      push_final(st, items, P.final_cap, it, kErrFinalCap);
+      push_final(st, items, P.final_cap, it, kErrFinalCap,
+                 P.refine && it.bits >= kRefineBits && it.bits != kBitsUnknown &&
+                     size > st->local.rank_max);
     } else {
       SegIn s;
       s.start = start;
       s.m = size;
       s.k_hint = 0;
+      s.range = kr;
       const uint32_t slot = atomicAdd(&st->nseg[par_out], 1u);
       if (slot < P.seg_cap) list_out[slot] = s;
       else atomicOr(&st->error, kErrSegCap);
@@ -1576,7 +1591,8 @@ int wide_scatter_blocks_per_sm(uint32_t kmax, int mode, bool stable) {
 // device error flag instead of being followed.
 __global__ void __launch_bounds__(256)
 k_init_segments(DevState* st, const uint64_t* offsets, uint32_t nseg, uint64_t n,
-                SegIn* list_l1, FinalItem* items, uint64_t seg_cap, uint64_t final_cap) {
+                SegIn* list_l1, FinalItem* items, uint64_t seg_cap, uint64_t final_cap,
+                int f64) {
   for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < nseg;
        s += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t a = offsets[s], b = offsets[s + 1];
@@ -1589,16 +1605,18 @@ k_init_segments(DevState* st, const uint64_t* offsets, uint32_t nseg, uint64_t n
     if (m <= (uint64_t)kBucketCap) {
       FinalItem f;
       f.start = a;
-      f.idx_base = a;
+      f.aux = a;
       f.size = (uint32_t)m;
       f.where = kWhereInput;
       f.kind = m == 1 ? kKindCopy : kKindSort;
-      push_final(st, items, final_cap, f, kErrFinalCap);
+      f.bits = kBitsUnknown;
+      push_final(st, items, final_cap, f, kErrFinalCap, f64 != 0 && m > st->local.rank_max);
     } else {
       SegIn in;
       in.start = a;
       in.m = (uint32_t)m;
       in.k_hint = 0;
+      in.range = KeyRange{0, ~0ULL, 0, 0};
       const uint32_t slot = atomicAdd(&st->nseg[1], 1u);
       if (slot < seg_cap) list_l1[slot] = in;
       else atomicOr(&st->error, kErrSegCap);
@@ -1608,11 +1626,11 @@ k_init_segments(DevState* st, const uint64_t* offsets, uint32_t nseg, uint64_t n
 
 void launch_init_segments(const LaunchEnv& e, DevState* st, const uint64_t* offsets,
                           uint32_t nseg, uint64_t n, SegIn* list_l1, FinalItem* items,
-                          uint64_t seg_cap, uint64_t final_cap) {
+                          uint64_t seg_cap, uint64_t final_cap, int f64) {
   Scope sc(e, "init_segments");
   const int grid = (int)umin64((nseg + 255) / 256 + 1, (uint64_t)e.num_sms * 8);
   k_init_segments<<<grid, 256, 0, e.stream>>>(st, offsets, nseg, n, list_l1, items, seg_cap,
-                                              final_cap);
+                                              final_cap, f64);
 }
 
 void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const SegIn* list_in,

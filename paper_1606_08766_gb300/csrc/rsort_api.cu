@@ -133,7 +133,7 @@ void layout(Plan& p) {
     return at;
   };
   p.off_state = take(sizeof(DevState));
-  p.off_items = take((size_t)kNumClasses * p.final_cap * sizeof(FinalItem));
+  p.off_items = take((size_t)kNumLists * p.final_cap * sizeof(FinalItem));
   if (p.need_tmp) {
     p.off_tmp_key = take(p.n * 8);
     p.off_tmp_idx = take(p.n * 4);
@@ -289,7 +289,7 @@ void set_attributes_once(int device) {
 void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const LaunchEnv& e, DevState* st,
                               FinalItem* items, SegIn* const lists[2], rsort_key_type type,
                               const void* d_keys_in, const Dst& out, const Dst& tmp,
-                              uint64_t seed, uint32_t k1) {
+                              uint64_t seed, uint32_t k1, bool segmented) {
   // Level 1 scatters into the output buffer unless the input is that buffer
   // (an in-place sort): its equality buckets, final when kept in position
   // order, then need no copy.  Later levels alternate with the scratch
@@ -303,6 +303,7 @@ void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const 
     // (the in-SM sort orders (key, position) pairs either way; level 1's
     // default leaves it to the device); a level's input is in position order
     // only after stable levels, and level 1's order is read on the device
+    P.refine = segmented && type == RSORT_KEY_F64;
     P.stable = L == 1 ? c->level1_stable : c->deep_levels_stable;
     P.in_order = L == 1 ? 1 : (L == 2 || c->deep_levels_stable ? kOrderAuto : 0);
     Src src;
@@ -321,8 +322,8 @@ void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const 
                  at<uint32_t>(ws, p.off_hist), at<uint32_t>(ws, p.off_sums), items, kmax,
                  L == p.levels, 1, nullptr, p.n, 0);
   }
-  launch_local_sort(e, st, items, p.final_cap, (const uint64_t*)d_keys_in, out, tmp,
-                    type == RSORT_KEY_F64);
+  launch_local_sort(e, st, items, p.final_cap, p.direct ? 1 : p.final_cap,
+                    (const uint64_t*)d_keys_in, out, tmp, type == RSORT_KEY_F64, segmented);
 }
 
 rsort_status set_tunable(rsort_ctx* c, const char* name, long long v) {
@@ -554,11 +555,15 @@ rsort_status enqueue_sort(rsort_ctx* c, Workspace& ws, const LaunchEnv& e, rsort
   DevState* st = at<DevState>(ws, p.off_state);
   FinalItem* items = at<FinalItem>(ws, p.off_items);
   SegIn* lists[2] = {at<SegIn>(ws, p.off_list0), at<SegIn>(ws, p.off_list1)};
-  launch_init_plain(e, st, lists[1], items, n, k1, p.direct, p.final_cap);
   Dst out{(uint64_t*)d_keys_out, d_perm_out};
-  Dst tmp{at<uint64_t>(ws, p.off_tmp_key), at<uint32_t>(ws, p.off_tmp_idx)};
-  enqueue_levels_and_local(c, ws, p, e, st, items, lists, type, d_keys_in, out, tmp, seed, k1);
   if (st_out) *st_out = st;
+  if (p.direct && direct_sort_takes(e.local, n)) {
+    launch_direct_sort(e, st, (const uint64_t*)d_keys_in, out, (uint32_t)n, type == RSORT_KEY_F64);
+    return RSORT_OK;
+  }
+  launch_init_plain(e, st, lists[1], items, n, k1, p.direct, p.final_cap);
+  Dst tmp{at<uint64_t>(ws, p.off_tmp_key), at<uint32_t>(ws, p.off_tmp_idx)};
+  enqueue_levels_and_local(c, ws, p, e, st, items, lists, type, d_keys_in, out, tmp, seed, k1, false);
   return RSORT_OK;
 }
 
@@ -574,10 +579,10 @@ rsort_status enqueue_segmented(rsort_ctx* c, Workspace& ws, const LaunchEnv& e,
   SegIn* lists[2] = {at<SegIn>(ws, p.off_list0), at<SegIn>(ws, p.off_list1)};
   launch_init_plain(e, st, lists[1], items, 0, 0, 0, p.final_cap);  // reset the control block
   launch_init_segments(e, st, d_offsets, num_segments, n, lists[1], items, p.seg_cap,
-                       p.final_cap);
+                       p.final_cap, type == RSORT_KEY_F64);
   Dst out{(uint64_t*)d_keys_out, d_perm_out};
   Dst tmp{at<uint64_t>(ws, p.off_tmp_key), at<uint32_t>(ws, p.off_tmp_idx)};
-  enqueue_levels_and_local(c, ws, p, e, st, items, lists, type, d_keys_in, out, tmp, seed, 0);
+  enqueue_levels_and_local(c, ws, p, e, st, items, lists, type, d_keys_in, out, tmp, seed, 0, true);
   if (st_out) *st_out = st;
   return RSORT_OK;
 }
@@ -860,7 +865,8 @@ rsort_status rsort_sort(rsort_ctx* c, rsort_key_type type, const void* d_keys_in
     const double mean = opt_stats->p ? (double)n / opt_stats->p : (double)n;
     opt_stats->max_over_mean = mean > 0 ? opt_stats->max_bucket / mean : 0.0;
     opt_stats->final_buckets = 0;
-    for (int i = 0; i < kNumClasses; ++i) opt_stats->final_buckets += h.nfinal_c[i];
+    // (kListCrowd's buckets are on their class's list too)
+    for (int i = 0; i < kListCrowd; ++i) opt_stats->final_buckets += h.nfinal_c[i];
     // per key: level 1's classify reads 8 B and writes a 2-byte bucket id,
     // its scatter reads 8 + 2 and writes 12; a deeper level reads 8 and
     // writes 2, then reads 12 + 2 and writes 12; the in-SM sort reads and

@@ -27,8 +27,7 @@ constexpr int kSampleChunk = 8192;                // sample sort: pairs per CTA 
 constexpr int kSampleThreads = 512;               // sample sort CTA
 constexpr int kDeepOversample = 16;               // samples per bucket at levels >= 2
 constexpr int kMaxLevels = 3;                     // partition levels before fallback
-constexpr int kLocalThreads = 256;                // in-SM bucket sort CTA
-constexpr int kLocalItems = 16;                   // kLocalThreads * kLocalItems = kBucketCap
+constexpr int kLocalThreads = 256;                // in-SM quicksort CTA
 constexpr int kRankMax = 64;                      // rank-by-counting up to this size
 constexpr int kScanTile = 4096;                   // device scan tile (1024 x 4)
 constexpr int kUnitMaxK = 1024;                   // buckets of the whole-unit scatter
@@ -49,7 +48,15 @@ enum : int {
   kClassMid = 2,     // <= kMidCap keys
   kClassMedium = 3,  // <= kBucketCap keys
   kClassBig = 4,
-  kNumClasses = 5
+  kNumClasses = 5,
+  // a batch's float64 buckets that span many octaves (segments straight from
+  // the input, and the buckets around zero): lists of their own per size class,
+  // sorted with bins refined to the keys' density (their bit patterns crowd a
+  // few octaves, so equal-width bins would not do)
+  kListRefine = 5,   // + (class - kClassSmall)
+  // buckets in which a class kernel found crowded bins
+  kListCrowd = 8,
+  kNumLists = 9
 };
 // Which in-SM algorithm finished a bucket (rsort_stats.algo_elems counts the
 // elements each one handled):
@@ -80,11 +87,19 @@ struct LocalPlan {
   uint8_t algo[3] = {kLocalBins, kLocalBins, kLocalBins};  // small, mid, medium
 };
 
+// Range of the keys of a segment or bucket, as far as splitters bound it.
+struct KeyRange {
+  uint64_t lo, hi;  // inclusive
+  uint32_t known;   // bit 0: lo is a bound, bit 1: hi is
+  uint32_t pad;
+};
+
 // A segment waiting to be partitioned (input of a level).
 struct SegIn {
   uint64_t start;   // absolute position (identical in every buffer)
   uint32_t m;       // elements
   uint32_t k_hint;  // buckets requested (>= 1), or 0 to choose from m
+  KeyRange range;   // of its keys
 };
 
 // A segment being partitioned at the current level (written by the plan).
@@ -105,22 +120,30 @@ struct LevelSeg {
   uint32_t nunits;      // histogram units: nchunks (CTA chunks) or 8 * nchunks (warp sub-chunks)
   uint32_t W;           // keys per chunk of this segment (all chunks equal but the last)
   uint32_t pad;
+  KeyRange range;       // of the segment's keys
 };
 
 // A bucket handed to the in-SM sort.
 struct FinalItem {
   uint64_t start;     // absolute position of its first element
-  uint64_t idx_base;  // position - idx_base = original position (input only)
+  uint64_t aux;       // input: position - aux = original position;
+                      // otherwise the smallest key its splitters allow
   uint32_t size;
   uint16_t where;
-  uint16_t kind;
+  uint8_t kind;
+  uint8_t bits;       // bits of (largest - smallest key) the splitters allow
+                      // (not input), or kBitsUnknown
 };
+constexpr uint8_t kBitsUnknown = 255;
+// float64 buckets whose key range has at least this many bits span 32 octaves
+constexpr uint8_t kRefineBits = 57;
 
 // Device-resident control block of one call.
 struct DevState {
   uint32_t nseg[2];         // segment lists (ping-pong by level parity)
-  uint32_t nfinal_c[kNumClasses];  // final items per size class
-  uint32_t cursor_c[kNumClasses];  // work counters of the in-SM sort kernels
+  uint32_t nfinal_c[kNumLists];  // final items per list
+  uint32_t cursor_c[kNumLists];  // work counters of the in-SM sort kernels
+  uint32_t cursor_rest;               // work counter of k_local_rest
   uint64_t class_elems[kNumClasses];  // elements handed to each size class
   uint64_t algo_elems[kNumAlgos];     // elements finished by each in-SM algorithm
   LocalPlan local;                    // the call's in-SM size classes and algorithms
@@ -198,6 +221,8 @@ struct LevelParams {
                           // small-footprint atomic-ranked kernel
   int bulk_classify = 0;  // 1: the id-storing classify stages its keys by
                           // bulk copies (16-byte aligned key arrays)
+  int refine = 0;         // 1: buckets of kRefineBits bits or more go to the
+                          // lists of buckets whose bins will need refining
 };
 
 // AMS-sort overpartitioning of a one-segment partition step: b*k fine
@@ -314,31 +339,36 @@ __device__ __forceinline__ void block_bitonic_sort(uint64_t* sk, uint32_t* si, i
 
 __host__ __device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
 
-// Appends a final bucket to the work list of its size class
-// (items holds kNumClasses lists of cap entries each).
+// Appends a final bucket to the work list of its size class (items holds
+// kNumLists lists of cap entries each); refine: to the class's list of buckets
+// whose bins will need refining, if the class is sorted by bins.
 __device__ __forceinline__ void push_final(DevState* st, FinalItem* items, uint64_t cap,
-                                           const FinalItem& f, uint32_t err_flag) {
+                                           const FinalItem& f, uint32_t err_flag,
+                                           bool refine = false) {
   const int cls = f.kind == kKindCopy ? kClassCopy
                   : f.kind == kKindBig ? kClassBig
                   : (f.size <= st->local.small_cap
                          ? kClassSmall
                          : (f.size <= st->local.mid_cap ? kClassMid : kClassMedium));
-  // one atomic per (warp, class): the lanes appending to the same list share it
+  // one atomic per (warp, list): the lanes appending to the same list share it
+  const int list = refine && cls >= kClassSmall && cls <= kClassMedium &&
+                           st->local.algo[cls - kClassSmall] == kLocalBins
+                       ? kListRefine + (cls - kClassSmall) : cls;
   const uint32_t act = __activemask();
-  const uint32_t peers = __match_any_sync(act, (uint32_t)cls);
+  const uint32_t peers = __match_any_sync(act, (uint32_t)list);
   const int leader = __ffs(peers) - 1;
   const int lane = threadIdx.x & 31;
   uint32_t base = 0;
   const uint32_t keys = __reduce_add_sync(peers, f.size);
   if (lane == leader) {
-    base = atomicAdd(&st->nfinal_c[cls], (uint32_t)__popc(peers));
+    base = atomicAdd(&st->nfinal_c[list], (uint32_t)__popc(peers));
     atomicAdd((unsigned long long*)&st->class_elems[cls], (unsigned long long)keys);
   }
   base = __shfl_sync(peers, base, leader);
   uint32_t lt;
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
   const uint32_t slot = base + __popc(peers & lt);
-  if (slot < cap) items[(uint64_t)cls * cap + slot] = f;
+  if (slot < cap) items[(uint64_t)list * cap + slot] = f;
   else atomicOr(&st->error, err_flag);
 }
 __host__ __device__ __forceinline__ uint64_t umax64(uint64_t a, uint64_t b) { return a > b ? a : b; }
@@ -386,7 +416,7 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
                   uint64_t n_total, int unmap_out, const Overpart* op = nullptr);
 void launch_init_segments(const LaunchEnv& e, DevState* st, const uint64_t* offsets,
                           uint32_t nseg, uint64_t n, SegIn* list_l1, FinalItem* items,
-                          uint64_t seg_cap, uint64_t final_cap);
+                          uint64_t seg_cap, uint64_t final_cap, int f64);
 void set_partition_kernel_attributes();
 // Binary-tree median approximation of n <= 2^24 keys (median_kernels.cu);
 // k in {2, 4, 8, 16, 32}.  Returns false for an unsupported k.
@@ -409,7 +439,14 @@ void launch_scatter_atomic(const LaunchEnv& e, const LevelParams& P, DevState* s
 void launch_scatter_units(const LaunchEnv& e, const LevelParams& P, DevState* st,
                           const LevelSeg* segs, Src src, const uint32_t* hist_scan, Dst dst,
                           uint32_t kmax, int unmap_out, const char* name);
-void launch_local_sort(const LaunchEnv& e, DevState* st, const FinalItem* items,
-                       uint64_t item_cap, const uint64_t* in_key, Dst out, Dst tmp, int f64);
+// max_items: upper bound on the call's final buckets; segmented: some of them
+// may be segments straight from the input.
+void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t item_cap,
+                       uint64_t max_items, const uint64_t* in_key, Dst out, Dst tmp, int f64,
+                       bool segmented);
+// A whole sort of n <= kBucketCap keys in one launch, control block included.
+void launch_direct_sort(const LaunchEnv& e, DevState* st, const uint64_t* in_key, Dst out,
+                        uint32_t n, int f64);
+bool direct_sort_takes(const LocalPlan& local, uint64_t n);
 
 }  // namespace rsort
