@@ -281,6 +281,7 @@ void set_attributes_once(int device) {
   set_partition_kernel_attributes();
   set_local_kernel_attributes();
   set_unit_scatter_attributes();
+  set_median_kernel_attributes();
   done.push_back(device);
 }
 

@@ -139,7 +139,7 @@ constexpr uint8_t kBitsUnknown = 255;
 constexpr uint8_t kRefineBits = 57;
 
 // Device-resident control block of one call.
-struct DevState {
+struct alignas(16) DevState {
   uint32_t nseg[2];         // segment lists (ping-pong by level parity)
   uint32_t nfinal_c[kNumLists];  // final items per list
   uint32_t cursor_c[kNumLists];  // work counters of the in-SM sort kernels
@@ -421,6 +421,7 @@ void set_partition_kernel_attributes();
 // Binary-tree median approximation of n <= 2^24 keys (median_kernels.cu);
 // k in {2, 4, 8, 16, 32}.  Returns false for an unsupported k.
 size_t tree_median_scratch_bytes(uint64_t n);
+void set_median_kernel_attributes();
 bool launch_tree_median(const LaunchEnv& e, const uint64_t* keys, uint32_t n, int f64,
                         uint32_t k, uint64_t seed, void* scratch, uint64_t* out_pos);
 void launch_plain_groups(const LaunchEnv& e, const uint64_t* offsets, uint32_t k,
