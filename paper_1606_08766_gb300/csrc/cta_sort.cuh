@@ -326,32 +326,48 @@ __device__ __forceinline__ void order_bins(uint32_t m, const BinShape& g, const 
 // The bins are refined once: bin b, whose c elements start at slot lo, is cut
 // into 2c equal parts numbered from 2 lo, so the 2m parts of all bins fit the
 // counters, are in key order, and follow the keys' density.  A key's part is
-// its offset in the bin times 2c over the bin's width 2^shift.  A part that is
-// crowded still (copies of a key, or keys in a cluster far narrower than a
-// bin) sends the bucket to the bitonic sort.  Returns the algorithm that
+// its offset in the bin times 2c over the bin's width 2^shift; where the bins
+// are one key wide (shift 0: copies of a few neighbouring keys) it is the
+// offset of its position in the range of all positions.  A part that is
+// crowded still (copies of keys far apart, or keys in a cluster far narrower
+// than a bin) sends the bucket to the bitonic sort.  Returns the algorithm that
 // finished.  Not inlined: it would cost the common path registers.
 //   One rsort_sort of 3001 normal float64 keys, by the bitonic network over
 //   shared memory and six launches: 90 us; with refined bins and one launch
 //   (k_direct_sort): 15 us.
 template <int NT, int ITEMS>
 __device__ __noinline__ int cta_sort_crowded(uint32_t m, uint64_t mn, int shift, CtaSortSmem s,
-                                             uint64_t* scan_sm) {
+                                             uint64_t* scan_sm, uint64_t* red) {
   const uint32_t tid = threadIdx.x;
-  if (shift > 0) {
+  {
     const BinShape g = bin_shape<NT>(m);
     __shared__ uint32_t s_nmulti;
     uint64_t key[ITEMS];
     uint32_t idx[ITEMS], bs[ITEMS];
+    uint64_t imn = ~0ULL, imx = 0;
 #pragma unroll
     for (int r = 0; r < ITEMS; ++r) {
       const uint32_t e = r * NT + tid;
       if (e < m) {
         key[r] = s.k[e];
         idx[r] = s.i[e];
+        imn = idx[r] < imn ? idx[r] : imn;
+        imx = idx[r] > imx ? idx[r] : imx;
+      }
+    }
+    int pshift = 0;  // positions' range in bits, when they order the parts
+    if (shift == 0) {
+      block_minmax_u64<NT>(imn, imx, red);
+      pshift = imx > imn ? 64 - __clzll((long long)(imx - imn)) : 1;
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      if (r * NT + tid < m) {
         const uint32_t b = (uint32_t)((key[r] - mn) >> shift);
         const uint32_t lo = bin_start(s.hist, b, g.lp);
         const uint32_t hi = b + 1 < g.nb ? bin_start(s.hist, b + 1, g.lp) : m;
-        const uint64_t off = (key[r] - mn) << (64 - shift);
+        const uint64_t off = shift ? (key[r] - mn) << (64 - shift)
+                                   : ((uint64_t)idx[r] - imn) << (64 - pshift);
         bs[r] = 2 * lo + (uint32_t)__umul64hi(off, (uint64_t)(2 * (hi - lo)));
       }
     }
@@ -496,7 +512,7 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
       if (e < m) { s.k[e] = key[r]; s.i[e] = idx[r]; }
     }
     __syncthreads();
-    const int how = cta_sort_crowded<NT, ITEMS>(m, mn, shift, s, scan_sm);
+    const int how = cta_sort_crowded<NT, ITEMS>(m, mn, shift, s, scan_sm, red);
     // (no register of the pairs is kept across the call)
 #pragma unroll
     for (int r = 0; r < ITEMS; ++r) {

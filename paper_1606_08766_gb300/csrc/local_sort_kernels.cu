@@ -252,7 +252,6 @@ k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
   __shared__ FinalItem s_f;
   __shared__ uint32_t s_nmulti;
   constexpr int kList = REFINE ? kListRefine + (CLS - kClassSmall) : CLS;
-  const FinalItem* list = items + (uint64_t)kList * cap;
   const uint32_t nitems = (uint32_t)umin64(st->nfinal_c[kList], cap);
   const uint32_t rank_max = min(st->local.rank_max, (uint32_t)NT);
   const uint32_t tid = threadIdx.x;
@@ -282,7 +281,7 @@ k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
   // (which starts at the grid's size)
   FinalItem f{};
   if (blockIdx.x < nitems) {
-    f = list[blockIdx.x];
+    f = items[item_slot(kList, blockIdx.x, cap)];
     load(f);
   }
   while (f.size) {
@@ -301,7 +300,7 @@ k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
         si[tid] = idx[0];
       }
       if (tid == 0) {
-        if (claim < nitems) fn = list[claim];
+        if (claim < nitems) fn = items[item_slot(kList, claim, cap)];
         s_f = fn;
         count_algo(st->algo_elems, kAlgoRank, m);
       }
@@ -351,7 +350,7 @@ k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
           const uint32_t old = atomicAdd(&hist[h >> 1], 1u << sh);
           hr[r] = (h << 16) | ((old >> sh) & 0xffffu);
         });
-        if (tid == 0 && pass == 0 && claim < nitems) fn = list[claim];
+        if (tid == 0 && pass == 0 && claim < nitems) fn = items[item_slot(kList, claim, cap)];
         __syncthreads();  // (2) counts complete
         uint32_t sum = 0, any = 0;
 #pragma unroll
@@ -419,7 +418,7 @@ k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
         // crowded: the bucket goes to k_local_rest's list
         if (tid == 0) {
           const uint32_t slot = atomicAdd(&st->nfinal_c[kListCrowd], 1u);
-          if (slot < cap) items[(uint64_t)kListCrowd * cap + slot] = f;
+          if (slot < cap) items[item_slot(kListCrowd, slot, cap)] = f;
           else atomicOr(&st->error, kErrFinalCap);
         }
         __syncthreads();
@@ -562,7 +561,7 @@ k_local_rest(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, uint32_
         from = end[q];
       }
     }
-    const FinalItem f = items[(uint64_t)l * cap + (at - from)];
+    const FinalItem f = items[item_slot(l, at - from, cap)];
     if (threadIdx.x == 0) s_next = gridDim.x + atomicAdd(&st->cursor_rest, 1u);
     if (l == kClassCopy) {
       if (f.where != kWhereOut || B.f64) {  // else already in place

@@ -120,6 +120,7 @@ extern "C" rsort_status rsort_partition_noalloc(rsort_key_type type, const void*
   P.schunk_cap = samp / kSampleChunk + 2;
   P.bucket_cap = kk;
   P.level1_oversample = 1;
+  P.hinted = 1;
   P.classifier = 0;
   P.warp_direct = 0;
   P.wide_scatter_k = 1 << 30;  // always the 2048-key sub-tile scatter
@@ -151,12 +152,11 @@ extern "C" rsort_status rsort_partition_noalloc(rsort_key_type type, const void*
   e.launches = nullptr;
   // The control block is reset by the first kernel; every other scratch word
   // read later is written earlier in the same call.
-  launch_init_plain(e, st, list1, items, n, k, 0, 1);
   Src src{(const uint64_t*)d_keys_in, nullptr, type == RSORT_KEY_F64};
   Dst dst{(uint64_t*)d_keys_out, d_pos_out};
   launch_level(e, P, st, list1, list0, segs, src, dst, kWhereOut, samp_key, samp_idx, ssamp_key,
                ssamp_idx, hist_arr, sums, items, (int)kk, 1, 0, d_offsets_out, n,
-               type == RSORT_KEY_F64);
+               type == RSORT_KEY_F64, nullptr, k, nullptr);
   if (cudaGetLastError() != cudaSuccess) return RSORT_ECUDA;
   return RSORT_OK;
 }

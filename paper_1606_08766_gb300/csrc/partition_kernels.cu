@@ -2,7 +2,7 @@
 // (Appendix "Robust Multi-Level Sample Sort" of Axtmann & Sanders,
 // arXiv 1606.08766) over a device-resident list of segments:
 //
-//   plan -> sample -> sort the sample -> classify + per-chunk histograms ->
+//   plan -> sample and sort the sample -> classify + per-chunk histograms ->
 //   exclusive scan -> scatter -> collect the buckets
 //
 // The scatter keeps input order inside every bucket (the partition step's
@@ -16,6 +16,7 @@
 // segment are its k virtual partitions, and the MPI_Alltoallv data exchange of
 // the paper's sample sort becomes the scan + scatter through HBM.
 #include <cstdio>
+#include <type_traits>
 
 #include "async_copy.cuh"
 #include "cta_sort.cuh"
@@ -41,9 +42,8 @@ struct Scope {
 // Kernels
 // ---------------------------------------------------------------------------
 
-__global__ void k_init_plain(DevState* st, SegIn* list_l1, FinalItem* items, uint64_t n,
-                             uint32_t k1, int direct, uint64_t final_cap, LocalPlan local) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Control block of a call, before its first level.
+__device__ __forceinline__ void reset_state(DevState* st, const LocalPlan& local) {
   st->local = local;
   st->nseg[0] = st->nseg[1] = 0;
   for (int c = 0; c < kNumLists; ++c) {
@@ -61,198 +61,287 @@ __global__ void k_init_plain(DevState* st, SegIn* list_l1, FinalItem* items, uin
   st->total_schunks = st->total_buckets = 0;
   st->big_items = 0;
   for (int i = 0; i < 4; ++i) st->level_elems[i] = 0;
+  st->l1_eq = st->l1_nb = st->l1_ordered = 0;
+}
+
+// Start of a call on a list of segments (n == 0), or of a sort of n keys that
+// one CTA sorts.
+__global__ void k_init_plain(DevState* st, FinalItem* items, uint64_t n, uint64_t final_cap,
+                             LocalPlan local) {
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  reset_state(st, local);
   if (n == 0) return;
-  if (direct) {
-    FinalItem f;
-    f.start = 0;
-    f.aux = 0;
-    f.size = (uint32_t)n;
-    f.where = kWhereInput;
-    f.kind = n == 1 ? kKindCopy : kKindSort;
-    f.bits = kBitsUnknown;
-    push_final(st, items, final_cap, f, kErrFinalCap);
+  FinalItem f;
+  f.start = 0;
+  f.aux = 0;
+  f.size = (uint32_t)n;
+  f.where = kWhereInput;
+  f.kind = n == 1 ? kKindCopy : kKindSort;
+  f.bits = kBitsUnknown;
+  push_final(st, items, final_cap, f, kErrFinalCap);
+}
+
+// Buckets and samples of a segment of m elements (in k: its bucket count).
+__device__ __forceinline__ uint32_t segment_samples(uint32_t m, uint32_t k, bool hinted,
+                                                    const LevelParams& P) {
+  const uint64_t a = hinted && P.level1_oversample ? 16ull * ceil_log2_dev(k)
+                                                   : (uint64_t)kDeepOversample;
+  return (uint32_t)umin64(umin64(m, a * k), P.samp_max);
+}
+
+__device__ __forceinline__ void fill_segment(LevelSeg& s, uint64_t start, uint32_t m, uint32_t k,
+                                             uint32_t S, uint32_t nch, const LevelParams& P,
+                                             const KeyRange& range) {
+  s.start = start;
+  s.seed = P.level == 1 ? P.seed : splitmix64_at(P.seed, ((uint64_t)P.level << 40) ^ start);
+  s.m = m;
+  s.k = k;
+  s.S = S;
+  s.nchunks = nch;
+  s.nschunks = (S + kSampleChunk - 1) / kSampleChunk;
+  s.nunits = nch * (P.warp_direct ? kPartWarps : 1);
+  // equal chunks inside the segment (the level's W bounds their size)
+  s.W = nch ? (uint32_t)(((uint64_t)m + nch - 1) / nch) : P.W;
+  s.pad = 0;
+  s.range = range;
+}
+
+// Per-segment parameters and prefix sums of one level.  CTA t takes segments
+// [t, t + 1) * kPlanThreads.  With one CTA k_level_plan does everything; a level
+// that may have more segments runs k_plan_sums first, which leaves every CTA's
+// six sums in plan_sums, and each CTA of k_level_plan adds up those before its
+// own (33,000 segments: one CTA in a loop over tiles 197 us, a run of segments
+// per thread 256, the two launches 30).
+constexpr int kPlanThreads = 1024;
+
+// Samples, chunks, histogram counters, sample chunks, buckets and elements of
+// segment g of list_in (zeros past the end).
+__device__ __forceinline__ SegIn plan_shape(const SegIn* list_in, uint32_t g, uint32_t G,
+                                            const LevelParams& P, uint32_t kmax_level,
+                                            uint64_t (&v)[6]) {
+  SegIn in{};
+#pragma unroll
+  for (int i = 0; i < 6; ++i) v[i] = 0;
+  if (g >= G) return in;
+  in = list_in[g];
+  uint32_t k;
+  if (in.k_hint >= 1) {
+    k = min(in.k_hint, kmax_level);
   } else {
-    SegIn s;
-    s.start = 0;
-    s.m = (uint32_t)n;
-    s.k_hint = k1;
-    s.range = KeyRange{0, ~0ULL, 0, 0};
-    list_l1[0] = s;
-    st->nseg[1] = 1;  // level 1 reads list parity 1
+    const uint32_t cls = ceil_log2_dev(in.m);
+    const uint32_t tb = (cls <= 32 && P.target_by_class[cls]) ? P.target_by_class[cls]
+                                                              : P.target_bucket;
+    const uint32_t want = in.m / tb + (in.m % tb ? 1u : 0u);
+    k = max(2u, min(want, kmax_level));
+  }
+  const uint32_t S = segment_samples(in.m, k, in.k_hint >= 1, P);
+  const uint32_t nch = in.m / P.W + (in.m % P.W ? 1u : 0u);
+  v[0] = S;
+  v[1] = nch;
+  v[2] = (uint64_t)k * nch * (P.warp_direct ? kPartWarps : 1);
+  v[3] = (S + kSampleChunk - 1) / kSampleChunk;
+  v[4] = k;
+  v[5] = in.m;
+  return in;
+}
+
+__global__ void __launch_bounds__(kPlanThreads)
+k_plan_sums(const DevState* st, const SegIn* list_in, LevelParams P, int par_in,
+            uint32_t kmax_level, uint64_t* plan_sums) {
+  __shared__ uint64_t sm[kPlanThreads / 32];
+  const uint32_t G = st->nseg[par_in];
+  if (G > P.seg_cap || (uint64_t)blockIdx.x * kPlanThreads >= G) return;
+  uint64_t v[6];
+  plan_shape(list_in, blockIdx.x * kPlanThreads + threadIdx.x, G, P, kmax_level, v);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    uint64_t tot;
+    block_excl_scan_u64<kPlanThreads>(v[i], &tot, sm);
+    if (threadIdx.x == 0) plan_sums[blockIdx.x * 6 + i] = tot;
   }
 }
 
-// Per-segment parameters and prefix sums of one level (one CTA).
-constexpr int kPlanThreads = 1024;
 __global__ void __launch_bounds__(kPlanThreads)
 k_level_plan(DevState* st, const SegIn* list_in, LevelSeg* segs, LevelParams P, int par_in,
-             uint32_t kmax_level) {
+             uint32_t kmax_level, const uint64_t* plan_sums, uint32_t* chunk_seg) {
   __shared__ uint64_t sm[kPlanThreads / 32];
-  __shared__ uint64_t carry[6];
-  __shared__ uint32_t sG;
-  if (threadIdx.x == 0) {
-    uint32_t G = st->nseg[par_in];
-    st->nseg[par_in ^ 1] = 0;
-    if (G > P.seg_cap) {
-      atomicOr(&st->error, kErrSegCap);
-      G = 0;
+  const uint32_t G0 = st->nseg[par_in];
+  const bool over = G0 > P.seg_cap;
+  const uint32_t G = over ? 0u : G0;
+  const uint32_t ncta = max(1u, (G + kPlanThreads - 1) / kPlanThreads);
+  const uint32_t t = blockIdx.x;
+  if (t >= ncta) return;
+  uint64_t before[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    uint64_t x = 0;
+    for (uint32_t q = threadIdx.x; q < t; q += kPlanThreads) x += plan_sums[q * 6 + i];
+    before[i] = 0;
+    if (t > 0) block_excl_scan_u64<kPlanThreads>(x, &before[i], sm);
+  }
+  const uint32_t g = t * kPlanThreads + threadIdx.x;
+  uint64_t v[6], ex[6], tot[6];
+  const SegIn in = plan_shape(list_in, g, G, P, kmax_level, v);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    ex[i] = before[i] + block_excl_scan_u64<kPlanThreads>(v[i], &tot[i], sm);
+    tot[i] += before[i];
+  }
+  // (every CTA's totals up to its own tile: beyond a capacity, the last CTA's
+  // check fails too and the level is not run)
+  uint32_t err = 0;
+  if (tot[0] > P.samp_cap) err |= kErrSampleCap;
+  if (tot[1] > P.chunk_cap) err |= kErrChunkCap;
+  if (tot[2] > P.hist_cap) err |= kErrHistCap;
+  if (tot[3] > P.schunk_cap) err |= kErrSchunkCap;
+  if (tot[4] > P.bucket_cap) err |= kErrBucketCap;
+  if (g < G) {
+    LevelSeg s;
+    fill_segment(s, in.start, in.m, (uint32_t)v[4], (uint32_t)v[0], (uint32_t)v[1], P, in.range);
+    s.samp_off = ex[0];
+    s.chunk_off = ex[1];
+    s.hist_off = ex[2];
+    s.schunk_off = ex[3];
+    s.bkt_off = ex[4];
+    s.delta = in.start - ex[5];
+    segs[g] = s;
+  }
+  if (err == 0) {
+    // the segment of every chunk: a thread its segment's few, a warp the many
+    const uint32_t nch = (uint32_t)v[1];
+    const bool many = nch > 8;
+    if (!many)
+      for (uint32_t c = 0; c < nch; ++c) chunk_seg[ex[1] + c] = g;
+    uint32_t left = __ballot_sync(0xffffffffu, many);
+    while (left) {
+      const int l = __ffs(left) - 1;
+      left &= left - 1;
+      const uint64_t c0 = __shfl_sync(0xffffffffu, ex[1], l);
+      const uint32_t n = __shfl_sync(0xffffffffu, nch, l);
+      const uint32_t gl = __shfl_sync(0xffffffffu, g, l);
+      for (uint32_t c = threadIdx.x & 31; c < n; c += 32) chunk_seg[c0 + c] = gl;
     }
+  }
+  if (threadIdx.x != 0 || t + 1 != ncta) return;
+  st->nseg[par_in ^ 1] = 0;
+  if (over) err |= kErrSegCap;
+  if (err) {
+    atomicOr(&st->error, err);
+    st->cur_nseg = 0;
+    st->total_samples = st->total_chunks = st->total_hist = 0;
+    st->total_schunks = st->total_buckets = 0;
+  } else {
+    st->cur_nseg = G;
+    st->total_samples = tot[0];
+    st->total_chunks = tot[1];
+    st->total_hist = tot[2];
+    st->total_schunks = tot[3];
+    st->total_buckets = tot[4];
     if (G) st->levels_used = P.level;
-    if (P.level == 1) {
-      st->l1_eq = 0;
-      st->l1_nb = 0;
-      st->l1_ordered = 0;
-    }
-    sG = G;
-    for (int i = 0; i < 6; ++i) carry[i] = 0;
-  }
-  __syncthreads();
-  const uint32_t G = sG;
-  for (uint32_t base = 0; base < G; base += kPlanThreads) {
-    const uint32_t g = base + threadIdx.x;
-    uint64_t v[6] = {0, 0, 0, 0, 0, 0};
-    SegIn in{};
-    uint32_t k = 0, S = 0, nch = 0, nsch = 0;
-    if (g < G) {
-      in = list_in[g];
-      if (in.k_hint >= 1) {
-        k = min(in.k_hint, kmax_level);
-      } else {
-        const uint32_t cls = ceil_log2_dev(in.m);
-        const uint32_t tb = (cls <= 32 && P.target_by_class[cls]) ? P.target_by_class[cls]
-                                                                  : P.target_bucket;
-        const uint64_t want = ((uint64_t)in.m + tb - 1) / tb;
-        k = (uint32_t)umax64(2, umin64(want, kmax_level));
-      }
-      const uint64_t a = (in.k_hint >= 1 && P.level1_oversample)
-                             ? 16ull * ceil_log2_dev(k) : (uint64_t)kDeepOversample;
-      S = (uint32_t)umin64(in.m, a * k);
-      nch = (uint32_t)((in.m + (uint64_t)P.W - 1) / P.W);
-      nsch = (S + kSampleChunk - 1) / kSampleChunk;
-      v[0] = S;
-      v[1] = nch;
-      v[2] = (uint64_t)k * nch * (P.warp_direct ? kPartWarps : 1);
-      v[3] = nsch;
-      v[4] = k;
-      v[5] = in.m;
-    }
-    uint64_t ex[6], tot[6];
-    for (int i = 0; i < 6; ++i) ex[i] = block_excl_scan_u64<kPlanThreads>(v[i], &tot[i], sm);
-    if (g < G) {
-      LevelSeg s;
-      s.start = in.start;
-      s.seed = P.level == 1 ? P.seed
-                            : splitmix64_at(P.seed, ((uint64_t)P.level << 40) ^ in.start);
-      s.samp_off = carry[0] + ex[0];
-      s.chunk_off = carry[1] + ex[1];
-      s.hist_off = carry[2] + ex[2];
-      s.schunk_off = carry[3] + ex[3];
-      s.bkt_off = carry[4] + ex[4];
-      s.delta = in.start - (carry[5] + ex[5]);
-      s.m = in.m;
-      s.k = k;
-      s.S = S;
-      s.nchunks = nch;
-      s.nschunks = nsch;
-      s.nunits = nch * (P.warp_direct ? kPartWarps : 1);
-      // equal chunks inside the segment (the level's W bounds their size)
-      s.W = nch ? (uint32_t)(((uint64_t)in.m + nch - 1) / nch) : P.W;
-      s.pad = 0;
-      s.range = in.range;
-      segs[g] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0)
-      for (int i = 0; i < 6; ++i) carry[i] += tot[i];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    uint32_t err = 0;
-    if (carry[0] > P.samp_cap) err |= kErrSampleCap;
-    if (carry[1] > P.chunk_cap) err |= kErrChunkCap;
-    if (carry[2] > P.hist_cap) err |= kErrHistCap;
-    if (carry[3] > P.schunk_cap) err |= kErrSchunkCap;
-    if (carry[4] > P.bucket_cap) err |= kErrBucketCap;
-    if (err) {
-      atomicOr(&st->error, err);
-      st->cur_nseg = 0;
-      st->total_samples = st->total_chunks = st->total_hist = 0;
-      st->total_schunks = st->total_buckets = 0;
-    } else {
-      st->cur_nseg = G;
-      st->total_samples = carry[0];
-      st->total_chunks = carry[1];
-      st->total_hist = carry[2];
-      st->total_schunks = carry[3];
-      st->total_buckets = carry[4];
-      if (P.level >= 1 && P.level <= 4) st->level_elems[P.level - 1] = carry[5];
-    }
+    if (P.level == 1) st->l1_nb = (uint32_t)umin64(tot[4], 0xffffffffull);
+    if (P.level >= 1 && P.level <= 4) st->level_elems[P.level - 1] = tot[5];
   }
 }
 
-// Step 1: stratified random samples, each carrying its position.  Sample j of
-// a segment of m elements with S samples comes from positions
-// [floor(j*m/S), floor((j+1)*m/S)) at offset splitmix64(seed, j) mod size.
-__global__ void __launch_bounds__(256)
-k_sample(const DevState* st, const LevelSeg* segs, Src src, uint64_t* samp_key,
-         uint32_t* samp_idx) {
-  const uint64_t total = st->total_samples;
-  const uint32_t G = st->cur_nseg;
-  // every CTA draws a contiguous range of samples, so a thread's segment
-  // changes rarely and the segment search runs once per segment, not per sample
-  const uint64_t span = (total + gridDim.x - 1) / gridDim.x;
-  const uint64_t s0 = (uint64_t)blockIdx.x * span;
-  const uint64_t s1 = umin64(total, s0 + span);
-  uint32_t g = 0;
-  uint64_t g_lo = 1, g_hi = 0;  // sample range of the cached segment (empty)
-  for (uint64_t s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
-    if (s < g_lo || s >= g_hi) {
-      g = find_seg(segs, G, s, [](const LevelSeg& x) { return x.samp_off; });
-      g_lo = segs[g].samp_off;
-      g_hi = g_lo + segs[g].S;
-    }
-    const LevelSeg& sg = segs[g];
-    const uint64_t j = s - sg.samp_off;
-    const uint64_t lo = (j * sg.m) / sg.S, hi = ((j + 1) * sg.m) / sg.S;
-    const uint64_t pos = lo + splitmix64_at(sg.seed, j) % (hi - lo);
-    const uint64_t at = sg.start + pos;
-    samp_key[s] = load_key(src, at);
-    samp_idx[s] = src.idx ? src.idx[at] : (uint32_t)pos;
+// Sample positions of a segment of m elements with S samples: sample j comes
+// from positions [floor(j*m/S), floor((j+1)*m/S)) at offset splitmix64(seed, j)
+// mod size.  The quotients need no 64-bit division per sample: with m = q S + r,
+// floor(j*m/S) = j q + floor(j r / S), and j r < S^2 is divided by a multiply
+// with ceil(2^64 / S) (exact while S < 2^21: j r S < 2^63); a stratum holds q
+// or q + 1 positions, whose remainders come from a multiply with
+// floor((2^64 - 1) / size), at most two too small.
+struct SampleDraw {
+  uint64_t inv, magic0, magic1, seed;
+  uint32_t q, r, S;
+  __device__ __forceinline__ SampleDraw(uint32_t m, uint32_t S_, uint64_t seed_)
+      : seed(seed_), S(S_) {
+    q = m / S;
+    r = m - q * S;
+    inv = ~0ULL / S + 1;  // (S = 1 wraps to 0: r is 0 then)
+    magic0 = ~0ULL / q;   // q >= 1 (S <= m)
+    magic1 = ~0ULL / (q + 1);
   }
-}
+  __device__ __forceinline__ uint32_t position(uint32_t j) const {
+    const uint64_t x = (uint64_t)j * r;
+    const uint32_t f0 = (uint32_t)__umul64hi(x, inv);
+    const uint32_t f1 = (uint32_t)__umul64hi(x + r, inv);
+    const uint32_t size = q + (f1 - f0);
+    const uint64_t z = splitmix64_at(seed, j);
+    uint64_t rem = z - __umul64hi(z, f1 != f0 ? magic1 : magic0) * size;
+    if (rem >= size) rem -= size;
+    if (rem >= size) rem -= size;
+    return j * q + f0 + (uint32_t)rem;
+  }
+};
+static_assert(16u * 11 * kMaxK < (1u << 21), "sample counts the exact division covers");
 
-// Step 2a: sort chunks of up to kSampleChunk sample pairs in one CTA each
-// (cta_sort_pairs).  Single-chunk samples go straight to the sorted-sample
-// array.  Samples are drawn in segment order, which is position order when
-// the segment's level input is (in_order).
-__global__ void __launch_bounds__(kSampleThreads, 1)
-k_sample_sort_chunks(const DevState* st, const LevelSeg* segs, uint64_t* samp_key,
-                     uint32_t* samp_idx, uint64_t* ssamp_key, uint32_t* ssamp_idx,
-                     int in_order) {
-  constexpr int NT = kSampleThreads, IT = kSampleChunk / kSampleThreads;
+// Start of a one-segment call, made by the first launch itself (n == 0: the
+// level's segments come from its plan).
+struct PlainStart {
+  uint64_t n = 0;
+  uint32_t k = 0;     // buckets
+  uint32_t S = 0;     // samples
+  uint32_t nch = 0;   // chunks
+  LocalPlan local;
+};
+
+// Steps 1 and 2a: stratified random samples, each carrying its position, drawn
+// straight into the registers of the CTA that sorts them.  Sample chunk c of
+// nschunks takes samples c, c + nschunks, ...: every chunk represents the whole
+// segment (the merge below takes its ranges from one chunk), in position order
+// when the segment's level input is (in_order).  A segment with one chunk is
+// done here.  Serves the chunks of more than min_len samples.  A one-segment
+// call's control block and segment are written here too.
+template <int NT, int IT, int MINB>
+__global__ void __launch_bounds__(NT, MINB)
+k_sample_sort(DevState* st, LevelSeg* segs, Src src, uint64_t* samp_key, uint32_t* samp_idx,
+              uint64_t* ssamp_key, uint32_t* ssamp_idx, int in_order, uint32_t min_len,
+              PlainStart ps, LevelParams P) {
+  constexpr uint32_t kCap = NT * IT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CtaSortSmem s;
   s.k = (uint64_t*)smem_raw;
-  s.i = (uint32_t*)(s.k + kSampleChunk);
-  s.hist = s.i + kSampleChunk;
+  s.i = (uint32_t*)(s.k + kCap);
+  s.hist = s.i + kCap;
   __shared__ uint64_t red[2 * NT / 32];
   __shared__ uint64_t scan_sm[NT / 32];
-  const uint64_t total = st->total_schunks;
-  const uint32_t G = st->cur_nseg;
+  LevelSeg sg;
+  if (ps.n) {
+    fill_segment(sg, 0, (uint32_t)ps.n, ps.k, ps.S, ps.nch, P, KeyRange{0, ~0ULL, 0, 0});
+    sg.samp_off = sg.chunk_off = sg.hist_off = sg.schunk_off = sg.bkt_off = sg.delta = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      reset_state(st, ps.local);
+      segs[0] = sg;
+      st->levels_used = P.level;
+      st->cur_nseg = 1;
+      st->total_samples = sg.S;
+      st->total_chunks = sg.nchunks;
+      st->total_hist = (uint64_t)sg.k * sg.nunits;
+      st->total_schunks = sg.nschunks;
+      st->total_buckets = sg.k;
+      st->l1_nb = sg.k;
+      st->level_elems[0] = sg.m;
+    }
+  }
+  const uint64_t total = ps.n ? sg.nschunks : st->total_schunks;
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = find_seg(segs, G, c, [](const LevelSeg& x) { return x.schunk_off; });
-    const LevelSeg sg = segs[g];
-    const uint64_t cl = c - sg.schunk_off;
-    const uint64_t base = sg.samp_off + cl * kSampleChunk;
-    const uint32_t len = (uint32_t)umin64(kSampleChunk, sg.S - cl * kSampleChunk);
+    if (!ps.n) sg = segs[c];  // (one sample chunk a segment)
+    const uint32_t cl = (uint32_t)(c - sg.schunk_off);
+    const uint32_t each = sg.S / sg.nschunks, more = sg.S % sg.nschunks;
+    const uint32_t len = each + (cl < more ? 1u : 0u);
+    if (len <= min_len || len > kCap) continue;
+    const uint64_t base = sg.samp_off + (uint64_t)cl * each + min(cl, more);
+    const SampleDraw draw(sg.m, sg.S, sg.seed);
     uint64_t key[IT];
     uint32_t idx[IT];
 #pragma unroll
     for (int r = 0; r < IT; ++r) {
       const uint32_t e = r * NT + threadIdx.x;
       if (e < len) {
-        key[r] = samp_key[base + e];
-        idx[r] = samp_idx[base + e];
+        const uint32_t pos = draw.position(cl + e * sg.nschunks);
+        const uint64_t at = sg.start + pos;
+        key[r] = load_key(src, at);
+        idx[r] = src.idx ? src.idx[at] : pos;
       }
     }
     cta_sort_pairs<NT, IT>(key, idx, len,
@@ -269,48 +358,113 @@ k_sample_sort_chunks(const DevState* st, const LevelSeg* segs, uint64_t* samp_ke
   }
 }
 
-// Step 2b: merge sorted chunks by ranking (the fast work-inefficient ranking
-// idea of Appendix "Fast Work-Inefficient Ranking": the rank of an element is
-// its rank in its own sorted sequence plus its ranks in the other sorted
-// sequences).
-__global__ void __launch_bounds__(256)
-k_sample_merge_rank(const DevState* st, const LevelSeg* segs, const uint64_t* samp_key,
-                    const uint32_t* samp_idx, uint64_t* ssamp_key, uint32_t* ssamp_idx) {
-  const uint64_t total = st->total_samples;
-  const uint32_t G = st->cur_nseg;
-  // contiguous sample range per CTA, segment searched once per segment
-  const uint64_t span = (total + gridDim.x - 1) / gridDim.x;
-  const uint64_t s0 = (uint64_t)blockIdx.x * span;
-  const uint64_t s1 = umin64(total, s0 + span);
-  uint32_t g = 0;
-  uint64_t g_lo = 1, g_hi = 0;
-  for (uint64_t s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
-    if (s < g_lo || s >= g_hi) {
-      g = find_seg(segs, G, s, [](const LevelSeg& x) { return x.samp_off; });
-      g_lo = segs[g].samp_off;
-      g_hi = g_lo + segs[g].S;
+// Step 2b: merge the sorted chunks of a one-segment level.  CTA i takes the
+// pairs between two quantiles of chunk 0 (chunks are alike, so about S/gridDim
+// pairs): a binary search per chunk finds their runs, the sum of the runs'
+// starts is their place in the sorted sample (the rank of an element is its
+// rank in its own sorted sequence plus its ranks in the others, Appendix "Fast
+// Work-Inefficient Ranking"), and the CTA sorts them in shared memory.  A range
+// that does not fit is placed pair by pair by its ranks.
+//   163,840 samples in 20 chunks: ranking every pair in every other chunk
+//   81 us, this form 19 us.
+constexpr int kMergeThreads = 512;
+constexpr int kMergeItems = 8;
+constexpr uint32_t kMergeRange = 1024;   // pairs a CTA is given on average
+constexpr uint32_t kMaxSampleChunks = 64;
+static_assert(16u * 11 * kMaxK <= kMaxSampleChunks * kSampleChunk, "a run per sample chunk");
+__global__ void __launch_bounds__(kMergeThreads, 2)
+k_sample_merge(const LevelSeg* segs, const uint64_t* samp_key, const uint32_t* samp_idx,
+               uint64_t* ssamp_key, uint32_t* ssamp_idx) {
+  constexpr int NT = kMergeThreads, IT = kMergeItems;
+  constexpr uint32_t kCap = NT * IT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  CtaSortSmem s;
+  s.k = (uint64_t*)smem_raw;
+  s.i = (uint32_t*)(s.k + kCap);
+  s.hist = s.i + kCap;
+  __shared__ uint64_t red[2 * NT / 32];
+  __shared__ uint64_t scan_sm[NT / 32];
+  __shared__ uint32_t s_lo[kMaxSampleChunks];       // first pair of every chunk's run
+  __shared__ uint32_t s_at[kMaxSampleChunks + 1];   // runs' starts in the range
+  const LevelSeg& sg = segs[0];
+  const uint32_t nch = sg.nschunks, S = sg.S, tid = threadIdx.x;
+  const uint32_t each = S / nch, more = S % nch;
+  auto chunk_len = [&](uint32_t c) { return each + (c < more ? 1u : 0u); };
+  auto chunk_at = [&](uint32_t c) { return sg.samp_off + (uint64_t)c * each + min(c, more); };
+  // pairs of chunk c below the pair (k, i)
+  auto rank_in = [&](uint32_t c, uint64_t k, uint32_t i) {
+    const uint64_t b = chunk_at(c);
+    uint32_t lo = 0, hi = chunk_len(c);
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi) >> 1;
+      const uint64_t km = samp_key[b + mid];
+      if (km < k || (km == k && samp_idx[b + mid] < i)) lo = mid + 1;
+      else hi = mid;
     }
-    const LevelSeg& sg = segs[g];
-    if (sg.nschunks <= 1) continue;
-    const uint64_t j = s - sg.samp_off;
-    const uint32_t c = (uint32_t)(j / kSampleChunk);
-    const uint64_t myk = samp_key[s];
-    const uint32_t myi = samp_idx[s];
-    uint64_t rank = j - (uint64_t)c * kSampleChunk;
-    for (uint32_t c2 = 0; c2 < sg.nschunks; ++c2) {
-      if (c2 == c) continue;
-      const uint64_t b0 = sg.samp_off + (uint64_t)c2 * kSampleChunk;
-      const uint64_t len = umin64(kSampleChunk, sg.S - (uint64_t)c2 * kSampleChunk);
-      uint64_t lo = 0, hi = len;
-      while (lo < hi) {
-        const uint64_t mid = (lo + hi) >> 1;
-        if (pair_less(samp_key[b0 + mid], samp_idx[b0 + mid], myk, myi)) lo = mid + 1;
-        else hi = mid;
-      }
-      rank += lo;
+    return lo;
+  };
+  const uint32_t l0 = chunk_len(0);
+  const uint32_t q0 = (uint32_t)(((uint64_t)blockIdx.x * l0) / gridDim.x);
+  const uint32_t q1 = (uint32_t)(((uint64_t)(blockIdx.x + 1) * l0) / gridDim.x);
+  const bool last = blockIdx.x + 1 == gridDim.x;
+  if (tid < 2 * nch) {  // both ends of every run at once
+    const uint32_t c = tid >> 1, q = tid & 1 ? q1 : q0;
+    uint32_t r;
+    if (tid & 1 ? last : blockIdx.x == 0) r = tid & 1 ? chunk_len(c) : 0u;
+    else r = rank_in(c, samp_key[chunk_at(0) + q], samp_idx[chunk_at(0) + q]);
+    if (tid & 1) s_at[c + 1] = r;
+    else s_lo[c] = r;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    uint32_t run = 0;
+    s_at[0] = 0;
+    for (uint32_t c = 0; c < nch; ++c) {
+      run += s_at[c + 1] - s_lo[c];
+      s_at[c + 1] = run;
     }
-    ssamp_key[sg.samp_off + rank] = myk;
-    ssamp_idx[sg.samp_off + rank] = myi;
+  }
+  __syncthreads();
+  const uint32_t cnt = s_at[nch];
+  uint64_t out = sg.samp_off;
+  for (uint32_t c = 0; c < nch; ++c) out += s_lo[c];
+  auto source = [&](uint32_t e) {  // slot of the range's pair e
+    uint32_t lo = 0, hi = nch;
+    while (hi - lo > 1) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if (s_at[mid] <= e) lo = mid;
+      else hi = mid;
+    }
+    return chunk_at(lo) + s_lo[lo] + (e - s_at[lo]);
+  };
+  if (cnt == 0) return;
+  if (cnt > kCap) {
+    for (uint32_t e = tid; e < cnt; e += NT) {
+      const uint64_t at = source(e);
+      const uint64_t k = samp_key[at];
+      const uint32_t i = samp_idx[at];
+      uint64_t r = sg.samp_off;
+      for (uint32_t c = 0; c < nch; ++c) r += rank_in(c, k, i);
+      ssamp_key[r] = k;
+      ssamp_idx[r] = i;
+    }
+    return;
+  }
+  uint64_t key[IT];
+  uint32_t idx[IT];
+#pragma unroll
+  for (int r = 0; r < IT; ++r) {
+    const uint32_t e = r * NT + tid;
+    if (e < cnt) {
+      const uint64_t at = source(e);
+      key[r] = samp_key[at];
+      idx[r] = samp_idx[at];
+    }
+  }
+  cta_sort_pairs<NT, IT>(key, idx, cnt, [] { return false; }, s, red, scan_sm, nullptr);
+  for (uint32_t t = tid; t < cnt; t += NT) {
+    ssamp_key[out + t] = s.k[t];
+    ssamp_idx[out + t] = s.i[t];
   }
 }
 
@@ -451,7 +605,7 @@ k_classify_count(const DevState* st, const LevelSeg* segs, Src src, const uint64
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t cur_g = 0xffffffffu;
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = find_seg(segs, G, c, [](const LevelSeg& x) { return x.chunk_off; });
+    const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
     const LevelSeg sg = segs[g];
     __syncthreads();
     if (g != cur_g) {
@@ -533,7 +687,9 @@ k_classify_count(const DevState* st, const LevelSeg* segs, Src src, const uint64
   }
 }
 
-// Step 5b: exclusive scan of the histogram counters (three launches).
+// Step 5b: exclusive scan of the histogram counters: sums of tiles of
+// kScanTile, then every CTA adds up the sums before its tile (a few thousand
+// words at most) and scans the tile.
 __global__ void __launch_bounds__(1024)
 k_scan_reduce(const DevState* st, const uint32_t* a, uint32_t* sums) {
   __shared__ uint64_t sm[32];
@@ -550,28 +706,9 @@ k_scan_reduce(const DevState* st, const uint32_t* a, uint32_t* sums) {
   if (threadIdx.x == 0) sums[blockIdx.x] = (uint32_t)tot;
 }
 
-__global__ void __launch_bounds__(1024)
-k_scan_sums(const DevState* st, uint32_t* sums) {
-  __shared__ uint64_t sm[32];
-  const uint64_t total = st->total_hist;
-  const uint64_t ntiles = (total + kScanTile - 1) / kScanTile;
-  uint64_t carry = 0;
-  for (uint64_t b = 0; b < ntiles; b += 1024) {
-    const uint64_t i = b + threadIdx.x;
-    const uint64_t v = i < ntiles ? sums[i] : 0;
-    uint64_t tot;
-    const uint64_t ex = block_excl_scan_u64<1024>(v, &tot, sm);
-    if (i < ntiles) sums[i] = (uint32_t)(carry + ex);
-    carry += tot;
-  }
-}
-
-__global__ void __launch_bounds__(1024)
-k_scan_down(const DevState* st, uint32_t* a, const uint32_t* sums) {
-  __shared__ uint64_t sm[32];
-  const uint64_t total = st->total_hist;
-  const uint64_t base = (uint64_t)blockIdx.x * kScanTile;
-  if (base >= total) return;
+// One tile of the scan by 1024 threads; returns the tile's sum.
+__device__ __forceinline__ uint32_t scan_tile(uint32_t* a, uint64_t base, uint64_t total,
+                                              uint32_t before, uint64_t* sm) {
   uint32_t x[4];
   uint64_t v = 0;
   for (int r = 0; r < 4; ++r) {
@@ -580,12 +717,25 @@ k_scan_down(const DevState* st, uint32_t* a, const uint32_t* sums) {
     v += x[r];
   }
   uint64_t tot;
-  uint64_t run = block_excl_scan_u64<1024>(v, &tot, sm) + sums[blockIdx.x];
+  uint64_t run = block_excl_scan_u64<1024>(v, &tot, sm) + before;
   for (int r = 0; r < 4; ++r) {
     const uint64_t i = base + threadIdx.x * 4 + r;
     if (i < total) a[i] = (uint32_t)run;
     run += x[r];
   }
+  return (uint32_t)tot;
+}
+
+__global__ void __launch_bounds__(1024)
+k_scan_down(const DevState* st, uint32_t* a, const uint32_t* sums) {
+  __shared__ uint64_t sm[32];
+  const uint64_t total = st->total_hist;
+  const uint64_t base = (uint64_t)blockIdx.x * kScanTile;
+  if (base >= total) return;
+  uint64_t pre = 0, before;
+  for (uint32_t t = threadIdx.x; t < blockIdx.x; t += 1024) pre += sums[t];
+  block_excl_scan_u64<1024>(pre, &before, sm);
+  scan_tile(a, base, total, (uint32_t)before, sm);
 }
 
 // Step 5c: scatter.  Every chunk streams through two ST-key sub-tile buffers
@@ -645,7 +795,7 @@ k_scatter(const DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk
   uint8_t* my_win = sm.wwin + (size_t)warp * kmax;
   uint32_t cur_g = 0xffffffffu;
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = find_seg(segs, G, c, [](const LevelSeg& x) { return x.chunk_off; });
+    const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
     const LevelSeg sg = segs[g];
     __syncthreads();
     if (g != cur_g) {
@@ -899,7 +1049,7 @@ k_classify_count_wd(const DevState* st, const LevelSeg* segs, Src src, const uin
   uint64_t* stk = sm.skey + (size_t)warp * kWdStages * kWdKeys;
   uint32_t cur_g = 0xffffffffu;
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = find_seg(segs, G, c, [](const LevelSeg& x) { return x.chunk_off; });
+    const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
     const LevelSeg sg = segs[g];
     __syncthreads();
     if (g != cur_g) {
@@ -980,7 +1130,7 @@ k_scatter_wd(const DevState* st, const LevelSeg* segs, Src src, const uint64_t* 
   uint32_t* sti = sm.sidx + (size_t)warp * kWdStages * kWdKeys;
   uint32_t cur_g = 0xffffffffu;
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = find_seg(segs, G, c, [](const LevelSeg& x) { return x.chunk_off; });
+    const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
     const LevelSeg sg = segs[g];
     __syncthreads();
     if (g != cur_g) {
@@ -1053,33 +1203,6 @@ k_scatter_wd(const DevState* st, const LevelSeg* segs, Src src, const uint64_t* 
   }
 }
 
-// Level 1 with its order left to the device (LevelParams::stable ==
-// kOrderAuto): counts the level's equality buckets, those whose two bounding
-// splitters hold one key (every element of such a bucket has that key, so in
-// position order it is final and skips the levels below).  The scatter and
-// the collect keep input order when they are at least 1/kAutoOrderShare of
-// the buckets (duplicate-heavy inputs) and rank by atomics otherwise.
-__global__ void __launch_bounds__(256)
-k_l1_order(DevState* st, const LevelSeg* segs, const uint64_t* ssk) {
-  const uint64_t total = st->total_buckets;
-  const uint32_t G = st->cur_nseg;
-  uint32_t cnt = 0;
-  for (uint64_t f = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; f < total;
-       f += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t g = find_seg(segs, G, f, [](const LevelSeg& x) { return x.bkt_off; });
-    const LevelSeg& sg = segs[g];
-    const uint32_t b = (uint32_t)(f - sg.bkt_off);
-    if (b >= 1 && b + 1 < sg.k)
-      cnt += ssk[sg.samp_off + ((uint64_t)b * sg.S) / sg.k] ==
-                     ssk[sg.samp_off + ((uint64_t)(b + 1) * sg.S) / sg.k]
-                 ? 1u : 0u;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
-  if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(&st->l1_eq, cnt);
-  if (blockIdx.x == 0 && threadIdx.x == 0) st->l1_nb = (uint32_t)umin64(total, 0xffffffffull);
-}
-
 // Collect the buckets of the level: bucket sizes follow from the scanned
 // histogram.  Buckets that fit one SM, equality buckets of a stable level on
 // input in position order (both bounding splitters share one key, so every
@@ -1087,10 +1210,12 @@ k_l1_order(DevState* st, const LevelSeg* segs, const uint64_t* ssk) {
 // and empty ones are final; the rest become segments of the next level.
 // Otherwise an equality bucket is a bucket like any other, and its elements
 // arrive at the in-SM sort in no particular order.
-__global__ void __launch_bounds__(256)
-k_collect(DevState* st, const LevelSeg* segs, const uint64_t* ssk, const uint32_t* hist_scan,
-          SegIn* list_out, int par_out, FinalItem* items, LevelParams P, uint16_t where,
-          int last_level, int emit_final, uint64_t* offsets_out) {
+__device__ __forceinline__ void collect_buckets(DevState* st, const LevelSeg* segs,
+                                                const uint64_t* ssk, const uint32_t* hist_scan,
+                                                SegIn* list_out, int par_out, FinalItem* items,
+                                                const LevelParams& P, uint16_t where,
+                                                int last_level, int emit_final,
+                                                uint64_t* offsets_out) {
   const uint64_t total = st->total_buckets;
   const uint32_t G = st->cur_nseg;
   // buckets keep position order only if the level is stable and its input
@@ -1154,6 +1279,31 @@ k_collect(DevState* st, const LevelSeg* segs, const uint64_t* ssk, const uint32_
       else atomicOr(&st->error, kErrSegCap);
     }
   }
+}
+
+__global__ void __launch_bounds__(256)
+k_collect(DevState* st, const LevelSeg* segs, const uint64_t* ssk, const uint32_t* hist_scan,
+          SegIn* list_out, int par_out, FinalItem* items, LevelParams P, uint16_t where,
+          int last_level, int emit_final, uint64_t* offsets_out) {
+  collect_buckets(st, segs, ssk, hist_scan, list_out, par_out, items, P, where, last_level,
+                  emit_final, offsets_out);
+}
+
+// Scan and collect of a one-segment level with few counters, by one CTA in one
+// launch instead of three.
+constexpr uint64_t kSmallScan = 4 * kScanTile;
+__global__ void __launch_bounds__(1024)
+k_scan_collect(DevState* st, const LevelSeg* segs, const uint64_t* ssk, uint32_t* hist,
+               SegIn* list_out, int par_out, FinalItem* items, LevelParams P, uint16_t where,
+               int last_level, int emit_final, uint64_t* offsets_out) {
+  __shared__ uint64_t sm[32];
+  const uint64_t total = st->total_hist;
+  uint32_t before = 0;
+  for (uint64_t base = 0; base < total; base += kScanTile)
+    before += scan_tile(hist, base, total, before, sm);
+  __syncthreads();
+  collect_buckets(st, segs, ssk, hist, list_out, par_out, items, P, where, last_level, emit_final,
+                  offsets_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -1481,15 +1631,26 @@ void launch_plain_groups(const LaunchEnv& e, const uint64_t* offsets, uint32_t k
   k_plain_groups<<<(k + 256) / 256, 256, 0, e.stream>>>(offsets, k, fine_out, first_out);
 }
 
-void launch_init_plain(const LaunchEnv& e, DevState* st, SegIn* list0, FinalItem* items,
-                       uint64_t n, uint32_t k1, int direct, uint64_t final_cap) {
+void launch_init_plain(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t n,
+                       uint64_t final_cap) {
   Scope sc(e, "init");
-  k_init_plain<<<1, 32, 0, e.stream>>>(st, list0, items, n, k1, direct, final_cap, e.local);
+  k_init_plain<<<1, 32, 0, e.stream>>>(st, items, n, final_cap, e.local);
+}
+
+template <int NT, int IT, int MINB>
+void set_sample_sort_attributes() {
+  cudaFuncSetAttribute(k_sample_sort<NT, IT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       NT * IT * kCtaSortBytesPerElem);
 }
 
 void set_partition_kernel_attributes() {
-  cudaFuncSetAttribute(k_sample_sort_chunks, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kSampleChunk * kCtaSortBytesPerElem);
+  set_sample_sort_attributes<128, 8, 8>();
+  set_sample_sort_attributes<256, 16, 2>();
+  set_sample_sort_attributes<512, 8, 1>();
+  set_sample_sort_attributes<512, 16, 1>();
+  set_sample_sort_attributes<1024, 8, 1>();
+  cudaFuncSetAttribute(k_sample_merge, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       kMergeThreads * kMergeItems * kCtaSortBytesPerElem);
   const size_t c = umax64(part_smem_bytes(kMaxK, false, 0), part_smem_bytes(kMaxK, false, 1));
   const size_t s = umax64(part_smem_bytes(kMaxK, true, 0), part_smem_bytes(kMaxK, true, 1));
   cudaFuncSetAttribute(k_classify_count<kCStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1633,44 +1794,100 @@ void launch_init_segments(const LaunchEnv& e, DevState* st, const uint64_t* offs
                                               final_cap, f64);
 }
 
+namespace {
+
+// Samples of a deeper level's segments: the expected segment decides the shape
+// of the CTAs that draw and sort them (LevelParams::samp_max bounds the rest).
+template <int NT, int IT, int MINB>
+void launch_sample_sort(const LaunchEnv& e, const char* name, uint64_t chunks, DevState* st,
+                        LevelSeg* segs, const Src& src, uint64_t* samp_key, uint32_t* samp_idx,
+                        uint64_t* ssamp_key, uint32_t* ssamp_idx, uint32_t min_len,
+                        const PlainStart& ps, const LevelParams& P) {
+  Scope sc(e, name);
+  k_sample_sort<NT, IT, MINB>
+      <<<grid_for(chunks, 1, e.num_sms * MINB), NT, NT * IT * kCtaSortBytesPerElem, e.stream>>>(
+          st, segs, src, samp_key, samp_idx, ssamp_key, ssamp_idx, P.in_order, min_len, ps, P);
+}
+
+}  // namespace
+
+// k_plain: buckets of a call's only segment, [0, n_total) of the input (level 1
+// of a sort or partition, started by this launch); 0: the segments of list_in.
 void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const SegIn* list_in,
                   SegIn* list_out, LevelSeg* segs, Src src, Dst dst, uint16_t dst_where,
                   uint64_t* samp_key, uint32_t* samp_idx, uint64_t* ssamp_key,
                   uint32_t* ssamp_idx, uint32_t* hist, uint32_t* block_sums, FinalItem* items,
                   int kmax_level, int last_level, int emit_final, uint64_t* offsets_out,
-                  uint64_t /*n_total*/, int unmap_out, const Overpart* op) {
+                  uint64_t n_total, int unmap_out, const Overpart* op, uint32_t k_plain,
+                  uint64_t* plan_sums) {
   const int par_in = P.level & 1;
   const int sms = e.num_sms;
-  static const char* kNames[kMaxLevels + 1][11] = {
-      {"L?.plan", "L?.sample", "L?.sample_sort", "L?.sample_merge", "L?.classify",
-       "L?.scan_reduce", "L?.scan_sums", "L?.scan_down", "L?.scatter", "L?.collect", "L?.order"},
-      {"L1.plan", "L1.sample", "L1.sample_sort", "L1.sample_merge", "L1.classify",
-       "L1.scan_reduce", "L1.scan_sums", "L1.scan_down", "L1.scatter", "L1.collect", "L1.order"},
-      {"L2.plan", "L2.sample", "L2.sample_sort", "L2.sample_merge", "L2.classify",
-       "L2.scan_reduce", "L2.scan_sums", "L2.scan_down", "L2.scatter", "L2.collect", "L2.order"},
-      {"L3.plan", "L3.sample", "L3.sample_sort", "L3.sample_merge", "L3.classify",
-       "L3.scan_reduce", "L3.scan_sums", "L3.scan_down", "L3.scatter", "L3.collect", "L3.order"}};
+  static const char* kNames[kMaxLevels + 1][8] = {
+      {"L?.plan", "L?.sample_sort", "L?.sample_merge", "L?.classify", "L?.scan_reduce",
+       "L?.scan_down", "L?.scatter", "L?.collect"},
+      {"L1.plan", "L1.sample_sort", "L1.sample_merge", "L1.classify", "L1.scan_reduce",
+       "L1.scan_down", "L1.scatter", "L1.collect"},
+      {"L2.plan", "L2.sample_sort", "L2.sample_merge", "L2.classify", "L2.scan_reduce",
+       "L2.scan_down", "L2.scatter", "L2.collect"},
+      {"L3.plan", "L3.sample_sort", "L3.sample_merge", "L3.classify", "L3.scan_reduce",
+       "L3.scan_down", "L3.scatter", "L3.collect"}};
   const char* const* nm = kNames[(P.level >= 1 && P.level <= kMaxLevels) ? P.level : 0];
-  {
-    Scope sc(e, nm[0]);
-    k_level_plan<<<1, kPlanThreads, 0, e.stream>>>(st, list_in, segs, P, par_in,
-                                                  (uint32_t)kmax_level);
-  }
-  {
-    Scope sc(e, nm[1]);
-    k_sample<<<grid_for(P.samp_cap, 256, sms * 8), 256, 0, e.stream>>>(st, segs, src, samp_key,
-                                                                       samp_idx);
-  }
-  {
-    Scope sc(e, nm[2]);
-    const int smem = kSampleChunk * kCtaSortBytesPerElem;
-    k_sample_sort_chunks<<<grid_for(P.schunk_cap, 1, sms), kSampleThreads, smem, e.stream>>>(
-        st, segs, samp_key, samp_idx, ssamp_key, ssamp_idx, P.in_order);
-  }
-  {
-    Scope sc(e, nm[3]);
-    k_sample_merge_rank<<<grid_for(P.samp_cap, 256, sms * 8), 256, 0, e.stream>>>(
-        st, segs, samp_key, samp_idx, ssamp_key, ssamp_idx);
+  PlainStart ps;
+  uint64_t plain_hist = 0;  // counters of a one-segment level
+  if (k_plain) {
+    ps.n = n_total;
+    ps.k = k_plain;
+    ps.nch = (uint32_t)((n_total + P.W - 1) / P.W);
+    uint32_t lg = 0;
+    while ((1ull << lg) < k_plain) ++lg;
+    const uint64_t a = P.hinted ? 16ull * lg : (uint64_t)P.oversample;
+    ps.S = (uint32_t)umin64(umin64(n_total, a * k_plain), P.samp_max);
+    ps.local = e.local;
+    plain_hist = (uint64_t)k_plain * ps.nch * (P.warp_direct ? kPartWarps : 1);
+    const uint64_t nsch = (ps.S + kSampleChunk - 1) / kSampleChunk;
+    auto draw = [&](auto nt, auto it) {
+      launch_sample_sort<decltype(nt)::value, decltype(it)::value, 1>(
+          e, nm[1], umax64(nsch, 1), st, segs, src, samp_key, samp_idx, ssamp_key, ssamp_idx, 0,
+          ps, P);
+    };
+    // one CTA a chunk: the more threads the shorter
+    if (ps.S <= 4096)
+      draw(std::integral_constant<int, 512>(), std::integral_constant<int, 8>());
+    else
+      draw(std::integral_constant<int, 1024>(), std::integral_constant<int, 8>());
+    if (nsch > 1) {
+      Scope sc(e, nm[2]);
+      const int smem = kMergeThreads * kMergeItems * kCtaSortBytesPerElem;
+      k_sample_merge<<<(int)((ps.S + kMergeRange - 1) / kMergeRange), kMergeThreads, smem,
+                       e.stream>>>(segs, samp_key, samp_idx, ssamp_key, ssamp_idx);
+    }
+  } else {
+    {
+      Scope sc(e, nm[0]);
+      const int ctas = grid_for(umin64(P.seg_cap, P.max_segs), kPlanThreads, 1 << 22);
+      if (ctas > 1) {
+        k_plan_sums<<<ctas, kPlanThreads, 0, e.stream>>>(st, list_in, P, par_in,
+                                                         (uint32_t)kmax_level, plan_sums);
+        if (e.launches) ++*e.launches;
+      }
+      k_level_plan<<<ctas, kPlanThreads, 0, e.stream>>>(
+          st, list_in, segs, P, par_in, (uint32_t)kmax_level, plan_sums, src.chunk_seg);
+    }
+    // (every segment has at most kMaxKDeep buckets, so one sample chunk)
+    static_assert(kMaxKDeep * kDeepOversample <= kSampleChunk, "one sample chunk a segment");
+    if (P.samp_max <= 1024) {
+      launch_sample_sort<128, 8, 8>(e, nm[1], P.schunk_cap, st, segs, src, samp_key, samp_idx,
+                                    ssamp_key, ssamp_idx, 0, ps, P);
+    } else if (P.samp_max <= 4096) {
+      launch_sample_sort<256, 16, 2>(e, nm[1], P.schunk_cap, st, segs, src, samp_key, samp_idx,
+                                     ssamp_key, ssamp_idx, 0, ps, P);
+    } else {
+      // segments of any size: small samples by small CTAs, the others by large
+      launch_sample_sort<128, 8, 8>(e, nm[1], P.schunk_cap, st, segs, src, samp_key, samp_idx,
+                                    ssamp_key, ssamp_idx, 0, ps, P);
+      launch_sample_sort<512, 16, 1>(e, nm[1], P.schunk_cap, st, segs, src, samp_key, samp_idx,
+                                     ssamp_key, ssamp_idx, 1024, ps, P);
+    }
   }
   if (op) launch_overpartition(e, P, segs, src, ssamp_key, ssamp_idx, *op);
   const int mode = P.classifier | (P.no_tie_break ? 2 : 0);
@@ -1711,20 +1928,14 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
   const bool atomics = !units && P.atomic_scatter && !stable && !P.warp_direct &&
                        src.bid != nullptr && atomic_scatter_fits((uint32_t)kmax_level);
   if (!units && !atomics && (P.warp_direct || kmax_level >= 1024)) src.bid = nullptr;
-  // level 1 with its order left to the device: count its equality buckets
-  // (without the unit scatter the level stays unordered)
-  if (units && P.stable == kOrderAuto) {
-    Scope sc(e, nm[10]);
-    k_l1_order<<<grid_for(P.bucket_cap, 256, sms * 4), 256, 0, e.stream>>>(st, segs, ssamp_key);
-  }
   // Deeper levels keep the staged classify below, which stores the ids as
   // well: with many short chunks it measured faster (1.00 vs 1.09 ms at 2^28
   // keys) than the register-streaming one.
   if (units && P.level == 1) {
     launch_classify_ids(e, P, st, segs, src, ssamp_key, ssamp_idx, hist, (uint32_t)kmax_level,
-                        mode, nm[4]);
+                        mode, nm[3]);
   } else {
-    Scope sc(e, nm[4]);
+    Scope sc(e, nm[3]);
     if (P.warp_direct)
       k_classify_count_wd<<<grid_wd_c, kPartThreads, smem_wd, e.stream>>>(
           st, segs, src, ssamp_key, ssamp_idx, hist, P.W, (uint32_t)kmax_level, mode);
@@ -1735,25 +1946,30 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
       k_classify_count<kCStages><<<grid_c, kPartThreads, smem_c, e.stream>>>(
           st, segs, src, ssamp_key, ssamp_idx, hist, P.W, (uint32_t)kmax_level, mode);
   }
-  const int scan_grid = (int)((P.hist_cap + kScanTile - 1) / kScanTile);
-  {
+  const bool small_scan = k_plain && plain_hist <= kSmallScan;
+  if (small_scan) {
     Scope sc(e, nm[5]);
-    k_scan_reduce<<<scan_grid > 0 ? scan_grid : 1, 1024, 0, e.stream>>>(st, hist, block_sums);
-  }
-  {
-    Scope sc(e, nm[6]);
-    k_scan_sums<<<1, 1024, 0, e.stream>>>(st, block_sums);
-  }
-  {
-    Scope sc(e, nm[7]);
-    k_scan_down<<<scan_grid > 0 ? scan_grid : 1, 1024, 0, e.stream>>>(st, hist, block_sums);
+    k_scan_collect<<<1, 1024, 0, e.stream>>>(st, segs, ssamp_key, hist, list_out, par_in ^ 1,
+                                             items, P, dst_where, last_level, emit_final,
+                                             offsets_out);
+  } else {
+    const uint64_t most = k_plain ? plain_hist : P.hist_cap;
+    const int scan_grid = (int)umax64((most + kScanTile - 1) / kScanTile, 1);
+    {
+      Scope sc(e, nm[4]);
+      k_scan_reduce<<<scan_grid, 1024, 0, e.stream>>>(st, hist, block_sums);
+    }
+    {
+      Scope sc(e, nm[5]);
+      k_scan_down<<<scan_grid, 1024, 0, e.stream>>>(st, hist, block_sums);
+    }
   }
   if (units) {
-    launch_scatter_units(e, P, st, segs, src, hist, dst, (uint32_t)kmax_level, unmap_out, nm[8]);
+    launch_scatter_units(e, P, st, segs, src, hist, dst, (uint32_t)kmax_level, unmap_out, nm[6]);
   } else if (atomics) {
-    launch_scatter_atomic(e, P, st, segs, src, hist, dst, (uint32_t)kmax_level, unmap_out, nm[8]);
+    launch_scatter_atomic(e, P, st, segs, src, hist, dst, (uint32_t)kmax_level, unmap_out, nm[6]);
   } else {
-    Scope sc(e, nm[8]);
+    Scope sc(e, nm[6]);
     if (P.warp_direct)
       k_scatter_wd<<<grid_wd_s, kPartThreads, smem_wd, e.stream>>>(
           st, segs, src, ssamp_key, ssamp_idx, hist, dst, P.W, (uint32_t)kmax_level, unmap_out,
@@ -1784,8 +2000,8 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
              e.stream>>>(st, segs, src, ssamp_key, ssamp_idx, hist, dst, P.W,
                          (uint32_t)kmax_level, unmap_out, mode);
   }
-  {
-    Scope sc(e, nm[9]);
+  if (!small_scan) {
+    Scope sc(e, nm[7]);
     k_collect<<<grid_for(P.bucket_cap, 256, sms * 8), 256, 0, e.stream>>>(
         st, segs, ssamp_key, hist, list_out, par_in ^ 1, items, P, dst_where, last_level,
         emit_final, offsets_out);

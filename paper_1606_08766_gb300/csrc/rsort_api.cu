@@ -96,6 +96,9 @@ struct Plan {
   uint64_t n = 0;
   uint32_t k1 = 0;          // level-1 buckets (0: automatic)
   int levels = 0;           // partition levels to launch
+  uint32_t k_plain = 0;     // level-1 buckets of a one-segment call
+  uint32_t oversample1 = kDeepOversample;  // its samples per bucket when automatic
+  uint32_t samp_max = 0xffffffffu;         // most samples of a deeper segment
   int direct = 0;           // n small enough for one in-SM sort
   uint32_t W1 = 0, Wd = 0;  // chunk sizes (level 1, deeper levels)
   uint64_t seg_cap = 0, samp_cap = 0, hist_cap = 0, chunk_cap = 0, schunk_cap = 0;
@@ -115,7 +118,7 @@ struct Plan {
   // arena offsets
   size_t off_tmp_key = 0, off_tmp_idx = 0, off_samp_key = 0, off_samp_idx = 0;
   size_t off_ssamp_key = 0, off_ssamp_idx = 0, off_hist = 0, off_sums = 0, off_segs = 0;
-  size_t off_list0 = 0, off_list1 = 0, off_items = 0, off_state = 0, off_fine = 0, off_bid = 0;
+  size_t off_plan = 0, off_chunk = 0, off_list0 = 0, off_list1 = 0, off_items = 0, off_state = 0, off_fine = 0, off_bid = 0;
   size_t total = 0;
 };
 
@@ -133,7 +136,7 @@ void layout(Plan& p) {
     return at;
   };
   p.off_state = take(sizeof(DevState));
-  p.off_items = take((size_t)kNumLists * p.final_cap * sizeof(FinalItem));
+  p.off_items = take((size_t)kNumItemArrays * p.final_cap * sizeof(FinalItem));
   if (p.need_tmp) {
     p.off_tmp_key = take(p.n * 8);
     p.off_tmp_idx = take(p.n * 4);
@@ -147,6 +150,8 @@ void layout(Plan& p) {
   p.off_hist = take(p.hist_cap * 4);
   p.off_sums = take((p.hist_cap / kScanTile + 2) * 4);
   p.off_segs = take(p.seg_cap * sizeof(LevelSeg));
+  p.off_plan = take(plan_sum_words(p.seg_cap) * 8);
+  p.off_chunk = take(p.chunk_cap * 4);
   p.off_list0 = take(p.seg_cap * sizeof(SegIn));
   p.off_list1 = take(p.seg_cap * sizeof(SegIn));
   p.total = o;
@@ -154,7 +159,11 @@ void layout(Plan& p) {
 
 // Capacities of the sample-sort levels for n elements, level-1 fan-out k1
 // (0: automatic) and g1 level-1 segments.
-void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int levels) {
+// fine: chunks as small as the call needs to spread over the GPU (false: no
+// smaller than one scatter sub-tile, 65536 keys at the deeper levels, which
+// takes the least scratch).
+void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int levels,
+                 bool fine) {
   p.n = n;
   p.k1 = k1;
   // Levels the sizes call for (at most the max_levels tunable): the sample
@@ -182,14 +191,51 @@ void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int
              3 * mean1 <= 2 * (uint64_t)kMaxKDeep * tmin)
       needed = 2;
     levels = std::min(levels, needed);
+    // most samples of a deeper segment: its expected size is mean1, twice that
+    // is far outside what the sampling leaves; the bound lets small CTAs sort
+    // small samples (a segment beyond it only gets fewer samples a bucket)
+    if (g1 == 1) {
+      const uint64_t k2 = std::min<uint64_t>(2 * mean1 / tmin + 1, kMaxKDeep);
+      p.samp_max = k2 * kDeepOversample <= 1024   ? 1024
+                   : k2 * kDeepOversample <= 4096 ? 4096
+                                                  : kMaxKDeep * kDeepOversample;
+    }
   }
   p.levels = levels;
+  if (g1 == 1) {
+    const uint32_t cls = ceil_log2_host((uint32_t)n);
+    const uint32_t tb = p.target_by_class[cls] ? p.target_by_class[cls] : p.target_bucket;
+    p.k_plain = k1 >= 2 ? k1
+                        : (uint32_t)std::max<uint64_t>(
+                              2, std::min<uint64_t>((n + tb - 1) / tb, kMaxKDeep));
+    // buckets above the target that no further level will cut: 16 samples a
+    // bucket leave some beyond kBucketCap (at 2539 expected keys one in 150, at
+    // 2730 keys and 64 samples still one in 10^4), which one CTA each then
+    // merge-sorts; with 128, 1.5 times the mean is 5 deviations away
+    if (k1 < 2 && levels == 1 && n / p.k_plain > tb) p.oversample1 = 8 * kDeepOversample;
+  }
   // level 1 of one segment: 6 chunks per SM, so grids of 1, 2, 3 or 6 resident
   // CTAs per SM all get the same number of chunks
   const uint64_t per = (n + 6ull * num_sms - 1) / (6ull * num_sms);
   p.W1 = (uint32_t)std::max<uint64_t>(kSubTile, align_up(per, kSubTile));
-  if (g1 > 1) p.W1 = 65536;
   p.Wd = 65536;
+  if (fine) {
+    // calls below 6 scatter sub-tiles an SM: a whole number of chunks per SM,
+    // each at most one sub-tile (kFineTile keys) and at least kMinChunk keys, so
+    // that 10^5 keys keep 98 SMs busy instead of 25
+    const uint64_t j = (n + (uint64_t)num_sms * kFineTile - 1) / ((uint64_t)num_sms * kFineTile);
+    if (j < 6) {
+      const uint64_t chunks = (uint64_t)num_sms * std::max<uint64_t>(2, j);
+      p.W1 = (uint32_t)std::max<uint64_t>(kMinChunk, align_up((n + chunks - 1) / chunks, 64));
+    }
+    // deeper levels aim at four chunks an SM (2^20 keys over 64 segments: one
+    // chunk a segment kept 64 SMs busy)
+    const uint64_t perd = (n + 4ull * num_sms - 1) / (4ull * num_sms);
+    p.Wd = (uint32_t)std::min<uint64_t>(65536,
+                                        std::max<uint64_t>(kMinDeepChunk,
+                                                           align_up(perd, kMinDeepChunk)));
+  }
+  if (g1 > 1) p.W1 = p.Wd;
   const uint64_t segs_deep = n / (kBucketCap + 1) + 1;
   p.seg_cap = std::max<uint64_t>(g1, segs_deep);
   const uint32_t kmax1 = k1 >= 2 ? k1 : kMaxKDeep;
@@ -200,17 +246,19 @@ void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int
   // level 1
   p.bucket_cap1 = k1 >= 2 ? (uint64_t)k1 * g1 : n / tmin + g1 + 1;
   p.bucket_cap1 = std::min<uint64_t>(p.bucket_cap1, (uint64_t)kmax1 * g1);
-  const uint64_t a1 = k1 >= 2 ? 16ull * ceil_log2_host(k1) : (uint64_t)kDeepOversample;
+  const uint64_t a1 = k1 >= 2 ? 16ull * ceil_log2_host(k1) : (uint64_t)p.oversample1;
   p.samp_cap1 = std::min<uint64_t>(n, a1 * p.bucket_cap1);
   p.chunk_cap1 = n / p.W1 + g1 + 1;
-  // (x kPartWarps: a warp-direct level has one histogram unit per warp sub-chunk)
-  p.hist_cap1 = ((uint64_t)kmax1 * (n / p.W1) + p.bucket_cap1) * kPartWarps;
+  // (a warp-direct level has one histogram unit per warp sub-chunk)
+  const uint64_t units1 = (int)kmax1 <= p.wd_max_k ? kPartWarps : 1;
+  p.hist_cap1 = ((uint64_t)kmax1 * (n / p.W1) + p.bucket_cap1) * units1;
   p.schunk_cap1 = p.samp_cap1 / kSampleChunk + g1 + 1;
   // deeper levels
   const uint64_t bucket_capd = n / tmin + segs_deep + 1;
   const uint64_t samp_capd = std::min<uint64_t>(n, (uint64_t)kDeepOversample * bucket_capd);
   const uint64_t chunk_capd = n / p.Wd + segs_deep + 1;
-  const uint64_t hist_capd = ((uint64_t)kMaxKDeep * (n / p.Wd) + bucket_capd) * kPartWarps;
+  const uint64_t unitsd = kMaxKDeep <= p.wd_max_k ? kPartWarps : 1;
+  const uint64_t hist_capd = ((uint64_t)kMaxKDeep * (n / p.Wd) + bucket_capd) * unitsd;
   const uint64_t schunk_capd = samp_capd / kSampleChunk + segs_deep + 1;
   const bool deep = levels > 1;
   p.bucket_cap = std::max<uint64_t>(p.bucket_cap1, deep ? bucket_capd : 0);
@@ -241,6 +289,9 @@ LevelParams level_params(const Plan& p, int level, uint64_t seed, int kmax_level
     P.schunk_cap = p.schunk_cap;
     P.bucket_cap = p.bucket_cap;
   }
+  P.samp_max = level == 1 ? 0xffffffffu : p.samp_max;
+  P.hinted = p.k1 >= 2;
+  P.oversample = p.oversample1;
   P.level1_oversample = 1;
   P.classifier = p.classifier;
   P.warp_direct = kmax_level <= p.wd_max_k ? 1 : 0;
@@ -304,6 +355,7 @@ void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const 
     // (the in-SM sort orders (key, position) pairs either way; level 1's
     // default leaves it to the device); a level's input is in position order
     // only after stable levels, and level 1's order is read on the device
+    if (L == 2 && !segmented) P.max_segs = p.k_plain;  // (level 1's buckets)
     P.refine = segmented && type == RSORT_KEY_F64;
     P.stable = L == 1 ? c->level1_stable : c->deep_levels_stable;
     P.in_order = L == 1 ? 1 : (L == 2 || c->deep_levels_stable ? kOrderAuto : 0);
@@ -315,13 +367,15 @@ void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const 
       src = Src{prev.key, prev.idx, 0};
     }
     src.bid = at<uint16_t>(ws, p.off_bid);
+    src.chunk_seg = at<uint32_t>(ws, p.off_chunk);
     const Dst& dst = level_dst(L);
     const uint16_t where = &dst == &tmp ? kWhereTmp : kWhereOut;
     launch_level(e, P, st, lists[L & 1], lists[(L + 1) & 1], at<LevelSeg>(ws, p.off_segs), src,
                  dst, where, at<uint64_t>(ws, p.off_samp_key), at<uint32_t>(ws, p.off_samp_idx),
                  at<uint64_t>(ws, p.off_ssamp_key), at<uint32_t>(ws, p.off_ssamp_idx),
                  at<uint32_t>(ws, p.off_hist), at<uint32_t>(ws, p.off_sums), items, kmax,
-                 L == p.levels, 1, nullptr, p.n, 0);
+                 L == p.levels, 1, nullptr, p.n, 0, nullptr,
+                 L == 1 && !segmented ? p.k_plain : 0u, at<uint64_t>(ws, p.off_plan));
   }
   launch_local_sort(e, st, items, p.final_cap, p.direct ? 1 : p.final_cap,
                     (const uint64_t*)d_keys_in, out, tmp, type == RSORT_KEY_F64, segmented);
@@ -506,12 +560,19 @@ Plan plan_sort(rsort_ctx* c, uint64_t n, uint32_t p_virtual) {
   if (n <= (uint64_t)kBucketCap) {
     p.n = n;
     p.direct = 1;
-    p.final_cap = 4;
+    p.final_cap = 2;
     p.seg_cap = 1;
     p.need_tmp = false;
     p.levels = 0;
   } else {
-    plan_levels(p, n, k1, 1, c->num_sms, c->max_levels);
+    const Plan q = p;
+    plan_levels(p, n, k1, 1, c->num_sms, c->max_levels, true);
+    p.need_tmp = true;
+    layout(p);
+    if (c->budget == 0 || p.total <= c->budget) return p;
+    // the budget counts: the plan that takes the least scratch
+    p = q;
+    plan_levels(p, n, k1, 1, c->num_sms, c->max_levels, false);
     p.need_tmp = true;
   }
   layout(p);
@@ -529,10 +590,15 @@ Plan plan_segmented(rsort_ctx* c, uint64_t n, uint32_t num_segments) {
   p.atomic_scatter = c->atomic_scatter;
   p.bulk_classify = c->bulk_classify;
   const uint64_t g1 = std::min<uint64_t>(num_segments, n / (kBucketCap + 1) + 1);
-  plan_levels(p, n, 0, std::max<uint64_t>(g1, 2), c->num_sms, c->max_levels);
-  p.final_cap += num_segments;
-  p.need_tmp = true;
-  layout(p);
+  const Plan q = p;
+  for (const bool fine : {true, false}) {
+    p = q;
+    plan_levels(p, n, 0, std::max<uint64_t>(g1, 2), c->num_sms, c->max_levels, fine);
+    p.final_cap += num_segments;
+    p.need_tmp = true;
+    layout(p);
+    if (c->budget == 0 || p.total <= c->budget) break;
+  }
   return p;
 }
 
@@ -562,7 +628,7 @@ rsort_status enqueue_sort(rsort_ctx* c, Workspace& ws, const LaunchEnv& e, rsort
     launch_direct_sort(e, st, (const uint64_t*)d_keys_in, out, (uint32_t)n, type == RSORT_KEY_F64);
     return RSORT_OK;
   }
-  launch_init_plain(e, st, lists[1], items, n, k1, p.direct, p.final_cap);
+  if (p.direct) launch_init_plain(e, st, items, n, p.final_cap);  // (a level starts itself)
   Dst tmp{at<uint64_t>(ws, p.off_tmp_key), at<uint32_t>(ws, p.off_tmp_idx)};
   enqueue_levels_and_local(c, ws, p, e, st, items, lists, type, d_keys_in, out, tmp, seed, k1, false);
   return RSORT_OK;
@@ -578,7 +644,7 @@ rsort_status enqueue_segmented(rsort_ctx* c, Workspace& ws, const LaunchEnv& e,
   DevState* st = at<DevState>(ws, p.off_state);
   FinalItem* items = at<FinalItem>(ws, p.off_items);
   SegIn* lists[2] = {at<SegIn>(ws, p.off_list0), at<SegIn>(ws, p.off_list1)};
-  launch_init_plain(e, st, lists[1], items, 0, 0, 0, p.final_cap);  // reset the control block
+  launch_init_plain(e, st, items, 0, p.final_cap);  // reset the control block
   launch_init_segments(e, st, d_offsets, num_segments, n, lists[1], items, p.seg_cap,
                        p.final_cap, type == RSORT_KEY_F64);
   Dst out{(uint64_t*)d_keys_out, d_perm_out};
@@ -743,20 +809,24 @@ rsort_status partition_impl(rsort_ctx* c, rsort_key_type type, const void* d_key
   p.atomic_scatter = c->atomic_scatter;
   p.bulk_classify = c->bulk_classify;
   const uint32_t kk = k < 2 ? 2 : k;  // capacities as for two buckets when k = 1
-  plan_levels(p, n, kk, 1, c->num_sms, 1);
-  p.final_cap = 4;
-  p.need_tmp = false;
-  if (over > 1) {
-    p.samp_extra = (uint64_t)kk + 2;
-    p.fine_cap = 2 * (uint64_t)K + 8;  // counters, prefix sums, search state
+  const Plan q = p;
+  for (const bool fine : {true, false}) {
+    p = q;
+    plan_levels(p, n, kk, 1, c->num_sms, 1, fine);
+    p.final_cap = 1;
+    p.need_tmp = false;
+    if (over > 1) {
+      p.samp_extra = (uint64_t)kk + 2;
+      p.fine_cap = 2 * (uint64_t)K + 8;  // counters, prefix sums, search state
+    }
+    layout(p);
+    if (c->budget == 0 || p.total <= c->budget) break;
   }
-  layout(p);
   Workspace& ws = c->ws;
   rsort_status rs = ensure_workspace(c, ws, p.total, s);
   if (rs != RSORT_OK) return latch(c, rs);
   DevState* st = at<DevState>(ws, p.off_state);
   SegIn* list1 = at<SegIn>(ws, p.off_list1);
-  launch_init_plain(e, st, list1, at<FinalItem>(ws, p.off_items), n, k, 0, p.final_cap);
   LevelParams P = level_params(p, 1, seed, (int)kk);
   P.no_tie_break = tie_break ? 0 : 1;
   Src src{(const uint64_t*)d_keys_in, nullptr, type == RSORT_KEY_F64};
@@ -775,7 +845,7 @@ rsort_status partition_impl(rsort_ctx* c, rsort_key_type type, const void* d_key
                at<uint64_t>(ws, p.off_ssamp_key), at<uint32_t>(ws, p.off_ssamp_idx),
                at<uint32_t>(ws, p.off_hist), at<uint32_t>(ws, p.off_sums),
                at<FinalItem>(ws, p.off_items), (int)kk, 1, 0, d_offsets_out, n,
-               type == RSORT_KEY_F64, over > 1 ? &op : nullptr);
+               type == RSORT_KEY_F64, over > 1 ? &op : nullptr, k, nullptr);
   if (over == 1 && (d_fine_out || d_first_out))
     launch_plain_groups(e, d_offsets_out, k, d_fine_out, d_first_out);
   return cuda_status(c);

@@ -17,6 +17,9 @@ constexpr int kPartWarps = kPartThreads / 32;
 constexpr int kItems = 16;                        // keys per lane per sub-tile
 constexpr int kWarpSpan = 32 * kItems;            // 512 consecutive keys per warp
 constexpr int kSubTile = kPartThreads * kItems;   // 4096 keys staged per sub-tile
+constexpr int kMinChunk = 1024;                   // smallest level-1 chunk of a small call
+constexpr int kFineTile = 6144;                   // keys of an unordered scatter sub-tile
+constexpr int kMinDeepChunk = 4096;               // smallest chunk at levels >= 2
 constexpr int kMaxK = 2048;                       // buckets per partition step
 constexpr int kMaxKDeep = 512;                    // buckets at levels >= 2
 constexpr int kMaxFine = 10240;                   // fine partitions of an overpartitioned step
@@ -56,8 +59,20 @@ enum : int {
   kListRefine = 5,   // + (class - kClassSmall)
   // buckets in which a class kernel found crowded bins
   kListCrowd = 8,
-  kNumLists = 9
+  kNumLists = 9,
+  kNumItemArrays = 5
 };
+
+// Slot of a list's item i among kNumItemArrays arrays of cap items.  A bucket
+// is on one list only, except that a class's may be on kListCrowd as well; so
+// two lists share an array, one from its start and one from its end:
+// copies | oversize, each class | its refine list, and the crowded ones alone.
+__host__ __device__ __forceinline__ uint64_t item_slot(int list, uint64_t i, uint64_t cap) {
+  if (list == kListCrowd) return 4 * cap + i;
+  if (list == kClassBig) return cap - 1 - i;
+  if (list >= kListRefine) return (uint64_t)(list - kListRefine + 2) * cap - 1 - i;
+  return (uint64_t)list * cap + i;
+}
 // Which in-SM algorithm finished a bucket (rsort_stats.algo_elems counts the
 // elements each one handled):
 enum : int {
@@ -197,6 +212,12 @@ struct LevelParams {
   uint32_t W;           // keys per classify/scatter chunk
   uint64_t seed;
   uint64_t samp_cap, hist_cap, chunk_cap, seg_cap, final_cap, schunk_cap, bucket_cap;
+  uint64_t max_segs = ~0ull;        // segments the level can have (seg_cap aside)
+  uint32_t samp_max = 0xffffffffu;  // at most this many samples a segment
+  // a one-segment level: 1: its bucket count was asked for (16 ceil(log2 k)
+  // samples a bucket, the paper's rule), 0: it is automatic (oversample)
+  int hinted = 0;
+  uint32_t oversample = kDeepOversample;
   int level1_oversample;  // 1: a = 16 ceil(log2 k) for hinted k (the paper's rule)
   int classifier;         // 0: splitter tree, 1: leading-bits table
   int warp_direct;        // 1: per-warp sub-chunks scattered straight to HBM
@@ -246,6 +267,9 @@ struct Src {
   // [n + 16] bucket of every element by position, written by the classify
   // pass and read by the scatter (nullptr: the scatter classifies again)
   uint16_t* bid = nullptr;
+  // segment of every chunk of the level, written by its plan (not read when
+  // the level has one segment)
+  uint32_t* chunk_seg = nullptr;
 };
 struct Dst {
   uint64_t* key;
@@ -339,8 +363,8 @@ __device__ __forceinline__ void block_bitonic_sort(uint64_t* sk, uint32_t* si, i
 
 __host__ __device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
 
-// Appends a final bucket to the work list of its size class (items holds
-// kNumLists lists of cap entries each); refine: to the class's list of buckets
+// Appends a final bucket to the work list of its size class (items: see
+// item_slot); refine: to the class's list of buckets
 // whose bins will need refining, if the class is sorted by bins.
 __device__ __forceinline__ void push_final(DevState* st, FinalItem* items, uint64_t cap,
                                            const FinalItem& f, uint32_t err_flag,
@@ -368,7 +392,7 @@ __device__ __forceinline__ void push_final(DevState* st, FinalItem* items, uint6
   uint32_t lt;
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
   const uint32_t slot = base + __popc(peers & lt);
-  if (slot < cap) items[(uint64_t)list * cap + slot] = f;
+  if (slot < cap) items[item_slot(list, slot, cap)] = f;
   else atomicOr(&st->error, err_flag);
 }
 __host__ __device__ __forceinline__ uint64_t umax64(uint64_t a, uint64_t b) { return a > b ? a : b; }
@@ -406,14 +430,17 @@ struct LaunchEnv {
   LocalPlan local;      // in-SM size classes and algorithms (written to DevState at init)
 };
 
-void launch_init_plain(const LaunchEnv& e, DevState* st, SegIn* list0, FinalItem* items,
-                       uint64_t n, uint32_t k1, int direct, uint64_t final_cap);
+void launch_init_plain(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t n,
+                       uint64_t final_cap);
 void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const SegIn* list_in,
                   SegIn* list_out, LevelSeg* segs, Src src, Dst dst, uint16_t dst_where,
                   uint64_t* samp_key, uint32_t* samp_idx, uint64_t* ssamp_key,
                   uint32_t* ssamp_idx, uint32_t* hist, uint32_t* block_sums, FinalItem* items,
                   int kmax_level, int last_level, int emit_final, uint64_t* offsets_out,
-                  uint64_t n_total, int unmap_out, const Overpart* op = nullptr);
+                  uint64_t n_total, int unmap_out, const Overpart* op, uint32_t k_plain,
+                  uint64_t* plan_sums);
+// plan_sums words a level of at most seg_cap segments needs.
+inline uint64_t plan_sum_words(uint64_t seg_cap) { return (seg_cap / 1024 + 1) * 6; }
 void launch_init_segments(const LaunchEnv& e, DevState* st, const uint64_t* offsets,
                           uint32_t nseg, uint64_t n, SegIn* list_l1, FinalItem* items,
                           uint64_t seg_cap, uint64_t final_cap, int f64);

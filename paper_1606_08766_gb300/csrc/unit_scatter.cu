@@ -83,6 +83,22 @@ __device__ __forceinline__ uint64_t conv_key(uint64_t k, int conv) {
 // ---------------------------------------------------------------------------
 // Classify with stored bucket ids
 // ---------------------------------------------------------------------------
+// Level 1 with its order left to the device (LevelParams::stable ==
+// kOrderAuto): the classify counts the level's equality buckets, those whose
+// two bounding splitters hold one key (every element of such a bucket has that
+// key, so in position order it is final and skips the levels below), one
+// segment's by the CTA of its first chunk.  The scatter and the collect keep
+// input order when they are at least 1/kAutoOrderShare of the buckets
+// (duplicate-heavy inputs) and rank by atomics otherwise.
+template <int NT>
+__device__ __forceinline__ void count_equality_buckets(DevState* st, const Splitters& sp) {
+  uint32_t cnt = 0;
+  for (uint32_t j = threadIdx.x; j + 1 < sp.nspl; j += NT) cnt += sp.key[j] == sp.key[j + 1];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
+  if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(&st->l1_eq, cnt);
+}
+
 constexpr int kCiPairs = 4;  // 16-byte loads (two keys) per thread per step
 // steps ahead of the current one whose keys are asked into L2 (0 or 1: none;
 // the next step's keys are already in registers)
@@ -92,8 +108,8 @@ constexpr int kCiPrefetch = 2;
 // MAP: the keys are float64 bit patterns, mapped to the order map on load.
 template <int NT, bool VEC, bool MAP>
 __global__ void __launch_bounds__(NT, 3)
-k_classify_ids(const DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
-               const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode) {
+k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
+               const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode, bool count_eq) {
   constexpr int R = 2 * kCiPairs;  // keys per thread per step
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Splitters sp;
@@ -123,7 +139,7 @@ k_classify_ids(const DevState* st, const LevelSeg* segs, Src src, const uint64_t
   const int lane = threadIdx.x & 31;
   uint32_t cur_g = 0xffffffffu;
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = find_seg(segs, G, c, [](const LevelSeg& x) { return x.chunk_off; });
+    const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
     const LevelSeg sg = segs[g];
     __syncthreads();
     if (g != cur_g) {
@@ -133,6 +149,7 @@ k_classify_ids(const DevState* st, const LevelSeg* segs, Src src, const uint64_t
     for (uint32_t b = threadIdx.x; b < sg.k; b += NT) cnt[b] = 0;
     __syncthreads();
     const uint64_t cl = c - sg.chunk_off;
+    if (count_eq && cl == 0) count_equality_buckets<NT>(st, sp);
     const uint64_t cs = sg.start + cl * sg.W;
     const uint64_t ce = umin64(cs + sg.W, sg.start + sg.m);
     // pairs start at the even position at or below cs (16-byte aligned when
@@ -280,7 +297,8 @@ __host__ __device__ inline size_t classify_bulk_smem_bytes(size_t common) {
 template <int NC>
 __global__ void __launch_bounds__(NC + 32, 2)
 k_classify_bulk(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
-                const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode, size_t common) {
+                const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode, size_t common,
+                bool count_eq) {
   constexpr int NT = NC + 32;
   constexpr int NCW = NC / 32;         // consumer warps
   constexpr int SK = kCbStageKeys;
@@ -332,7 +350,7 @@ k_classify_bulk(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk
   uint32_t next = 0;   // stages issued (producer) / consumed (consumers) so far
   uint32_t cur_g = 0xffffffffu;
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = find_seg(segs, G, c, [](const LevelSeg& x) { return x.chunk_off; });
+    const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
     const LevelSeg sg = segs[g];
     if (__syncthreads_or(s_abort != 0)) break;
     if (g != cur_g) {
@@ -342,6 +360,7 @@ k_classify_bulk(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk
     for (uint32_t b = tid; b < sg.k; b += NT) cnt[b] = 0;
     __syncthreads();
     const uint64_t cl = c - sg.chunk_off;
+    if (count_eq && cl == 0) count_equality_buckets<NT>(st, sp);
     const uint64_t cs = sg.start + cl * sg.W;
     const uint64_t ce = umin64(cs + sg.W, sg.start + sg.m);
     const uint64_t ps = cs & ~1ull, pe = ce & ~1ull;
@@ -562,13 +581,10 @@ __device__ __forceinline__ void rank_by_atomics(const uint32_t (&bid)[IT], uint3
 // and a prefix over the warps); otherwise (a full sort's level 1, whose
 // buckets the in-SM sort orders by (key, position) anyway) every element takes
 // its rank from one shared-memory atomic on its bucket's counter.
-// auto_order: level 1 with its order decided on the device; the kernel
-// returns at once unless the decision (l1_auto_ordered) is its own form.
 template <int NT, int IT, bool HAS_IDX, bool STABLE>
-__global__ void __launch_bounds__(NT, 1)
-k_scatter_units(const DevState* st, const LevelSeg* segs, Src src, const uint32_t* hist_scan,
-                Dst dst, uint32_t kmax, int conv, uint32_t aoff, bool auto_order) {
-  if (auto_order && l1_auto_ordered(st) != STABLE) return;
+__device__ __forceinline__ void scatter_units(const DevState* st, const LevelSeg* segs, Src src,
+                                              const uint32_t* hist_scan, Dst dst, uint32_t kmax,
+                                              int conv, uint32_t aoff) {
   constexpr int NW = NT / 32;
   constexpr int ST = NT * IT;
   static_assert(ST + kUnit < (1 << kMetaUnitShift), "sorted slots fit the meta word");
@@ -620,7 +636,7 @@ k_scatter_units(const DevState* st, const LevelSeg* segs, Src src, const uint32_
     for (uint32_t b = tid; b < kmax; b += NT) ucnt[b] = 0;
 
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = find_seg(segs, G, c, [](const LevelSeg& x) { return x.chunk_off; });
+    const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
     const LevelSeg sg = segs[g];
     const uint32_t k = sg.k;
     const int nbits = k > 32 ? 5 : (int)ceil_log2_dev(k);
@@ -928,6 +944,34 @@ k_scatter_units(const DevState* st, const LevelSeg* segs, Src src, const uint32_
   }
 }
 
+template <int NT, int IT, bool HAS_IDX, bool STABLE>
+__global__ void __launch_bounds__(NT, 1)
+k_scatter_units(const DevState* st, const LevelSeg* segs, Src src, const uint32_t* hist_scan,
+                Dst dst, uint32_t kmax, int conv, uint32_t aoff, bool auto_order) {
+  // (level 1 with its order decided on the device: both forms are launched and
+  // the one not chosen returns at once)
+  if (auto_order && l1_auto_ordered(st) != STABLE) return;
+  scatter_units<NT, IT, HAS_IDX, STABLE>(st, segs, src, hist_scan, dst, kmax, conv, aoff);
+}
+
+// Level 1 with its order decided on the device: either form, in one launch.  It
+// spares a small call one launch; the two forms in one kernel cost registers
+// and scheduling (2^28 keys: 2.06 -> 2.24 ms), so calls with long chunks launch
+// both.
+constexpr uint32_t kAutoOneLaunchW = kFineTile;
+static_assert(kUsThreadsAny * kUsItemsAny == kFineTile, "fine chunks are one sub-tile");
+static_assert(kUsThreads == kUsThreadsAny, "both forms run with the same threads");
+__global__ void __launch_bounds__(kUsThreads, 1)
+k_scatter_units_auto(const DevState* st, const LevelSeg* segs, Src src, const uint32_t* hist_scan,
+                     Dst dst, uint32_t kmax, int conv, uint32_t aoff) {
+  if (l1_auto_ordered(st))
+    scatter_units<kUsThreads, kUsItems, false, true>(st, segs, src, hist_scan, dst, kmax, conv,
+                                                     aoff);
+  else
+    scatter_units<kUsThreadsAny, kUsItemsAny, false, false>(st, segs, src, hist_scan, dst, kmax,
+                                                            conv, aoff);
+}
+
 // ---------------------------------------------------------------------------
 // Scatter of an unordered level (a full sort's levels after the first): the
 // in-SM sort orders (key, position) pairs, so elements of a bucket may leave
@@ -967,7 +1011,7 @@ k_scatter_atomic(const DevState* st, const LevelSeg* segs, Src src, const uint32
   const int lane = tid & 31, warp = tid >> 5;
   const uint32_t q0 = (uint32_t)warp * (IT * 32) + lane;
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = find_seg(segs, G, c, [](const LevelSeg& x) { return x.chunk_off; });
+    const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
     const LevelSeg sg = segs[g];
     const uint32_t k = sg.k;
     const uint64_t cl = c - sg.chunk_off;
@@ -1090,6 +1134,8 @@ void set_unit_scatter_attributes() {
         cudaFuncSetAttribute(k_scatter_units<kUsThreadsAny, kUsItemsAny, true, false>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)limit) != cudaSuccess ||
+        cudaFuncSetAttribute(k_scatter_units_auto, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)limit) != cudaSuccess ||
         cudaFuncSetAttribute(k_scatter_units<kUsThreadsAny, kUsItemsAny, false, false>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)limit) != cudaSuccess)
@@ -1116,7 +1162,7 @@ void launch_classify_ids(const LaunchEnv& e, const LevelParams& P, DevState* st,
     const uint64_t grid = umin64(P.chunk_cap, (uint64_t)e.num_sms * nb);
     Scope sc(e, name);
     k_classify_bulk<256><<<(int)(grid ? grid : 1), 256 + 32, smem, e.stream>>>(
-        st, segs, src, ssk, ssi, hist, kmax, mode, common);
+        st, segs, src, ssk, ssi, hist, kmax, mode, common, P.stable == kOrderAuto);
     return;
   }
   const size_t smem = classify_ids_smem_bytes(kmax, mode);
@@ -1127,20 +1173,21 @@ void launch_classify_ids(const LaunchEnv& e, const LevelParams& P, DevState* st,
   const uint64_t grid = umin64(P.chunk_cap, (uint64_t)e.num_sms * nb);
   // 16-byte pair loads need a 16-byte aligned key array
   const int vec = ((uintptr_t)src.key & 15) == 0;
+  const bool eq = P.stable == kOrderAuto;
   Scope sc(e, name);
   const int g = (int)(grid ? grid : 1);
   if (vec && src.map_f64)
     k_classify_ids<256, true, true><<<g, 256, smem, e.stream>>>(st, segs, src, ssk, ssi, hist,
-                                                                kmax, mode);
+                                                                kmax, mode, eq);
   else if (vec)
     k_classify_ids<256, true, false><<<g, 256, smem, e.stream>>>(st, segs, src, ssk, ssi, hist,
-                                                                 kmax, mode);
+                                                                 kmax, mode, eq);
   else if (src.map_f64)
     k_classify_ids<256, false, true><<<g, 256, smem, e.stream>>>(st, segs, src, ssk, ssi, hist,
-                                                                 kmax, mode);
+                                                                 kmax, mode, eq);
   else
     k_classify_ids<256, false, false><<<g, 256, smem, e.stream>>>(st, segs, src, ssk, ssi, hist,
-                                                                  kmax, mode);
+                                                                  kmax, mode, eq);
 }
 
 void launch_scatter_atomic(const LaunchEnv& e, const LevelParams& P, DevState* st,
@@ -1181,7 +1228,12 @@ void launch_scatter_units(const LaunchEnv& e, const LevelParams& P, DevState* st
   const int g = (int)(grid ? grid : 1);
   const size_t smem_s = us_smem_bytes(kmax, kUsThreads, kUsItems, true);
   const size_t smem_a = us_smem_bytes(kmax, kUsThreadsAny, kUsItemsAny, false);
-  const bool autoo = P.stable == kOrderAuto;
+  const bool autoo = P.stable == kOrderAuto;  // (level 1: no stored positions)
+  if (autoo && P.W <= kAutoOneLaunchW) {
+    k_scatter_units_auto<<<g, kUsThreads, umax64(smem_s, smem_a), e.stream>>>(
+        st, segs, src, hist_scan, dst, kmax, conv, aoff);
+    return;
+  }
   if (P.stable == 1 || autoo) {
     if (src.idx)
       k_scatter_units<kUsThreads, kUsItems, true, true><<<g, kUsThreads, smem_s, e.stream>>>(
@@ -1190,8 +1242,6 @@ void launch_scatter_units(const LaunchEnv& e, const LevelParams& P, DevState* st
       k_scatter_units<kUsThreads, kUsItems, false, true><<<g, kUsThreads, smem_s, e.stream>>>(
           st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
   }
-  // with the order left to the device both forms launch; the one not chosen
-  // returns at once
   if (autoo && e.launches) ++*e.launches;
   if (P.stable != 1 || autoo) {
     if (src.idx)
