@@ -386,10 +386,10 @@ rsort_status rsort_phase_times(rsort_ctx *ctx, const char **names, double *ms,
  *   wide_scatter_k  levels with at least this many buckets stage 4096-key
  *                sub-tiles with 512 threads when shared memory allows
  *                (default 1024).
- *   warp_direct_max_k  partition levels with at most this many buckets per
- *                segment classify and scatter per warp sub-chunk straight to
- *                HBM; larger levels stage every sub-tile through shared
- *                memory (default 0: always staged).
+ *   warp_direct_max_k  (0..2048, default 0) accepted for existing tune tables;
+ *                no effect: every level stages its sub-tiles through shared
+ *                memory, which measured 3x faster than scattering straight
+ *                from the warps.
  * Errors: EINVAL for an unknown name or an out-of-range value. */
 rsort_status rsort_set_tunable(rsort_ctx *ctx, const char *name, int64_t value);
 rsort_status rsort_get_tunable(rsort_ctx *ctx, const char *name, int64_t *value);

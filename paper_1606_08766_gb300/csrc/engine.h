@@ -56,8 +56,8 @@ struct rsort_ctx {
   // tunable "classifier": 0 splitter tree, 1 leading-bits table (default: the
   // table; both give the same buckets and the table measured faster on GB300)
   int classifier = 1;
-  // tunable "warp_direct_max_k": warp-direct kernels up to this k (default off:
-  // direct scattered stores measured ~3x slower than shared-memory combining)
+  // tunable "warp_direct_max_k": kept for existing tune tables, without effect
+  // (scattering straight from the warps was 3x slower than through shared memory)
   int wd_max_k = 0;
   // tunable "wide_scatter_k": levels with at least this many buckets stage
   // 4096-key sub-tiles with 512 threads (longer runs per bucket)

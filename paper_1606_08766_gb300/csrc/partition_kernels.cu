@@ -99,7 +99,7 @@ __device__ __forceinline__ void fill_segment(LevelSeg& s, uint64_t start, uint32
   s.S = S;
   s.nchunks = nch;
   s.nschunks = (S + kSampleChunk - 1) / kSampleChunk;
-  s.nunits = nch * (P.warp_direct ? kPartWarps : 1);
+  s.nunits = nch;
   // equal chunks inside the segment (the level's W bounds their size)
   s.W = nch ? (uint32_t)(((uint64_t)m + nch - 1) / nch) : P.W;
   s.pad = 0;
@@ -138,7 +138,7 @@ __device__ __forceinline__ SegIn plan_shape(const SegIn* list_in, uint32_t g, ui
   const uint32_t nch = in.m / P.W + (in.m % P.W ? 1u : 0u);
   v[0] = S;
   v[1] = nch;
-  v[2] = (uint64_t)k * nch * (P.warp_direct ? kPartWarps : 1);
+  v[2] = (uint64_t)k * nch;
   v[3] = (S + kSampleChunk - 1) / kSampleChunk;
   v[4] = k;
   v[5] = in.m;
@@ -494,7 +494,7 @@ constexpr size_t kSBufBytes = (size_t)kST * (8 + 4 + 2);
 // mode: bit 0 the classifier (0 tree, 1 table), bit 1 no tie-breaking.
 __host__ __device__ inline size_t part_common_bytes(uint32_t kmax, int mode) {
   const size_t Kp = next_pow2_u32(kmax);
-  size_t b = (mode & 1) == 0 ? Kp * 8 : ((size_t)4 << table_bits_for((uint32_t)Kp));
+  size_t b = (mode & 1) == 0 ? Kp * 8 : table_bytes((uint32_t)Kp);
   b += (size_t)kmax * 8 + (size_t)kmax * 4 + (size_t)kmax * 2 + (size_t)kmax * 4;
   return (b + 15) & ~(size_t)15;
 }
@@ -528,8 +528,8 @@ __device__ inline PartSmem carve(unsigned char* base, uint32_t kmax, bool scatte
     s.sp.tree = (uint64_t*)p;
     p += Kp * 8;
   } else {
-    s.sp.tbl = (uint32_t*)p;
-    p += (size_t)4 << table_bits_for((uint32_t)Kp);
+    s.sp.tbl = (uint16_t*)p;
+    p += table_bytes((uint32_t)Kp);
   }
   s.sp.key = (uint64_t*)p; p += (size_t)kmax * 8;
   s.sp.idx = (uint32_t*)p; p += (size_t)kmax * 4;
@@ -989,220 +989,6 @@ k_scatter(const DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk
   }
 }
 
-// ---------------------------------------------------------------------------
-// Warp-direct variant of steps 4-5a / 5c.  Every chunk is split into
-// kPartWarps contiguous warp sub-chunks; the histogram has one unit per
-// (chunk, warp).  A warp streams its own sub-chunk through kWdStages
-// cp.async stages of kWdKeys keys (warp-level waits only), ranks elements
-// among equal buckets with match counting, and writes them straight to HBM
-// from warp-private running offsets.  No block barrier inside a chunk; the
-// order inside a bucket is still the input order.
-// ---------------------------------------------------------------------------
-constexpr int kWdItems = 4;                   // keys per lane per stage
-constexpr int kWdKeys = 32 * kWdItems;        // keys per warp per stage
-constexpr int kWdStages = 2;
-
-__host__ __device__ inline size_t wd_smem_bytes(uint32_t kmax, int mode) {
-  return part_common_bytes(kmax, mode) + (size_t)kPartWarps * kmax * 4 +
-         (size_t)kPartWarps * kWdStages * kWdKeys * (8 + 4);
-}
-
-struct WdSmem {
-  Splitters sp;
-  uint32_t* rows;   // [kPartWarps][kmax]: counts (classify) / next position (scatter)
-  uint64_t* skey;   // [kPartWarps][kWdStages][kWdKeys]
-  uint32_t* sidx;   // [kPartWarps][kWdStages][kWdKeys]
-};
-
-__device__ inline WdSmem carve_wd(unsigned char* base, uint32_t kmax, int mode) {
-  PartSmem ps = carve(base, kmax, false, mode);
-  WdSmem w;
-  w.sp = ps.sp;
-  unsigned char* p = base + part_common_bytes(kmax, mode);
-  w.rows = (uint32_t*)p;
-  p += (size_t)kPartWarps * kmax * 4;
-  w.skey = (uint64_t*)p;
-  p += (size_t)kPartWarps * kWdStages * kWdKeys * 8;
-  w.sidx = (uint32_t*)p;
-  return w;
-}
-
-// This warp's sub-chunk [ws, we) of chunk [cs, ce).
-__device__ __forceinline__ void warp_subchunk(uint64_t cs, uint64_t ce, int warp, uint64_t& ws,
-                                              uint64_t& we) {
-  const uint64_t cnt = ce - cs;
-  const uint64_t wsz = (cnt + kPartWarps - 1) / kPartWarps;
-  ws = cs + umin64((uint64_t)warp * wsz, cnt);
-  we = cs + umin64((uint64_t)(warp + 1) * wsz, cnt);
-}
-
-__global__ void __launch_bounds__(kPartThreads, 3)
-k_classify_count_wd(const DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
-                    const uint32_t* ssi, uint32_t* hist, uint32_t W, uint32_t kmax, int mode) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  WdSmem sm = carve_wd(smem_raw, kmax, mode);
-  const uint64_t pol = l2_evict_first_policy();
-  const uint64_t total = st->total_chunks;
-  const uint32_t G = st->cur_nseg;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t* row = sm.rows + (size_t)warp * kmax;
-  uint64_t* stk = sm.skey + (size_t)warp * kWdStages * kWdKeys;
-  uint32_t cur_g = 0xffffffffu;
-  for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
-    const LevelSeg sg = segs[g];
-    __syncthreads();
-    if (g != cur_g) {
-      load_splitters<kPartThreads>(sg, ssk, ssi, sm.sp);
-      cur_g = g;
-    }
-    const uint32_t k = sg.k;
-    for (uint32_t b = lane; b < k; b += 32) row[b] = 0;
-    const uint64_t cl = c - sg.chunk_off;
-    const uint64_t cs = sg.start + cl * sg.W;
-    const uint64_t ce = umin64(cs + sg.W, sg.start + sg.m);
-    uint64_t ws, we;
-    warp_subchunk(cs, ce, warp, ws, we);
-    const uint64_t nsteps = (we - ws + kWdKeys - 1) / kWdKeys;
-    auto issue = [&](uint64_t t) {
-      if (t < nsteps) {
-        const uint64_t b0 = ws + t * kWdKeys;
-        uint64_t* dstk = stk + (t % kWdStages) * kWdKeys;
-#pragma unroll
-        for (int r = 0; r < kWdItems; ++r) {
-          const uint32_t q = r * 32 + lane;
-          if (b0 + q < we) cp_async_8(dstk + q, src.key + b0 + q, pol);
-        }
-      }
-      cp_async_commit();
-    };
-    issue(0);
-    __syncwarp();
-    for (uint64_t t = 0; t < nsteps; ++t) {
-      issue(t + 1);
-      cp_async_wait<1>();
-      __syncwarp();
-      const uint64_t b0 = ws + t * kWdKeys;
-      const uint64_t* sk = stk + (t % kWdStages) * kWdKeys;
-      uint64_t key[kWdItems];
-#pragma unroll
-      for (int r = 0; r < kWdItems; ++r) {
-        const uint32_t q = r * 32 + lane;
-        const uint64_t kv = b0 + q < we ? sk[q] : 0;
-        key[r] = src.map_f64 ? f64_to_ordered(kv) : kv;
-      }
-      uint32_t bk[kWdItems];
-      // (never past the sub-chunk: a padding slot's result is discarded)
-      classify_batch<kWdItems>(key, bk, [&](int r) {
-        const uint64_t pos = b0 + r * 32 + lane;
-        if (pos >= we) return 0u;
-        return src.idx ? src.idx[pos] : (uint32_t)(pos - sg.start);
-      }, sm.sp);
-#pragma unroll
-      for (int r = 0; r < kWdItems; ++r) {
-        const bool v = b0 + r * 32 + lane < we;
-        const uint32_t b = v ? bk[r] : 0xffffffffu;
-        const uint32_t peers = __match_any_sync(0xffffffffu, b);
-        if (v && lane == __ffs(peers) - 1) row[b] += __popc(peers);
-        __syncwarp();
-      }
-    }
-    cp_async_wait<0>();
-    __syncwarp();
-    for (uint32_t b = lane; b < k; b += 32)
-      hist[sg.hist_off + (uint64_t)b * sg.nunits + cl * kPartWarps + warp] = row[b];
-  }
-}
-
-__global__ void __launch_bounds__(kPartThreads, 3)
-k_scatter_wd(const DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
-             const uint32_t* ssi, const uint32_t* hist_scan, Dst dst, uint32_t W, uint32_t kmax,
-             int unmap_out, int mode) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  WdSmem sm = carve_wd(smem_raw, kmax, mode);
-  const uint64_t pol = l2_evict_first_policy();
-  const uint64_t total = st->total_chunks;
-  const uint32_t G = st->cur_nseg;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t ltmask = lanemask_lt();
-  uint32_t* row = sm.rows + (size_t)warp * kmax;
-  uint64_t* stk = sm.skey + (size_t)warp * kWdStages * kWdKeys;
-  uint32_t* sti = sm.sidx + (size_t)warp * kWdStages * kWdKeys;
-  uint32_t cur_g = 0xffffffffu;
-  for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
-    const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
-    const LevelSeg sg = segs[g];
-    __syncthreads();
-    if (g != cur_g) {
-      load_splitters<kPartThreads>(sg, ssk, ssi, sm.sp);
-      cur_g = g;
-    }
-    const uint32_t k = sg.k;
-    const uint64_t cl = c - sg.chunk_off;
-    for (uint32_t b = lane; b < k; b += 32)
-      row[b] = (uint32_t)(hist_scan[sg.hist_off + (uint64_t)b * sg.nunits + cl * kPartWarps +
-                                    warp] + sg.delta);
-    const uint64_t cs = sg.start + cl * sg.W;
-    const uint64_t ce = umin64(cs + sg.W, sg.start + sg.m);
-    uint64_t ws, we;
-    warp_subchunk(cs, ce, warp, ws, we);
-    const uint64_t nsteps = (we - ws + kWdKeys - 1) / kWdKeys;
-    auto issue = [&](uint64_t t) {
-      if (t < nsteps) {
-        const uint64_t b0 = ws + t * kWdKeys;
-        const size_t so = (t % kWdStages) * kWdKeys;
-#pragma unroll
-        for (int r = 0; r < kWdItems; ++r) {
-          const uint32_t q = r * 32 + lane;
-          if (b0 + q < we) {
-            cp_async_8(stk + so + q, src.key + b0 + q, pol);
-            if (src.idx) cp_async_4(sti + so + q, src.idx + b0 + q, pol);
-          }
-        }
-      }
-      cp_async_commit();
-    };
-    issue(0);
-    __syncwarp();
-    for (uint64_t t = 0; t < nsteps; ++t) {
-      issue(t + 1);
-      cp_async_wait<1>();
-      __syncwarp();
-      const uint64_t b0 = ws + t * kWdKeys;
-      const size_t so = (t % kWdStages) * kWdKeys;
-      uint64_t key[kWdItems];
-      uint32_t idx[kWdItems];
-#pragma unroll
-      for (int r = 0; r < kWdItems; ++r) {
-        const uint32_t q = r * 32 + lane;
-        const bool v = b0 + q < we;
-        const uint64_t kv = v ? stk[so + q] : 0;
-        key[r] = src.map_f64 ? f64_to_ordered(kv) : kv;
-        idx[r] = v ? (src.idx ? sti[so + q] : (uint32_t)(b0 + q - sg.start)) : 0;
-      }
-      uint32_t bk[kWdItems];
-      classify_batch<kWdItems>(key, bk, [&](int r) { return idx[r]; }, sm.sp);
-#pragma unroll
-      for (int r = 0; r < kWdItems; ++r) {
-        const bool v = b0 + r * 32 + lane < we;
-        const uint32_t b = v ? bk[r] : 0xffffffffu;
-        const uint32_t peers = __match_any_sync(0xffffffffu, b);
-        const uint32_t c0 = v ? row[b] : 0;
-        __syncwarp();
-        if (v && lane == __ffs(peers) - 1) row[b] = c0 + __popc(peers);
-        __syncwarp();
-        if (v) {
-          const uint64_t d = (uint64_t)c0 + __popc(peers & ltmask);
-          dst.key[d] = unmap_out ? ordered_to_f64(key[r]) : key[r];
-          dst.idx[d] = idx[r];
-        }
-      }
-    }
-    cp_async_wait<0>();
-    __syncwarp();
-  }
-}
-
 // Collect the buckets of the level: bucket sizes follow from the scanned
 // histogram.  Buckets that fit one SM, equality buckets of a stable level on
 // input in position order (both bounding splitters share one key, so every
@@ -1326,7 +1112,7 @@ constexpr int kGreedyThreads = 1024;
 
 __host__ __device__ inline size_t fine_smem_bytes(uint32_t K) {
   const uint32_t Kp = next_pow2_u32(K);
-  return ((size_t)4 << table_bits_for(Kp)) + (size_t)K * (8 + 4 + 4 + 2);
+  return table_bytes(Kp) + (size_t)K * (8 + 4 + 4 + 2);
 }
 
 __host__ __device__ inline size_t greedy_smem_bytes(uint32_t K, uint32_t k) {
@@ -1347,8 +1133,8 @@ k_fine_count(const LevelSeg* segs, Src src, const uint64_t* ssk, const uint32_t*
   sp.ntb = ntb;
   sp.tree = nullptr;
   unsigned char* p = smem_raw;
-  sp.tbl = (uint32_t*)p;
-  p += (size_t)4 << table_bits_for(next_pow2_u32(K));
+  sp.tbl = (uint16_t*)p;
+  p += table_bytes(next_pow2_u32(K));
   sp.key = (uint64_t*)p;
   p += (size_t)K * 8;
   sp.idx = (uint32_t*)p;
@@ -1694,19 +1480,6 @@ void set_partition_kernel_attributes() {
   cudaFuncSetAttribute(k_group_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)greedy_smem_bytes(kMaxFine, kMaxK));
   cudaGetLastError();  // a refused attribute only disables the variant
-  const size_t w = umax64(wd_smem_bytes(kMaxK, 0), wd_smem_bytes(kMaxK, 1));
-  cudaFuncSetAttribute(k_classify_count_wd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w);
-  cudaFuncSetAttribute(k_scatter_wd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w);
-}
-
-int wd_blocks_per_sm(uint32_t kmax, bool scatter, int mode) {
-  int nb = 0;
-  const size_t smem = wd_smem_bytes(kmax, mode);
-  if (scatter)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_scatter_wd, kPartThreads, smem);
-  else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_classify_count_wd, kPartThreads, smem);
-  return nb > 0 ? nb : 1;
 }
 
 // Resident CTAs per SM of the classify / scatter kernels for a bucket bound.
@@ -1843,7 +1616,7 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
     const uint64_t a = P.hinted ? 16ull * lg : (uint64_t)P.oversample;
     ps.S = (uint32_t)umin64(umin64(n_total, a * k_plain), P.samp_max);
     ps.local = e.local;
-    plain_hist = (uint64_t)k_plain * ps.nch * (P.warp_direct ? kPartWarps : 1);
+    plain_hist = (uint64_t)k_plain * ps.nch;
     const uint64_t nsch = (ps.S + kSampleChunk - 1) / kSampleChunk;
     auto draw = [&](auto nt, auto it) {
       launch_sample_sort<decltype(nt)::value, decltype(it)::value, 1>(
@@ -1903,19 +1676,13 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
   const bool stable = P.stable == 1;
   const int grid_s = grid_for(P.chunk_cap, 1,
                               sms * part_blocks_per_sm((uint32_t)kmax_level, true, mode, stable));
-  const size_t smem_wd = wd_smem_bytes((uint32_t)kmax_level, mode);
-  const int grid_wd_c =
-      grid_for(P.chunk_cap, 1, sms * wd_blocks_per_sm((uint32_t)kmax_level, false, mode));
-  const int grid_wd_s =
-      grid_for(P.chunk_cap, 1, sms * wd_blocks_per_sm((uint32_t)kmax_level, true, mode));
-  const bool wide = !P.warp_direct && kmax_level >= P.wide_scatter_k &&
+  const bool wide = kmax_level >= P.wide_scatter_k &&
                     scatter_smem_bytes((uint32_t)kmax_level, mode, 16, 4096, stable) <=
                         g_wide_scatter_smem_max;
   // A stable level with at most kUnitMaxK buckets classifies once, storing
   // every element's bucket id, and scatters whole 8-element units
   // (unit_scatter.cu).  Otherwise stored bucket ids spare the staged scatter
-  // its second classification, except in the warp-direct scatter and at
-  // 1024+ buckets, where the staged scatter's L2-resident write frontiers
+  // its second classification, except at 1024+ buckets, where the staged scatter's L2-resident write frontiers
   // were the bottleneck and the extra id stream measured slower.
   // With atomic_scatter, an unordered level (a full sort's levels after the
   // first) keeps the ids of its classify pass and ranks by shared-memory
@@ -1923,23 +1690,17 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
   // scatter at 2^28 keys with ~171 buckets per segment; a tuner candidate).
   // (a level that need not keep input order -- a full sort's levels -- has
   // the unit scatter rank by shared-memory atomics)
-  const bool units = P.unit_scatter && !P.warp_direct && src.bid != nullptr &&
+  const bool units = P.unit_scatter && src.bid != nullptr &&
                      kmax_level > 32 && unit_scatter_fits((uint32_t)kmax_level);
-  const bool atomics = !units && P.atomic_scatter && !stable && !P.warp_direct &&
+  const bool atomics = !units && P.atomic_scatter && !stable &&
                        src.bid != nullptr && atomic_scatter_fits((uint32_t)kmax_level);
-  if (!units && !atomics && (P.warp_direct || kmax_level >= 1024)) src.bid = nullptr;
-  // Deeper levels keep the staged classify below, which stores the ids as
-  // well: with many short chunks it measured faster (1.00 vs 1.09 ms at 2^28
-  // keys) than the register-streaming one.
-  if (units && P.level == 1) {
+  if (!units && !atomics && kmax_level >= 1024) src.bid = nullptr;
+  if (units) {
     launch_classify_ids(e, P, st, segs, src, ssamp_key, ssamp_idx, hist, (uint32_t)kmax_level,
                         mode, nm[3]);
   } else {
     Scope sc(e, nm[3]);
-    if (P.warp_direct)
-      k_classify_count_wd<<<grid_wd_c, kPartThreads, smem_wd, e.stream>>>(
-          st, segs, src, ssamp_key, ssamp_idx, hist, P.W, (uint32_t)kmax_level, mode);
-    else if (deep_c)
+    if (deep_c)
       k_classify_count<kCStagesDeep><<<grid_c, kPartThreads, smem_cd, e.stream>>>(
           st, segs, src, ssamp_key, ssamp_idx, hist, P.W, (uint32_t)kmax_level, mode);
     else
@@ -1970,11 +1731,7 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
     launch_scatter_atomic(e, P, st, segs, src, hist, dst, (uint32_t)kmax_level, unmap_out, nm[6]);
   } else {
     Scope sc(e, nm[6]);
-    if (P.warp_direct)
-      k_scatter_wd<<<grid_wd_s, kPartThreads, smem_wd, e.stream>>>(
-          st, segs, src, ssamp_key, ssamp_idx, hist, dst, P.W, (uint32_t)kmax_level, unmap_out,
-          mode);
-    else if (wide && stable)
+    if (wide && stable)
       k_scatter<512, 4096, true>
           <<<grid_for(P.chunk_cap, 1,
                       sms * wide_scatter_blocks_per_sm((uint32_t)kmax_level, mode, true)),

@@ -106,7 +106,6 @@ struct Plan {
   uint64_t samp_cap1 = 0, hist_cap1 = 0, chunk_cap1 = 0, schunk_cap1 = 0, bucket_cap1 = 0;
   bool need_tmp = false;
   int classifier = 0;       // 0: splitter tree, 1: leading-bits table
-  int wd_max_k = 0;         // levels with at most this many buckets run warp-direct
   int wide_scatter_k = 1024;  // levels with at least this many buckets use wide sub-tiles
   uint32_t target_bucket = kTargetBucket;  // automatic fan-out target
   uint32_t target_by_class[33] = {};       // per segment-size class (0: target_bucket)
@@ -191,11 +190,11 @@ void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int
              3 * mean1 <= 2 * (uint64_t)kMaxKDeep * tmin)
       needed = 2;
     levels = std::min(levels, needed);
-    // most samples of a deeper segment: its expected size is mean1, twice that
-    // is far outside what the sampling leaves; the bound lets small CTAs sort
-    // small samples (a segment beyond it only gets fewer samples a bucket)
+    // most samples of a deeper segment: its expected size is mean1, 1.45 times
+    // that is far outside what the sampling leaves; the bound lets small CTAs
+    // sort small samples (a larger segment only gets fewer samples a bucket)
     if (g1 == 1) {
-      const uint64_t k2 = std::min<uint64_t>(2 * mean1 / tmin + 1, kMaxKDeep);
+      const uint64_t k2 = std::min<uint64_t>(145 * mean1 / (100 * tmin) + 1, kMaxKDeep);
       p.samp_max = k2 * kDeepOversample <= 1024   ? 1024
                    : k2 * kDeepOversample <= 4096 ? 4096
                                                   : kMaxKDeep * kDeepOversample;
@@ -249,16 +248,13 @@ void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int
   const uint64_t a1 = k1 >= 2 ? 16ull * ceil_log2_host(k1) : (uint64_t)p.oversample1;
   p.samp_cap1 = std::min<uint64_t>(n, a1 * p.bucket_cap1);
   p.chunk_cap1 = n / p.W1 + g1 + 1;
-  // (a warp-direct level has one histogram unit per warp sub-chunk)
-  const uint64_t units1 = (int)kmax1 <= p.wd_max_k ? kPartWarps : 1;
-  p.hist_cap1 = ((uint64_t)kmax1 * (n / p.W1) + p.bucket_cap1) * units1;
+  p.hist_cap1 = (uint64_t)kmax1 * (n / p.W1) + p.bucket_cap1;
   p.schunk_cap1 = p.samp_cap1 / kSampleChunk + g1 + 1;
   // deeper levels
   const uint64_t bucket_capd = n / tmin + segs_deep + 1;
   const uint64_t samp_capd = std::min<uint64_t>(n, (uint64_t)kDeepOversample * bucket_capd);
   const uint64_t chunk_capd = n / p.Wd + segs_deep + 1;
-  const uint64_t unitsd = kMaxKDeep <= p.wd_max_k ? kPartWarps : 1;
-  const uint64_t hist_capd = ((uint64_t)kMaxKDeep * (n / p.Wd) + bucket_capd) * unitsd;
+  const uint64_t hist_capd = (uint64_t)kMaxKDeep * (n / p.Wd) + bucket_capd;
   const uint64_t schunk_capd = samp_capd / kSampleChunk + segs_deep + 1;
   const bool deep = levels > 1;
   p.bucket_cap = std::max<uint64_t>(p.bucket_cap1, deep ? bucket_capd : 0);
@@ -269,7 +265,7 @@ void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int
   p.final_cap = p.bucket_cap1 + (uint64_t)(levels - 1) * bucket_capd + 4;
 }
 
-LevelParams level_params(const Plan& p, int level, uint64_t seed, int kmax_level) {
+LevelParams level_params(const Plan& p, int level, uint64_t seed) {
   LevelParams P;
   P.level = level;
   P.W = level == 1 ? p.W1 : p.Wd;
@@ -294,7 +290,6 @@ LevelParams level_params(const Plan& p, int level, uint64_t seed, int kmax_level
   P.oversample = p.oversample1;
   P.level1_oversample = 1;
   P.classifier = p.classifier;
-  P.warp_direct = kmax_level <= p.wd_max_k ? 1 : 0;
   P.wide_scatter_k = p.wide_scatter_k;
   P.target_bucket = p.target_bucket;
   for (int i = 0; i <= 32; ++i) P.target_by_class[i] = p.target_by_class[i];
@@ -350,7 +345,7 @@ void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const 
   auto level_dst = [&](int L) -> const Dst& { return ((L + l1_out) & 1) ? tmp : out; };
   for (int L = 1; L <= p.levels; ++L) {
     const int kmax = L == 1 ? (k1 >= 2 ? (int)k1 : kMaxKDeep) : kMaxKDeep;
-    LevelParams P = level_params(p, L, seed, kmax);
+    LevelParams P = level_params(p, L, seed);
     // the levels keep input order inside buckets or not as the tunables say
     // (the in-SM sort orders (key, position) pairs either way; level 1's
     // default leaves it to the device); a level's input is in position order
@@ -549,7 +544,6 @@ namespace {
 Plan plan_sort(rsort_ctx* c, uint64_t n, uint32_t p_virtual) {
   Plan p;
   p.classifier = c->classifier;
-  p.wd_max_k = c->wd_max_k;
   p.wide_scatter_k = c->wide_scatter_k;
   p.target_bucket = c->target_bucket;
   for (int i = 0; i <= 32; ++i) p.target_by_class[i] = c->target_by_class[i];
@@ -582,7 +576,6 @@ Plan plan_sort(rsort_ctx* c, uint64_t n, uint32_t p_virtual) {
 Plan plan_segmented(rsort_ctx* c, uint64_t n, uint32_t num_segments) {
   Plan p;
   p.classifier = c->classifier;
-  p.wd_max_k = c->wd_max_k;
   p.wide_scatter_k = c->wide_scatter_k;
   p.target_bucket = c->target_bucket;
   for (int i = 0; i <= 32; ++i) p.target_by_class[i] = c->target_by_class[i];
@@ -801,7 +794,6 @@ rsort_status partition_impl(rsort_ctx* c, rsort_key_type type, const void* d_key
   }
   Plan p;
   p.classifier = c->classifier;
-  p.wd_max_k = c->wd_max_k;
   p.wide_scatter_k = c->wide_scatter_k;
   p.target_bucket = c->target_bucket;
   for (int i = 0; i <= 32; ++i) p.target_by_class[i] = c->target_by_class[i];
@@ -827,7 +819,7 @@ rsort_status partition_impl(rsort_ctx* c, rsort_key_type type, const void* d_key
   if (rs != RSORT_OK) return latch(c, rs);
   DevState* st = at<DevState>(ws, p.off_state);
   SegIn* list1 = at<SegIn>(ws, p.off_list1);
-  LevelParams P = level_params(p, 1, seed, (int)kk);
+  LevelParams P = level_params(p, 1, seed);
   P.no_tie_break = tie_break ? 0 : 1;
   Src src{(const uint64_t*)d_keys_in, nullptr, type == RSORT_KEY_F64};
   src.bid = at<uint16_t>(ws, p.off_bid);

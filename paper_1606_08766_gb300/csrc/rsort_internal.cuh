@@ -132,7 +132,7 @@ struct LevelSeg {
   uint32_t S;
   uint32_t nchunks;
   uint32_t nschunks;
-  uint32_t nunits;      // histogram units: nchunks (CTA chunks) or 8 * nchunks (warp sub-chunks)
+  uint32_t nunits;      // histogram units (one per chunk)
   uint32_t W;           // keys per chunk of this segment (all chunks equal but the last)
   uint32_t pad;
   KeyRange range;       // of the segment's keys
@@ -220,7 +220,6 @@ struct LevelParams {
   uint32_t oversample = kDeepOversample;
   int level1_oversample;  // 1: a = 16 ceil(log2 k) for hinted k (the paper's rule)
   int classifier;         // 0: splitter tree, 1: leading-bits table
-  int warp_direct;        // 1: per-warp sub-chunks scattered straight to HBM
   int wide_scatter_k;     // levels with at least this many buckets scatter 4096-key sub-tiles
   uint32_t target_bucket; // automatic fan-out aims at buckets of this many keys
   // per segment-size class c = ceil(log2 m): the fan-out target for segments

@@ -52,19 +52,24 @@ __device__ __forceinline__ uint64_t load_key(const Src& s, uint64_t pos) {
 //   tree   the branchless implicit search tree of Super Scalar Sample Sort that
 //          the appendix names: the keys in Eytzinger order, padded with
 //          UINT64_MAX to Kp - 1 = next_pow2(k) - 1 nodes;
-//   table  a lookup table over the leading bits of (key - smallest splitter
-//          key) giving, for every bin, the range of splitters whose key falls
-//          in it; a key is located by one table read and a binary search over
-//          its bin's splitters (a full binary search when keys cluster).
+//   table  a lookup table of 4 to 8 bins per splitter over the leading bits of
+//          (key - smallest splitter key) giving every bin's first splitter; a
+//          key steps from there to the first splitter that is not smaller, one
+//          or two reads, as long as no bin holds more than kLinearMax; else it
+//          searches its bin's splitters by halving.  float64 keys, whose bit
+//          patterns crowd a few octaves of a range of thousands, get bins of
+//          equal width in value instead where that keeps them small (2*10^7
+//          normal keys, 512 buckets: 194 us with 150 splitters in a bin, 81).
 // A key equal to splitter keys is then placed among the run of those
 // splitters by its position (tie_break).
 // ---------------------------------------------------------------------------
-constexpr int kTableBitsMax = 12;
+constexpr int kTableBitsMax = 13;
+constexpr uint32_t kLinearMax = 6;
 
 struct Splitters {
   uint64_t* tree;   // [Kp]   node i at tree[i], i = 1..Kp-1          (tree mode)
-  uint32_t* tbl;    // [2^tbits] packed (first, end) splitter of a bin (table mode)
-  uint64_t* key;    // [k-1]  sorted splitter keys
+  uint16_t* tbl;    // [2^tbits] first splitter of a bin (table mode)
+  uint64_t* key;    // [k]    sorted splitter keys, then UINT64_MAX
   uint32_t* idx;    // [k-1]  their positions (tie-breakers)
   uint16_t* rend;   // [k-1]  end of the run of splitters whose key equals key[j]
   uint64_t lo, hi;  // smallest / largest splitter key
@@ -72,40 +77,113 @@ struct Splitters {
   int tbits;        // table bits
   uint32_t tmax;    // last table entry (2^tbits - 1)
   int shift;        // key bits dropped before the table index
+  int linear;       // 1: no bin holds more than kLinearMax splitters
+  int by_value;     // 1: bins of equal width in float64 value
+  float flo, fscale;  // value of the smallest splitter, bins per unit
   int mode;         // 0 tree, 1 table
   int ntb;          // 1: no tie-breaking, classify by key only (ablation)
   uint32_t nspl;    // k - 1
 };
 
 __host__ __device__ inline int table_bits_for(uint32_t kp) {
-  const int b = log2_u32(kp) + 1;
+  const int b = log2_u32(kp) + 2;
   return b < kTableBitsMax ? b : kTableBitsMax;
 }
+__host__ __device__ inline size_t table_bytes(uint32_t kp) {
+  return (size_t)2 << table_bits_for(kp);
+}
 
-template <int NT>
+// Bin of a key in the table.  Monotone in the key either way: the conversion to
+// float, the subtraction and the product round monotonically, and the keys
+// beyond the largest splitter (infinities and NaNs among them) take the last
+// bin.
+__device__ __forceinline__ uint32_t bin_by_bits(uint64_t x, const Splitters& sp) {
+  const uint64_t t = (x > sp.lo ? x - sp.lo : 0ull) >> sp.shift;
+  return t < sp.tmax ? (uint32_t)t : sp.tmax;
+}
+__device__ __forceinline__ uint32_t bin_by_value(uint64_t x, const Splitters& sp) {
+  const float v = (float)__longlong_as_double((long long)ordered_to_f64(x));
+  const uint32_t t = __float2uint_rz(__fmul_rn(__fsub_rn(v, sp.flo), sp.fscale));
+  return x > sp.hi || t > sp.tmax ? sp.tmax : t;
+}
+
+// Fills the table by a histogram of the splitters' bins and its exclusive scan;
+// returns the largest bin's splitters (the same in every thread).
+template <int NT, typename BinFn>
+__device__ __forceinline__ uint32_t build_table(const Splitters& sp, BinFn bin_of) {
+  __shared__ uint32_t s_scan[NT / 32];
+  __shared__ uint32_t s_max;
+  const uint32_t words = (sp.tmax + 1) / 2;
+  uint32_t* w = reinterpret_cast<uint32_t*>(sp.tbl);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (uint32_t q = threadIdx.x; q < words; q += NT) w[q] = 0;
+  if (threadIdx.x == 0) s_max = 0;
+  __syncthreads();
+  for (uint32_t j = threadIdx.x; j < sp.nspl; j += NT) {
+    const uint32_t t = bin_of(sp.key[j]);
+    atomicAdd(&w[t >> 1], 1u << ((t & 1) << 4));
+  }
+  __syncthreads();
+  const uint32_t per = (words + NT - 1) / NT;
+  const uint32_t q0 = min(threadIdx.x * per, words), q1 = min(q0 + per, words);
+  uint32_t sum = 0, most = 0;
+  for (uint32_t q = q0; q < q1; ++q) {
+    const uint32_t a = w[q] & 0xffffu, b = w[q] >> 16;
+    sum += a + b;
+    most = max(most, max(a, b));
+  }
+  uint32_t inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  most = __reduce_max_sync(0xffffffffu, most);
+  if (lane == 31) s_scan[warp] = inc;
+  if (lane == 0) atomicMax(&s_max, most);
+  __syncthreads();
+  uint32_t at = inc - sum;
+  for (int q = 0; q < warp; ++q) at += s_scan[q];
+  for (uint32_t q = q0; q < q1; ++q) {
+    const uint32_t a = w[q] & 0xffffu, b = w[q] >> 16;
+    w[q] = at | ((at + a) << 16);
+    at += a + b;
+  }
+  most = s_max;
+  __syncthreads();
+  return most;
+}
+
+// F64: the keys are mapped float64 patterns (bins by value are tried).
+template <int NT, bool F64 = false>
 __device__ void load_splitters(const LevelSeg& sg, const uint64_t* ssk, const uint32_t* ssi,
                                Splitters& sp) {
   const uint32_t k = sg.k;
   const uint32_t Kp = next_pow2_u32(k);
   sp.nspl = k - 1;
   sp.logK = log2_u32(Kp);
+  // (j + 1) S < 2^32: at most kMaxFine splitters of 16 * 11 * kMaxK samples
+  static_assert((uint64_t)kMaxFine * 16 * 11 * kMaxK < (1ull << 32), "32-bit sample ranks");
   for (uint32_t j = threadIdx.x; j < sp.nspl; j += NT) {
-    const uint64_t r = ((uint64_t)(j + 1) * sg.S) / k;
+    const uint32_t r = (j + 1) * sg.S / k;
     sp.key[j] = ssk[sg.samp_off + r];
     sp.idx[j] = ssi[sg.samp_off + r];
   }
+  if (threadIdx.x == 0) sp.key[sp.nspl] = ~0ULL;
   __syncthreads();
   // end of every run of equal splitter keys (keys are sorted, so the run of
   // key[j] is contiguous); tie-breaks search positions inside the run only
   for (uint32_t j = threadIdx.x; j < sp.nspl; j += NT) {
     const uint64_t kj = sp.key[j];
     uint32_t lo = j + 1, hi = sp.nspl;
+    if (lo < hi && sp.key[lo] != kj) hi = lo;
     while (lo < hi) {
       const uint32_t mid = (lo + hi) >> 1;
       if (sp.key[mid] == kj) lo = mid + 1; else hi = mid;
     }
     sp.rend[j] = (uint16_t)lo;
   }
+  sp.by_value = 0;
   if (sp.mode == 0) {
     for (uint32_t i = threadIdx.x + 1; i < Kp; i += NT) {
       const int d = 31 - __clz(i);
@@ -120,19 +198,26 @@ __device__ void load_splitters(const LevelSeg& sg, const uint64_t* ssk, const ui
     const int bits = range ? 64 - __clzll((long long)range) : 0;
     sp.tbits = table_bits_for(Kp);
     sp.shift = bits > sp.tbits ? bits - sp.tbits : 0;
-    const uint32_t T = 1u << sp.tbits;
-    sp.tmax = T - 1;
-    // first splitter whose bin is >= t, by binary search over the sorted keys
-    auto first_at_least = [&](uint32_t t) {
-      uint32_t lo = 0, hi = sp.nspl;
-      while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (((sp.key[mid] - sp.lo) >> sp.shift) < t) lo = mid + 1; else hi = mid;
+    sp.tmax = (1u << sp.tbits) - 1;
+    uint32_t most = build_table<NT>(sp, [&](uint64_t x) { return bin_by_bits(x, sp); });
+    if (F64 && most > kLinearMax) {
+      const double vlo = __longlong_as_double((long long)ordered_to_f64(sp.lo));
+      const double vhi = __longlong_as_double((long long)ordered_to_f64(sp.hi));
+      const float flo = (float)vlo, fscale = (float)(sp.tmax + 1) / ((float)vhi - flo);
+      // (finite values, and a finite scale; NaNs fail every comparison)
+      if (vlo > -1e37 && vhi < 1e37 && fscale > 0.0f && fscale < 1e37f) {
+        sp.flo = flo;
+        sp.fscale = fscale;
+        const uint32_t mv = build_table<NT>(sp, [&](uint64_t x) { return bin_by_value(x, sp); });
+        if (mv <= kLinearMax || 2 * mv < most) {
+          sp.by_value = 1;
+          most = mv;
+        } else {
+          build_table<NT>(sp, [&](uint64_t x) { return bin_by_bits(x, sp); });
+        }
       }
-      return lo;
-    };
-    for (uint32_t t = threadIdx.x; t < T; t += NT)
-      sp.tbl[t] = first_at_least(t) | (first_at_least(t + 1) << 16);
+    }
+    sp.linear = most <= kLinearMax;
   } else {
     // no splitters: one bin, empty, so every key lands in bucket 0
     sp.lo = 0;
@@ -140,6 +225,7 @@ __device__ void load_splitters(const LevelSeg& sg, const uint64_t* ssk, const ui
     sp.tbits = 0;
     sp.tmax = 0;
     sp.shift = 0;
+    sp.linear = 0;
     if (threadIdx.x == 0) sp.tbl[0] = 0;
   }
   __syncthreads();
@@ -225,43 +311,50 @@ __device__ __forceinline__ void classify_batch_tree(const uint64_t (&x)[R], uint
   }
 }
 
-// Same result through the leading-bits table: one table read per element, then
-// a lower-bound search over the splitters of its bin (usually 0-2 of them).
+// Same result through the table: one table read per element, then the first
+// splitter of its bin that is not smaller, step by step where the bins are
+// small (usually the first one read) and by halving otherwise.
 // PAIRS: elements 2j and 2j+1 sit at consecutive positions whenever
 // valid(2j) and valid(2j+1); when both tie with the same run of splitter keys,
 // the second element's bucket is the first's or the next (splitter positions
 // are distinct, so at most one more of them lies below it): one comparison
 // instead of a search.
-template <int R, bool PAIRS = false, typename PosFn, typename ValidFn>
+template <int R, bool PAIRS = false, bool F64 = false, typename PosFn, typename ValidFn>
 __device__ __forceinline__ void classify_batch_table(const uint64_t (&x)[R], uint32_t (&b)[R],
                                                      PosFn pos_of, ValidFn valid,
                                                      const Splitters& sp) {
   // A key below the smallest splitter reads bin 0 and one above the largest
   // the last bin: each then finds no splitter on its far side, so no case
   // needs its own branch.
-  uint32_t pr[R];
+  uint64_t ub[R];  // key of the first splitter that is not smaller
+  if (sp.linear) {
+    if (F64 && sp.by_value) {
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const uint64_t t = (x[r] > sp.lo ? x[r] - sp.lo : 0ull) >> sp.shift;
-    pr[r] = sp.tbl[t < sp.tmax ? (uint32_t)t : sp.tmax];
-  }
-  bool prev_tied = false;
-  uint32_t prev_b = 0;
+      for (int r = 0; r < R; ++r) b[r] = sp.tbl[bin_by_value(x[r], sp)];
+    } else {
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    uint32_t bb;
-    bool tied = false;
-    {
-      uint32_t lo = pr[r] & 0xffffu, hi = pr[r] >> 16;
-      const uint32_t end = hi;
-      uint64_t ub = ~0ULL;
+      for (int r = 0; r < R; ++r) b[r] = sp.tbl[bin_by_bits(x[r], sp)];
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) ub[r] = sp.key[b[r]];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      // (the key after the last splitter is the largest there is)
+      while (ub[r] < x[r]) ub[r] = sp.key[++b[r]];
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const uint32_t t = F64 && sp.by_value ? bin_by_value(x[r], sp) : bin_by_bits(x[r], sp);
+      uint32_t lo = sp.tbl[t], hi = t < sp.tmax ? (uint32_t)sp.tbl[t + 1] : sp.nspl;
+      uint64_t u = sp.key[hi];
       // the bin's first splitter may already bound x (always so when a run of
       // copies of x fills the bin): then no search is needed
       if (lo < hi) {
         const uint64_t k0 = sp.key[lo];
         if (k0 >= x[r]) {
           hi = lo;
-          ub = k0;
+          u = k0;
         } else {
           ++lo;
         }
@@ -273,23 +366,31 @@ __device__ __forceinline__ void classify_batch_table(const uint64_t (&x)[R], uin
           lo = mid + 1;
         } else {
           hi = mid;
-          ub = km;
+          u = km;
         }
       }
-      bb = lo;
-      tied = !sp.ntb && bb < end && ub == x[r];
-      if (tied) {
-        if (PAIRS && (r & 1) && prev_tied && x[r] == x[r - 1] && valid(r - 1) && valid(r)) {
-          const uint32_t re = sp.rend[bb];
-          bb = prev_b + (prev_b < re && sp.idx[prev_b] < pos_of(r) ? 1u : 0u);
-        } else {
-          bb = tie_break(bb, x[r], pos_of(r), sp);
-        }
+      b[r] = lo;
+      ub[r] = u;
+    }
+  }
+  if (sp.ntb) return;
+  bool tie = false;
+#pragma unroll
+  for (int r = 0; r < R; ++r) tie |= ub[r] == x[r];
+  if (!tie) return;
+  bool prev_tied = false;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const bool tied = ub[r] == x[r] && b[r] < sp.nspl;
+    if (tied) {
+      if (PAIRS && (r & 1) && prev_tied && x[r] == x[r - 1] && valid(r - 1) && valid(r)) {
+        const uint32_t re = sp.rend[b[r]], pb = b[r - 1];
+        b[r] = pb + (pb < re && sp.idx[pb] < pos_of(r) ? 1u : 0u);
+      } else {
+        b[r] = tie_break(b[r], x[r], pos_of(r), sp);
       }
     }
-    b[r] = bb;
     prev_tied = tied;
-    prev_b = bb;
   }
 }
 
@@ -302,12 +403,12 @@ __device__ __forceinline__ void classify_batch(const uint64_t (&x)[R], uint32_t 
 
 // The same for elements in consecutive-position pairs (see
 // classify_batch_table); valid(e) says whether element e is a real element.
-template <int R, typename PosFn, typename ValidFn>
+template <int R, bool F64, typename PosFn, typename ValidFn>
 __device__ __forceinline__ void classify_batch_pairs(const uint64_t (&x)[R], uint32_t (&b)[R],
                                                      PosFn pos_of, ValidFn valid,
                                                      const Splitters& sp) {
   if (sp.mode == 0) classify_batch_tree<R>(x, b, pos_of, sp);
-  else classify_batch_table<R, true>(x, b, pos_of, valid, sp);
+  else classify_batch_table<R, true, F64>(x, b, pos_of, valid, sp);
 }
 
 

@@ -104,6 +104,13 @@ constexpr int kCiPairs = 4;  // 16-byte loads (two keys) per thread per step
 // the next step's keys are already in registers)
 constexpr int kCiPrefetch = 2;
 
+// Bound by shared-memory wavefronts (79 % of the SM's rate: table, splitter and
+// counter accesses at random banks).  What got it there, 2^28 uniform keys, level
+// 1 / level 2: a table step to the first splitter that is not smaller instead of
+// a search (0.92 -> 0.82 ms at level 1), steps that lie inside the chunk without
+// checks or 64-bit index arithmetic (0.82 -> 0.60), this kernel instead of one
+// staged by cp.async at the deeper levels (0.96 -> 0.87, then 0.66).  Four CTAs
+// per SM (64 registers) 0.81 / 0.72, four keys a thread 0.92 / 0.86.
 // VEC: the key array is 16-byte aligned (pairs are read by 16-byte loads);
 // MAP: the keys are float64 bit patterns, mapped to the order map on load.
 template <int NT, bool VEC, bool MAP>
@@ -125,8 +132,8 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
       sp.tree = (uint64_t*)p;
       p += Kp * 8;
     } else {
-      sp.tbl = (uint32_t*)p;
-      p += (size_t)4 << table_bits_for((uint32_t)Kp);
+      sp.tbl = (uint16_t*)p;
+      p += table_bytes((uint32_t)Kp);
     }
     sp.key = (uint64_t*)p; p += (size_t)kmax * 8;
     sp.idx = (uint32_t*)p; p += (size_t)kmax * 4;
@@ -143,7 +150,7 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
     const LevelSeg sg = segs[g];
     __syncthreads();
     if (g != cur_g) {
-      load_splitters<NT>(sg, ssk, ssi, sp);
+      load_splitters<NT, MAP>(sg, ssk, ssi, sp);
       cur_g = g;
     }
     for (uint32_t b = threadIdx.x; b < sg.k; b += NT) cnt[b] = 0;
@@ -187,11 +194,27 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
       prefetch_l2_range(src.key + a, src.key + e);
     };
     for (int d = 2; d < kCiPrefetch; ++d) prefetch((uint64_t)d * NT * kCiPairs);
+    constexpr uint64_t kStep = (uint64_t)NT * kCiPairs;  // pairs per step
+    // steps [w0, w1) hold only pairs inside the chunk: they are read, stored and
+    // counted without a check (the first step may start one key before the
+    // chunk, the last may be short)
+    const uint64_t w0 = VEC ? (ps == cs ? 0 : kStep) : ~0ull;
+    const uint64_t w1 = VEC ? npairs / kStep * kStep : 0;
+    auto load_step = [&](uint64_t p0, uint64_t (&x)[R]) {
+      if (VEC && p0 < w1) {  // (whole pairs, also where the first key is not the chunk's)
+        const uint64_t* kp = src.key + ps + 2 * (p0 + threadIdx.x);
+#pragma unroll
+        for (int r = 0; r < kCiPairs; ++r)
+          ld_stream_v2(x[2 * r], x[2 * r + 1], kp + 2 * r * NT, pol);
+      } else {
+        load(p0, x);
+      }
+    };
     uint64_t x[R], xn[R];
-    if (npairs > 0) load(0, x);
-    for (uint64_t p0 = 0; p0 < npairs; p0 += (uint64_t)NT * kCiPairs) {
-      prefetch(p0 + (uint64_t)kCiPrefetch * NT * kCiPairs);
-      load(p0 + (uint64_t)NT * kCiPairs, xn);
+    if (npairs > 0) load_step(0, x);
+    for (uint64_t p0 = 0; p0 < npairs; p0 += kStep) {
+      prefetch(p0 + (uint64_t)kCiPrefetch * kStep);
+      load_step(p0 + kStep, xn);
       uint64_t key[R];
 #pragma unroll
       for (int e = 0; e < R; ++e) key[e] = MAP ? f64_to_ordered(x[e]) : x[e];
@@ -206,47 +229,48 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
         const uint64_t pos = pos_at(e);
         return (p0 + (uint64_t)(e >> 1) * NT + threadIdx.x) < npairs && pos >= cs && pos < ce;
       };
-      classify_batch_pairs<R>(key, bk, [&](int e) {
+      classify_batch_pairs<R, MAP>(key, bk, [&](int e) {
         if (!valid(e)) return 0u;
         const uint64_t pos = pos_at(e);
         return src.idx ? src.idx[pos] : (uint32_t)(pos - sg.start);
       }, [&](int e) { return valid(e) && src.idx == nullptr; }, sp);
-      // a step whose pairs all lie inside the chunk stores them whole
-      const bool whole = ps == cs && p0 + (uint64_t)NT * kCiPairs <= npairs &&
-                         ps + 2 * (p0 + (uint64_t)NT * kCiPairs) <= ce;
       // runs of one bucket across the warp (duplicate-heavy inputs) take one
       // atomic per warp and slot; otherwise one atomic per key
       const uint32_t b0 = __shfl_sync(0xffffffffu, bk[0], 0);
       const bool skewed = __popc(__ballot_sync(0xffffffffu, bk[0] == b0)) > 8;
-      uint32_t vmask = 0;  // valid elements of the step
+      if (p0 >= w0 && p0 < w1) {
+        uint16_t* bp = src.bid + ps + 2 * (p0 + threadIdx.x);
 #pragma unroll
-      for (int r = 0; r < kCiPairs; ++r) {
-        const uint64_t j = p0 + (uint64_t)r * NT + threadIdx.x;
-        const uint64_t pos = ps + 2 * j;
-        const bool v0 = whole || (j < npairs && pos >= cs && pos < ce);
-        const bool v1 = whole || (j < npairs && pos + 1 < ce);
-        if (whole || (v0 && v1)) {
-          *reinterpret_cast<uint32_t*>(src.bid + pos) = bk[2 * r] | (bk[2 * r + 1] << 16);
-        } else if (v0) {
-          src.bid[pos] = (uint16_t)bk[2 * r];
-        } else if (v1) {
-          src.bid[pos + 1] = (uint16_t)bk[2 * r + 1];
+        for (int r = 0; r < kCiPairs; ++r)
+          *reinterpret_cast<uint32_t*>(bp + 2 * r * NT) = bk[2 * r] | (bk[2 * r + 1] << 16);
+        if (!skewed) {
+#pragma unroll
+          for (int e = 0; e < R; ++e) atomicAdd(&cnt[bk[e]], 1u);
+        } else {
+#pragma unroll
+          for (int e = 0; e < R; ++e) {
+            const uint32_t bl = __shfl_sync(0xffffffffu, bk[e], 0);
+            if (__all_sync(0xffffffffu, bk[e] == bl)) {
+              if (lane == 0) atomicAdd(&cnt[bl], 32u);
+            } else {
+              atomicAdd(&cnt[bk[e]], 1u);
+            }
+          }
         }
-        vmask |= ((v0 ? 1u : 0u) | (v1 ? 2u : 0u)) << (2 * r);
-      }
-      if (!skewed) {
-#pragma unroll
-        for (int e = 0; e < R; ++e)
-          if ((vmask >> e) & 1u) atomicAdd(&cnt[bk[e]], 1u);
       } else {
 #pragma unroll
-        for (int e = 0; e < R; ++e) {
-          const bool v = (vmask >> e) & 1u;
-          const uint32_t bl = __shfl_sync(0xffffffffu, bk[e], 0);
-          if (__all_sync(0xffffffffu, v && bk[e] == bl)) {
-            if (lane == 0) atomicAdd(&cnt[bl], 32u);
-          } else if (v) {
-            atomicAdd(&cnt[bk[e]], 1u);
+        for (int r = 0; r < kCiPairs; ++r) {
+          const uint64_t j = p0 + (uint64_t)r * NT + threadIdx.x;
+          const uint64_t pos = ps + 2 * j;
+          const bool v0 = j < npairs && pos >= cs && pos < ce;
+          const bool v1 = j < npairs && pos + 1 < ce;
+          if (v0) {
+            src.bid[pos] = (uint16_t)bk[2 * r];
+            atomicAdd(&cnt[bk[2 * r]], 1u);
+          }
+          if (v1) {
+            src.bid[pos + 1] = (uint16_t)bk[2 * r + 1];
+            atomicAdd(&cnt[bk[2 * r + 1]], 1u);
           }
         }
       }
@@ -260,9 +284,9 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
       const uint64_t raw = ld_stream_u64(src.key + pos, pol);
       uint64_t k1[1] = {MAP ? f64_to_ordered(raw) : raw};
       uint32_t b1[1];
-      classify_batch<1>(k1, b1, [&](int) {
+      classify_batch_pairs<1, MAP>(k1, b1, [&](int) {
         return src.idx ? src.idx[pos] : (uint32_t)(pos - sg.start);
-      }, sp);
+      }, [](int) { return false; }, sp);
       src.bid[pos] = (uint16_t)b1[0];
       atomicAdd(&cnt[b1[0]], 1u);
     }
@@ -320,8 +344,8 @@ k_classify_bulk(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk
       sp.tree = (uint64_t*)p;
       p += Kp * 8;
     } else {
-      sp.tbl = (uint32_t*)p;
-      p += (size_t)4 << table_bits_for((uint32_t)Kp);
+      sp.tbl = (uint16_t*)p;
+      p += table_bytes((uint32_t)Kp);
     }
     sp.key = (uint64_t*)p; p += (size_t)kmax * 8;
     sp.idx = (uint32_t*)p; p += (size_t)kmax * 4;
@@ -1089,7 +1113,7 @@ size_t g_us_smem_max = 0;
 
 size_t classify_ids_smem_bytes(uint32_t kmax, int mode) {
   const size_t Kp = next_pow2_u32(kmax);
-  size_t b = (mode & 1) == 0 ? Kp * 8 : ((size_t)4 << table_bits_for((uint32_t)Kp));
+  size_t b = (mode & 1) == 0 ? Kp * 8 : table_bytes((uint32_t)Kp);
   b += (size_t)kmax * (8 + 4 + 4 + 2);
   return (b + 15) & ~(size_t)15;
 }
