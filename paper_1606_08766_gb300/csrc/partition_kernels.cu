@@ -171,6 +171,17 @@ k_level_plan(DevState* st, const SegIn* list_in, LevelSeg* segs, LevelParams P, 
   const uint32_t ncta = max(1u, (G + kPlanThreads - 1) / kPlanThreads);
   const uint32_t t = blockIdx.x;
   if (t >= ncta) return;
+  if (P.fit_chunks && gridDim.x == 1) {
+    // few elements may have come this far (duplicate-heavy input): they are
+    // spread over as many chunks as all elements would be (the chunk and
+    // histogram capacities count those chunks and one more per segment)
+    const uint32_t gm = threadIdx.x;
+    uint64_t sum;
+    block_excl_scan_u64<kPlanThreads>(gm < G ? list_in[gm].m : 0u, &sum, sm);
+    const uint64_t w = (sum + P.fit_chunks - 1) / P.fit_chunks;
+    P.W = (uint32_t)umin64(P.W, umax64(kMinDeepChunk,
+                                       (w + kMinDeepChunk - 1) / kMinDeepChunk * kMinDeepChunk));
+  }
   uint64_t before[6];
 #pragma unroll
   for (int i = 0; i < 6; ++i) {

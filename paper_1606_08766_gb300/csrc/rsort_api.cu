@@ -98,6 +98,7 @@ struct Plan {
   int levels = 0;           // partition levels to launch
   uint32_t k_plain = 0;     // level-1 buckets of a one-segment call
   uint32_t oversample1 = kDeepOversample;  // its samples per bucket when automatic
+  bool fine = false;        // chunks as small as the call needs
   uint32_t samp_max = 0xffffffffu;         // most samples of a deeper segment
   int direct = 0;           // n small enough for one in-SM sort
   uint32_t W1 = 0, Wd = 0;  // chunk sizes (level 1, deeper levels)
@@ -165,6 +166,7 @@ void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int
                  bool fine) {
   p.n = n;
   p.k1 = k1;
+  p.fine = fine;
   // Levels the sizes call for (at most the max_levels tunable): the sample
   // keeps a level's largest bucket within ~1.5x its mean, so a level-1
   // bucket holds up to 1.5 n / k1 keys (an automatic fan-out aims at the
@@ -351,6 +353,7 @@ void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const 
     // default leaves it to the device); a level's input is in position order
     // only after stable levels, and level 1's order is read on the device
     if (L == 2 && !segmented) P.max_segs = p.k_plain;  // (level 1's buckets)
+    if (L > 1 && p.fine) P.fit_chunks = (uint32_t)(p.n / p.Wd);
     P.refine = segmented && type == RSORT_KEY_F64;
     P.stable = L == 1 ? c->level1_stable : c->deep_levels_stable;
     P.in_order = L == 1 ? 1 : (L == 2 || c->deep_levels_stable ? kOrderAuto : 0);

@@ -212,6 +212,8 @@ struct LevelParams {
   uint32_t W;           // keys per classify/scatter chunk
   uint64_t seed;
   uint64_t samp_cap, hist_cap, chunk_cap, seg_cap, final_cap, schunk_cap, bucket_cap;
+  uint32_t fit_chunks = 0;          // chunks a deeper level's elements are spread
+                                    // over, however few (0: chunks of W keys)
   uint64_t max_segs = ~0ull;        // segments the level can have (seg_cap aside)
   uint32_t samp_max = 0xffffffffu;  // at most this many samples a segment
   // a one-segment level: 1: its bucket count was asked for (16 ceil(log2 k)

@@ -10,21 +10,18 @@
 //                  bucket histogram.  Keys stream through 16-byte loads (two
 //                  keys each) straight into registers.
 //
-// k_scatter_units  reads keys and stored bucket ids of 4096-element sub-tiles
-//                  (registers, the next sub-tile's loads in flight while the
-//                  current one is processed), ranks every element among the
-//                  elements of its bucket (warp order, then lane order: input
-//                  order, so buckets keep input order), counting-sorts the
-//                  sub-tile into shared memory, and writes every bucket's run
-//                  in whole UNITS of 8 elements -- 64 bytes of keys and 32
-//                  bytes of positions, aligned in the output -- each stored by
-//                  8 consecutive lanes of one warp instruction, so every output
-//                  sector is written whole and once.  A bucket's incomplete
-//                  last unit (at most 7 elements) waits in a per-bucket carry
-//                  area in shared memory and goes out with the bucket's next
-//                  elements.  Only the first and last unit of a bucket in a
-//                  chunk, shared with the neighbouring chunks' ranges, are
-//                  written in part.
+// k_scatter_units  reads keys and stored bucket ids of a sub-tile into
+//                  registers, ranks every element among the elements of its
+//                  bucket (stable: warp order, then lane order), and writes
+//                  every bucket's run in whole UNITS of 8 elements -- 64 bytes
+//                  of keys and 32 bytes of positions, aligned in the output --
+//                  each stored by 8 consecutive lanes of one warp instruction,
+//                  so every output sector is written whole and once.  Elements
+//                  that fill units go through a bucket-sorted sub-tile in
+//                  shared memory; a bucket's others (at most 7) wait in its
+//                  carry slots and go out with its next elements.  Only the
+//                  first and last unit of a bucket in a chunk, shared with the
+//                  neighbouring chunks' ranges, are written in part.
 //
 // The carry area holds 7 (key, position) slots per bucket, so the scatter
 // serves levels with at most kUnitMaxK buckets.
@@ -494,26 +491,29 @@ k_classify_bulk(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk
 // ---------------------------------------------------------------------------
 // Scatter in whole units
 // ---------------------------------------------------------------------------
-// The stable scatter keeps per-warp counters and winner slots (512 threads,
-// 4096-element sub-tiles); the unordered one needs one counter per bucket,
-// and the room that frees holds longer sub-tiles (more elements per thread).
-constexpr int kUsThreads = 512;        // stable
-constexpr int kUsItems = 8;
-constexpr int kUsThreadsAny = 512;     // unordered (6144-element sub-tiles)
-constexpr int kUsItemsAny = 12;
+// The stable scatter keeps per-warp counters and winner slots; the unordered one
+// needs one counter per bucket, and the room that frees holds longer sub-tiles
+// (more elements per thread).  Up to kUsSmallK buckets two CTAs of 256 threads
+// share an SM, each other's barriers and latencies overlapping (2^28 keys, level
+// 2: 1.70 -> 1.61 ms; 100,000 segments 2.20 -> 1.90); above, the carry area
+// leaves room for one, of 512 threads (640, 768 and 1024 threads with fewer
+// elements each measured 1.97, 2.00 and 2.05 ms against 1.91 at level 1).
+constexpr int kUsThreads = 512;
+constexpr int kUsThreadsSmall = 256;
+constexpr int kUsItems = 8;        // per thread, stable
+constexpr int kUsItemsAny = 12;    // unordered
+constexpr uint32_t kUsSmallK = 512;
 // sub-tiles ahead whose bytes are asked into L2 when a sub-tile starts (0:
-// none): with 1, the next sub-tile's register loads, issued after this one's
-// placement, find their bytes on the way (measured at 2^28 keys: distance 1
-// 2.23 -> 2.08 ms, 2 -> 2.12, 3 -> 2.18)
+// none): with 1, the next sub-tile's register loads find their bytes on the way
 constexpr int kUsPrefetch = 1;
 // a bucket with at most this many whole units in a sub-tile writes their
-// records itself; more (skewed inputs) send the sub-tile through the unit
-// marks and a block max-scan instead
+// records itself; those of the others (skewed inputs) are written by a warp
+// each from a list
 constexpr int kUsDirectUnits = 16;
-// bits of the per-bucket meta word
-constexpr int kMetaUnitShift = 14;     // sorted slot + 8 below (14 bits)
-constexpr int kMetaCarryShift = 25;    // first unit (11 bits) below
-constexpr int kMetaPhShift = 28;       // carry count (3 bits) below, phantoms (3 bits)
+// bits of the per-bucket sub-tile word (info)
+constexpr int kInfoSlotBits = 13;      // first sorted slot
+constexpr int kInfoUnitShift = 13;     // elements that leave in whole units (14 bits)
+constexpr int kInfoCarryShift = 27;    // carry slot of the first one that does not (3 bits)
 // bits of the second word of a per-unit record (the first is the output
 // position of the unit's slot 0)
 constexpr int kRecFirstShift = 14;     // sorted slot of slot 0 + 8 (14 bits) below
@@ -523,42 +523,23 @@ __host__ __device__ inline uint32_t us_max_units(uint32_t kmax, uint32_t st) {
   return (st + kCarry * kmax) / kUnit + 1;
 }
 
+// Buckets of a sub-tile of st elements that can have more than kUsDirectUnits
+// units.
+__host__ __device__ constexpr uint32_t us_max_big(uint32_t st) {
+  return st / (kUsDirectUnits * kUnit) + 1;
+}
+
 __host__ __device__ inline size_t us_smem_bytes(uint32_t kmax, uint32_t nt, uint32_t it,
                                                 bool stable) {
   const uint32_t nw = nt / 32, st = nt * it;
   size_t b = 0;
-  b += (size_t)st * 8;                           // sorted keys
-  b += (size_t)kmax * kCarry * 8;                // carried keys
+  b += (size_t)(st + kmax * kCarry) * 8;         // sorted keys, carried keys
   b += (size_t)us_max_units(kmax, st) * 8;       // per-unit records
-  b += (size_t)st * 4;                           // sorted positions
-  b += (size_t)kmax * kCarry * 4;                // carried positions
-  b += (size_t)kmax * 8;                         // per-bucket obase + meta
-  b += (size_t)(kmax + 1) * 4;                   // sbase
+  b += (size_t)(st + kmax * kCarry) * 4;         // sorted positions, carried ones
+  b += (size_t)kmax * 12;                        // per-bucket obase, meta, info
   b += stable ? (size_t)nw * cnt_stride(kmax) * 2 : (size_t)kmax * 4;  // counters
-  b += (size_t)us_max_units(kmax, st) * 2 + 2;   // unit -> bucket
   b += stable ? (size_t)nw * kmax : 0;           // per-warp winner slots
   return (b + 15) & ~(size_t)15;
-}
-
-// Exclusive max-scan of one u32 per thread over the block (NT % 32 == 0);
-// sm holds NT/32 words.
-template <int NT>
-__device__ __forceinline__ uint32_t block_excl_max_u32(uint32_t v, uint32_t* sm) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  uint32_t x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x = max(x, y);
-  }
-  if (lane == 31) sm[w] = x;
-  __syncthreads();
-  uint32_t pre = 0;
-  for (int q = 0; q < w; ++q) pre = max(pre, sm[q]);
-  const uint32_t y = __shfl_up_sync(0xffffffffu, x, 1);
-  const uint32_t excl = max(pre, lane > 0 ? y : 0u);
-  __syncthreads();
-  return excl;
 }
 
 // Ranks every valid element (bucket id != 0xffffffff) of a thread's IT among
@@ -605,46 +586,52 @@ __device__ __forceinline__ void rank_by_atomics(const uint32_t (&bid)[IT], uint3
 // and a prefix over the warps); otherwise (a full sort's level 1, whose
 // buckets the in-SM sort orders by (key, position) anyway) every element takes
 // its rank from one shared-memory atomic on its bucket's counter.
+//
+// The kernel is bound by shared-memory wavefronts and by the latency between
+// its barriers (one CTA per SM), so every element goes through shared memory
+// once: from the elements of its bucket before it and the bucket's carry it
+// knows whether it leaves in a whole unit of this sub-tile (then it goes to its
+// sorted slot) or stays (then it waits in its thread's registers until the old
+// carry has been written out, and goes to its carry slot).  Copying the
+// incomplete units from the sorted slots to the carry area instead took 0.44 of
+// 1.39 shared-memory wavefronts per element.  2^28 uniform keys: level 1 2.03 ->
+// 1.91 ms, level 2 1.79 -> 1.70.
 template <int NT, int IT, bool HAS_IDX, bool STABLE>
 __device__ __forceinline__ void scatter_units(const DevState* st, const LevelSeg* segs, Src src,
                                               const uint32_t* hist_scan, Dst dst, uint32_t kmax,
                                               int conv, uint32_t aoff) {
   constexpr int NW = NT / 32;
   constexpr int ST = NT * IT;
-  static_assert(ST + kUnit < (1 << kMetaUnitShift), "sorted slots fit the meta word");
-  static_assert(((ST + kCarry * kUnitMaxK) / kUnit) < (1 << (kMetaCarryShift - kMetaUnitShift)),
-                "unit indices fit the meta word");
+  static_assert(ST <= (1 << kInfoSlotBits), "sorted slots fit the info word");
   static_assert(ST + kUnit < (1 << kRecFirstShift) && kUnitMaxK <= (1 << (32 - kRecBucketShift)),
                 "sorted slots and buckets fit the unit record");
+  static_assert((ST + kCarry * kUnitMaxK) / kUnit < (1 << 17), "units fit the packed scan");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* p = smem_raw;
-  uint64_t* skey = (uint64_t*)p; p += (size_t)ST * 8;
-  uint64_t* ckey = (uint64_t*)p; p += (size_t)kmax * kCarry * 8;
+  // sorted slots, then bucket b's carry slots from ST + 7 b on
+  uint64_t* skey = (uint64_t*)p; p += (size_t)(ST + kmax * kCarry) * 8;
   const uint32_t umax = us_max_units(kmax, ST);
   // per whole unit of the sub-tile: its output position, and the sorted slot
   // of its slot 0 + 8 | (carry count | phantoms << 3) << 14 | bucket << 20
   // (carry count and phantoms only in a bucket's first unit)
   uint2* urec = (uint2*)p; p += (size_t)umax * 8;
-  uint32_t* sidx = (uint32_t*)p; p += (size_t)ST * 4;
-  uint32_t* cidx = (uint32_t*)p; p += (size_t)kmax * kCarry * 4;
-  // per-bucket state (two flat word arrays, so that both the bucket-ordered
-  // and the interleaved phases touch consecutive words):
+  uint32_t* sidx = (uint32_t*)p; p += (size_t)(ST + kmax * kCarry) * 4;
+  // per-bucket state:
   //   obase  output position of the bucket's current unit start (mod 2^32)
-  //   meta   sorted slot of that unit's first slot + 8 (14 bits; the unit
-  //          may begin with up to 7 carried slots) | first unit in the unit
-  //          list << 14 (11 bits) | carry count << 25 | phantoms << 28
+  //   meta   carry count | phantoms << 3
+  //   info   of the sub-tile: first sorted slot | elements that leave in whole
+  //          units << 13 | carry slot of the first one that stays << 27
   uint32_t* obase = (uint32_t*)p; p += (size_t)kmax * 4;
   uint32_t* meta = (uint32_t*)p; p += (size_t)kmax * 4;
-  uint32_t* sbase = (uint32_t*)p; p += (size_t)(kmax + 1) * 4;
+  uint32_t* info = (uint32_t*)p; p += (size_t)kmax * 4;
   const uint32_t kst = cnt_stride(kmax);
   uint16_t* wcnt = (uint16_t*)p;
   p += STABLE ? (size_t)NW * kst * 2 : (size_t)kmax * 4;
-  uint16_t* unit_b = (uint16_t*)p; p += (size_t)umax * 2 + 2;
   uint8_t* wwin = (uint8_t*)p;
-  __shared__ uint64_t scan_sm[NW];
-  __shared__ uint32_t max_sm[NW];
-  __shared__ uint32_t s_big;  // some bucket has more than kUsDirectUnits units
-  if (threadIdx.x == 0) s_big = 0;
+  __shared__ __align__(16) uint32_t s_scan[NW];
+  __shared__ uint4 s_bigs[us_max_big(ST)];  // buckets of many units: first record, units, record
+  __shared__ uint32_t s_nbig;
+  if (threadIdx.x == 0) s_nbig = 0;
 
   const uint64_t pol = l2_evict_first_policy();
   const uint64_t total = st->total_chunks;
@@ -655,7 +642,6 @@ __device__ __forceinline__ void scatter_units(const DevState* st, const LevelSeg
   uint16_t* my_cnt = wcnt + (size_t)warp * kst;
   uint8_t* my_win = wwin + (size_t)warp * kmax;
   uint32_t* ucnt = reinterpret_cast<uint32_t*>(wcnt);  // unordered: one counter per bucket
-  for (uint32_t u = tid; u < umax; u += NT) unit_b[u] = 0;
   if (!STABLE)
     for (uint32_t b = tid; b < kmax; b += NT) ucnt[b] = 0;
 
@@ -672,32 +658,46 @@ __device__ __forceinline__ void scatter_units(const DevState* st, const LevelSeg
     const uint32_t per = (k + NT - 1) / NT;
     const uint32_t bb0 = min(tid * per, k);
     const uint32_t bb1 = min(bb0 + per, k);
-    __syncthreads();  // the previous chunk is done with every shared array
-    // output state of every bucket: the chunk's first position p0, the unit
-    // start at or below it (units start at positions = aoff mod 8) and the
-    // slots before p0 in that unit (phantoms: held, never written)
-    for (uint32_t b = tid; b < k; b += NT) {
-      const uint32_t p0 = (uint32_t)(hist_scan[sg.hist_off + (uint64_t)b * sg.nunits + cl] +
-                                     sg.delta);
-      const uint32_t a = (p0 - aoff) & (kUnit - 1);
-      obase[b] = p0 - a;
-      meta[b] = (a << kMetaCarryShift) | (a << kMetaPhShift);
-    }
     const uint32_t q0 = (uint32_t)warp * (IT * 32) + lane;
     uint64_t key[IT];
     uint32_t idx[IT], bid[IT];
-    auto load = [&](uint64_t s, uint64_t (&kk)[IT], uint32_t (&ii)[IT], uint32_t (&bb)[IT]) {
+    // (a whole sub-tile is loaded without checks, at constant offsets from one
+    // address per array)
+    auto load_bid = [&](uint64_t s) {
+      if (s >= nst) return;
       const uint64_t b0 = cs + s * ST;
+      const uint16_t* bp = src.bid + b0 + q0;
+      if (b0 + ST <= ce) {
 #pragma unroll
-      for (int r = 0; r < IT; ++r) {
-        const uint64_t pos = b0 + q0 + r * 32;
-        kk[r] = 0;
-        ii[r] = 0;
-        bb[r] = 0xffffffffu;
-        if (s < nst && pos < ce) {
-          kk[r] = ld_stream_u64(src.key + pos, pol);
-          if (HAS_IDX) ii[r] = ld_stream_u32(src.idx + pos, pol);
-          bb[r] = ld_stream_u16(src.bid + pos, pol);
+        for (int r = 0; r < IT; ++r) bid[r] = ld_stream_u16(bp + r * 32, pol);
+      } else {
+        const uint32_t left = (uint32_t)(ce - b0);
+#pragma unroll
+        for (int r = 0; r < IT; ++r) {
+          bid[r] = 0xffffffffu;
+          if (q0 + r * 32 < left) bid[r] = ld_stream_u16(bp + r * 32, pol);
+        }
+      }
+    };
+    auto load_key = [&](uint64_t s) {
+      if (s >= nst) return;
+      const uint64_t b0 = cs + s * ST;
+      const uint64_t* kp = src.key + b0 + q0;
+      const uint32_t* ip = HAS_IDX ? src.idx + b0 + q0 : nullptr;
+      if (b0 + ST <= ce) {
+#pragma unroll
+        for (int r = 0; r < IT; ++r) {
+          key[r] = ld_stream_u64(kp + r * 32, pol);
+          if (HAS_IDX) idx[r] = ld_stream_u32(ip + r * 32, pol);
+        }
+      } else {
+        const uint32_t left = (uint32_t)(ce - b0);
+#pragma unroll
+        for (int r = 0; r < IT; ++r) {
+          if (q0 + r * 32 < left) {
+            key[r] = ld_stream_u64(kp + r * 32, pol);
+            if (HAS_IDX) idx[r] = ld_stream_u32(ip + r * 32, pol);
+          }
         }
       }
     };
@@ -709,8 +709,20 @@ __device__ __forceinline__ void scatter_units(const DevState* st, const LevelSeg
       if (HAS_IDX) prefetch_l2_range(src.idx + a, src.idx + e);
       prefetch_l2_range(src.bid + a, src.bid + e);
     };
+    load_bid(0);
+    load_key(0);
     for (int d = 1; d < kUsPrefetch; ++d) prefetch(d);
-    load(0, key, idx, bid);
+    __syncthreads();  // the previous chunk is done with every shared array
+    // output state of every bucket: the chunk's first position p0, the unit
+    // start at or below it (units start at positions = aoff mod 8) and the
+    // slots before p0 in that unit (phantoms: held, never written)
+    for (uint32_t b = tid; b < k; b += NT) {
+      const uint32_t p0 = (uint32_t)(hist_scan[sg.hist_off + (uint64_t)b * sg.nunits + cl] +
+                                     sg.delta);
+      const uint32_t a = (p0 - aoff) & (kUnit - 1);
+      obase[b] = p0 - a;
+      meta[b] = a | (a << 3);
+    }
     for (uint64_t s = 0; s < nst; ++s) {
       prefetch(s + kUsPrefetch);
       // -- 1. rank every element among its bucket's elements of this warp
@@ -771,22 +783,26 @@ __device__ __forceinline__ void scatter_units(const DevState* st, const LevelSeg
       }
       }  // mixed window
       }  // STABLE
-      __syncthreads();  // (A) every warp's counts are in
-      // -- 2. per bucket: exclusive prefix over the warps' counts (in place),
-      //    the bucket's elements t in this sub-tile, its virtual run
-      //    (carry + t) and the whole units u of that run; then one block scan
-      //    of (u, t) places every bucket's elements in the sorted sub-tile and
-      //    its units in the unit list, and a bucket with few units writes
-      //    their records
-      uint32_t loc_t = 0, loc_u = 0;
+      __syncthreads();  // (A) every warp's counts are in; the old carry is in place
+      // -- 2. per bucket: its elements t in this sub-tile (stable: the exclusive
+      //    prefix over the warps' counts, in place), its virtual run (carry +
+      //    t), the whole units u of that run and the elements w among t that
+      //    fill them; one block scan of (u, w) places its elements in the
+      //    sorted sub-tile and its units in the record list; its output state
+      //    moves on by u units
+      uint32_t loc = 0;  // w | u << 15
+      auto shape = [&](uint32_t t, uint32_t cb, uint32_t& u, uint32_t& w) {
+        u = (cb + t) / kUnit;
+        w = u ? kUnit * u - cb : 0u;
+      };
       if constexpr (!STABLE) {
         for (uint32_t b = bb0; b < bb1; ++b) {
           const uint32_t t = ucnt[b];
           ucnt[b] = 0;  // ready for the next sub-tile (its atomics follow barriers)
-          const uint32_t u = (((meta[b] >> kMetaCarryShift) & 7u) + t) / kUnit;
-          sbase[b] = t | (u << 16);
-          loc_t += t;
-          loc_u += u;
+          uint32_t u, w;
+          shape(t, meta[b] & 7u, u, w);
+          info[b] = t;
+          loc += w | (u << 15);
         }
       } else {
         uint32_t b = bb0;
@@ -802,10 +818,10 @@ __device__ __forceinline__ void scatter_units(const DevState* st, const LevelSeg
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const uint32_t t = h ? (tot2 >> 16) : (tot2 & 0xffffu);
-            const uint32_t u = (((meta[b + h] >> kMetaCarryShift) & 7u) + t) / kUnit;
-            sbase[b + h] = t | (u << 16);
-            loc_t += t;
-            loc_u += u;
+            uint32_t u, w;
+            shape(t, meta[b + h] & 7u, u, w);
+            info[b + h] = t;
+            loc += w | (u << 15);
           }
         }
         for (; b < bb1; ++b) {
@@ -816,160 +832,140 @@ __device__ __forceinline__ void scatter_units(const DevState* st, const LevelSeg
             wcnt[(size_t)w * kst + b] = (uint16_t)t;
             t += cnt;
           }
-          const uint32_t u = (((meta[b] >> kMetaCarryShift) & 7u) + t) / kUnit;
-          sbase[b] = t | (u << 16);
-          loc_t += t;
-          loc_u += u;
+          uint32_t u, w;
+          shape(t, meta[b] & 7u, u, w);
+          info[b] = t;
+          loc += w | (u << 15);
         }
       }
-      uint64_t tot;
-      const uint64_t ex =
-          block_excl_scan_u64<NT>(((uint64_t)loc_u << 32) | loc_t, &tot, scan_sm);
+      uint32_t inc = loc;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      if (lane == 31) s_scan[warp] = inc;
+      __syncthreads();  // (A2) warp sums
+      uint32_t tot = 0, at = inc - loc;
+#pragma unroll
+      for (int q = 0; q < NW; ++q) {
+        const uint32_t v = s_scan[q];
+        at += q < warp ? v : 0u;
+        tot += v;
+      }
       {
-        uint32_t run_t = (uint32_t)ex, run_u = (uint32_t)(ex >> 32);
-        bool big = false;
+        uint32_t run_w = at & 0x7fffu, run_u = at >> 15;
         for (uint32_t b = bb0; b < bb1; ++b) {
-          const uint32_t tu = sbase[b], t = tu & 0xffffu, u = tu >> 16;
-          const uint32_t m = meta[b];
-          const uint32_t cb = (m >> kMetaCarryShift) & 7u;
-          sbase[b] = run_t;
-          meta[b] = (m & (0x3fu << kMetaCarryShift)) | (run_u << kMetaUnitShift) |
-                    (run_t + kUnit - cb);
-          if (u > (uint32_t)kUsDirectUnits) {
-            big = true;
-          } else if (u) {
+          const uint32_t t = info[b], m = meta[b], cb = m & 7u;
+          uint32_t u, w;
+          shape(t, cb, u, w);
+          info[b] = (run_w & ((1u << kInfoSlotBits) - 1)) | (w << kInfoUnitShift) |
+                    ((u ? 0u : cb) << kInfoCarryShift);
+          // (an incomplete first unit keeps its phantoms)
+          meta[b] = u ? (cb + t) % kUnit : (cb + t) | (m & 0x38u);
+          if (u) {
             const uint32_t ob = obase[b];
-            const uint32_t qv = run_t + kUnit - cb;
-            urec[run_u] = make_uint2(ob, qv | (((m >> kMetaCarryShift) & 0x3fu) << kRecFirstShift) |
-                                             (b << kRecBucketShift));
-            for (uint32_t d = 1; d < u; ++d)
-              urec[run_u + d] = make_uint2(ob + kUnit * d, (qv + kUnit * d) | (b << kRecBucketShift));
+            obase[b] = ob + kUnit * u;
+            const uint32_t qv = (run_w + kUnit - cb) | (b << kRecBucketShift);
+            const uint2 first = make_uint2(ob, qv | ((m & 0x3fu) << kRecFirstShift));
+            if (u > (uint32_t)kUsDirectUnits) {
+              s_bigs[atomicAdd(&s_nbig, 1u)] = make_uint4(run_u, u, first.x, first.y);
+            } else {
+              urec[run_u] = first;
+              for (uint32_t d = 1; d < u; ++d)
+                urec[run_u + d] = make_uint2(ob + kUnit * d, qv + kUnit * d);
+            }
           }
-          run_t += t;
+          run_w += w;
           run_u += u;
         }
-        if (big) s_big = 1u;
       }
-      const uint32_t U = (uint32_t)(tot >> 32);
-      if (tid == 0) sbase[k] = (uint32_t)tot;
-      __syncthreads();  // (B) bucket bases and unit marks are in
-      // -- 3. if a bucket had too many units to write their records: the
-      //    bucket of every unit (marks carry bucket + 1 at a bucket's first
-      //    unit; an inclusive max-scan fills the rest) and every unit's record
-      //    (the marks are cleared for the next sub-tile); then the sub-tile
-      //    counting-sorted by bucket into shared memory
-      if (s_big) {
-        for (uint32_t b = bb0; b < bb1; ++b) {
-          const uint32_t m = meta[b];
-          const uint32_t uu = (((m >> kMetaCarryShift) & 7u) + sbase[b + 1] - sbase[b]) / kUnit;
-          if (uu) unit_b[(m >> kMetaUnitShift) & 0x7ffu] = (uint16_t)(b + 1);
-        }
-        __syncthreads();
-        const uint32_t upt = (U + NT - 1) / NT;
-        const uint32_t u0 = min(tid * upt, U), u1 = min(u0 + upt, U);
-        uint32_t m = 0;
-        for (uint32_t u = u0; u < u1; ++u) m = max(m, (uint32_t)unit_b[u]);
-        uint32_t run = block_excl_max_u32<NT>(m, max_sm);
-        for (uint32_t u = u0; u < u1; ++u) {
-          run = max(run, (uint32_t)unit_b[u]);
-          unit_b[u] = 0;
-          const uint32_t b = run - 1, mb = meta[b];
-          const uint32_t d = u - ((mb >> kMetaUnitShift) & 0x7ffu);  // unit of the bucket's run
-          const uint32_t first = d == 0 ? (mb >> kMetaCarryShift) & 0x3fu : 0u;
-          urec[u] = make_uint2(obase[b] + kUnit * d,
-                               ((mb & ((1u << kMetaUnitShift) - 1)) + kUnit * d) |
-                                   (first << kRecFirstShift) | (b << kRecBucketShift));
-        }
+      const uint32_t U = tot >> 15;
+      __syncthreads();  // (B) bucket bases and records are in
+      const uint32_t nbig = s_nbig;
+      for (uint32_t i = warp; i < nbig; i += NW) {
+        const uint4 e = s_bigs[i];
+        for (uint32_t d = lane; d < e.y; d += 32)
+          urec[e.x + d] = make_uint2(e.z + kUnit * d,
+                                     (d ? e.w & ~(0x3fu << kRecFirstShift) : e.w) + kUnit * d);
       }
+      // -- 3. elements that leave go to their sorted slots; the others keep
+      //    their carry slot (lrank) and wait
       const uint32_t pos0 = (uint32_t)(cs + s * ST - sg.start) + q0;  // implicit positions
+      if (conv) {
+#pragma unroll
+        for (int r = 0; r < IT; ++r) key[r] = conv_key(key[r], conv);
+      }
 #pragma unroll
       for (int r = 0; r < IT; ++r) {
         const uint32_t b = bid[r];
+        uint32_t wait = 0xffffffffu;
         if (b != 0xffffffffu) {
-          const uint32_t q = sbase[b] + (STABLE ? (uint32_t)my_cnt[b] : 0u) + lrank[r];
-          skey[q] = conv_key(key[r], conv);
-          sidx[q] = HAS_IDX ? idx[r] : pos0 + r * 32;
+          const uint32_t in = info[b];
+          const uint32_t w = (in >> kInfoUnitShift) & 0x3fffu;
+          const uint32_t rk = lrank[r] + (STABLE ? (uint32_t)my_cnt[b] : 0u);
+          const uint32_t q = (in & ((1u << kInfoSlotBits) - 1)) + rk;
+          if (rk < w) {
+            skey[q] = key[r];
+            sidx[q] = HAS_IDX ? idx[r] : pos0 + r * 32;
+          } else {
+            wait = ST + b * kCarry + (in >> kInfoCarryShift) + rk - w;
+          }
         }
+        lrank[r] = wait;
       }
-      __syncthreads();  // (C) the sorted sub-tile and the unit buckets are in
-      if (tid == 0) s_big = 0;
-      // the next sub-tile's loads go out now, into the same registers, and
-      // land while this one is written
-      load(s + 1, key, idx, bid);
+      // the next sub-tile's bucket ids go out now (they are ranked first)
+      load_bid(s + 1);
+      __syncthreads();  // (C) the sorted sub-tile and the records are in
+      if (tid == 0) s_nbig = 0;
       // -- 4. whole units out: 8 consecutive lanes store one unit (slots
       //    before the carry count come from the carry area, phantoms are
       //    skipped); one record lookup per slot
-      for (uint32_t e = tid; e < U * kUnit; e += NT) {
-        const uint32_t u = e / kUnit, j = e % kUnit;
-        const uint2 rc = urec[u];
-        const uint32_t cb = (rc.y >> kRecFirstShift) & 7u;
-        const uint32_t ph = (rc.y >> (kRecFirstShift + 3)) & 7u;
-        uint64_t kv;
-        uint32_t iv;
-        if (j < cb) {
-          const uint32_t cq = (rc.y >> kRecBucketShift) * kCarry + j;
-          kv = ckey[cq];
-          iv = cidx[cq];
-        } else {
-          const uint32_t q = (rc.y & ((1u << kRecFirstShift) - 1)) - kUnit + j;
-          kv = skey[q];
-          iv = sidx[q];
-        }
-        if (j >= ph) {
-          dst.key[rc.x + j] = kv;
-          dst.idx[rc.x + j] = iv;
+      {
+        const uint32_t j = tid % kUnit;
+#pragma unroll 2
+        for (uint32_t u = tid / kUnit; u < U; u += NT / kUnit) {
+          const uint2 rc = urec[u];
+          const uint32_t cb = (rc.y >> kRecFirstShift) & 7u;
+          const uint32_t ph = (rc.y >> (kRecFirstShift + 3)) & 7u;
+          const uint32_t q = j < cb ? ST + (rc.y >> kRecBucketShift) * kCarry + j
+                                    : (rc.y & ((1u << kRecFirstShift) - 1)) - kUnit + j;
+          const uint64_t kv = skey[q];
+          const uint32_t iv = sidx[q];
+          if (j >= ph) {
+            const uint32_t d = rc.x + j;  // (a bucket's first unit may start below 0)
+            dst.key[d] = kv;
+            dst.idx[d] = iv;
+          }
         }
       }
       __syncthreads();  // (D) carry slots are read
-      // -- 5. the incomplete last unit of every bucket becomes its carry
-      //    (buckets interleaved over the threads, so that neighbouring lanes
-      //    touch neighbouring carry rows; copies unrolled and predicated)
-      for (uint32_t b = tid; b < k; b += NT) {
-        const uint32_t m = meta[b];
-        const uint32_t cb = (m >> kMetaCarryShift) & 7u;
-        const uint32_t qb = (m & ((1u << kMetaUnitShift) - 1)) - kUnit;  // sorted slot of run slot 0
-        const uint32_t L = cb + (sbase[b + 1] - sbase[b]), u = L / kUnit, nc = L % kUnit;
-        // run slots [first, L) become carry slots [first - shift, L - shift)
-        const uint32_t first = u == 0 ? cb : kUnit * u;
-        const uint32_t shift = kUnit * u;
-        {
-          uint64_t ck[kCarry];
+      // -- 5. the elements that stay become their buckets' carry
 #pragma unroll
-          for (int j = 0; j < kCarry; ++j)
-            if (first + j < L) ck[j] = skey[qb + first + j];
-#pragma unroll
-          for (int j = 0; j < kCarry; ++j)
-            if (first + j < L) ckey[b * kCarry + first + j - shift] = ck[j];
+      for (int r = 0; r < IT; ++r) {
+        if (lrank[r] != 0xffffffffu) {
+          skey[lrank[r]] = key[r];
+          sidx[lrank[r]] = HAS_IDX ? idx[r] : pos0 + r * 32;
         }
-        {
-          uint32_t ci[kCarry];
-#pragma unroll
-          for (int j = 0; j < kCarry; ++j)
-            if (first + j < L) ci[j] = sidx[qb + first + j];
-#pragma unroll
-          for (int j = 0; j < kCarry; ++j)
-            if (first + j < L) cidx[b * kCarry + first + j - shift] = ci[j];
-        }
-        const uint32_t ph = u == 0 ? ((m >> kMetaPhShift) & 7u) : 0u;
-        obase[b] += shift;
-        meta[b] = (nc << kMetaCarryShift) | (ph << kMetaPhShift);
       }
+      load_key(s + 1);
     }
+    __syncthreads();  // the last carry is in place
     // the chunk's last, incomplete unit of every bucket (the rest of its
     // sectors belongs to the next chunk's range)
     for (uint32_t b = tid; b < k; b += NT) {
       const uint32_t m = meta[b], ob = obase[b];
-      const uint32_t cb = (m >> kMetaCarryShift) & 7u, ph = (m >> kMetaPhShift) & 7u;
+      const uint32_t cb = m & 7u, ph = m >> 3;
       for (uint32_t j = ph; j < cb; ++j) {
-        dst.key[ob + j] = ckey[b * kCarry + j];
-        dst.idx[ob + j] = cidx[b * kCarry + j];
+        dst.key[ob + j] = skey[ST + b * kCarry + j];
+        dst.idx[ob + j] = sidx[ST + b * kCarry + j];
       }
     }
   }
 }
 
 template <int NT, int IT, bool HAS_IDX, bool STABLE>
-__global__ void __launch_bounds__(NT, 1)
+__global__ void __launch_bounds__(NT, kUsThreads / NT)
 k_scatter_units(const DevState* st, const LevelSeg* segs, Src src, const uint32_t* hist_scan,
                 Dst dst, uint32_t kmax, int conv, uint32_t aoff, bool auto_order) {
   // (level 1 with its order decided on the device: both forms are launched and
@@ -983,17 +979,15 @@ k_scatter_units(const DevState* st, const LevelSeg* segs, Src src, const uint32_
 // and scheduling (2^28 keys: 2.06 -> 2.24 ms), so calls with long chunks launch
 // both.
 constexpr uint32_t kAutoOneLaunchW = kFineTile;
-static_assert(kUsThreadsAny * kUsItemsAny == kFineTile, "fine chunks are one sub-tile");
-static_assert(kUsThreads == kUsThreadsAny, "both forms run with the same threads");
-__global__ void __launch_bounds__(kUsThreads, 1)
+static_assert(kUsThreads * kUsItemsAny == kFineTile, "fine chunks are one sub-tile");
+template <int NT>
+__global__ void __launch_bounds__(NT, kUsThreads / NT)
 k_scatter_units_auto(const DevState* st, const LevelSeg* segs, Src src, const uint32_t* hist_scan,
                      Dst dst, uint32_t kmax, int conv, uint32_t aoff) {
   if (l1_auto_ordered(st))
-    scatter_units<kUsThreads, kUsItems, false, true>(st, segs, src, hist_scan, dst, kmax, conv,
-                                                     aoff);
+    scatter_units<NT, kUsItems, false, true>(st, segs, src, hist_scan, dst, kmax, conv, aoff);
   else
-    scatter_units<kUsThreadsAny, kUsItemsAny, false, false>(st, segs, src, hist_scan, dst, kmax,
-                                                            conv, aoff);
+    scatter_units<NT, kUsItemsAny, false, false>(st, segs, src, hist_scan, dst, kmax, conv, aoff);
 }
 
 // ---------------------------------------------------------------------------
@@ -1121,8 +1115,22 @@ size_t classify_ids_smem_bytes(uint32_t kmax, int mode) {
 bool unit_scatter_fits(uint32_t kmax) {
   return kmax <= (uint32_t)kUnitMaxK &&
          us_smem_bytes(kmax, kUsThreads, kUsItems, true) <= g_us_smem_max &&
-         us_smem_bytes(kmax, kUsThreadsAny, kUsItemsAny, false) <= g_us_smem_max;
+         us_smem_bytes(kmax, kUsThreads, kUsItemsAny, false) <= g_us_smem_max;
 }
+
+namespace {
+template <int NT>
+bool set_scatter_units_attributes(int limit) {
+  auto set = [&](auto* f) {
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) ==
+           cudaSuccess;
+  };
+  return set(k_scatter_units<NT, kUsItems, true, true>) &&
+         set(k_scatter_units<NT, kUsItems, false, true>) &&
+         set(k_scatter_units<NT, kUsItemsAny, true, false>) &&
+         set(k_scatter_units<NT, kUsItemsAny, false, false>) && set(k_scatter_units_auto<NT>);
+}
+}  // namespace
 
 void set_unit_scatter_attributes() {
   const int ci_smem = (int)umax64(classify_ids_smem_bytes(kMaxK, 0),
@@ -1143,26 +1151,14 @@ void set_unit_scatter_attributes() {
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   cudaFuncAttributes fa{};
   size_t limit = 0;
-  if (cudaFuncGetAttributes(&fa, k_scatter_units<kUsThreads, kUsItems, true, true>) == cudaSuccess &&
+  if (cudaFuncGetAttributes(&fa, k_scatter_units_auto<kUsThreads>) == cudaSuccess &&
       (size_t)optin > fa.sharedSizeBytes) {
     limit = (size_t)optin - fa.sharedSizeBytes;
     const size_t need = umax64(us_smem_bytes(kUnitMaxK, kUsThreads, kUsItems, true),
-                               us_smem_bytes(kUnitMaxK, kUsThreadsAny, kUsItemsAny, false));
+                               us_smem_bytes(kUnitMaxK, kUsThreads, kUsItemsAny, false));
     if (limit > need) limit = need;
-    if (cudaFuncSetAttribute(k_scatter_units<kUsThreads, kUsItems, true, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)limit) != cudaSuccess ||
-        cudaFuncSetAttribute(k_scatter_units<kUsThreads, kUsItems, false, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)limit) != cudaSuccess ||
-        cudaFuncSetAttribute(k_scatter_units<kUsThreadsAny, kUsItemsAny, true, false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)limit) != cudaSuccess ||
-        cudaFuncSetAttribute(k_scatter_units_auto, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)limit) != cudaSuccess ||
-        cudaFuncSetAttribute(k_scatter_units<kUsThreadsAny, kUsItemsAny, false, false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)limit) != cudaSuccess)
+    if (!set_scatter_units_attributes<kUsThreads>((int)limit) ||
+        !set_scatter_units_attributes<kUsThreadsSmall>((int)limit))
       limit = 0;
   }
   g_us_smem_max = limit;
@@ -1241,42 +1237,52 @@ bool atomic_scatter_fits(uint32_t kmax) {
   return kmax <= (uint32_t)kMaxK && sa_smem_bytes(kmax) <= sa_smem_bytes(kMaxK);
 }
 
+namespace {
+template <int NT>
+void launch_scatter_units_nt(const LaunchEnv& e, const LevelParams& P, DevState* st,
+                             const LevelSeg* segs, const Src& src, const uint32_t* hist_scan,
+                             const Dst& dst, uint32_t kmax, int conv, uint32_t aoff) {
+  const uint64_t grid = umin64(P.chunk_cap, (uint64_t)e.num_sms * (kUsThreads / NT));
+  const int g = (int)(grid ? grid : 1);
+  const size_t smem_s = us_smem_bytes(kmax, NT, kUsItems, true);
+  const size_t smem_a = us_smem_bytes(kmax, NT, kUsItemsAny, false);
+  const bool autoo = P.stable == kOrderAuto;  // (level 1: no stored positions)
+  if (autoo && P.W <= kAutoOneLaunchW) {
+    k_scatter_units_auto<NT><<<g, NT, umax64(smem_s, smem_a), e.stream>>>(
+        st, segs, src, hist_scan, dst, kmax, conv, aoff);
+    return;
+  }
+  if (P.stable == 1 || autoo) {
+    if (src.idx)
+      k_scatter_units<NT, kUsItems, true, true><<<g, NT, smem_s, e.stream>>>(
+          st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
+    else
+      k_scatter_units<NT, kUsItems, false, true><<<g, NT, smem_s, e.stream>>>(
+          st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
+  }
+  if (autoo && e.launches) ++*e.launches;
+  if (P.stable != 1 || autoo) {
+    if (src.idx)
+      k_scatter_units<NT, kUsItemsAny, true, false><<<g, NT, smem_a, e.stream>>>(
+          st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
+    else
+      k_scatter_units<NT, kUsItemsAny, false, false><<<g, NT, smem_a, e.stream>>>(
+          st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
+  }
+}
+}  // namespace
+
 void launch_scatter_units(const LaunchEnv& e, const LevelParams& P, DevState* st,
                           const LevelSeg* segs, Src src, const uint32_t* hist_scan, Dst dst,
                           uint32_t kmax, int unmap_out, const char* name) {
   const int conv = (src.map_f64 && !unmap_out) ? 1 : ((!src.map_f64 && unmap_out) ? 2 : 0);
   // units start where the output key address is 64-byte aligned
   const uint32_t aoff = (uint32_t)(((64 - ((uintptr_t)dst.key & 63)) & 63) / 8);
-  const uint64_t grid = umin64(P.chunk_cap, (uint64_t)e.num_sms);
   Scope sc(e, name);
-  const int g = (int)(grid ? grid : 1);
-  const size_t smem_s = us_smem_bytes(kmax, kUsThreads, kUsItems, true);
-  const size_t smem_a = us_smem_bytes(kmax, kUsThreadsAny, kUsItemsAny, false);
-  const bool autoo = P.stable == kOrderAuto;  // (level 1: no stored positions)
-  if (autoo && P.W <= kAutoOneLaunchW) {
-    k_scatter_units_auto<<<g, kUsThreads, umax64(smem_s, smem_a), e.stream>>>(
-        st, segs, src, hist_scan, dst, kmax, conv, aoff);
-    return;
-  }
-  if (P.stable == 1 || autoo) {
-    if (src.idx)
-      k_scatter_units<kUsThreads, kUsItems, true, true><<<g, kUsThreads, smem_s, e.stream>>>(
-          st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
-    else
-      k_scatter_units<kUsThreads, kUsItems, false, true><<<g, kUsThreads, smem_s, e.stream>>>(
-          st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
-  }
-  if (autoo && e.launches) ++*e.launches;
-  if (P.stable != 1 || autoo) {
-    if (src.idx)
-      k_scatter_units<kUsThreadsAny, kUsItemsAny, true, false>
-          <<<g, kUsThreadsAny, smem_a, e.stream>>>(st, segs, src, hist_scan, dst, kmax, conv,
-                                                   aoff, autoo);
-    else
-      k_scatter_units<kUsThreadsAny, kUsItemsAny, false, false>
-          <<<g, kUsThreadsAny, smem_a, e.stream>>>(st, segs, src, hist_scan, dst, kmax, conv,
-                                                   aoff, autoo);
-  }
+  if (kmax <= kUsSmallK)
+    launch_scatter_units_nt<kUsThreadsSmall>(e, P, st, segs, src, hist_scan, dst, kmax, conv, aoff);
+  else
+    launch_scatter_units_nt<kUsThreads>(e, P, st, segs, src, hist_scan, dst, kmax, conv, aoff);
 }
 
 }  // namespace rsort
