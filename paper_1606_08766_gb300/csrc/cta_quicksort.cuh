@@ -45,10 +45,10 @@ struct QsSmem {
 };
 
 // Shared memory of a QsSmem for `cap` elements, followed by the CtaSortSmem
-// of the base case (kQsBase elements).
+// of the base case (kQsBase elements, 256 threads).
 __host__ __device__ constexpr size_t qs_smem_bytes(size_t cap) {
   return cap * 24 + (size_t)kQsSample * 24 + (size_t)kQsSample * 2 + (size_t)kQsStack * 8 +
-         (size_t)kQsBase * kCtaSortBytesPerElem;
+         (size_t)(BinSort<256, kQsBase / 256>::kSmem);
 }
 
 __device__ inline QsSmem qs_carve(unsigned char* base, uint32_t cap) {
@@ -78,6 +78,7 @@ __device__ inline QsSmem qs_carve(unsigned char* base, uint32_t cap) {
 template <int NT>
 __device__ void cta_quicksort_pairs(const QsSmem& q, uint32_t m, uint64_t seed,
                                     uint64_t* scan_sm, uint64_t* red) {
+  static_assert(NT == 256, "qs_smem_bytes counts the base case of 256 threads");
   static_assert(kQsBase % NT == 0, "the base case holds kQsBase / NT elements per thread");
   constexpr int kBaseItems = kQsBase / NT;
   __shared__ uint32_t s_top;

@@ -9,8 +9,8 @@
 //                       (the ranking of Appendix "Fast Work-Inefficient
 //                       Ranking", all in one CTA)
 //   otherwise           split the bucket's key range [min, max] into
-//                       2 * next_pow2(m) equal-width bins (a counting sort in
-//                       shared memory), then order each bin that holds
+//                       two equal-width bins per slot of the CTA (a counting
+//                       sort in shared memory), then order each bin that holds
 //                       several elements by insertion (an element alone in
 //                       its bin is already in place); the bins of a bucket
 //                       are tiny unless its keys cluster
@@ -36,47 +36,80 @@ static_assert(kRankMax <= kLocalThreads, "rank-by-counting holds one element per
 struct CtaSortSmem {
   uint64_t* k;     // [cap]      cap = NT * ITEMS
   uint32_t* i;     // [cap]
-  uint32_t* hist;  // [cap + cap/4 + cap/2]  up to 2*cap 16-bit bin counters
-                   //   packed in pairs (one pad word after every thread's run
-                   //   of counter words), then the list of bins holding
-                   //   several elements
+  uint32_t* hist;  // BinSort's counters, then its list of bins to order
 };
 
-// Shared memory per element of capacity that a CtaSortSmem needs.
-constexpr int kCtaSortBytesPerElem = 8 + 4 + 4 + 1 + 2;
+// Layout of the bins of a CTA with IT slots a thread: 2 * NT * IT 16-bit
+// counters, two to a word, every thread's run of IT words 4 words apart from the
+// next, so that eight lanes' 16-byte accesses to their runs cover all banks;
+// then the end of the last bin, and the list of bins that hold several pairs.
+template <int NT, int IT>
+struct BinSort {
+  static constexpr int log2c(int x) { return x <= 1 ? 0 : 1 + log2c(x / 2); }
+  static constexpr int kCap = NT * IT;
+  static constexpr int kLogIt = log2c(IT);
+  static_assert((1 << kLogIt) == IT && IT % 4 == 0, "4, 8 or 16 slots a thread");
+  static constexpr int kRun = IT + 4;                       // words from run to run
+  static constexpr int kLogBins = log2c(2 * kCap);
+  static_assert((1 << kLogBins) == 2 * kCap, "two bins per slot");
+  static constexpr int kMulti = NT * kRun + 4;              // word of the list
+  // pairs, counters, the end of the last bin, the list
+  static constexpr size_t kSmem =
+      (size_t)kCap * 12 + (size_t)NT * kRun * 4 + 16 + (size_t)kCap;
+  // halfword of bin b's counter
+  static __device__ __forceinline__ uint32_t half_of(uint32_t b) {
+    return b + ((b >> (kLogIt + 1)) << 3);
+  }
+  // halfword of the bin after the one at halfword h
+  static __device__ __forceinline__ uint32_t next_half(uint32_t h) {
+    return h % (2 * kRun) == 2 * IT - 1 ? h + 9 : h + 1;
+  }
+};
 
-// Counter word w of a scan in which every thread owns 2^lp consecutive words
-// sits at w + (w >> lp): each thread's run starts one bank further on, so the
-// lanes of a warp walking their runs in step hit distinct banks.
-__device__ __forceinline__ uint32_t padded_word(uint32_t w, int lp) { return w + (w >> lp); }
+// Runs fn(r) for every slot r of a thread that some thread of the CTA fills
+// (m pairs, slot r holding element r*NT + tid), four slots per uniform branch.
+template <int NT, int IT, typename Fn>
+__device__ __forceinline__ void for_slots(uint32_t m, Fn fn) {
+#pragma unroll
+  for (int q = 0; q < IT; q += 4) {
+    if (q == 0 || m > (uint32_t)(q * NT)) {
+#pragma unroll
+      for (int r = q; r < q + 4; ++r)
+        if (r * NT + threadIdx.x < m) fn(r);
+    }
+  }
+}
 
+// Minimum and maximum of a 64-bit value over a warp: the high words, then the
+// low words of the lanes that hold the extreme high word (four redux instead of
+// twenty shuffles).
+__device__ __forceinline__ uint64_t warp_min_u64(uint64_t v) {
+  const uint32_t h = __reduce_min_sync(0xffffffffu, (uint32_t)(v >> 32));
+  const uint32_t l =
+      __reduce_min_sync(0xffffffffu, (uint32_t)(v >> 32) == h ? (uint32_t)v : 0xffffffffu);
+  return ((uint64_t)h << 32) | l;
+}
+__device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
+  const uint32_t h = __reduce_max_sync(0xffffffffu, (uint32_t)(v >> 32));
+  const uint32_t l = __reduce_max_sync(0xffffffffu, (uint32_t)(v >> 32) == h ? (uint32_t)v : 0u);
+  return ((uint64_t)h << 32) | l;
+}
+
+// Over the CTA, one barrier; red (2 * NT/32 words) may be written again after
+// the next barrier.
 template <int NT>
 __device__ __forceinline__ void block_minmax_u64(uint64_t& mn, uint64_t& mx, uint64_t* red) {
+  constexpr int NW = NT / 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t a = __shfl_xor_sync(0xffffffffu, mn, o);
-    const uint64_t b = __shfl_xor_sync(0xffffffffu, mx, o);
-    mn = a < mn ? a : mn;
-    mx = b > mx ? b : mx;
-  }
+  mn = warp_min_u64(mn);
+  mx = warp_max_u64(mx);
   if (lane == 0) {
     red[2 * w] = mn;
     red[2 * w + 1] = mx;
   }
   __syncthreads();
-  mn = red[0];
-  mx = red[1];
-#pragma unroll
-  for (int q = 1; q < NT / 32; ++q) {
-    mn = red[2 * q] < mn ? red[2 * q] : mn;
-    mx = red[2 * q + 1] > mx ? red[2 * q + 1] : mx;
-  }
-  __syncthreads();
-}
-
-__device__ __forceinline__ uint32_t bin_start(const uint32_t* hist, uint32_t b, int lp) {
-  return (hist[padded_word(b >> 1, lp)] >> ((b & 1) << 4)) & 0xffffu;
+  mn = warp_min_u64(lane < NW ? red[2 * lane] : ~0ULL);
+  mx = warp_max_u64(lane < NW ? red[2 * lane + 1] : 0ULL);
 }
 
 // After a sort in which the positions stood in for keys that were all equal
@@ -217,96 +250,108 @@ __device__ __forceinline__ void cta_bitonic_pairs(uint32_t m, const CtaSortSmem&
   block_bitonic_sort<NT>(s.k, s.i, (int)P);
 }
 
-// Layout of a bucket's bin counters: nb 16-bit counters packed in words, each
-// thread scanning a run of 2^lp of them.
-struct BinShape {
-  uint32_t nb, words, per;
-  int lp;
-};
-
-template <int NT>
-__device__ __forceinline__ BinShape bin_shape(uint32_t m) {
-  BinShape g;
-  g.nb = 2 * next_pow2_u32(m);
-  g.words = g.nb / 2;
-  g.per = (g.words + NT - 1) / NT;  // a power of two
-  g.lp = log2_u32(g.per);
-  return g;
-}
-
-template <int NT>
-__device__ __forceinline__ void clear_bins(const BinShape& g, uint32_t* hist) {
-  for (uint32_t w = threadIdx.x; w < g.words + (g.words >> g.lp); w += NT) hist[w] = 0;
-}
-
-// Counts one element of bin b; returns bin << 16 | rank inside the bin.
-__device__ __forceinline__ uint32_t count_bin(uint32_t b, const BinShape& g, uint32_t* hist) {
-  const uint32_t sh = (b & 1) << 4;
-  const uint32_t old = atomicAdd(&hist[padded_word(b >> 1, g.lp)], 1u << sh);
-  return (b << 16) | ((old >> sh) & 0xffffu);
-}
-
-// Exclusive scan of the counters in place (each thread a run of words), which
-// also finds out whether any bin is crowded (the same answer in every thread).
-template <int NT>
-__device__ __forceinline__ bool scan_bins(const BinShape& g, uint32_t* hist, uint64_t* scan_sm) {
-  const uint32_t w0 = threadIdx.x * g.per;
-  bool crowd = false;
-  uint32_t loc = 0;
-  for (uint32_t w = w0; w < w0 + g.per && w < g.words; ++w) {
-    const uint32_t v = hist[padded_word(w, g.lp)];
-    const uint32_t a = v & 0xffffu, b = v >> 16;
-    loc += a + b;
-    crowd |= a > (uint32_t)kBinLimit || b > (uint32_t)kBinLimit;
-  }
-  uint64_t tot;
-  uint32_t run = (uint32_t)block_excl_scan_u64<NT>(loc, &tot, scan_sm);
-  for (uint32_t w = w0; w < w0 + g.per && w < g.words; ++w) {
-    const uint32_t pw = padded_word(w, g.lp);
-    const uint32_t v = hist[pw];
-    const uint32_t lo = run, hi = run + (v & 0xffffu);
-    hist[pw] = lo | (hi << 16);
-    run = hi + (v >> 16);
-  }
-  return __syncthreads_or(crowd);
-}
-
-// Counting-sort scatter of the pairs into their bins; the second element to
-// land in a bin puts the bin on the list of bins that still need ordering.
-template <int NT, int ITEMS>
-__device__ __forceinline__ void place_in_bins(const uint64_t (&key)[ITEMS],
-                                              const uint32_t (&idx)[ITEMS],
-                                              const uint32_t (&bs)[ITEMS], uint32_t m,
-                                              const BinShape& g, const CtaSortSmem& s,
-                                              uint32_t* nmulti) {
-  constexpr uint32_t kCap = NT * ITEMS;
-  uint32_t* multi = s.hist + kCap + kCap / 4;
+template <int NT, int IT>
+__device__ __forceinline__ void clear_bins(uint32_t* hist) {
+  uint4* run = (uint4*)(hist + threadIdx.x * BinSort<NT, IT>::kRun);
 #pragma unroll
-  for (int r = 0; r < ITEMS; ++r) {
-    if (r * NT + threadIdx.x < m) {
-      const uint32_t b = bs[r] >> 16, o = bs[r] & 0xffffu;
-      const uint32_t p = bin_start(s.hist, b, g.lp) + o;
-      s.k[p] = key[r];
-      s.i[p] = idx[r];
-      if (o == 1) multi[atomicAdd(nmulti, 1u)] = b;
-    }
-  }
+  for (int q = 0; q < IT / 4; ++q) run[q] = make_uint4(0, 0, 0, 0);
 }
 
-// Orders every listed bin in place by insertion (at most kBinLimit elements;
-// an element alone in its bin is already in its final slot).
-template <int NT, int ITEMS>
-__device__ __forceinline__ void order_bins(uint32_t m, const BinShape& g, const CtaSortSmem& s,
-                                           uint32_t nmulti) {
-  constexpr uint32_t kCap = NT * ITEMS;
-  const uint32_t* multi = s.hist + kCap + kCap / 4;
+// Counts one pair of the bin whose counter is halfword h; returns h << 16 | its
+// rank inside the bin.
+__device__ __forceinline__ uint32_t count_bin(uint32_t h, uint32_t* hist) {
+  const uint32_t sh = (h & 1) << 4;
+  const uint32_t old = atomicAdd(&hist[h >> 1], 1u << sh);
+  return (h << 16) | ((old >> sh) & 0xffffu);
+}
+
+// Exclusive scan of the counters in place (m pairs; each thread its run of
+// words, a word's two counts added by one dp2a), one barrier inside; s_sum holds
+// NT/32 words.  Returns whether a bin holds kBinLimit pairs or more (the same in
+// every thread): one of the high bits of the OR of all counters.  The caller
+// synchronises before it reads the starts.
+template <int NT, int IT>
+__device__ __forceinline__ bool scan_bins(uint32_t* hist, uint32_t m, uint32_t* s_sum) {
+  using BS = BinSort<NT, IT>;
+  constexpr int NW = NT / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint4* run = (uint4*)(hist + threadIdx.x * BS::kRun);
+  uint32_t sum = 0, any = 0;
+#pragma unroll
+  for (int q = 0; q < IT / 4; ++q) {
+    const uint4 v = run[q];
+    sum = __dp2a_lo(v.x, 0x0101u, sum);
+    sum = __dp2a_lo(v.y, 0x0101u, sum);
+    sum = __dp2a_lo(v.z, 0x0101u, sum);
+    sum = __dp2a_lo(v.w, 0x0101u, sum);
+    any |= v.x | v.y | v.z | v.w;
+  }
+  uint32_t inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  static_assert((kBinLimit & (kBinLimit - 1)) == 0, "the crowd test reads high bits");
+  constexpr uint32_t kHigh = 0xffffu & ~(uint32_t)(kBinLimit - 1);
+  const bool crowd = __any_sync(0xffffffffu, (any & (kHigh | (kHigh << 16))) != 0);
+  if (lane == 31) s_sum[warp] = inc | (crowd ? 0x80000000u : 0u);
+  __syncthreads();
+  uint32_t pre = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    const uint32_t v = s_sum[w];
+    pre += w < warp ? v : 0u;
+    all |= v;
+  }
+  uint32_t at = (pre & 0xffffu) + inc - sum;  // (the sums' crowd flags fall away)
+#pragma unroll
+  for (int q = 0; q < IT / 4; ++q) {
+    uint4 v = run[q];
+    auto step = [&](uint32_t& w) {
+      const uint32_t c = w;
+      w = at * 0x10001u + (c << 16);
+      at = __dp2a_lo(c, 0x0101u, at);
+    };
+    step(v.x);
+    step(v.y);
+    step(v.z);
+    step(v.w);
+    run[q] = v;
+  }
+  if (threadIdx.x == NT - 1) ((uint16_t*)hist)[NT * BS::kRun * 2] = (uint16_t)m;
+  return (all >> 31) != 0;
+}
+
+// Counting-sort scatter of the pairs into their bins; the second one to land in
+// a bin puts the bin on the list of bins that still need ordering.
+template <int NT, int IT>
+__device__ __forceinline__ void place_in_bins(const uint64_t (&key)[IT], const uint32_t (&idx)[IT],
+                                              const uint32_t (&hr)[IT], uint32_t m,
+                                              const CtaSortSmem& s, uint32_t* nmulti) {
+  const uint16_t* half = (const uint16_t*)s.hist;
+  uint16_t* multi = (uint16_t*)(s.hist + BinSort<NT, IT>::kMulti);
+  for_slots<NT, IT>(m, [&](int r) {
+    const uint32_t h = hr[r] >> 16, o = hr[r] & 0xffffu;
+    const uint32_t p = half[h] + o;
+    s.k[p] = key[r];
+    s.i[p] = idx[r];
+    if (o == 1) multi[atomicAdd(nmulti, 1u)] = (uint16_t)h;
+  });
+}
+
+// Orders every listed bin in place by insertion (fewer than kBinLimit pairs; one
+// alone in its bin is already in its final slot).
+template <int NT, int IT>
+__device__ __forceinline__ void order_bins(const CtaSortSmem& s, uint32_t nmulti) {
+  const uint16_t* half = (const uint16_t*)s.hist;
+  const uint16_t* multi = (const uint16_t*)(s.hist + BinSort<NT, IT>::kMulti);
   for (uint32_t j = threadIdx.x; j < nmulti; j += NT) {
-    const uint32_t b = multi[j];
-    const uint32_t lo = bin_start(s.hist, b, g.lp);
-    const uint32_t hi = b + 1 < g.nb ? bin_start(s.hist, b + 1, g.lp) : m;
+    const uint32_t h = multi[j];
+    const uint32_t lo = half[h], cnt = half[BinSort<NT, IT>::next_half(h)] - lo;
     uint64_t* bk = s.k + lo;
     uint32_t* bi = s.i + lo;
-    for (uint32_t a = 1; a < hi - lo; ++a) {
+    for (uint32_t a = 1; a < cnt; ++a) {
       const uint64_t ka = bk[a];
       const uint32_t ia = bi[a];
       uint32_t q = a;
@@ -337,52 +382,46 @@ __device__ __forceinline__ void order_bins(uint32_t m, const BinShape& g, const 
 //   (k_direct_sort): 15 us.
 template <int NT, int ITEMS>
 __device__ __noinline__ int cta_sort_crowded(uint32_t m, uint64_t mn, int shift, CtaSortSmem s,
-                                             uint64_t* scan_sm, uint64_t* red) {
+                                             uint32_t* s_sum, uint64_t* red) {
+  using BS = BinSort<NT, ITEMS>;
   const uint32_t tid = threadIdx.x;
   {
-    const BinShape g = bin_shape<NT>(m);
     __shared__ uint32_t s_nmulti;
+    const uint16_t* half = (const uint16_t*)s.hist;
     uint64_t key[ITEMS];
-    uint32_t idx[ITEMS], bs[ITEMS];
+    uint32_t idx[ITEMS], hr[ITEMS];
     uint64_t imn = ~0ULL, imx = 0;
-#pragma unroll
-    for (int r = 0; r < ITEMS; ++r) {
+    for_slots<NT, ITEMS>(m, [&](int r) {
       const uint32_t e = r * NT + tid;
-      if (e < m) {
-        key[r] = s.k[e];
-        idx[r] = s.i[e];
-        imn = idx[r] < imn ? idx[r] : imn;
-        imx = idx[r] > imx ? idx[r] : imx;
-      }
-    }
+      key[r] = s.k[e];
+      idx[r] = s.i[e];
+      imn = idx[r] < imn ? idx[r] : imn;
+      imx = idx[r] > imx ? idx[r] : imx;
+    });
     int pshift = 0;  // positions' range in bits, when they order the parts
     if (shift == 0) {
       block_minmax_u64<NT>(imn, imx, red);
       pshift = imx > imn ? 64 - __clzll((long long)(imx - imn)) : 1;
     }
-#pragma unroll
-    for (int r = 0; r < ITEMS; ++r) {
-      if (r * NT + tid < m) {
-        const uint32_t b = (uint32_t)((key[r] - mn) >> shift);
-        const uint32_t lo = bin_start(s.hist, b, g.lp);
-        const uint32_t hi = b + 1 < g.nb ? bin_start(s.hist, b + 1, g.lp) : m;
-        const uint64_t off = shift ? (key[r] - mn) << (64 - shift)
-                                   : ((uint64_t)idx[r] - imn) << (64 - pshift);
-        bs[r] = 2 * lo + (uint32_t)__umul64hi(off, (uint64_t)(2 * (hi - lo)));
-      }
-    }
+    for_slots<NT, ITEMS>(m, [&](int r) {
+      const uint32_t h = BS::half_of((uint32_t)((key[r] - mn) >> shift));
+      const uint32_t lo = half[h], c = half[BS::next_half(h)] - lo;
+      const uint64_t off = shift ? (key[r] - mn) << (64 - shift)
+                                 : ((uint64_t)idx[r] - imn) << (64 - pshift);
+      hr[r] = BS::half_of(2 * lo + (uint32_t)__umul64hi(off, (uint64_t)(2 * c)));
+    });
     if (tid == 0) s_nmulti = 0;
     __syncthreads();
-    clear_bins<NT>(g, s.hist);
+    clear_bins<NT, ITEMS>(s.hist);
     __syncthreads();
-#pragma unroll
-    for (int r = 0; r < ITEMS; ++r)
-      if (r * NT + tid < m) bs[r] = count_bin(bs[r], g, s.hist);
+    for_slots<NT, ITEMS>(m, [&](int r) { hr[r] = count_bin(hr[r], s.hist); });
     __syncthreads();
-    if (!scan_bins<NT>(g, s.hist, scan_sm)) {
-      place_in_bins<NT, ITEMS>(key, idx, bs, m, g, s, &s_nmulti);
+    const bool crowd = scan_bins<NT, ITEMS>(s.hist, m, s_sum);
+    __syncthreads();
+    if (!crowd) {
+      place_in_bins<NT, ITEMS>(key, idx, hr, m, s, &s_nmulti);
       __syncthreads();
-      order_bins<NT, ITEMS>(m, g, s, s_nmulti);
+      order_bins<NT, ITEMS>(s, s_nmulti);
       __syncthreads();
       return kAlgoBins;
     }
@@ -411,7 +450,6 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
                                InOrderFn in_position_order, const CtaSortSmem& s, uint64_t* red,
                                uint64_t* scan_sm, uint64_t* algo, uint32_t rank_max = kRankMax,
                                bool force_bitonic = false, ReleaseFn released = ReleaseFn()) {
-  static_assert(ITEMS >= 4, "the padded counters need cap/4 >= NT words of slack");
   const uint32_t tid = threadIdx.x;
   if (m <= rank_max && m <= (uint32_t)NT) {
     count_algo(algo, kAlgoRank, m);
@@ -449,13 +487,10 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
     return;
   }
   uint64_t mn = ~0ULL, mx = 0;
-#pragma unroll
-  for (int r = 0; r < ITEMS; ++r) {
-    if (r * NT + tid < m) {
-      mn = key[r] < mn ? key[r] : mn;
-      mx = key[r] > mx ? key[r] : mx;
-    }
-  }
+  for_slots<NT, ITEMS>(m, [&](int r) {
+    mn = key[r] < mn ? key[r] : mn;
+    mx = key[r] > mx ? key[r] : mx;
+  });
   block_minmax_u64<NT>(mn, mx, red);
   if (mn == mx && in_position_order()) {
     count_algo(algo, kAlgoInOrder, m);
@@ -478,41 +513,42 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
     s_key_all = mn;
   }
   if (mn == mx) {
+    __syncthreads();  // (red is written again)
     mn = ~0ULL;
     mx = 0;
-#pragma unroll
-    for (int r = 0; r < ITEMS; ++r) {
-      if (r * NT + tid < m) {
-        key[r] = idx[r];
-        mn = key[r] < mn ? key[r] : mn;
-        mx = key[r] > mx ? key[r] : mx;
-      }
-    }
+    for_slots<NT, ITEMS>(m, [&](int r) {
+      key[r] = idx[r];
+      mn = key[r] < mn ? key[r] : mn;
+      mx = key[r] > mx ? key[r] : mx;
+    });
     block_minmax_u64<NT>(mn, mx, red);
   }
   // equal-width bins over [mn, mx]
-  const BinShape g = bin_shape<NT>(m);  // g.nb <= 2 * kCap
-  const int lognb = log2_u32(g.nb);
+  using BS = BinSort<NT, ITEMS>;
+  uint32_t* s_sum = (uint32_t*)scan_sm;
   const uint64_t range = mx - mn;
   const int bits = range ? 64 - __clzll((long long)range) : 0;
-  const int shift = bits > lognb ? bits - lognb : 0;
-  clear_bins<NT>(g, s.hist);
+  const int shift = bits > BS::kLogBins ? bits - BS::kLogBins : 0;
   __shared__ uint32_t s_nmulti;
+  clear_bins<NT, ITEMS>(s.hist);
   if (tid == 0) s_nmulti = 0;
   __syncthreads();
-  uint32_t bs[ITEMS];
-#pragma unroll
-  for (int r = 0; r < ITEMS; ++r)
-    if (r * NT + tid < m) bs[r] = count_bin((uint32_t)((key[r] - mn) >> shift), g, s.hist);
+  uint32_t hr[ITEMS];
+  for_slots<NT, ITEMS>(m, [&](int r) {
+    hr[r] = count_bin(BS::half_of((uint32_t)((key[r] - mn) >> shift)), s.hist);
+  });
   __syncthreads();
-  if (scan_bins<NT>(g, s.hist, scan_sm)) {
+  const bool crowd = scan_bins<NT, ITEMS>(s.hist, m, s_sum);
+  if (crowd) {
 #pragma unroll
     for (int r = 0; r < ITEMS; ++r) {
       const uint32_t e = r * NT + tid;
       if (e < m) { s.k[e] = key[r]; s.i[e] = idx[r]; }
     }
-    __syncthreads();
-    const int how = cta_sort_crowded<NT, ITEMS>(m, mn, shift, s, scan_sm, red);
+  }
+  __syncthreads();
+  if (crowd) {
+    const int how = cta_sort_crowded<NT, ITEMS>(m, mn, shift, s, s_sum, red);
     // (no register of the pairs is kept across the call)
 #pragma unroll
     for (int r = 0; r < ITEMS; ++r) {
@@ -525,10 +561,10 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
     return;
   }
   count_algo(algo, kAlgoBins, m);
-  place_in_bins<NT, ITEMS>(key, idx, bs, m, g, s, &s_nmulti);
+  place_in_bins<NT, ITEMS>(key, idx, hr, m, s, &s_nmulti);
   __syncthreads();
   released();
-  order_bins<NT, ITEMS>(m, g, s, s_nmulti);
+  order_bins<NT, ITEMS>(s, s_nmulti);
   __syncthreads();
   restore_common_key<NT>(s, m, s_by_pos, s_key_all);
 }

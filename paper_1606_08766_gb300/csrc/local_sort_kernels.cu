@@ -196,41 +196,6 @@ __device__ __forceinline__ int64_t next_item(DevState* st, int cls, uint64_t cap
 //     travel while this one is sorted, and its loads go out as soon as this
 //     one's pairs have left the registers.
 // ---------------------------------------------------------------------------
-template <int NT, int IT>
-struct BinSort {
-  static constexpr int kCap = NT * IT;
-  static constexpr int kLogIt = IT == 8 ? 3 : 4;
-  static_assert((1 << kLogIt) == IT, "8 or 16 slots a thread");
-  static constexpr int kRun = IT + 4;                       // counter words between two runs
-  static constexpr int kLogBins = kLogIt + 1 + (NT == 128 ? 7 : 8);
-  static_assert((1 << kLogBins) == 2 * kCap, "two bins per slot");
-  // counters, the end of the last bin, and the list of bins to order
-  static constexpr size_t kSmem =
-      (size_t)kCap * 12 + (size_t)NT * kRun * 4 + 16 + (size_t)kCap;
-  // halfword of bin b's counter
-  static __device__ __forceinline__ uint32_t half_of(uint32_t b) {
-    return b + ((b >> (kLogIt + 1)) << 3);
-  }
-  // halfword of the bin after the one at halfword h
-  static __device__ __forceinline__ uint32_t next_half(uint32_t h) {
-    return h % (2 * kRun) == 2 * IT - 1 ? h + 9 : h + 1;
-  }
-};
-
-// Runs fn(r) for every slot r of a thread that some thread of the CTA fills
-// (m pairs, slot r holding element r*NT + tid), four slots per uniform branch.
-template <int NT, int IT, typename Fn>
-__device__ __forceinline__ void for_slots(uint32_t m, Fn fn) {
-#pragma unroll
-  for (int q = 0; q < IT; q += 4) {
-    if (q == 0 || m > (uint32_t)(q * NT)) {
-#pragma unroll
-      for (int r = q; r < q + 4; ++r)
-        if (r * NT + threadIdx.x < m) fn(r);
-    }
-  }
-}
-
 // REFINE: crowded bins are refined once (as in cta_sort_crowded) before the
 // bucket is given up; the instantiations for a batch's float64 buckets that
 // span many octaves (a separate kernel for the same reason of registers).
@@ -340,9 +305,8 @@ k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
       if (tid == 0) s_nmulti = 0;
 #pragma unroll 1
       for (int pass = 0;; ++pass) {
+        clear_bins<NT, IT>(hist);
         uint4* run = (uint4*)(hist + tid * BS::kRun);
-#pragma unroll
-        for (int q = 0; q < IT / 4; ++q) run[q] = make_uint4(0, 0, 0, 0);
         __syncthreads();  // (1) counters clear; the previous bucket written out
         for_slots<NT, IT>(m, [&](int r) {
           const uint32_t h = hr[r];
@@ -661,6 +625,9 @@ constexpr int kMediumItems = kBucketCap / kMediumThreads;  // 16
 static_assert(kMediumThreads * kMediumItems == kBucketCap, "medium class fits one CTA");
 
 
+constexpr size_t kDirectSmem = BinSort<kDirectThreads, kBucketCap / kDirectThreads>::kSmem;
+constexpr size_t kRestSmem = BinSort<kRestThreads, kBucketCap / kRestThreads>::kSmem;
+
 // Calls whose buckets cannot outnumber this many per SM finish in one launch
 // of k_local_rest: 66 buckets (10^5 keys) 54 -> 15 us, 714 buckets (2^20 keys)
 // 43 -> 29 us against a launch per class; the class kernels sort a bucket in
@@ -691,13 +658,13 @@ void set_local_kernel_attributes() {
   set_class_attributes<kMediumThreads, kMediumItems, kClassMedium, kMediumPerSm,
                        kMediumPerSm>();
   cudaFuncSetAttribute(k_direct_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kBucketCap * kCtaSortBytesPerElem);
+                       (int)kDirectSmem);
   cudaFuncSetAttribute(k_local_quicksort<kLocalThreads, (int)kMidCap, kClassMid>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs_smem_bytes(kMidCap));
   cudaFuncSetAttribute(k_local_quicksort<kLocalThreads, kBucketCap, kClassMedium>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs_smem_bytes(kBucketCap));
   cudaFuncSetAttribute(k_local_rest, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kBucketCap * kCtaSortBytesPerElem);
+                       (int)kRestSmem);
 }
 
 bool direct_sort_takes(const LocalPlan& local, uint64_t n) {
@@ -713,7 +680,7 @@ void launch_direct_sort(const LaunchEnv& e, DevState* st, const uint64_t* in_key
   B.tmp = out;
   B.f64 = f64;
   Scope sc(e, "direct_sort");
-  k_direct_sort<<<1, kDirectThreads, kBucketCap * kCtaSortBytesPerElem, e.stream>>>(st, B, n,
+  k_direct_sort<<<1, kDirectThreads, kDirectSmem, e.stream>>>(st, B, n,
                                                                                     e.local);
 }
 
@@ -772,7 +739,7 @@ void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint6
   {
     Scope sc(e, "local_rest");
     const uint64_t grid = umin64(umax64(max_items, 1), (uint64_t)e.num_sms * 2);
-    k_local_rest<<<(int)grid, kRestThreads, kBucketCap * kCtaSortBytesPerElem, e.stream>>>(
+    k_local_rest<<<(int)grid, kRestThreads, kRestSmem, e.stream>>>(
         st, items, item_cap, B, lists, bitonic);
   }
 }

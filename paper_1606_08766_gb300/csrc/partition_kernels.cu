@@ -1437,7 +1437,7 @@ void launch_init_plain(const LaunchEnv& e, DevState* st, FinalItem* items, uint6
 template <int NT, int IT, int MINB>
 void set_sample_sort_attributes() {
   cudaFuncSetAttribute(k_sample_sort<NT, IT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       NT * IT * kCtaSortBytesPerElem);
+                       (int)BinSort<NT, IT>::kSmem);
 }
 
 void set_partition_kernel_attributes() {
@@ -1447,7 +1447,7 @@ void set_partition_kernel_attributes() {
   set_sample_sort_attributes<512, 16, 1>();
   set_sample_sort_attributes<1024, 8, 1>();
   cudaFuncSetAttribute(k_sample_merge, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kMergeThreads * kMergeItems * kCtaSortBytesPerElem);
+                       (int)BinSort<kMergeThreads, kMergeItems>::kSmem);
   const size_t c = umax64(part_smem_bytes(kMaxK, false, 0), part_smem_bytes(kMaxK, false, 1));
   const size_t s = umax64(part_smem_bytes(kMaxK, true, 0), part_smem_bytes(kMaxK, true, 1));
   cudaFuncSetAttribute(k_classify_count<kCStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1589,7 +1589,7 @@ void launch_sample_sort(const LaunchEnv& e, const char* name, uint64_t chunks, D
                         const PlainStart& ps, const LevelParams& P) {
   Scope sc(e, name);
   k_sample_sort<NT, IT, MINB>
-      <<<grid_for(chunks, 1, e.num_sms * MINB), NT, NT * IT * kCtaSortBytesPerElem, e.stream>>>(
+      <<<grid_for(chunks, 1, e.num_sms * MINB), NT, BinSort<NT, IT>::kSmem, e.stream>>>(
           st, segs, src, samp_key, samp_idx, ssamp_key, ssamp_idx, P.in_order, min_len, ps, P);
 }
 
@@ -1641,7 +1641,7 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
       draw(std::integral_constant<int, 1024>(), std::integral_constant<int, 8>());
     if (nsch > 1) {
       Scope sc(e, nm[2]);
-      const int smem = kMergeThreads * kMergeItems * kCtaSortBytesPerElem;
+      const size_t smem = BinSort<kMergeThreads, kMergeItems>::kSmem;
       k_sample_merge<<<(int)((ps.S + kMergeRange - 1) / kMergeRange), kMergeThreads, smem,
                        e.stream>>>(segs, samp_key, samp_idx, ssamp_key, ssamp_idx);
     }
