@@ -204,6 +204,7 @@ __device__ __forceinline__ int64_t next_item(DevState* st, int cls, uint64_t cap
 template <int NT, int IT, int CLS, int MINB, bool REFINE>
 __global__ void __launch_bounds__(NT, MINB)
 k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
+  pdl_entry();
   using BS = BinSort<NT, IT>;
   constexpr int NW = NT / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -452,6 +453,7 @@ k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
 template <int NT, int CAP, int CLS>
 __global__ void __launch_bounds__(NT, 1)
 k_local_quicksort(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, uint64_t seed) {
+  pdl_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const QsSmem q = qs_carve(smem_raw, CAP);
   __shared__ uint64_t scan_sm[NT / 32];
@@ -489,6 +491,7 @@ k_local_quicksort(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, ui
 __global__ void __launch_bounds__(kRestThreads, 2)
 k_local_rest(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, uint32_t lists,
              uint32_t bitonic) {
+  pdl_entry();
   constexpr int NT = kRestThreads, IT = kBucketCap / kRestThreads;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CtaSortSmem s;
@@ -562,6 +565,7 @@ k_local_rest(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, uint32_
 constexpr int kDirectThreads = 512;
 __global__ void __launch_bounds__(kDirectThreads, 1)
 k_direct_sort(DevState* st, Bufs B, uint32_t n, LocalPlan local) {
+  pdl_entry();
   constexpr int NT = kDirectThreads, IT = kBucketCap / kDirectThreads;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CtaSortSmem s;
@@ -638,8 +642,8 @@ template <int NT, int IT, int CLS, int MINB, bool REFINE>
 void launch_class(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t cap, const Bufs& B,
                   const char* name) {
   Scope sc(e, name);
-  k_local_sort<NT, IT, CLS, MINB, REFINE>
-      <<<e.num_sms * MINB, NT, BinSort<NT, IT>::kSmem, e.stream>>>(st, items, cap, B);
+  launch_kernel(e, k_local_sort<NT, IT, CLS, MINB, REFINE>, e.num_sms * MINB, NT,
+                BinSort<NT, IT>::kSmem, st, items, cap, B);
 }
 
 template <int NT, int IT, int CLS, int MINB, int MINBR>
@@ -680,8 +684,7 @@ void launch_direct_sort(const LaunchEnv& e, DevState* st, const uint64_t* in_key
   B.tmp = out;
   B.f64 = f64;
   Scope sc(e, "direct_sort");
-  k_direct_sort<<<1, kDirectThreads, kDirectSmem, e.stream>>>(st, B, n,
-                                                                                    e.local);
+  launch_kernel(e, k_direct_sort, 1, kDirectThreads, kDirectSmem, st, B, n, e.local);
 }
 
 void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t item_cap,
@@ -714,9 +717,9 @@ void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint6
   }
   if (algo[kClassMid - kClassSmall] == kLocalQuick) {
     Scope sc(e, "local_sort_mid");
-    k_local_quicksort<kLocalThreads, (int)kMidCap, kClassMid>
-        <<<e.num_sms * 2, kLocalThreads, qs_smem_bytes(kMidCap), e.stream>>>(
-            st, items, item_cap, B, 0x243f6a8885a308d3ULL);
+    launch_kernel(e, k_local_quicksort<kLocalThreads, (int)kMidCap, kClassMid>, e.num_sms * 2,
+                  kLocalThreads, qs_smem_bytes(kMidCap), st, items, item_cap, B,
+                  0x243f6a8885a308d3ULL);
   } else if (own(kClassMid)) {
     launch_class<kMidThreads, kMidItems, kClassMid, kMidPerSm, false>(e, st, items, item_cap, B,
                                                                       "local_sort_mid");
@@ -726,9 +729,9 @@ void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint6
   }
   if (algo[kClassMedium - kClassSmall] == kLocalQuick) {
     Scope sc(e, "local_sort_medium");
-    k_local_quicksort<kLocalThreads, kBucketCap, kClassMedium>
-        <<<e.num_sms * 2, kLocalThreads, qs_smem_bytes(kBucketCap), e.stream>>>(
-            st, items, item_cap, B, 0x9e3779b97f4a7c15ULL);
+    launch_kernel(e, k_local_quicksort<kLocalThreads, kBucketCap, kClassMedium>, e.num_sms * 2,
+                  kLocalThreads, qs_smem_bytes(kBucketCap), st, items, item_cap, B,
+                  0x9e3779b97f4a7c15ULL);
   } else if (own(kClassMedium)) {
     launch_class<kMediumThreads, kMediumItems, kClassMedium, kMediumPerSm, false>(
         e, st, items, item_cap, B, "local_sort_medium");
@@ -739,8 +742,8 @@ void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint6
   {
     Scope sc(e, "local_rest");
     const uint64_t grid = umin64(umax64(max_items, 1), (uint64_t)e.num_sms * 2);
-    k_local_rest<<<(int)grid, kRestThreads, kRestSmem, e.stream>>>(
-        st, items, item_cap, B, lists, bitonic);
+    launch_kernel(e, k_local_rest, (int)grid, kRestThreads, kRestSmem, st, items, item_cap, B,
+                  lists, bitonic);
   }
 }
 

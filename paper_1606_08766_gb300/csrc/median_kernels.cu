@@ -212,6 +212,7 @@ template <int K>
 __global__ void __launch_bounds__(kTmThreads)
 k_tm_leaves(const uint64_t* keys, uint32_t n, int f64, uint64_t seed, uint32_t leaves,
             TmWindows out, uint64_t* out_pos, uint32_t* error) {
+  pdl_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const TmLeafSmem<K> m(smem_raw);
   constexpr int H = K / 2;  // leaves a thread sorts
@@ -255,6 +256,7 @@ template <int K>
 __global__ void __launch_bounds__(kTmThreads)
 k_tm_windows(TmWindows in, uint32_t count, uint64_t seed, uint64_t leaves, TmWindows out,
              uint64_t* out_pos) {
+  pdl_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const TmWindowSmem<K> m(smem_raw);
   constexpr uint32_t kGroup = kTmEntries<K> / K;
@@ -300,13 +302,13 @@ void launch_k(const LaunchEnv& e, const uint64_t* keys, uint32_t n, int f64, uin
     p += w;
     p = (unsigned char*)(((uintptr_t)p + 15) & ~(uintptr_t)15);
   }
-  k_tm_leaves<K><<<w, kTmThreads, TmLeafSmem<K>::kBytes, e.stream>>>(
-      keys, n, f64, seed, leaves, lv[0], out, &st->error);
+  launch_kernel(e, k_tm_leaves<K>, w, kTmThreads, TmLeafSmem<K>::kBytes, keys, n, f64, seed, leaves,
+                lv[0], out, &st->error);
   for (int i = 0; w > 1; i ^= 1) {
     constexpr uint32_t kGroup = kTmEntries<K> / K;
     const uint32_t groups = w > kGroup ? w / kGroup : 1;
-    k_tm_windows<K><<<groups, kTmThreads, TmWindowSmem<K>::kBytes, e.stream>>>(
-        lv[i], w, seed, leaves, lv[i ^ 1], out);
+    launch_kernel(e, k_tm_windows<K>, groups, kTmThreads, TmWindowSmem<K>::kBytes, lv[i], w, seed,
+                  leaves, lv[i ^ 1], out);
     if (e.launches) ++*e.launches;
     w = groups;
   }

@@ -149,6 +149,7 @@ extern "C" rsort_status rsort_partition_noalloc(rsort_key_type type, const void*
   e.num_sms = sms;
   e.timer = nullptr;
   e.launches = nullptr;
+  e.overlap = n <= kOverlapMaxKeys;
   // The control block is reset by the first kernel; every other scratch word
   // read later is written earlier in the same call.
   Src src{(const uint64_t*)d_keys_in, nullptr, type == RSORT_KEY_F64};

@@ -68,6 +68,7 @@ __device__ __forceinline__ void reset_state(DevState* st, const LocalPlan& local
 // one CTA sorts.
 __global__ void k_init_plain(DevState* st, FinalItem* items, uint64_t n, uint64_t final_cap,
                              LocalPlan local) {
+  pdl_entry();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   reset_state(st, local);
   if (n == 0) return;
@@ -98,7 +99,7 @@ __device__ __forceinline__ void fill_segment(LevelSeg& s, uint64_t start, uint32
   s.k = k;
   s.S = S;
   s.nchunks = nch;
-  s.nschunks = (S + kSampleChunk - 1) / kSampleChunk;
+  s.nschunks = (S + P.sample_chunk - 1) / P.sample_chunk;
   s.nunits = nch;
   // equal chunks inside the segment (the level's W bounds their size)
   s.W = nch ? (uint32_t)(((uint64_t)m + nch - 1) / nch) : P.W;
@@ -148,6 +149,7 @@ __device__ __forceinline__ SegIn plan_shape(const SegIn* list_in, uint32_t g, ui
 __global__ void __launch_bounds__(kPlanThreads)
 k_plan_sums(const DevState* st, const SegIn* list_in, LevelParams P, int par_in,
             uint32_t kmax_level, uint64_t* plan_sums) {
+  pdl_entry();
   __shared__ uint64_t sm[kPlanThreads / 32];
   const uint32_t G = st->nseg[par_in];
   if (G > P.seg_cap || (uint64_t)blockIdx.x * kPlanThreads >= G) return;
@@ -164,6 +166,7 @@ k_plan_sums(const DevState* st, const SegIn* list_in, LevelParams P, int par_in,
 __global__ void __launch_bounds__(kPlanThreads)
 k_level_plan(DevState* st, const SegIn* list_in, LevelSeg* segs, LevelParams P, int par_in,
              uint32_t kmax_level, const uint64_t* plan_sums, uint32_t* chunk_seg) {
+  pdl_entry();
   __shared__ uint64_t sm[kPlanThreads / 32];
   const uint32_t G0 = st->nseg[par_in];
   const bool over = G0 > P.seg_cap;
@@ -308,6 +311,7 @@ __global__ void __launch_bounds__(NT, MINB)
 k_sample_sort(DevState* st, LevelSeg* segs, Src src, uint64_t* samp_key, uint32_t* samp_idx,
               uint64_t* ssamp_key, uint32_t* ssamp_idx, int in_order, uint32_t min_len,
               PlainStart ps, LevelParams P) {
+  pdl_entry();
   constexpr uint32_t kCap = NT * IT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CtaSortSmem s;
@@ -376,16 +380,17 @@ k_sample_sort(DevState* st, LevelSeg* segs, Src src, uint64_t* samp_key, uint32_
 // rank in its own sorted sequence plus its ranks in the others, Appendix "Fast
 // Work-Inefficient Ranking"), and the CTA sorts them in shared memory.  A range
 // that does not fit is placed pair by pair by its ranks.
-//   163,840 samples in 20 chunks: ranking every pair in every other chunk
+//   163,840 samples: ranking every pair in every other chunk
 //   81 us, this form 19 us.
 constexpr int kMergeThreads = 512;
 constexpr int kMergeItems = 8;
 constexpr uint32_t kMergeRange = 1024;   // pairs a CTA is given on average
-constexpr uint32_t kMaxSampleChunks = 64;
-static_assert(16u * 11 * kMaxK <= kMaxSampleChunks * kSampleChunk, "a run per sample chunk");
+constexpr uint32_t kMaxSampleChunks = 96;
+static_assert(16u * 11 * kMaxK <= kMaxSampleChunks * kSampleChunk / 2, "a run per sample chunk");
 __global__ void __launch_bounds__(kMergeThreads, 2)
 k_sample_merge(const LevelSeg* segs, const uint64_t* samp_key, const uint32_t* samp_idx,
                uint64_t* ssamp_key, uint32_t* ssamp_idx) {
+  pdl_entry();
   constexpr int NT = kMergeThreads, IT = kMergeItems;
   constexpr uint32_t kCap = NT * IT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -607,6 +612,7 @@ template <int STAGES>
 __global__ void __launch_bounds__(kPartThreads, STAGES == 2 ? 4 : 3)
 k_classify_count(const DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
                  const uint32_t* ssi, uint32_t* hist, uint32_t W, uint32_t kmax, int mode) {
+  pdl_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PartSmem sm = carve(smem_raw, kmax, false, mode);
   uint64_t* stage = (uint64_t*)sm.buf;
@@ -703,6 +709,7 @@ k_classify_count(const DevState* st, const LevelSeg* segs, Src src, const uint64
 // words at most) and scans the tile.
 __global__ void __launch_bounds__(1024)
 k_scan_reduce(const DevState* st, const uint32_t* a, uint32_t* sums) {
+  pdl_entry();
   __shared__ uint64_t sm[32];
   const uint64_t total = st->total_hist;
   const uint64_t base = (uint64_t)blockIdx.x * kScanTile;
@@ -739,6 +746,7 @@ __device__ __forceinline__ uint32_t scan_tile(uint32_t* a, uint64_t base, uint64
 
 __global__ void __launch_bounds__(1024)
 k_scan_down(const DevState* st, uint32_t* a, const uint32_t* sums) {
+  pdl_entry();
   __shared__ uint64_t sm[32];
   const uint64_t total = st->total_hist;
   const uint64_t base = (uint64_t)blockIdx.x * kScanTile;
@@ -767,6 +775,7 @@ __global__ void __launch_bounds__(NT, (NT <= 256 ? 2 : 1))
 k_scatter(const DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
           const uint32_t* ssi, const uint32_t* hist_scan, Dst dst, uint32_t W, uint32_t kmax,
           int unmap_out, int mode) {
+  pdl_entry();
   constexpr int NW = NT / 32;
   constexpr int IT = ST / NT;
   static_assert(IT * 32 * NW == ST, "warp w owns IT*32 consecutive keys of a sub-tile");
@@ -1082,6 +1091,7 @@ __global__ void __launch_bounds__(256)
 k_collect(DevState* st, const LevelSeg* segs, const uint64_t* ssk, const uint32_t* hist_scan,
           SegIn* list_out, int par_out, FinalItem* items, LevelParams P, uint16_t where,
           int last_level, int emit_final, uint64_t* offsets_out) {
+  pdl_entry();
   collect_buckets(st, segs, ssk, hist_scan, list_out, par_out, items, P, where, last_level,
                   emit_final, offsets_out);
 }
@@ -1093,6 +1103,7 @@ __global__ void __launch_bounds__(1024)
 k_scan_collect(DevState* st, const LevelSeg* segs, const uint64_t* ssk, uint32_t* hist,
                SegIn* list_out, int par_out, FinalItem* items, LevelParams P, uint16_t where,
                int last_level, int emit_final, uint64_t* offsets_out) {
+  pdl_entry();
   __shared__ uint64_t sm[32];
   const uint64_t total = st->total_hist;
   uint32_t before = 0;
@@ -1133,6 +1144,7 @@ __host__ __device__ inline size_t greedy_smem_bytes(uint32_t K, uint32_t k) {
 __global__ void __launch_bounds__(kFineThreads, 1)
 k_fine_count(const LevelSeg* segs, Src src, const uint64_t* ssk, const uint32_t* ssi,
              uint32_t over, int ntb, uint32_t* fine_cnt) {
+  pdl_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   LevelSeg sg = segs[0];
   const uint32_t K = sg.k * over;
@@ -1234,17 +1246,20 @@ __device__ __forceinline__ uint32_t greedy_count(const uint32_t* P, uint32_t K, 
 // The greedy's bound L is searched by the whole GPU.  k_group_prep (one CTA)
 // writes the prefix sums P of the fine sizes and the first bracket
 // [lo, hi] (hi always feasible); every k_group_search launch spreads
-// gridDim candidate bounds over the bracket, one per CTA, each checked by a
-// greedy scan over P in shared memory; k_group_narrow keeps the sub-bracket
-// below the smallest feasible candidate.  Four rounds of 3 CTAs per SM narrow
-// any bracket below 2^33 to one value, the smallest feasible bound;
-// k_group_finish (one CTA) runs the greedy scan with it.
-// search[0] = lo, search[1] = hi, search[2] = smallest feasible candidate index.
+// gridDim candidate bounds over the bracket the earlier rounds left, one per
+// CTA, each checked by a greedy scan over P in shared memory, and keeps the
+// smallest feasible candidate of the round; the next launch follows the rounds
+// to the bracket below it.  Four rounds of 3 CTAs per SM narrow any bracket below
+// 2^33 to one value, the smallest feasible bound; k_group_finish (one CTA) runs
+// the greedy scan with it.
+// search[0] = lo, search[1] = hi, search[2 + r] = smallest feasible candidate of
+// round r.
 constexpr int kSearchThreads = 256;
 constexpr int kSearchRounds = 4;
 
 __global__ void __launch_bounds__(kGreedyThreads, 1)
 k_group_prep(const LevelSeg* segs, Overpart op) {
+  pdl_entry();
   __shared__ uint64_t scan_sm[kGreedyThreads / 32];
   const LevelSeg sg = segs[0];
   const uint32_t k = sg.k, K = k * op.over;
@@ -1284,14 +1299,29 @@ k_group_prep(const LevelSeg* segs, Overpart op) {
     const uint64_t lo = avg > maxc ? avg : maxc;
     op.search[0] = lo;
     op.search[1] = avg + maxc > lo ? avg + maxc : lo;
-    op.search[2] = ~0ull;
+    for (int r = 0; r < kSearchRounds; ++r) op.search[2 + r] = ~0ull;
+  }
+}
+
+// The bracket after `rounds` rounds of T candidates.
+__device__ __forceinline__ void group_bracket(const Overpart& op, int rounds, uint64_t T,
+                                              uint64_t& lo, uint64_t& hi) {
+  lo = op.search[0];
+  hi = op.search[1];
+  for (int r = 0; r < rounds && lo < hi; ++r) {
+    const uint64_t t = op.search[2 + r];  // < T: the candidate hi is feasible
+    const uint64_t span = hi - lo;
+    hi = lo + (span * (t + 1)) / T;
+    lo = t == 0 ? lo : lo + (span * t) / T + 1;
   }
 }
 
 __global__ void __launch_bounds__(kSearchThreads)
-k_group_search(const LevelSeg* segs, Overpart op) {
+k_group_search(const LevelSeg* segs, Overpart op, int round) {
+  pdl_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const uint64_t lo = op.search[0], hi = op.search[1];
+  uint64_t lo, hi;
+  group_bracket(op, round, gridDim.x, lo, hi);
   if (lo >= hi) return;  // settled (the same for every CTA of this launch)
   const uint32_t k = segs[0].k, K = k * op.over;
   uint32_t* P = (uint32_t*)smem_raw;   // [K + 1]
@@ -1312,22 +1342,13 @@ k_group_search(const LevelSeg* segs, Overpart op) {
       j = nxt[j];
       ++g;
     }
-    if (g <= k) atomicMin((unsigned long long*)&op.search[2], (unsigned long long)t);
+    if (g <= k) atomicMin((unsigned long long*)&op.search[2 + round], (unsigned long long)t);
   }
 }
 
-__global__ void k_group_narrow(Overpart op, uint64_t T) {
-  const uint64_t lo = op.search[0], hi = op.search[1];
-  if (lo >= hi) return;
-  const uint64_t t = op.search[2];  // < T: the candidate hi is feasible
-  const uint64_t span = hi - lo;
-  op.search[1] = lo + (span * (t + 1)) / T;
-  op.search[0] = t == 0 ? lo : lo + (span * t) / T + 1;
-  op.search[2] = ~0ull;
-}
-
 __global__ void __launch_bounds__(kGreedyThreads, 1)
-k_group_finish(LevelSeg* segs, uint64_t* ssk, uint32_t* ssi, Overpart op) {
+k_group_finish(LevelSeg* segs, uint64_t* ssk, uint32_t* ssi, Overpart op, uint64_t T) {
+  pdl_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const LevelSeg sg = segs[0];
   const uint32_t k = sg.k, K = k * op.over;
@@ -1339,7 +1360,8 @@ k_group_finish(LevelSeg* segs, uint64_t* ssk, uint32_t* ssi, Overpart op) {
   __syncthreads();
   // the end of the group that would start at every fine partition, in
   // parallel; the scan from partition 0 then only follows these links
-  const uint64_t L = op.search[1];  // == search[0] once settled; always feasible
+  uint64_t lo, L;  // equal once settled; L is always feasible
+  group_bracket(op, kSearchRounds, T, lo, L);
   for (uint32_t j = tid; j < K; j += kGreedyThreads)
     nxt[j] = (uint16_t)greedy_next(P, K, j, L, op.over);
   __syncthreads();
@@ -1381,6 +1403,7 @@ k_group_finish(LevelSeg* segs, uint64_t* ssk, uint32_t* ssi, Overpart op) {
 // Without overpartitioning the fine partitions are the outputs themselves.
 __global__ void k_plain_groups(const uint64_t* offsets, uint32_t k, uint64_t* fine_out,
                                uint32_t* first_out) {
+  pdl_entry();
   for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g <= k; g += gridDim.x * blockDim.x) {
     if (fine_out && g < k) fine_out[g] = offsets[g + 1] - offsets[g];
     if (first_out) first_out[g] = g;
@@ -1403,20 +1426,18 @@ void launch_overpartition(const LaunchEnv& e, const LevelParams& P, LevelSeg* se
   cudaMemsetAsync(op.fine_cnt, 0, (size_t)K * 4, e.stream);
   {
     Scope sc(e, "L1.fine_count");
-    k_fine_count<<<e.num_sms, kFineThreads, fine_smem_bytes(K), e.stream>>>(
-        segs, src, ssk, ssi, op.over, P.no_tie_break, op.fine_cnt);
+    launch_kernel(e, k_fine_count, e.num_sms, kFineThreads, fine_smem_bytes(K), segs, src, ssk, ssi,
+                  op.over, P.no_tie_break, op.fine_cnt);
   }
   {
     Scope sc(e, "L1.group");
-    k_group_prep<<<1, kGreedyThreads, 0, e.stream>>>(segs, op);
+    launch_kernel(e, k_group_prep, 1, kGreedyThreads, 0, segs, op);
     const int grid = e.num_sms * 3;
-    for (int r = 0; r < kSearchRounds; ++r) {
-      k_group_search<<<grid, kSearchThreads, (size_t)(K + 1) * 4 + (size_t)K * 2, e.stream>>>(
-          segs, op);
-      k_group_narrow<<<1, 1, 0, e.stream>>>(op, (uint64_t)grid);
-    }
-    k_group_finish<<<1, kGreedyThreads, greedy_smem_bytes(K, k), e.stream>>>(segs, ssk, ssi,
-                                                                               op);
+    for (int r = 0; r < kSearchRounds; ++r)
+      launch_kernel(e, k_group_search, grid, kSearchThreads, (size_t)(K + 1) * 4 + (size_t)K * 2,
+                    segs, op, r);
+    launch_kernel(e, k_group_finish, 1, kGreedyThreads, greedy_smem_bytes(K, k), segs, ssk, ssi, op,
+                  (uint64_t)grid);
   }
 }
 
@@ -1425,13 +1446,13 @@ void launch_overpartition(const LaunchEnv& e, const LevelParams& P, LevelSeg* se
 void launch_plain_groups(const LaunchEnv& e, const uint64_t* offsets, uint32_t k,
                          uint64_t* fine_out, uint32_t* first_out) {
   Scope sc(e, "L1.group");
-  k_plain_groups<<<(k + 256) / 256, 256, 0, e.stream>>>(offsets, k, fine_out, first_out);
+  launch_kernel(e, k_plain_groups, (k + 256) / 256, 256, 0, offsets, k, fine_out, first_out);
 }
 
 void launch_init_plain(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t n,
                        uint64_t final_cap) {
   Scope sc(e, "init");
-  k_init_plain<<<1, 32, 0, e.stream>>>(st, items, n, final_cap, e.local);
+  launch_kernel(e, k_init_plain, 1, 32, 0, st, items, n, final_cap, e.local);
 }
 
 template <int NT, int IT, int MINB>
@@ -1538,6 +1559,7 @@ __global__ void __launch_bounds__(256)
 k_init_segments(DevState* st, const uint64_t* offsets, uint32_t nseg, uint64_t n,
                 SegIn* list_l1, FinalItem* items, uint64_t seg_cap, uint64_t final_cap,
                 int f64) {
+  pdl_entry();
   for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < nseg;
        s += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t a = offsets[s], b = offsets[s + 1];
@@ -1574,8 +1596,8 @@ void launch_init_segments(const LaunchEnv& e, DevState* st, const uint64_t* offs
                           uint64_t seg_cap, uint64_t final_cap, int f64) {
   Scope sc(e, "init_segments");
   const int grid = (int)umin64((nseg + 255) / 256 + 1, (uint64_t)e.num_sms * 8);
-  k_init_segments<<<grid, 256, 0, e.stream>>>(st, offsets, nseg, n, list_l1, items, seg_cap,
-                                              final_cap, f64);
+  launch_kernel(e, k_init_segments, grid, 256, 0, st, offsets, nseg, n, list_l1, items, seg_cap,
+                final_cap, f64);
 }
 
 namespace {
@@ -1588,9 +1610,9 @@ void launch_sample_sort(const LaunchEnv& e, const char* name, uint64_t chunks, D
                         uint64_t* ssamp_key, uint32_t* ssamp_idx, uint32_t min_len,
                         const PlainStart& ps, const LevelParams& P) {
   Scope sc(e, name);
-  k_sample_sort<NT, IT, MINB>
-      <<<grid_for(chunks, 1, e.num_sms * MINB), NT, BinSort<NT, IT>::kSmem, e.stream>>>(
-          st, segs, src, samp_key, samp_idx, ssamp_key, ssamp_idx, P.in_order, min_len, ps, P);
+  launch_kernel(e, k_sample_sort<NT, IT, MINB>, grid_for(chunks, 1, e.num_sms * MINB), NT,
+                BinSort<NT, IT>::kSmem, st, segs, src, samp_key, samp_idx, ssamp_key, ssamp_idx,
+                P.in_order, min_len, ps, P);
 }
 
 }  // namespace
@@ -1616,6 +1638,7 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
       {"L3.plan", "L3.sample_sort", "L3.sample_merge", "L3.classify", "L3.scan_reduce",
        "L3.scan_down", "L3.scatter", "L3.collect"}};
   const char* const* nm = kNames[(P.level >= 1 && P.level <= kMaxLevels) ? P.level : 0];
+  LevelParams PS = P;  // of the sample
   PlainStart ps;
   uint64_t plain_hist = 0;  // counters of a one-segment level
   if (k_plain) {
@@ -1628,34 +1651,36 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
     ps.S = (uint32_t)umin64(umin64(n_total, a * k_plain), P.samp_max);
     ps.local = e.local;
     plain_hist = (uint64_t)k_plain * ps.nch;
-    const uint64_t nsch = (ps.S + kSampleChunk - 1) / kSampleChunk;
+    // (more chunks than one: half as long, on twice the SMs)
+    if (ps.S > (uint32_t)kSampleChunk) PS.sample_chunk = kSampleChunk / 2;
+    const uint64_t nsch = (ps.S + PS.sample_chunk - 1) / PS.sample_chunk;
     auto draw = [&](auto nt, auto it) {
       launch_sample_sort<decltype(nt)::value, decltype(it)::value, 1>(
           e, nm[1], umax64(nsch, 1), st, segs, src, samp_key, samp_idx, ssamp_key, ssamp_idx, 0,
-          ps, P);
+          ps, PS);
     };
     // one CTA a chunk: the more threads the shorter
-    if (ps.S <= 4096)
+    if (ps.S <= 4096 || nsch > 1)
       draw(std::integral_constant<int, 512>(), std::integral_constant<int, 8>());
     else
       draw(std::integral_constant<int, 1024>(), std::integral_constant<int, 8>());
     if (nsch > 1) {
       Scope sc(e, nm[2]);
       const size_t smem = BinSort<kMergeThreads, kMergeItems>::kSmem;
-      k_sample_merge<<<(int)((ps.S + kMergeRange - 1) / kMergeRange), kMergeThreads, smem,
-                       e.stream>>>(segs, samp_key, samp_idx, ssamp_key, ssamp_idx);
+      launch_kernel(e, k_sample_merge, (int)((ps.S + kMergeRange - 1) / kMergeRange), kMergeThreads,
+                    smem, segs, samp_key, samp_idx, ssamp_key, ssamp_idx);
     }
   } else {
     {
       Scope sc(e, nm[0]);
       const int ctas = grid_for(umin64(P.seg_cap, P.max_segs), kPlanThreads, 1 << 22);
       if (ctas > 1) {
-        k_plan_sums<<<ctas, kPlanThreads, 0, e.stream>>>(st, list_in, P, par_in,
-                                                         (uint32_t)kmax_level, plan_sums);
+        launch_kernel(e, k_plan_sums, ctas, kPlanThreads, 0, st, list_in, P, par_in,
+                      (uint32_t)kmax_level, plan_sums);
         if (e.launches) ++*e.launches;
       }
-      k_level_plan<<<ctas, kPlanThreads, 0, e.stream>>>(
-          st, list_in, segs, P, par_in, (uint32_t)kmax_level, plan_sums, src.chunk_seg);
+      launch_kernel(e, k_level_plan, ctas, kPlanThreads, 0, st, list_in, segs, P, par_in,
+                    (uint32_t)kmax_level, plan_sums, src.chunk_seg);
     }
     // (every segment has at most kMaxKDeep buckets, so one sample chunk)
     static_assert(kMaxKDeep * kDeepOversample <= kSampleChunk, "one sample chunk a segment");
@@ -1690,11 +1715,11 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
   const bool wide = kmax_level >= P.wide_scatter_k &&
                     scatter_smem_bytes((uint32_t)kmax_level, mode, 16, 4096, stable) <=
                         g_wide_scatter_smem_max;
-  // A stable level with at most kUnitMaxK buckets classifies once, storing
-  // every element's bucket id, and scatters whole 8-element units
-  // (unit_scatter.cu).  Otherwise stored bucket ids spare the staged scatter
-  // its second classification, except at 1024+ buckets, where the staged scatter's L2-resident write frontiers
-  // were the bottleneck and the extra id stream measured slower.
+  // A level with at most kUnitMaxK buckets classifies once, storing every
+  // element's bucket id, and scatters whole 8-element units (unit_scatter.cu).
+  // Otherwise stored bucket ids spare the staged scatter its second
+  // classification, except at 1024+ buckets, where its L2-resident write
+  // frontiers were the bottleneck and the extra id stream measured slower.
   // With atomic_scatter, an unordered level (a full sort's levels after the
   // first) keeps the ids of its classify pass and ranks by shared-memory
   // atomics in the small-footprint scatter (measured slower than the staged
@@ -1712,28 +1737,27 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
   } else {
     Scope sc(e, nm[3]);
     if (deep_c)
-      k_classify_count<kCStagesDeep><<<grid_c, kPartThreads, smem_cd, e.stream>>>(
-          st, segs, src, ssamp_key, ssamp_idx, hist, P.W, (uint32_t)kmax_level, mode);
+      launch_kernel(e, k_classify_count<kCStagesDeep>, grid_c, kPartThreads, smem_cd, st, segs, src,
+                    ssamp_key, ssamp_idx, hist, P.W, (uint32_t)kmax_level, mode);
     else
-      k_classify_count<kCStages><<<grid_c, kPartThreads, smem_c, e.stream>>>(
-          st, segs, src, ssamp_key, ssamp_idx, hist, P.W, (uint32_t)kmax_level, mode);
+      launch_kernel(e, k_classify_count<kCStages>, grid_c, kPartThreads, smem_c, st, segs, src,
+                    ssamp_key, ssamp_idx, hist, P.W, (uint32_t)kmax_level, mode);
   }
   const bool small_scan = k_plain && plain_hist <= kSmallScan;
   if (small_scan) {
     Scope sc(e, nm[5]);
-    k_scan_collect<<<1, 1024, 0, e.stream>>>(st, segs, ssamp_key, hist, list_out, par_in ^ 1,
-                                             items, P, dst_where, last_level, emit_final,
-                                             offsets_out);
+    launch_kernel(e, k_scan_collect, 1, 1024, 0, st, segs, ssamp_key, hist, list_out, par_in ^ 1,
+                  items, P, dst_where, last_level, emit_final, offsets_out);
   } else {
     const uint64_t most = k_plain ? plain_hist : P.hist_cap;
     const int scan_grid = (int)umax64((most + kScanTile - 1) / kScanTile, 1);
     {
       Scope sc(e, nm[4]);
-      k_scan_reduce<<<scan_grid, 1024, 0, e.stream>>>(st, hist, block_sums);
+      launch_kernel(e, k_scan_reduce, scan_grid, 1024, 0, st, hist, block_sums);
     }
     {
       Scope sc(e, nm[5]);
-      k_scan_down<<<scan_grid, 1024, 0, e.stream>>>(st, hist, block_sums);
+      launch_kernel(e, k_scan_down, scan_grid, 1024, 0, st, hist, block_sums);
     }
   }
   if (units) {
@@ -1743,36 +1767,31 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
   } else {
     Scope sc(e, nm[6]);
     if (wide && stable)
-      k_scatter<512, 4096, true>
-          <<<grid_for(P.chunk_cap, 1,
-                      sms * wide_scatter_blocks_per_sm((uint32_t)kmax_level, mode, true)),
-             512, scatter_smem_bytes((uint32_t)kmax_level, mode, 16, 4096), e.stream>>>(
-              st, segs, src, ssamp_key, ssamp_idx, hist, dst, P.W, (uint32_t)kmax_level,
-              unmap_out, mode);
+      launch_kernel(e, k_scatter<512, 4096, true>,
+                    grid_for(P.chunk_cap, 1, sms * wide_scatter_blocks_per_sm((uint32_t)kmax_level, mode, true)),
+                    512, scatter_smem_bytes((uint32_t)kmax_level, mode, 16, 4096), st, segs, src,
+                    ssamp_key, ssamp_idx, hist, dst, P.W, (uint32_t)kmax_level, unmap_out, mode);
     else if (wide)
-      k_scatter<512, 4096, false>
-          <<<grid_for(P.chunk_cap, 1,
-                      sms * wide_scatter_blocks_per_sm((uint32_t)kmax_level, mode, false)),
-             512, scatter_smem_bytes((uint32_t)kmax_level, mode, 16, 4096, false), e.stream>>>(
-              st, segs, src, ssamp_key, ssamp_idx, hist, dst, P.W, (uint32_t)kmax_level,
-              unmap_out, mode);
+      launch_kernel(e, k_scatter<512, 4096, false>,
+                    grid_for(P.chunk_cap, 1, sms * wide_scatter_blocks_per_sm((uint32_t)kmax_level, mode, false)),
+                    512, scatter_smem_bytes((uint32_t)kmax_level, mode, 16, 4096, false), st, segs,
+                    src, ssamp_key, ssamp_idx, hist, dst, P.W, (uint32_t)kmax_level, unmap_out,
+                    mode);
     else if (stable)
-      k_scatter<kPartThreads, 2048, true>
-          <<<grid_s, kPartThreads, scatter_smem_bytes((uint32_t)kmax_level, mode, kPartWarps, 2048),
-             e.stream>>>(st, segs, src, ssamp_key, ssamp_idx, hist, dst, P.W,
-                         (uint32_t)kmax_level, unmap_out, mode);
+      launch_kernel(e, k_scatter<kPartThreads, 2048, true>, grid_s, kPartThreads,
+                    scatter_smem_bytes((uint32_t)kmax_level, mode, kPartWarps, 2048), st, segs, src,
+                    ssamp_key, ssamp_idx, hist, dst, P.W, (uint32_t)kmax_level, unmap_out, mode);
     else
-      k_scatter<kPartThreads, 2048, false>
-          <<<grid_s, kPartThreads,
-             scatter_smem_bytes((uint32_t)kmax_level, mode, kPartWarps, 2048, false),
-             e.stream>>>(st, segs, src, ssamp_key, ssamp_idx, hist, dst, P.W,
-                         (uint32_t)kmax_level, unmap_out, mode);
+      launch_kernel(e, k_scatter<kPartThreads, 2048, false>, grid_s, kPartThreads,
+                    scatter_smem_bytes((uint32_t)kmax_level, mode, kPartWarps, 2048, false), st,
+                    segs, src, ssamp_key, ssamp_idx, hist, dst, P.W, (uint32_t)kmax_level,
+                    unmap_out, mode);
   }
   if (!small_scan) {
     Scope sc(e, nm[7]);
-    k_collect<<<grid_for(P.bucket_cap, 256, sms * 8), 256, 0, e.stream>>>(
-        st, segs, ssamp_key, hist, list_out, par_in ^ 1, items, P, dst_where, last_level,
-        emit_final, offsets_out);
+    launch_kernel(e, k_collect, grid_for(P.bucket_cap, 256, sms * 8), 256, 0, st, segs, ssamp_key,
+                  hist, list_out, par_in ^ 1, items, P, dst_where, last_level, emit_final,
+                  offsets_out);
   }
 }
 

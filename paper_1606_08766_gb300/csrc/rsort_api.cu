@@ -118,7 +118,8 @@ struct Plan {
   // arena offsets
   size_t off_tmp_key = 0, off_tmp_idx = 0, off_samp_key = 0, off_samp_idx = 0;
   size_t off_ssamp_key = 0, off_ssamp_idx = 0, off_hist = 0, off_sums = 0, off_segs = 0;
-  size_t off_plan = 0, off_chunk = 0, off_list0 = 0, off_list1 = 0, off_items = 0, off_state = 0, off_fine = 0, off_bid = 0;
+  size_t off_plan = 0, off_chunk = 0, off_list0 = 0, off_list1 = 0, off_items = 0;
+  size_t off_state = 0, off_fine = 0, off_bid = 0;
   size_t total = 0;
 };
 
@@ -335,8 +336,8 @@ void set_attributes_once(int device) {
 
 // Enqueues the partition levels and the in-SM sort after the level-1 list and
 // the directly sortable items have been initialised.
-void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const LaunchEnv& e, DevState* st,
-                              FinalItem* items, SegIn* const lists[2], rsort_key_type type,
+void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const LaunchEnv& e,
+                              DevState* st, FinalItem* items, SegIn* const lists[2], rsort_key_type type,
                               const void* d_keys_in, const Dst& out, const Dst& tmp,
                               uint64_t seed, uint32_t k1, bool segmented) {
   // Level 1 scatters into the output buffer unless the input is that buffer
@@ -608,9 +609,11 @@ size_t segmented_scratch_bytes(rsort_ctx* c, uint64_t n, uint32_t num_segments) 
   return (n == 0 || num_segments == 0) ? 0 : plan_segmented(c, n, num_segments).total;
 }
 
-rsort_status enqueue_sort(rsort_ctx* c, Workspace& ws, const LaunchEnv& e, rsort_key_type type,
+rsort_status enqueue_sort(rsort_ctx* c, Workspace& ws, const LaunchEnv& env, rsort_key_type type,
                           const void* d_keys_in, void* d_keys_out, uint32_t* d_perm_out,
                           uint64_t n, uint32_t p_virtual, uint64_t seed, DevState** st_out) {
+  LaunchEnv e = env;
+  e.overlap = n <= kOverlapMaxKeys;
   Plan p = plan_sort(c, n, p_virtual);
   const uint32_t k1 = p_virtual >= 2 ? p_virtual : 0;
   rsort_status rs = ensure_workspace(c, ws, p.total, e.stream);
@@ -626,14 +629,17 @@ rsort_status enqueue_sort(rsort_ctx* c, Workspace& ws, const LaunchEnv& e, rsort
   }
   if (p.direct) launch_init_plain(e, st, items, n, p.final_cap);  // (a level starts itself)
   Dst tmp{at<uint64_t>(ws, p.off_tmp_key), at<uint32_t>(ws, p.off_tmp_idx)};
-  enqueue_levels_and_local(c, ws, p, e, st, items, lists, type, d_keys_in, out, tmp, seed, k1, false);
+  enqueue_levels_and_local(c, ws, p, e, st, items, lists, type, d_keys_in, out, tmp, seed, k1,
+                           false);
   return RSORT_OK;
 }
 
-rsort_status enqueue_segmented(rsort_ctx* c, Workspace& ws, const LaunchEnv& e,
+rsort_status enqueue_segmented(rsort_ctx* c, Workspace& ws, const LaunchEnv& env,
                                rsort_key_type type, const void* d_keys_in, void* d_keys_out,
                                uint32_t* d_perm_out, uint64_t n, const uint64_t* d_offsets,
                                uint32_t num_segments, uint64_t seed, DevState** st_out) {
+  LaunchEnv e = env;
+  e.overlap = n <= kOverlapMaxKeys;
   Plan p = plan_segmented(c, n, num_segments);
   rsort_status rs = ensure_workspace(c, ws, p.total, e.stream);
   if (rs != RSORT_OK) return rs;
@@ -777,6 +783,7 @@ rsort_status partition_impl(rsort_ctx* c, rsort_key_type type, const void* d_key
   cudaStream_t s = (cudaStream_t)stream;
   c->last_stream = s;
   LaunchEnv e = env_of(c, s);
+  e.overlap = n <= kOverlapMaxKeys;
   const uint32_t K = k * over;
   if (n == 0) {
     // every partition is empty; fine partition g is output g, or all fine
@@ -812,7 +819,7 @@ rsort_status partition_impl(rsort_ctx* c, rsort_key_type type, const void* d_key
     p.need_tmp = false;
     if (over > 1) {
       p.samp_extra = (uint64_t)kk + 2;
-      p.fine_cap = 2 * (uint64_t)K + 8;  // counters, prefix sums, search state
+      p.fine_cap = 2 * (uint64_t)K + 16;  // counters, prefix sums, search state
     }
     layout(p);
     if (c->budget == 0 || p.total <= c->budget) break;

@@ -214,6 +214,7 @@ struct LevelParams {
   uint64_t samp_cap, hist_cap, chunk_cap, seg_cap, final_cap, schunk_cap, bucket_cap;
   uint32_t fit_chunks = 0;          // chunks a deeper level's elements are spread
                                     // over, however few (0: chunks of W keys)
+  uint32_t sample_chunk = kSampleChunk;  // samples a CTA sorts (one-segment levels)
   uint64_t max_segs = ~0ull;        // segments the level can have (seg_cap aside)
   uint32_t samp_max = 0xffffffffu;  // at most this many samples a segment
   // a one-segment level: 1: its bucket count was asked for (16 ceil(log2 k)
@@ -255,7 +256,8 @@ struct Overpart {
   uint32_t over;         // b >= 2
   uint32_t* fine_cnt;    // [b*k] scratch counters (cleared by the launch)
   uint32_t* prefix;      // [b*k + 1] scratch: prefix sums of the fine sizes
-  uint64_t* search;      // [3] scratch: bracket of the greedy's bound, best candidate
+  uint64_t* search;      // [2 + rounds] scratch: first bracket of the greedy's
+                         // bound, smallest feasible candidate of every round
   uint64_t* fine_out;    // [b*k] fine partition sizes, or nullptr
   uint32_t* first_out;   // [k+1] first fine partition of every output, or nullptr
 };
@@ -306,6 +308,14 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   uint32_t m;
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
   return m;
+}
+
+// First statement of every kernel that launch_kernel starts: waits until the kernel
+// before it in the stream has completed and its writes are visible, then lets
+// the one after it be set up.  Without the launch attribute both do nothing.
+__device__ __forceinline__ void pdl_entry() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Exclusive block scan of one u64 per thread (NT threads, NT % 32 == 0).
@@ -413,9 +423,6 @@ __host__ __device__ __forceinline__ int log2_u32(uint32_t p) {  // p a power of 
   return l;
 }
 
-// ---------------------------------------------------------------------------
-// Host-side launchers (defined in the .cu files)
-// ---------------------------------------------------------------------------
 // Profiling hook owned by the context: CUDA events around every launch.
 struct KernelTimer {
   void begin(const char* name, cudaStream_t s);
@@ -429,7 +436,36 @@ struct LaunchEnv {
   KernelTimer* timer;   // may be null
   uint64_t* launches;   // launch counter
   LocalPlan local;      // in-SM size classes and algorithms (written to DevState at init)
+  bool overlap = true;  // launch_kernel: set kernels up while the one before runs
 };
+
+// Calls of more keys than this launch in the ordinary way: set up early, their
+// long passes took longer (2^28 keys: 7.07 -> 7.31 ms, scatter +0.07 ms and
+// classify +0.03 ms a pass), while 2^26 keys still gain 2 to 5 us a pass.
+constexpr uint64_t kOverlapMaxKeys = 1ull << 27;
+
+// Launches a kernel whose first statement is pdl_entry(): it may be set up on
+// the device while the kernel before it in the stream still runs (programmatic
+// stream serialization), which hides most of the gap between two dependent
+// launches -- a call is a chain of 5 to 20 of them, most a few microseconds long.
+//   10^5 keys (5 launches) 45 -> 36 us, 2^20 (14) 147 -> 117, 2*10^7 (20) 842 ->
+//   788, an overpartitioned step (16) 458 -> 407.
+template <typename... P, typename... A>
+inline void launch_kernel(const LaunchEnv& e, void (*kernel)(P...), uint64_t grid, uint32_t block,
+                          size_t smem, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = e.stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = e.overlap ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 
 void launch_init_plain(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t n,
                        uint64_t final_cap);

@@ -114,6 +114,7 @@ template <int NT, bool VEC, bool MAP>
 __global__ void __launch_bounds__(NT, 3)
 k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
                const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode, bool count_eq) {
+  pdl_entry();
   constexpr int R = 2 * kCiPairs;  // keys per thread per step
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Splitters sp;
@@ -320,6 +321,7 @@ __global__ void __launch_bounds__(NC + 32, 2)
 k_classify_bulk(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
                 const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode, size_t common,
                 bool count_eq) {
+  pdl_entry();
   constexpr int NT = NC + 32;
   constexpr int NCW = NC / 32;         // consumer warps
   constexpr int SK = kCbStageKeys;
@@ -968,6 +970,7 @@ template <int NT, int IT, bool HAS_IDX, bool STABLE>
 __global__ void __launch_bounds__(NT, kUsThreads / NT)
 k_scatter_units(const DevState* st, const LevelSeg* segs, Src src, const uint32_t* hist_scan,
                 Dst dst, uint32_t kmax, int conv, uint32_t aoff, bool auto_order) {
+  pdl_entry();
   // (level 1 with its order decided on the device: both forms are launched and
   // the one not chosen returns at once)
   if (auto_order && l1_auto_ordered(st) != STABLE) return;
@@ -984,6 +987,7 @@ template <int NT>
 __global__ void __launch_bounds__(NT, kUsThreads / NT)
 k_scatter_units_auto(const DevState* st, const LevelSeg* segs, Src src, const uint32_t* hist_scan,
                      Dst dst, uint32_t kmax, int conv, uint32_t aoff) {
+  pdl_entry();
   if (l1_auto_ordered(st))
     scatter_units<NT, kUsItems, false, true>(st, segs, src, hist_scan, dst, kmax, conv, aoff);
   else
@@ -1010,6 +1014,7 @@ template <int NT, bool HAS_IDX>
 __global__ void __launch_bounds__(NT, 4)
 k_scatter_atomic(const DevState* st, const LevelSeg* segs, Src src, const uint32_t* hist_scan,
                  Dst dst, uint32_t kmax, int conv) {
+  pdl_entry();
   constexpr int IT = kSaItems;
   constexpr int ST = NT * IT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1181,8 +1186,8 @@ void launch_classify_ids(const LaunchEnv& e, const LevelParams& P, DevState* st,
     if (nb < 1) nb = 1;
     const uint64_t grid = umin64(P.chunk_cap, (uint64_t)e.num_sms * nb);
     Scope sc(e, name);
-    k_classify_bulk<256><<<(int)(grid ? grid : 1), 256 + 32, smem, e.stream>>>(
-        st, segs, src, ssk, ssi, hist, kmax, mode, common, P.stable == kOrderAuto);
+    launch_kernel(e, k_classify_bulk<256>, (int)(grid ? grid : 1), 256 + 32, smem, st, segs, src,
+                  ssk, ssi, hist, kmax, mode, common, P.stable == kOrderAuto);
     return;
   }
   const size_t smem = classify_ids_smem_bytes(kmax, mode);
@@ -1197,17 +1202,17 @@ void launch_classify_ids(const LaunchEnv& e, const LevelParams& P, DevState* st,
   Scope sc(e, name);
   const int g = (int)(grid ? grid : 1);
   if (vec && src.map_f64)
-    k_classify_ids<256, true, true><<<g, 256, smem, e.stream>>>(st, segs, src, ssk, ssi, hist,
-                                                                kmax, mode, eq);
+    launch_kernel(e, k_classify_ids<256, true, true>, g, 256, smem, st, segs, src, ssk, ssi, hist,
+                  kmax, mode, eq);
   else if (vec)
-    k_classify_ids<256, true, false><<<g, 256, smem, e.stream>>>(st, segs, src, ssk, ssi, hist,
-                                                                 kmax, mode, eq);
+    launch_kernel(e, k_classify_ids<256, true, false>, g, 256, smem, st, segs, src, ssk, ssi, hist,
+                  kmax, mode, eq);
   else if (src.map_f64)
-    k_classify_ids<256, false, true><<<g, 256, smem, e.stream>>>(st, segs, src, ssk, ssi, hist,
-                                                                 kmax, mode, eq);
+    launch_kernel(e, k_classify_ids<256, false, true>, g, 256, smem, st, segs, src, ssk, ssi, hist,
+                  kmax, mode, eq);
   else
-    k_classify_ids<256, false, false><<<g, 256, smem, e.stream>>>(st, segs, src, ssk, ssi, hist,
-                                                                  kmax, mode, eq);
+    launch_kernel(e, k_classify_ids<256, false, false>, g, 256, smem, st, segs, src, ssk, ssi, hist,
+                  kmax, mode, eq);
 }
 
 void launch_scatter_atomic(const LaunchEnv& e, const LevelParams& P, DevState* st,
@@ -1226,11 +1231,11 @@ void launch_scatter_atomic(const LaunchEnv& e, const LevelParams& P, DevState* s
   const uint64_t grid = umin64(P.chunk_cap, (uint64_t)e.num_sms * nb);
   Scope sc(e, name);
   if (src.idx)
-    k_scatter_atomic<kSaThreads, true><<<(int)(grid ? grid : 1), kSaThreads, smem, e.stream>>>(
-        st, segs, src, hist_scan, dst, kmax, conv);
+    launch_kernel(e, k_scatter_atomic<kSaThreads, true>, (int)(grid ? grid : 1), kSaThreads, smem,
+                  st, segs, src, hist_scan, dst, kmax, conv);
   else
-    k_scatter_atomic<kSaThreads, false><<<(int)(grid ? grid : 1), kSaThreads, smem, e.stream>>>(
-        st, segs, src, hist_scan, dst, kmax, conv);
+    launch_kernel(e, k_scatter_atomic<kSaThreads, false>, (int)(grid ? grid : 1), kSaThreads, smem,
+                  st, segs, src, hist_scan, dst, kmax, conv);
 }
 
 bool atomic_scatter_fits(uint32_t kmax) {
@@ -1248,26 +1253,26 @@ void launch_scatter_units_nt(const LaunchEnv& e, const LevelParams& P, DevState*
   const size_t smem_a = us_smem_bytes(kmax, NT, kUsItemsAny, false);
   const bool autoo = P.stable == kOrderAuto;  // (level 1: no stored positions)
   if (autoo && P.W <= kAutoOneLaunchW) {
-    k_scatter_units_auto<NT><<<g, NT, umax64(smem_s, smem_a), e.stream>>>(
-        st, segs, src, hist_scan, dst, kmax, conv, aoff);
+    launch_kernel(e, k_scatter_units_auto<NT>, g, NT, umax64(smem_s, smem_a), st, segs, src,
+                  hist_scan, dst, kmax, conv, aoff);
     return;
   }
   if (P.stable == 1 || autoo) {
     if (src.idx)
-      k_scatter_units<NT, kUsItems, true, true><<<g, NT, smem_s, e.stream>>>(
-          st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
+      launch_kernel(e, k_scatter_units<NT, kUsItems, true, true>, g, NT, smem_s, st, segs, src,
+                    hist_scan, dst, kmax, conv, aoff, autoo);
     else
-      k_scatter_units<NT, kUsItems, false, true><<<g, NT, smem_s, e.stream>>>(
-          st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
+      launch_kernel(e, k_scatter_units<NT, kUsItems, false, true>, g, NT, smem_s, st, segs, src,
+                    hist_scan, dst, kmax, conv, aoff, autoo);
   }
   if (autoo && e.launches) ++*e.launches;
   if (P.stable != 1 || autoo) {
     if (src.idx)
-      k_scatter_units<NT, kUsItemsAny, true, false><<<g, NT, smem_a, e.stream>>>(
-          st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
+      launch_kernel(e, k_scatter_units<NT, kUsItemsAny, true, false>, g, NT, smem_a, st, segs, src,
+                    hist_scan, dst, kmax, conv, aoff, autoo);
     else
-      k_scatter_units<NT, kUsItemsAny, false, false><<<g, NT, smem_a, e.stream>>>(
-          st, segs, src, hist_scan, dst, kmax, conv, aoff, autoo);
+      launch_kernel(e, k_scatter_units<NT, kUsItemsAny, false, false>, g, NT, smem_a, st, segs, src,
+                    hist_scan, dst, kmax, conv, aoff, autoo);
   }
 }
 }  // namespace
