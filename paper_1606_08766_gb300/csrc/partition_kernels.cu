@@ -110,7 +110,7 @@ __device__ __forceinline__ void fill_segment(LevelSeg& s, uint64_t start, uint32
 // Per-segment parameters and prefix sums of one level.  CTA t takes segments
 // [t, t + 1) * kPlanThreads.  With one CTA k_level_plan does everything; a level
 // that may have more segments runs k_plan_sums first, which leaves every CTA's
-// six sums in plan_sums, and each CTA of k_level_plan adds up those before its
+// sums in plan_sums, and each CTA of k_level_plan adds up those before its
 // own (33,000 segments: one CTA in a loop over tiles 197 us, a run of segments
 // per thread 256, the two launches 30).
 constexpr int kPlanThreads = 1024;
@@ -146,6 +146,26 @@ __device__ __forceinline__ SegIn plan_shape(const SegIn* list_in, uint32_t g, ui
   return in;
 }
 
+// The six sums in four scans.  Samples, chunks, sample chunks and elements are
+// each at most one per element (below 2^32); buckets are not bounded like that,
+// but each brings a histogram counter, whose sum keeps 64 bits and fails its
+// capacity first.
+constexpr int kPlanScans = 4;
+__device__ __forceinline__ void pack_plan(const uint64_t (&v)[6], uint64_t (&pk)[kPlanScans]) {
+  pk[0] = v[0] | (v[1] << 32);
+  pk[1] = v[2];
+  pk[2] = v[3] | (v[4] << 32);
+  pk[3] = v[5];
+}
+__device__ __forceinline__ void unpack_plan(const uint64_t (&pk)[kPlanScans], uint64_t (&v)[6]) {
+  v[0] = pk[0] & 0xffffffffu;
+  v[1] = pk[0] >> 32;
+  v[2] = pk[1];
+  v[3] = pk[2] & 0xffffffffu;
+  v[4] = pk[2] >> 32;
+  v[5] = pk[3];
+}
+
 __global__ void __launch_bounds__(kPlanThreads)
 k_plan_sums(const DevState* st, const SegIn* list_in, LevelParams P, int par_in,
             uint32_t kmax_level, uint64_t* plan_sums) {
@@ -153,13 +173,14 @@ k_plan_sums(const DevState* st, const SegIn* list_in, LevelParams P, int par_in,
   __shared__ uint64_t sm[kPlanThreads / 32];
   const uint32_t G = st->nseg[par_in];
   if (G > P.seg_cap || (uint64_t)blockIdx.x * kPlanThreads >= G) return;
-  uint64_t v[6];
+  uint64_t v[6], pk[kPlanScans];
   plan_shape(list_in, blockIdx.x * kPlanThreads + threadIdx.x, G, P, kmax_level, v);
+  pack_plan(v, pk);
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
+  for (int i = 0; i < kPlanScans; ++i) {
     uint64_t tot;
-    block_excl_scan_u64<kPlanThreads>(v[i], &tot, sm);
-    if (threadIdx.x == 0) plan_sums[blockIdx.x * 6 + i] = tot;
+    block_excl_scan_u64<kPlanThreads>(pk[i], &tot, sm);
+    if (threadIdx.x == 0) plan_sums[blockIdx.x * kPlanScans + i] = tot;
   }
 }
 
@@ -185,21 +206,27 @@ k_level_plan(DevState* st, const SegIn* list_in, LevelSeg* segs, LevelParams P, 
     P.W = (uint32_t)umin64(P.W, umax64(kMinDeepChunk,
                                        (w + kMinDeepChunk - 1) / kMinDeepChunk * kMinDeepChunk));
   }
-  uint64_t before[6];
+  uint64_t before[kPlanScans];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
+  for (int i = 0; i < kPlanScans; ++i) {
     uint64_t x = 0;
-    for (uint32_t q = threadIdx.x; q < t; q += kPlanThreads) x += plan_sums[q * 6 + i];
+    for (uint32_t q = threadIdx.x; q < t; q += kPlanThreads) x += plan_sums[q * kPlanScans + i];
     before[i] = 0;
     if (t > 0) block_excl_scan_u64<kPlanThreads>(x, &before[i], sm);
   }
   const uint32_t g = t * kPlanThreads + threadIdx.x;
-  uint64_t v[6], ex[6], tot[6];
+  uint64_t v[6], pk[kPlanScans], ex[6], tot[6];
   const SegIn in = plan_shape(list_in, g, G, P, kmax_level, v);
+  pack_plan(v, pk);
+  {
+    uint64_t sum[kPlanScans];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    ex[i] = before[i] + block_excl_scan_u64<kPlanThreads>(v[i], &tot[i], sm);
-    tot[i] += before[i];
+    for (int i = 0; i < kPlanScans; ++i) {
+      pk[i] = before[i] + block_excl_scan_u64<kPlanThreads>(pk[i], &sum[i], sm);
+      sum[i] += before[i];
+    }
+    unpack_plan(pk, ex);
+    unpack_plan(sum, tot);
   }
   // (every CTA's totals up to its own tile: beyond a capacity, the last CTA's
   // check fails too and the level is not run)

@@ -477,7 +477,7 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
                   uint64_t n_total, int unmap_out, const Overpart* op, uint32_t k_plain,
                   uint64_t* plan_sums);
 // plan_sums words a level of at most seg_cap segments needs.
-inline uint64_t plan_sum_words(uint64_t seg_cap) { return (seg_cap / 1024 + 1) * 6; }
+inline uint64_t plan_sum_words(uint64_t seg_cap) { return (seg_cap / 1024 + 1) * 4; }
 void launch_init_segments(const LaunchEnv& e, DevState* st, const uint64_t* offsets,
                           uint32_t nseg, uint64_t n, SegIn* list_l1, FinalItem* items,
                           uint64_t seg_cap, uint64_t final_cap, int f64);

@@ -493,17 +493,18 @@ k_classify_bulk(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk
 // ---------------------------------------------------------------------------
 // Scatter in whole units
 // ---------------------------------------------------------------------------
-// The stable scatter keeps per-warp counters and winner slots; the unordered one
-// needs one counter per bucket, and the room that frees holds longer sub-tiles
-// (more elements per thread).  Up to kUsSmallK buckets two CTAs of 256 threads
+// The stable scatter keeps 16-bit counters per warp and bucket (its per-warp
+// winner slots lie in the sorted slots, unused while it ranks), the unordered
+// one a counter per bucket; with that 12 elements a thread fit either (stable
+// with 8: partition of 2^26 keys, 1024 buckets 750 -> 709 us, duplicate-heavy
+// 2^26 keys 566 -> 520).  Up to kUsSmallK buckets two CTAs of 256 threads
 // share an SM, each other's barriers and latencies overlapping (2^28 keys, level
 // 2: 1.70 -> 1.61 ms; 100,000 segments 2.20 -> 1.90); above, the carry area
 // leaves room for one, of 512 threads (640, 768 and 1024 threads with fewer
 // elements each measured 1.97, 2.00 and 2.05 ms against 1.91 at level 1).
 constexpr int kUsThreads = 512;
 constexpr int kUsThreadsSmall = 256;
-constexpr int kUsItems = 8;        // per thread, stable
-constexpr int kUsItemsAny = 12;    // unordered
+constexpr int kUsItems = 12;       // elements per thread
 constexpr uint32_t kUsSmallK = 512;
 // sub-tiles ahead whose bytes are asked into L2 when a sub-tile starts (0:
 // none): with 1, the next sub-tile's register loads find their bytes on the way
@@ -531,6 +532,10 @@ __host__ __device__ constexpr uint32_t us_max_big(uint32_t st) {
   return st / (kUsDirectUnits * kUnit) + 1;
 }
 
+// Per-warp counter rows start on 16-byte boundaries (they are cleared by 16-byte
+// stores).
+__host__ __device__ inline uint32_t us_cnt_stride(uint32_t kmax) { return (kmax + 7) & ~7u; }
+
 __host__ __device__ inline size_t us_smem_bytes(uint32_t kmax, uint32_t nt, uint32_t it,
                                                 bool stable) {
   const uint32_t nw = nt / 32, st = nt * it;
@@ -539,8 +544,8 @@ __host__ __device__ inline size_t us_smem_bytes(uint32_t kmax, uint32_t nt, uint
   b += (size_t)us_max_units(kmax, st) * 8;       // per-unit records
   b += (size_t)(st + kmax * kCarry) * 4;         // sorted positions, carried ones
   b += (size_t)kmax * 12;                        // per-bucket obase, meta, info
-  b += stable ? (size_t)nw * cnt_stride(kmax) * 2 : (size_t)kmax * 4;  // counters
-  b += stable ? (size_t)nw * kmax : 0;           // per-warp winner slots
+  b = (b + 15) & ~(size_t)15;
+  b += stable ? (size_t)nw * us_cnt_stride(kmax) * 2 : (size_t)kmax * 4;  // counters
   return (b + 15) & ~(size_t)15;
 }
 
@@ -626,10 +631,13 @@ __device__ __forceinline__ void scatter_units(const DevState* st, const LevelSeg
   uint32_t* obase = (uint32_t*)p; p += (size_t)kmax * 4;
   uint32_t* meta = (uint32_t*)p; p += (size_t)kmax * 4;
   uint32_t* info = (uint32_t*)p; p += (size_t)kmax * 4;
-  const uint32_t kst = cnt_stride(kmax);
+  p = smem_raw + (((p - smem_raw) + 15) & ~(size_t)15);
+  const uint32_t kst = us_cnt_stride(kmax);
   uint16_t* wcnt = (uint16_t*)p;
-  p += STABLE ? (size_t)NW * kst * 2 : (size_t)kmax * 4;
-  uint8_t* wwin = (uint8_t*)p;
+  // [NW][kmax] winner lanes, in the sorted slots (written out when ranking starts)
+  uint8_t* wwin = (uint8_t*)skey;
+  static_assert(!STABLE || (size_t)ST * 8 >= (size_t)NW * kUnitMaxK,
+                "the winner slots fit the sorted keys");
   __shared__ __align__(16) uint32_t s_scan[NW];
   __shared__ uint4 s_bigs[us_max_big(ST)];  // buckets of many units: first record, units, record
   __shared__ uint32_t s_nbig;
@@ -734,7 +742,8 @@ __device__ __forceinline__ void scatter_units(const DevState* st, const LevelSeg
       if constexpr (!STABLE) {
         rank_by_atomics<IT>(bid, lrank, ucnt, lane, ltmask);
       } else {
-      for (uint32_t q = lane; q < (k + 1) / 2; q += 32) ((uint32_t*)my_cnt)[q] = 0;
+      for (uint32_t q = lane; q < (k + 7) / 8; q += 32)
+        ((uint4*)my_cnt)[q] = make_uint4(0, 0, 0, 0);
       __syncwarp();
       // a warp whose whole window lies in one bucket (runs of copies of a
       // key) ranks its elements by their place in the window
@@ -980,18 +989,25 @@ k_scatter_units(const DevState* st, const LevelSeg* segs, Src src, const uint32_
 // Level 1 with its order decided on the device: either form, in one launch.  It
 // spares a small call one launch; the two forms in one kernel cost registers
 // and scheduling (2^28 keys: 2.06 -> 2.24 ms), so calls with long chunks launch
-// both.
+// both, the likelier first (the empty one's CTAs then start while it ends:
+// 2*10^7 float64 keys 799 -> 791 us).  Its stable form keeps 8 elements a thread
+// (48 served sorts of up to 2^22 keys: 1220 us, with 12 1245).
 constexpr uint32_t kAutoOneLaunchW = kFineTile;
-static_assert(kUsThreads * kUsItemsAny == kFineTile, "fine chunks are one sub-tile");
+static_assert(kUsThreads * kUsItems == kFineTile, "fine chunks are one sub-tile");
+constexpr int kUsItemsAuto = 8;  // of its stable form
+__host__ inline size_t us_smem_bytes_auto(uint32_t kmax, uint32_t nt) {
+  return umax64(us_smem_bytes(kmax, nt, kUsItemsAuto, true),
+                us_smem_bytes(kmax, nt, kUsItems, false));
+}
 template <int NT>
 __global__ void __launch_bounds__(NT, kUsThreads / NT)
 k_scatter_units_auto(const DevState* st, const LevelSeg* segs, Src src, const uint32_t* hist_scan,
                      Dst dst, uint32_t kmax, int conv, uint32_t aoff) {
   pdl_entry();
   if (l1_auto_ordered(st))
-    scatter_units<NT, kUsItems, false, true>(st, segs, src, hist_scan, dst, kmax, conv, aoff);
+    scatter_units<NT, kUsItemsAuto, false, true>(st, segs, src, hist_scan, dst, kmax, conv, aoff);
   else
-    scatter_units<NT, kUsItemsAny, false, false>(st, segs, src, hist_scan, dst, kmax, conv, aoff);
+    scatter_units<NT, kUsItems, false, false>(st, segs, src, hist_scan, dst, kmax, conv, aoff);
 }
 
 // ---------------------------------------------------------------------------
@@ -1120,7 +1136,7 @@ size_t classify_ids_smem_bytes(uint32_t kmax, int mode) {
 bool unit_scatter_fits(uint32_t kmax) {
   return kmax <= (uint32_t)kUnitMaxK &&
          us_smem_bytes(kmax, kUsThreads, kUsItems, true) <= g_us_smem_max &&
-         us_smem_bytes(kmax, kUsThreads, kUsItemsAny, false) <= g_us_smem_max;
+         us_smem_bytes(kmax, kUsThreads, kUsItems, false) <= g_us_smem_max;
 }
 
 namespace {
@@ -1132,8 +1148,8 @@ bool set_scatter_units_attributes(int limit) {
   };
   return set(k_scatter_units<NT, kUsItems, true, true>) &&
          set(k_scatter_units<NT, kUsItems, false, true>) &&
-         set(k_scatter_units<NT, kUsItemsAny, true, false>) &&
-         set(k_scatter_units<NT, kUsItemsAny, false, false>) && set(k_scatter_units_auto<NT>);
+         set(k_scatter_units<NT, kUsItems, true, false>) &&
+         set(k_scatter_units<NT, kUsItems, false, false>) && set(k_scatter_units_auto<NT>);
 }
 }  // namespace
 
@@ -1160,7 +1176,7 @@ void set_unit_scatter_attributes() {
       (size_t)optin > fa.sharedSizeBytes) {
     limit = (size_t)optin - fa.sharedSizeBytes;
     const size_t need = umax64(us_smem_bytes(kUnitMaxK, kUsThreads, kUsItems, true),
-                               us_smem_bytes(kUnitMaxK, kUsThreads, kUsItemsAny, false));
+                               us_smem_bytes(kUnitMaxK, kUsThreads, kUsItems, false));
     if (limit > need) limit = need;
     if (!set_scatter_units_attributes<kUsThreads>((int)limit) ||
         !set_scatter_units_attributes<kUsThreadsSmall>((int)limit))
@@ -1250,28 +1266,28 @@ void launch_scatter_units_nt(const LaunchEnv& e, const LevelParams& P, DevState*
   const uint64_t grid = umin64(P.chunk_cap, (uint64_t)e.num_sms * (kUsThreads / NT));
   const int g = (int)(grid ? grid : 1);
   const size_t smem_s = us_smem_bytes(kmax, NT, kUsItems, true);
-  const size_t smem_a = us_smem_bytes(kmax, NT, kUsItemsAny, false);
+  const size_t smem_a = us_smem_bytes(kmax, NT, kUsItems, false);
   const bool autoo = P.stable == kOrderAuto;  // (level 1: no stored positions)
   if (autoo && P.W <= kAutoOneLaunchW) {
-    launch_kernel(e, k_scatter_units_auto<NT>, g, NT, umax64(smem_s, smem_a), st, segs, src,
+    launch_kernel(e, k_scatter_units_auto<NT>, g, NT, us_smem_bytes_auto(kmax, NT), st, segs, src,
                   hist_scan, dst, kmax, conv, aoff);
     return;
   }
+  if (P.stable != 1 || autoo) {
+    if (src.idx)
+      launch_kernel(e, k_scatter_units<NT, kUsItems, true, false>, g, NT, smem_a, st, segs, src,
+                    hist_scan, dst, kmax, conv, aoff, autoo);
+    else
+      launch_kernel(e, k_scatter_units<NT, kUsItems, false, false>, g, NT, smem_a, st, segs, src,
+                    hist_scan, dst, kmax, conv, aoff, autoo);
+  }
+  if (autoo && e.launches) ++*e.launches;
   if (P.stable == 1 || autoo) {
     if (src.idx)
       launch_kernel(e, k_scatter_units<NT, kUsItems, true, true>, g, NT, smem_s, st, segs, src,
                     hist_scan, dst, kmax, conv, aoff, autoo);
     else
       launch_kernel(e, k_scatter_units<NT, kUsItems, false, true>, g, NT, smem_s, st, segs, src,
-                    hist_scan, dst, kmax, conv, aoff, autoo);
-  }
-  if (autoo && e.launches) ++*e.launches;
-  if (P.stable != 1 || autoo) {
-    if (src.idx)
-      launch_kernel(e, k_scatter_units<NT, kUsItemsAny, true, false>, g, NT, smem_a, st, segs, src,
-                    hist_scan, dst, kmax, conv, aoff, autoo);
-    else
-      launch_kernel(e, k_scatter_units<NT, kUsItemsAny, false, false>, g, NT, smem_a, st, segs, src,
                     hist_scan, dst, kmax, conv, aoff, autoo);
   }
 }
