@@ -316,9 +316,9 @@ __device__ __forceinline__ void classify_batch_tree(const uint64_t (&x)[R], uint
 // small (usually the first one read) and by halving otherwise.
 // PAIRS: elements 2j and 2j+1 sit at consecutive positions whenever
 // valid(2j) and valid(2j+1); when both tie with the same run of splitter keys,
-// the second element's bucket is the first's or the next (splitter positions
-// are distinct, so at most one more of them lies below it): one comparison
-// instead of a search.
+// the second element's bucket is the first's or the next: one comparison instead
+// of a search.  (Only one splitter position can lie between the two elements,
+// but with fewer samples than buckets several splitters share it.)
 template <int R, bool PAIRS = false, bool F64 = false, typename PosFn, typename ValidFn>
 __device__ __forceinline__ void classify_batch_table(const uint64_t (&x)[R], uint32_t (&b)[R],
                                                      PosFn pos_of, ValidFn valid,
@@ -384,8 +384,10 @@ __device__ __forceinline__ void classify_batch_table(const uint64_t (&x)[R], uin
     const bool tied = ub[r] == x[r] && b[r] < sp.nspl;
     if (tied) {
       if (PAIRS && (r & 1) && prev_tied && x[r] == x[r - 1] && valid(r - 1) && valid(r)) {
-        const uint32_t re = sp.rend[b[r]], pb = b[r - 1];
-        b[r] = pb + (pb < re && sp.idx[pb] < pos_of(r) ? 1u : 0u);
+        const uint32_t re = sp.rend[b[r]], pos = pos_of(r);
+        uint32_t pb = b[r - 1];
+        while (pb < re && sp.idx[pb] < pos) ++pb;
+        b[r] = pb;
       } else {
         b[r] = tie_break(b[r], x[r], pos_of(r), sp);
       }
