@@ -1165,7 +1165,7 @@ __host__ __device__ inline size_t fine_smem_bytes(uint32_t K) {
 }
 
 __host__ __device__ inline size_t greedy_smem_bytes(uint32_t K, uint32_t k) {
-  return (size_t)(K + 1) * 4 + (size_t)(k + 1) * 4 + (size_t)K * 2;
+  return (size_t)(K + 1) * 4 + (size_t)(k + 1) * 4 + (size_t)(K + 1) * 4;
 }
 
 __global__ void __launch_bounds__(kFineThreads, 1)
@@ -1259,15 +1259,18 @@ __device__ __forceinline__ uint32_t greedy_next(const uint32_t* P, uint32_t K, u
   return a;
 }
 
-// Groups the greedy scan opens under bound L (stops counting past kmax).
-__device__ __forceinline__ uint32_t greedy_count(const uint32_t* P, uint32_t K, uint64_t L,
-                                                 uint32_t kmax, uint32_t guess) {
-  uint32_t g = 0, j = 0;
-  while (j < K && g <= kmax) {
-    j = greedy_next(P, K, j, L, guess);
-    ++g;
-  }
-  return g == 0 ? 1 : g;
+// link[j] = link[link[j]] in the other of two arrays, for all j <= K: after i of
+// these a link leads 2^i groups on.  Following single links is a chain of as
+// many dependent shared-memory reads as there are groups (256 groups: 4.4 us a
+// launch), doubling them takes log2 of that many short passes.
+__device__ __forceinline__ void double_links(uint16_t*& link, uint16_t*& spare, uint32_t K,
+                                             uint32_t nt) {
+#pragma unroll 4
+  for (uint32_t j = threadIdx.x; j <= K; j += nt) spare[j] = link[link[j]];
+  __syncthreads();
+  uint16_t* t = link;
+  link = spare;
+  spare = t;
 }
 
 // The greedy's bound L is searched by the whole GPU.  k_group_prep (one CTA)
@@ -1352,25 +1355,27 @@ k_group_search(const LevelSeg* segs, Overpart op, int round) {
   if (lo >= hi) return;  // settled (the same for every CTA of this launch)
   const uint32_t k = segs[0].k, K = k * op.over;
   uint32_t* P = (uint32_t*)smem_raw;   // [K + 1]
-  uint16_t* nxt = (uint16_t*)(P + K + 1);  // [K]
+  uint16_t* nxt = (uint16_t*)(P + K + 1);  // [K + 1]
+  uint16_t* spare = nxt + K + 1;           // [K + 1]
   for (uint32_t j = threadIdx.x; j <= K; j += kSearchThreads) P[j] = op.prefix[j];
   __syncthreads();
   // this CTA's candidate bound (the last CTA's is hi): the end of the group
-  // that would start at every fine partition, in parallel, then one thread
-  // counts the groups of the scan from partition 0 by following the links
+  // that would start at every fine partition (the end links to itself); the
+  // bound holds if k groups from partition 0 reach the end
   const uint64_t t = blockIdx.x, T = gridDim.x;
   const uint64_t L = lo + ((hi - lo) * (t + 1)) / T;
   for (uint32_t j = threadIdx.x; j < K; j += kSearchThreads)
     nxt[j] = (uint16_t)greedy_next(P, K, j, L, op.over);
+  if (threadIdx.x == 0) nxt[K] = (uint16_t)K;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t g = 0, j = 0;
-    while (j < K && g <= k) {
-      j = nxt[j];
-      ++g;
-    }
-    if (g <= k) atomicMin((unsigned long long*)&op.search[2 + round], (unsigned long long)t);
+  uint32_t at = 0;  // the same in every thread
+  for (uint32_t left = k; left != 0; left >>= 1) {
+    if (left & 1) at = nxt[at];
+    if (at == K) break;
+    if (left > 1) double_links(nxt, spare, K, kSearchThreads);
   }
+  if (threadIdx.x == 0 && at == K)
+    atomicMin((unsigned long long*)&op.search[2 + round], (unsigned long long)t);
 }
 
 __global__ void __launch_bounds__(kGreedyThreads, 1)
@@ -1381,27 +1386,27 @@ k_group_finish(LevelSeg* segs, uint64_t* ssk, uint32_t* ssi, Overpart op, uint64
   const uint32_t k = sg.k, K = k * op.over;
   uint32_t* P = (uint32_t*)smem_raw;                 // [K + 1]
   uint32_t* first = P + K + 1;                       // [k + 1]
-  uint16_t* nxt = (uint16_t*)(first + k + 1);        // [K] (K <= kMaxFine < 2^16)
+  uint16_t* nxt = (uint16_t*)(first + k + 1);        // [K + 1] (K <= kMaxFine < 2^16)
+  uint16_t* spare = nxt + K + 1;                     // [K + 1]
   const uint32_t tid = threadIdx.x;
   for (uint32_t j = tid; j <= K; j += kGreedyThreads) P[j] = op.prefix[j];
   __syncthreads();
   // the end of the group that would start at every fine partition, in
-  // parallel; the scan from partition 0 then only follows these links
+  // parallel; the scan from partition 0 then only follows these links: the
+  // starts of groups [2^i, 2^(i + 1)) are 2^i groups on from those before
   uint64_t lo, L;  // equal once settled; L is always feasible
   group_bracket(op, kSearchRounds, T, lo, L);
   for (uint32_t j = tid; j < K; j += kGreedyThreads)
     nxt[j] = (uint16_t)greedy_next(P, K, j, L, op.over);
-  __syncthreads();
   if (tid == 0) {
-    uint32_t g = 0, j = 0;
-    while (j < K && g < k) {
-      first[g++] = j;
-      j = nxt[j];
-    }
-    if (g == 0) first[g++] = 0;
-    for (; g <= k; ++g) first[g] = K;
+    nxt[K] = (uint16_t)K;
+    first[0] = 0;
   }
   __syncthreads();
+  for (uint32_t d = 1; d <= k; d <<= 1) {
+    for (uint32_t g = d + tid; g < 2 * d && g <= k; g += kGreedyThreads) first[g] = nxt[first[g - d]];
+    double_links(nxt, spare, K, kGreedyThreads);  // (its barrier also ends this step)
+  }
   // group boundaries become the splitters of the k-way step, stored after the
   // sample: entry g (g = 1..k-1) is fine splitter first[g] (an element-free
   // sentinel above every pair when the group is empty and past the end)
@@ -1420,6 +1425,11 @@ k_group_finish(LevelSeg* segs, uint64_t* ssk, uint32_t* ssi, Overpart op, uint64
   }
   if (op.first_out)
     for (uint32_t g = tid; g <= k; g += kGreedyThreads) op.first_out[g] = first[g];
+  // the group of every fine partition (the sizes are no longer needed)
+  for (uint32_t g = tid; g < k; g += kGreedyThreads) {
+    const uint32_t end = g + 1 < k ? first[g + 1] : K;
+    for (uint32_t j = first[g]; j < end; ++j) op.fine_cnt[j] = g;
+  }
   __syncthreads();
   if (tid == 0) {
     segs[0].samp_off = extra;
@@ -1447,11 +1457,14 @@ inline int grid_for(uint64_t work, int per_block, int max_blocks) {
 
 namespace {
 
-void launch_overpartition(const LaunchEnv& e, const LevelParams& P, LevelSeg* segs, Src src,
-                          uint64_t* ssk, uint32_t* ssi, const Overpart& op) {
+void launch_overpartition(const LaunchEnv& e, const LevelParams& P, DevState* st, LevelSeg* segs,
+                          Src src, uint64_t* ssk, uint32_t* ssi, const Overpart& op,
+                          bool fine_ids) {
   const uint32_t k = op.k, K = op.k * op.over;
   cudaMemsetAsync(op.fine_cnt, 0, (size_t)K * 4, e.stream);
-  {
+  if (fine_ids) {
+    launch_fine_ids(e, P, st, segs, src, ssk, ssi, op, "L1.fine_count");
+  } else {
     Scope sc(e, "L1.fine_count");
     launch_kernel(e, k_fine_count, e.num_sms, kFineThreads, fine_smem_bytes(K), segs, src, ssk, ssi,
                   op.over, P.no_tie_break, op.fine_cnt);
@@ -1461,7 +1474,7 @@ void launch_overpartition(const LaunchEnv& e, const LevelParams& P, LevelSeg* se
     launch_kernel(e, k_group_prep, 1, kGreedyThreads, 0, segs, op);
     const int grid = e.num_sms * 3;
     for (int r = 0; r < kSearchRounds; ++r)
-      launch_kernel(e, k_group_search, grid, kSearchThreads, (size_t)(K + 1) * 4 + (size_t)K * 2,
+      launch_kernel(e, k_group_search, grid, kSearchThreads, (size_t)(K + 1) * 8,
                     segs, op, r);
     launch_kernel(e, k_group_finish, 1, kGreedyThreads, greedy_smem_bytes(K, k), segs, ssk, ssi, op,
                   (uint64_t)grid);
@@ -1535,7 +1548,7 @@ void set_partition_kernel_attributes() {
   cudaFuncSetAttribute(k_fine_count, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)fine_smem_bytes(kMaxFine));
   cudaFuncSetAttribute(k_group_search, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)((kMaxFine + 1) * 4 + kMaxFine * 2));
+                       (kMaxFine + 1) * 8);
   cudaFuncSetAttribute(k_group_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)greedy_smem_bytes(kMaxFine, kMaxK));
   cudaGetLastError();  // a refused attribute only disables the variant
@@ -1725,7 +1738,6 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
                                      ssamp_key, ssamp_idx, 1024, ps, P);
     }
   }
-  if (op) launch_overpartition(e, P, segs, src, ssamp_key, ssamp_idx, *op);
   const int mode = P.classifier | (P.no_tie_break ? 2 : 0);
   const size_t smem_c = part_smem_bytes((uint32_t)kmax_level, false, mode);
   const size_t smem_s = part_smem_bytes((uint32_t)kmax_level, true, mode);
@@ -1758,7 +1770,15 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
   const bool atomics = !units && P.atomic_scatter && !stable &&
                        src.bid != nullptr && atomic_scatter_fits((uint32_t)kmax_level);
   if (!units && !atomics && kmax_level >= 1024) src.bid = nullptr;
-  if (units) {
+  // the ids of an overpartitioned step's fine partitions are stored instead, and
+  // mapped to buckets after the greedy has grouped them
+  const bool fine_ids = op && units && stable && !P.bulk_classify &&
+                        n_total >= kFineIdsMin * op->k * op->over &&
+                        fine_ids_fit(op->k * op->over);
+  if (op) launch_overpartition(e, P, st, segs, src, ssamp_key, ssamp_idx, *op, fine_ids);
+  if (fine_ids) {
+    launch_map_ids(e, P, st, segs, src, *op, hist, nm[3]);
+  } else if (units) {
     launch_classify_ids(e, P, st, segs, src, ssamp_key, ssamp_idx, hist, (uint32_t)kmax_level,
                         mode, nm[3]);
   } else {

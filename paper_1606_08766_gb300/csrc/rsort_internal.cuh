@@ -254,7 +254,8 @@ struct LevelParams {
 struct Overpart {
   uint32_t k;            // outputs (the segment's k)
   uint32_t over;         // b >= 2
-  uint32_t* fine_cnt;    // [b*k] scratch counters (cleared by the launch)
+  uint32_t* fine_cnt;    // [b*k] scratch counters (cleared by the launch), then the
+                         // output of every fine partition
   uint32_t* prefix;      // [b*k + 1] scratch: prefix sums of the fine sizes
   uint64_t* search;      // [2 + rounds] scratch: first bracket of the greedy's
                          // bound, smallest feasible candidate of every round
@@ -494,6 +495,22 @@ void set_local_kernel_attributes();
 // Classify with stored bucket ids and the whole-unit scatter (unit_scatter.cu).
 void set_unit_scatter_attributes();
 bool unit_scatter_fits(uint32_t kmax);
+// An overpartitioned step whose scatter reads stored ids classifies once, into
+// fine partitions (launch_fine_ids; sizes to op.fine_cnt), and maps those ids
+// to buckets when the greedy has left the bucket of every fine partition in
+// op.fine_cnt (launch_map_ids).  The fine splitters must leave room for two CTAs
+// per SM, and a fine partition hold kFineIdsMin elements: below, the fill of two or
+// three tables per SM instead of one costs more than the second classification
+// (classified twice -> once: 2^23 keys, 2560 fine partitions 263 -> 241 us, 5120 315
+// -> 313; 2^22 keys 182 -> 188, 227 -> 240).
+constexpr uint64_t kFineIdsMin = 2048;
+bool fine_ids_fit(uint32_t K);
+void launch_fine_ids(const LaunchEnv& e, const LevelParams& P, DevState* st, const LevelSeg* segs,
+                     Src src, const uint64_t* ssk, const uint32_t* ssi, const Overpart& op,
+                     const char* name);
+void launch_map_ids(const LaunchEnv& e, const LevelParams& P, const DevState* st,
+                    const LevelSeg* segs, Src src, const Overpart& op, uint32_t* hist,
+                    const char* name);
 void launch_classify_ids(const LaunchEnv& e, const LevelParams& P, DevState* st,
                          const LevelSeg* segs, Src src, const uint64_t* ssk, const uint32_t* ssi,
                          uint32_t* hist, uint32_t kmax, int mode, const char* name);

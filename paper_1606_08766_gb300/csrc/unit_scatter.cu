@@ -110,10 +110,13 @@ constexpr int kCiPrefetch = 2;
 // per SM (64 registers) 0.81 / 0.72, four keys a thread 0.92 / 0.86.
 // VEC: the key array is 16-byte aligned (pairs are read by 16-byte loads);
 // MAP: the keys are float64 bit patterns, mapped to the order map on load.
-template <int NT, bool VEC, bool MAP>
+// FINE: the segment is cut by the over * k - 1 splitters of its fine partitions
+// instead; their sizes over the whole level are added to hist[over * k].
+template <int NT, bool VEC, bool MAP, bool FINE = false>
 __global__ void __launch_bounds__(NT, 3)
 k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
-               const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode, bool count_eq) {
+               const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode, bool count_eq,
+               uint32_t over) {
   pdl_entry();
   constexpr int R = 2 * kCiPairs;  // keys per thread per step
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -145,13 +148,16 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
   uint32_t cur_g = 0xffffffffu;
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
     const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
-    const LevelSeg sg = segs[g];
+    LevelSeg sg = segs[g];
+    // (no sample, no fine splitters: every element is in fine partition 0)
+    if (FINE) sg.k = sg.S > 0 ? sg.k * over : 1;
     __syncthreads();
+    if (!FINE || g != cur_g)
+      for (uint32_t b = threadIdx.x; b < sg.k; b += NT) cnt[b] = 0;
     if (g != cur_g) {
       load_splitters<NT, MAP>(sg, ssk, ssi, sp);
       cur_g = g;
     }
-    for (uint32_t b = threadIdx.x; b < sg.k; b += NT) cnt[b] = 0;
     __syncthreads();
     const uint64_t cl = c - sg.chunk_off;
     if (count_eq && cl == 0) count_equality_buckets<NT>(st, sp);
@@ -289,8 +295,109 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
       atomicAdd(&cnt[b1[0]], 1u);
     }
     __syncthreads();
+    if (!FINE)
+      for (uint32_t b = threadIdx.x; b < sg.k; b += NT)
+        hist[sg.hist_off + (uint64_t)b * sg.nunits + cl] = cnt[b];
+  }
+  if (FINE && cur_g != 0xffffffffu)
+    for (uint32_t b = threadIdx.x; b <= sp.nspl; b += NT)
+      if (cnt[b]) atomicAdd(&hist[b], cnt[b]);
+}
+
+// The second half of an overpartitioned step's classify: the stored fine ids
+// become bucket ids (map[f]: the bucket of fine partition f) and are counted
+// per chunk.  A bucket's splitters are fine splitters, so this is the bucket a
+// second classification would find; it reads 2 bytes an element instead of 8
+// and searches nothing (2^24 keys, 256 buckets of 2560 fine partitions: the
+// step 390 -> 350 us).
+constexpr int kMapThreads = 256;
+constexpr int kMapVecs = 4;  // 16-byte loads per thread per step
+
+__host__ __device__ inline size_t map_ids_smem_bytes(uint32_t K, uint32_t kmax) {
+  return (size_t)kmax * 4 + (((size_t)K * 2 + 15) & ~(size_t)15);
+}
+
+__global__ void __launch_bounds__(kMapThreads)
+k_map_ids(const DevState* st, const LevelSeg* segs, Src src, const uint32_t* map, uint32_t over,
+          uint32_t* hist, uint32_t kmax) {
+  pdl_entry();
+  constexpr int NT = kMapThreads;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint32_t* cnt = (uint32_t*)smem_raw;        // [kmax]
+  uint16_t* to = (uint16_t*)(cnt + kmax);     // [k over]
+  const uint64_t total = st->total_chunks;
+  if (blockIdx.x >= total) return;
+  const LevelSeg sg = segs[0];  // (the step has one segment)
+  for (uint32_t f = threadIdx.x; f < sg.k * over; f += NT) to[f] = (uint16_t)map[f];
+  const int lane = threadIdx.x & 31;
+  for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
+    __syncthreads();
+    for (uint32_t b = threadIdx.x; b < sg.k; b += NT) cnt[b] = 0;
+    __syncthreads();
+    const uint64_t cs = sg.start + c * sg.W;
+    const uint64_t ce = umin64(cs + sg.W, sg.start + sg.m);
+    // [cs, a0) and [a1, ce) singly, the 16-byte aligned part between in vectors
+    const uint64_t head = ((16 - ((uintptr_t)(src.bid + cs) & 15)) & 15) / 2;
+    const uint64_t a0 = umin64(cs + head, ce);
+    const uint64_t nv = (ce - a0) / 8;
+    const uint64_t a1 = a0 + nv * 8;
+    const uint32_t singles = (uint32_t)((a0 - cs) + (ce - a1));
+    if (threadIdx.x < singles) {
+      const uint64_t pos = threadIdx.x < a0 - cs ? cs + threadIdx.x
+                                                 : a1 + (threadIdx.x - (a0 - cs));
+      const uint32_t b = to[src.bid[pos]];
+      src.bid[pos] = (uint16_t)b;
+      atomicAdd(&cnt[b], 1u);
+    }
+    uint4* vec = reinterpret_cast<uint4*>(src.bid + a0);
+    for (uint64_t v0 = 0; v0 < nv; v0 += (uint64_t)NT * kMapVecs) {
+      uint4 x[kMapVecs];
+#pragma unroll
+      for (int r = 0; r < kMapVecs; ++r) {
+        const uint64_t v = v0 + (uint64_t)r * NT + threadIdx.x;
+        x[r] = v < nv ? vec[v] : make_uint4(0, 0, 0, 0);
+      }
+#pragma unroll
+      for (int r = 0; r < kMapVecs; ++r) {
+        const uint64_t v = v0 + (uint64_t)r * NT + threadIdx.x;
+        const bool in = v < nv;
+        uint32_t b[8];
+        const uint32_t w[4] = {x[r].x, x[r].y, x[r].z, x[r].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          b[2 * e] = to[w[e] & 0xffffu];
+          b[2 * e + 1] = to[w[e] >> 16];
+        }
+        if (in)
+          vec[v] = make_uint4(b[0] | (b[1] << 16), b[2] | (b[3] << 16), b[4] | (b[5] << 16),
+                              b[6] | (b[7] << 16));
+        // a warp whose elements all lie in one bucket (runs of copies of a key)
+        // takes one atomic, one where many do takes one a slot that agrees
+        const uint32_t b0 = __shfl_sync(0xffffffffu, b[0], 0);
+        bool same = in;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) same = same && b[e] == b0;
+        if (__all_sync(0xffffffffu, same)) {
+          if (lane == 0) atomicAdd(&cnt[b0], 256u);
+        } else if (__popc(__ballot_sync(0xffffffffu, in && b[0] == b0)) > 8) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const uint32_t bl = __shfl_sync(0xffffffffu, b[e], 0);
+            if (__all_sync(0xffffffffu, in && b[e] == bl)) {
+              if (lane == 0) atomicAdd(&cnt[bl], 32u);
+            } else if (in) {
+              atomicAdd(&cnt[b[e]], 1u);
+            }
+          }
+        } else if (in) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) atomicAdd(&cnt[b[e]], 1u);
+        }
+      }
+    }
+    __syncthreads();
     for (uint32_t b = threadIdx.x; b < sg.k; b += NT)
-      hist[sg.hist_off + (uint64_t)b * sg.nunits + cl] = cnt[b];
+      hist[sg.hist_off + (uint64_t)b * sg.nunits + c] = cnt[b];
   }
 }
 
@@ -1164,6 +1271,16 @@ void set_unit_scatter_attributes() {
                        cudaFuncAttributeMaxDynamicSharedMemorySize, ci_smem);
   cudaFuncSetAttribute(k_classify_ids<256, false, true>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, ci_smem);
+  const int fine_smem = (int)classify_ids_smem_bytes(kMaxFine, 1);
+  cudaFuncSetAttribute(k_classify_ids<256, true, false, true>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, fine_smem);
+  cudaFuncSetAttribute(k_classify_ids<256, true, true, true>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, fine_smem);
+  cudaFuncSetAttribute(k_classify_ids<256, false, false, true>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, fine_smem);
+  cudaFuncSetAttribute(k_classify_ids<256, false, true, true>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, fine_smem);
+  static_assert((size_t)kMaxFine * 2 + kUnitMaxK * 4 + 16 <= 48 * 1024, "k_map_ids' default limit");
   cudaFuncSetAttribute(k_classify_bulk<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)classify_bulk_smem_bytes(umax64(classify_ids_smem_bytes(kMaxK, 0),
                                                             classify_ids_smem_bytes(kMaxK, 1))));
@@ -1190,6 +1307,44 @@ void set_unit_scatter_attributes() {
   cudaGetLastError();
 }
 
+namespace {
+// Resident CTAs per SM of k_classify_ids (0: its shared memory does not fit).
+template <bool FINE>
+int classify_ids_blocks(size_t smem) {
+  int nb = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &nb, k_classify_ids<256, true, false, FINE>, 256, smem) != cudaSuccess) {
+    cudaGetLastError();
+    nb = 0;
+  }
+  return nb;
+}
+
+template <bool FINE>
+void launch_classify_ids_as(const LaunchEnv& e, uint64_t chunk_cap, DevState* st,
+                            const LevelSeg* segs, const Src& src, const uint64_t* ssk,
+                            const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode, bool eq,
+                            uint32_t over) {
+  const size_t smem = classify_ids_smem_bytes(kmax, mode);
+  const int nb = classify_ids_blocks<FINE>(smem);
+  const uint64_t grid = umin64(chunk_cap, (uint64_t)e.num_sms * (nb < 1 ? 1 : nb));
+  const int g = (int)(grid ? grid : 1);
+  auto go = [&](auto* kernel) {
+    launch_kernel(e, kernel, g, 256, smem, st, segs, src, ssk, ssi, hist, kmax, mode, eq, over);
+  };
+  // 16-byte pair loads need a 16-byte aligned key array
+  const bool vec = ((uintptr_t)src.key & 15) == 0;
+  if (vec && src.map_f64)
+    go(k_classify_ids<256, true, true, FINE>);
+  else if (vec)
+    go(k_classify_ids<256, true, false, FINE>);
+  else if (src.map_f64)
+    go(k_classify_ids<256, false, true, FINE>);
+  else
+    go(k_classify_ids<256, false, false, FINE>);
+}
+}  // namespace
+
 void launch_classify_ids(const LaunchEnv& e, const LevelParams& P, DevState* st,
                          const LevelSeg* segs, Src src, const uint64_t* ssk, const uint32_t* ssi,
                          uint32_t* hist, uint32_t kmax, int mode, const char* name) {
@@ -1206,29 +1361,33 @@ void launch_classify_ids(const LaunchEnv& e, const LevelParams& P, DevState* st,
                   ssk, ssi, hist, kmax, mode, common, P.stable == kOrderAuto);
     return;
   }
-  const size_t smem = classify_ids_smem_bytes(kmax, mode);
-  int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_classify_ids<256, true, false>, 256,
-                                                smem);
-  if (nb < 1) nb = 1;
-  const uint64_t grid = umin64(P.chunk_cap, (uint64_t)e.num_sms * nb);
-  // 16-byte pair loads need a 16-byte aligned key array
-  const int vec = ((uintptr_t)src.key & 15) == 0;
-  const bool eq = P.stable == kOrderAuto;
   Scope sc(e, name);
-  const int g = (int)(grid ? grid : 1);
-  if (vec && src.map_f64)
-    launch_kernel(e, k_classify_ids<256, true, true>, g, 256, smem, st, segs, src, ssk, ssi, hist,
-                  kmax, mode, eq);
-  else if (vec)
-    launch_kernel(e, k_classify_ids<256, true, false>, g, 256, smem, st, segs, src, ssk, ssi, hist,
-                  kmax, mode, eq);
-  else if (src.map_f64)
-    launch_kernel(e, k_classify_ids<256, false, true>, g, 256, smem, st, segs, src, ssk, ssi, hist,
-                  kmax, mode, eq);
-  else
-    launch_kernel(e, k_classify_ids<256, false, false>, g, 256, smem, st, segs, src, ssk, ssi, hist,
-                  kmax, mode, eq);
+  launch_classify_ids_as<false>(e, P.chunk_cap, st, segs, src, ssk, ssi, hist, kmax, mode,
+                                P.stable == kOrderAuto, 0);
+}
+
+bool fine_ids_fit(uint32_t K) {
+  return classify_ids_blocks<true>(classify_ids_smem_bytes(K, 1)) >= 2;
+}
+
+void launch_fine_ids(const LaunchEnv& e, const LevelParams& P, DevState* st, const LevelSeg* segs,
+                     Src src, const uint64_t* ssk, const uint32_t* ssi, const Overpart& op,
+                     const char* name) {
+  Scope sc(e, name);
+  launch_classify_ids_as<true>(e, P.chunk_cap, st, segs, src, ssk, ssi, op.fine_cnt,
+                               op.k * op.over, 1 | (P.no_tie_break ? 2 : 0), false, op.over);
+}
+
+void launch_map_ids(const LaunchEnv& e, const LevelParams& P, const DevState* st,
+                    const LevelSeg* segs, Src src, const Overpart& op, uint32_t* hist,
+                    const char* name) {
+  const size_t smem = map_ids_smem_bytes(op.k * op.over, op.k);
+  int nb = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_map_ids, kMapThreads, smem);
+  const uint64_t grid = umin64(P.chunk_cap, (uint64_t)e.num_sms * (nb < 1 ? 1 : nb));
+  Scope sc(e, name);
+  launch_kernel(e, k_map_ids, (int)(grid ? grid : 1), kMapThreads, smem, st, segs, src,
+                op.fine_cnt, op.over, hist, op.k);
 }
 
 void launch_scatter_atomic(const LaunchEnv& e, const LevelParams& P, DevState* st,
