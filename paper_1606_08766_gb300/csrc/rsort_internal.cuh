@@ -513,7 +513,7 @@ void launch_map_ids(const LaunchEnv& e, const LevelParams& P, const DevState* st
                     const char* name);
 void launch_classify_ids(const LaunchEnv& e, const LevelParams& P, DevState* st,
                          const LevelSeg* segs, Src src, const uint64_t* ssk, const uint32_t* ssi,
-                         uint32_t* hist, uint32_t kmax, int mode, const char* name);
+                         uint32_t* hist, uint32_t kmax, int mode, bool bands, const char* name);
 bool atomic_scatter_fits(uint32_t kmax);
 void launch_scatter_atomic(const LaunchEnv& e, const LevelParams& P, DevState* st,
                            const LevelSeg* segs, Src src, const uint32_t* hist_scan, Dst dst,

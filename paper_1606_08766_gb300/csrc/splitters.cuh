@@ -244,10 +244,8 @@ __device__ void load_splitters(const LevelSeg& sg, const uint64_t* ssk, const ui
 // run (many copies of one key) holds positions of a stratified sample, close
 // to evenly spaced: the search starts at an interpolated guess and gallops
 // to a bracket around the answer, a few steps instead of log2 of the run.
-__device__ __forceinline__ uint32_t tie_break(uint32_t bb, uint64_t x, uint32_t i,
+__device__ __forceinline__ uint32_t tie_break(uint32_t lo, uint32_t hi, uint32_t i,
                                               const Splitters& sp) {
-  (void)x;
-  uint32_t lo = bb, hi = sp.rend[bb];
   if (hi - lo > 8) {
     const uint32_t p0 = sp.idx[lo], p1 = sp.idx[hi - 1];
     if (i <= p0) return lo;
@@ -284,6 +282,20 @@ __device__ __forceinline__ uint32_t tie_break(uint32_t bb, uint64_t x, uint32_t 
   return lo;
 }
 
+// The band of every run of splitters for a chunk of positions [p0, p1] (level 1,
+// whose positions rise with the element): band[j], j the run's first splitter,
+// holds the buckets of the two positions when their key ties with the run, first |
+// last << 16.  A sample puts a run's splitters far apart, so nearly always the two
+// are the same and a tie needs no search.  The caller's barrier makes the bands
+// visible.
+template <int NT>
+__device__ __forceinline__ void load_bands(uint32_t p0, uint32_t p1, uint32_t* band,
+                                           const Splitters& sp) {
+  for (uint32_t j = threadIdx.x; j < sp.nspl; j += NT)
+    if (j == 0 || sp.key[j] != sp.key[j - 1])
+      band[j] = tie_break(j, sp.rend[j], p0, sp) | (tie_break(j, sp.rend[j], p1, sp) << 16);
+}
+
 template <int R, typename PosFn>
 __device__ __forceinline__ void classify_batch_tree(const uint64_t (&x)[R], uint32_t (&b)[R],
                                                     PosFn pos_of, const Splitters& sp) {
@@ -306,7 +318,7 @@ __device__ __forceinline__ void classify_batch_tree(const uint64_t (&x)[R], uint
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     uint32_t bb = j[r] - (1u << sp.logK);
-    if (!sp.ntb && bb < sp.nspl && ub[r] == x[r]) bb = tie_break(bb, x[r], pos_of(r), sp);
+    if (!sp.ntb && bb < sp.nspl && ub[r] == x[r]) bb = tie_break(bb, sp.rend[bb], pos_of(r), sp);
     b[r] = bb;
   }
 }
@@ -389,7 +401,7 @@ __device__ __forceinline__ void classify_batch_table(const uint64_t (&x)[R], uin
         while (pb < re && sp.idx[pb] < pos) ++pb;
         b[r] = pb;
       } else {
-        b[r] = tie_break(b[r], x[r], pos_of(r), sp);
+        b[r] = tie_break(b[r], sp.rend[b[r]], pos_of(r), sp);
       }
     }
     prev_tied = tied;
@@ -413,5 +425,39 @@ __device__ __forceinline__ void classify_batch_pairs(const uint64_t (&x)[R], uin
   else classify_batch_table<R, true, F64>(x, b, pos_of, valid, sp);
 }
 
+// The same for a table whose splitters hold runs, with the bands of the chunk:
+// runs fill bins, so the bin's first splitter nearly always bounds the key, and
+// the others search the bin.
+template <int R, bool F64, typename PosFn>
+__device__ __forceinline__ void classify_batch_bands(const uint64_t (&x)[R], uint32_t (&b)[R],
+                                                     PosFn pos_of, const uint32_t* band,
+                                                     const Splitters& sp) {
+  uint64_t ub[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    b[r] = F64 && sp.by_value ? bin_by_value(x[r], sp) : bin_by_bits(x[r], sp);
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const uint32_t t = b[r];
+    b[r] = sp.tbl[t];
+    ub[r] = sp.key[b[r]];
+    if (ub[r] < x[r]) {
+      uint32_t lo = b[r] + 1, hi = t < sp.tmax ? (uint32_t)sp.tbl[t + 1] : sp.nspl;
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (sp.key[mid] < x[r]) lo = mid + 1; else hi = mid;
+      }
+      b[r] = lo;
+      ub[r] = sp.key[lo];
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (ub[r] == x[r] && b[r] < sp.nspl) {
+      const uint32_t w = band[b[r]], lo = w & 0xffffu, hi = w >> 16;
+      b[r] = lo == hi ? lo : tie_break(lo, hi, pos_of(r), sp);
+    }
+  }
+}
 
 }  // namespace rsort

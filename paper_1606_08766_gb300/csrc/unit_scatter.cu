@@ -110,9 +110,14 @@ constexpr int kCiPrefetch = 2;
 // per SM (64 registers) 0.81 / 0.72, four keys a thread 0.92 / 0.86.
 // VEC: the key array is 16-byte aligned (pairs are read by 16-byte loads);
 // MAP: the keys are float64 bit patterns, mapped to the order map on load.
+// BANDS: one segment and long chunks (kBandMinW); if some splitters are equal, ties
+// are placed by bands (load_bands) instead of a search each: duplicate-heavy 2^26
+// keys 434 -> 251 us.  Distinct keys pay 2 % of the pass for looking (2^26 keys 168 ->
+// 172 us), so the other levels take the form without; a loop of its own for either
+// case cost them 20 % (spilled registers).
 // FINE: the segment is cut by the over * k - 1 splitters of its fine partitions
 // instead; their sizes over the whole level are added to hist[over * k].
-template <int NT, bool VEC, bool MAP, bool FINE = false>
+template <int NT, bool VEC, bool MAP, bool FINE, bool BANDS>
 __global__ void __launch_bounds__(NT, 3)
 k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
                const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode, bool count_eq,
@@ -139,6 +144,7 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
     sp.key = (uint64_t*)p; p += (size_t)kmax * 8;
     sp.idx = (uint32_t*)p; p += (size_t)kmax * 4;
     cnt = (uint32_t*)p; p += (size_t)kmax * 4;
+    if (BANDS) p += (size_t)kmax * 4;  // (the bands, after the counters)
     sp.rend = (uint16_t*)p;
   }
   const uint64_t pol = l2_evict_first_policy();
@@ -146,6 +152,7 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
   const uint32_t G = st->cur_nseg;
   const int lane = threadIdx.x & 31;
   uint32_t cur_g = 0xffffffffu;
+  int runs = 0;  // BANDS: some splitter keys are equal
   for (uint64_t c = blockIdx.x; c < total; c += gridDim.x) {
     const uint32_t g = seg_of_chunk(src.chunk_seg, G, c);
     LevelSeg sg = segs[g];
@@ -157,12 +164,19 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
     if (g != cur_g) {
       load_splitters<NT, MAP>(sg, ssk, ssi, sp);
       cur_g = g;
+      if (BANDS) {
+        int eq = 0;
+        for (uint32_t j = threadIdx.x; j + 1 < sp.nspl; j += NT) eq |= sp.key[j] == sp.key[j + 1];
+        runs = __syncthreads_or(eq);
+      }
     }
-    __syncthreads();
     const uint64_t cl = c - sg.chunk_off;
-    if (count_eq && cl == 0) count_equality_buckets<NT>(st, sp);
     const uint64_t cs = sg.start + cl * sg.W;
     const uint64_t ce = umin64(cs + sg.W, sg.start + sg.m);
+    if (BANDS && runs)
+      load_bands<NT>((uint32_t)(cs - sg.start), (uint32_t)(ce - 1 - sg.start), cnt + kmax, sp);
+    __syncthreads();
+    if (count_eq && cl == 0) count_equality_buckets<NT>(st, sp);
     // pairs start at the even position at or below cs (16-byte aligned when
     // the key array is).  VEC: every pair wholly before ce is read by one
     // 16-byte load, from a position clamped into that range (pairs past it
@@ -233,11 +247,17 @@ k_classify_ids(DevState* st, const LevelSeg* segs, Src src, const uint64_t* ssk,
         const uint64_t pos = pos_at(e);
         return (p0 + (uint64_t)(e >> 1) * NT + threadIdx.x) < npairs && pos >= cs && pos < ce;
       };
-      classify_batch_pairs<R, MAP>(key, bk, [&](int e) {
-        if (!valid(e)) return 0u;
-        const uint64_t pos = pos_at(e);
-        return src.idx ? src.idx[pos] : (uint32_t)(pos - sg.start);
-      }, [&](int e) { return valid(e) && src.idx == nullptr; }, sp);
+      if (BANDS && runs) {
+        classify_batch_bands<R, MAP>(key, bk, [&](int e) {
+          return valid(e) ? (uint32_t)(pos_at(e) - sg.start) : 0u;
+        }, cnt + kmax, sp);
+      } else {
+        classify_batch_pairs<R, MAP>(key, bk, [&](int e) {
+          if (!valid(e)) return 0u;
+          const uint64_t pos = pos_at(e);
+          return src.idx ? src.idx[pos] : (uint32_t)(pos - sg.start);
+        }, [&](int e) { return valid(e) && src.idx == nullptr; }, sp);
+      }
       // runs of one bucket across the warp (duplicate-heavy inputs) take one
       // atomic per warp and slot; otherwise one atomic per key
       const uint32_t b0 = __shfl_sync(0xffffffffu, bk[0], 0);
@@ -1233,10 +1253,10 @@ size_t g_us_smem_max = 0;
 
 }  // namespace
 
-size_t classify_ids_smem_bytes(uint32_t kmax, int mode) {
+size_t classify_ids_smem_bytes(uint32_t kmax, int mode, bool bands = false) {
   const size_t Kp = next_pow2_u32(kmax);
   size_t b = (mode & 1) == 0 ? Kp * 8 : table_bytes((uint32_t)Kp);
-  b += (size_t)kmax * (8 + 4 + 4 + 2);
+  b += (size_t)kmax * (8 + 4 + 4 + 2 + (bands ? 4 : 0));
   return (b + 15) & ~(size_t)15;
 }
 
@@ -1260,26 +1280,25 @@ bool set_scatter_units_attributes(int limit) {
 }
 }  // namespace
 
+namespace {
+template <bool FINE, bool BANDS>
+void set_classify_ids_attributes(uint32_t kmax) {
+  const int smem = (int)umax64(FINE ? 0 : classify_ids_smem_bytes(kmax, 0, BANDS),
+                               classify_ids_smem_bytes(kmax, 1, BANDS));
+  auto set = [&](auto* f) {
+    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  };
+  set(k_classify_ids<256, true, false, FINE, BANDS>);
+  set(k_classify_ids<256, true, true, FINE, BANDS>);
+  set(k_classify_ids<256, false, false, FINE, BANDS>);
+  set(k_classify_ids<256, false, true, FINE, BANDS>);
+}
+}  // namespace
+
 void set_unit_scatter_attributes() {
-  const int ci_smem = (int)umax64(classify_ids_smem_bytes(kMaxK, 0),
-                                  classify_ids_smem_bytes(kMaxK, 1));
-  cudaFuncSetAttribute(k_classify_ids<256, true, false>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, ci_smem);
-  cudaFuncSetAttribute(k_classify_ids<256, true, true>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, ci_smem);
-  cudaFuncSetAttribute(k_classify_ids<256, false, false>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, ci_smem);
-  cudaFuncSetAttribute(k_classify_ids<256, false, true>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, ci_smem);
-  const int fine_smem = (int)classify_ids_smem_bytes(kMaxFine, 1);
-  cudaFuncSetAttribute(k_classify_ids<256, true, false, true>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, fine_smem);
-  cudaFuncSetAttribute(k_classify_ids<256, true, true, true>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, fine_smem);
-  cudaFuncSetAttribute(k_classify_ids<256, false, false, true>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, fine_smem);
-  cudaFuncSetAttribute(k_classify_ids<256, false, true, true>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, fine_smem);
+  set_classify_ids_attributes<false, false>(kMaxK);
+  set_classify_ids_attributes<false, true>(kMaxK);
+  set_classify_ids_attributes<true, false>(kMaxFine);
   static_assert((size_t)kMaxFine * 2 + kUnitMaxK * 4 + 16 <= 48 * 1024, "k_map_ids' default limit");
   cudaFuncSetAttribute(k_classify_bulk<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)classify_bulk_smem_bytes(umax64(classify_ids_smem_bytes(kMaxK, 0),
@@ -1309,24 +1328,24 @@ void set_unit_scatter_attributes() {
 
 namespace {
 // Resident CTAs per SM of k_classify_ids (0: its shared memory does not fit).
-template <bool FINE>
-int classify_ids_blocks(size_t smem) {
+template <bool FINE, bool BANDS>
+int classify_ids_blocks(uint32_t kmax, int mode) {
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &nb, k_classify_ids<256, true, false, FINE>, 256, smem) != cudaSuccess) {
+          &nb, k_classify_ids<256, true, false, FINE, BANDS>, 256,
+          classify_ids_smem_bytes(kmax, mode, BANDS)) != cudaSuccess) {
     cudaGetLastError();
     nb = 0;
   }
   return nb;
 }
 
-template <bool FINE>
-void launch_classify_ids_as(const LaunchEnv& e, uint64_t chunk_cap, DevState* st,
+template <bool FINE, bool BANDS>
+void launch_classify_ids_as(const LaunchEnv& e, uint64_t chunk_cap, int nb, DevState* st,
                             const LevelSeg* segs, const Src& src, const uint64_t* ssk,
                             const uint32_t* ssi, uint32_t* hist, uint32_t kmax, int mode, bool eq,
                             uint32_t over) {
-  const size_t smem = classify_ids_smem_bytes(kmax, mode);
-  const int nb = classify_ids_blocks<FINE>(smem);
+  const size_t smem = classify_ids_smem_bytes(kmax, mode, BANDS);
   const uint64_t grid = umin64(chunk_cap, (uint64_t)e.num_sms * (nb < 1 ? 1 : nb));
   const int g = (int)(grid ? grid : 1);
   auto go = [&](auto* kernel) {
@@ -1335,19 +1354,20 @@ void launch_classify_ids_as(const LaunchEnv& e, uint64_t chunk_cap, DevState* st
   // 16-byte pair loads need a 16-byte aligned key array
   const bool vec = ((uintptr_t)src.key & 15) == 0;
   if (vec && src.map_f64)
-    go(k_classify_ids<256, true, true, FINE>);
+    go(k_classify_ids<256, true, true, FINE, BANDS>);
   else if (vec)
-    go(k_classify_ids<256, true, false, FINE>);
+    go(k_classify_ids<256, true, false, FINE, BANDS>);
   else if (src.map_f64)
-    go(k_classify_ids<256, false, true, FINE>);
+    go(k_classify_ids<256, false, true, FINE, BANDS>);
   else
-    go(k_classify_ids<256, false, false, FINE>);
+    go(k_classify_ids<256, false, false, FINE, BANDS>);
 }
+
 }  // namespace
 
 void launch_classify_ids(const LaunchEnv& e, const LevelParams& P, DevState* st,
                          const LevelSeg* segs, Src src, const uint64_t* ssk, const uint32_t* ssi,
-                         uint32_t* hist, uint32_t kmax, int mode, const char* name) {
+                         uint32_t* hist, uint32_t kmax, int mode, bool bands, const char* name) {
   if (P.bulk_classify && ((uintptr_t)src.key & 15) == 0) {
     // keys staged by bulk copies (needs a 16-byte aligned key array)
     const size_t common = classify_ids_smem_bytes(kmax, mode);
@@ -1362,20 +1382,28 @@ void launch_classify_ids(const LaunchEnv& e, const LevelParams& P, DevState* st,
     return;
   }
   Scope sc(e, name);
-  launch_classify_ids_as<false>(e, P.chunk_cap, st, segs, src, ssk, ssi, hist, kmax, mode,
-                                P.stable == kOrderAuto, 0);
+  // bands where the room for them costs no resident CTA
+  const bool eq = P.stable == kOrderAuto;
+  const int nb = classify_ids_blocks<false, false>(kmax, mode);
+  if (bands && (mode & 3) == 1 && classify_ids_blocks<false, true>(kmax, mode) >= nb)
+    launch_classify_ids_as<false, true>(e, P.chunk_cap, nb, st, segs, src, ssk, ssi, hist, kmax,
+                                        mode, eq, 0);
+  else
+    launch_classify_ids_as<false, false>(e, P.chunk_cap, nb, st, segs, src, ssk, ssi, hist, kmax,
+                                         mode, eq, 0);
 }
 
-bool fine_ids_fit(uint32_t K) {
-  return classify_ids_blocks<true>(classify_ids_smem_bytes(K, 1)) >= 2;
-}
+bool fine_ids_fit(uint32_t K) { return classify_ids_blocks<true, false>(K, 1) >= 2; }
 
 void launch_fine_ids(const LaunchEnv& e, const LevelParams& P, DevState* st, const LevelSeg* segs,
                      Src src, const uint64_t* ssk, const uint32_t* ssi, const Overpart& op,
                      const char* name) {
   Scope sc(e, name);
-  launch_classify_ids_as<true>(e, P.chunk_cap, st, segs, src, ssk, ssi, op.fine_cnt,
-                               op.k * op.over, 1 | (P.no_tie_break ? 2 : 0), false, op.over);
+  const uint32_t K = op.k * op.over;
+  const int mode = 1 | (P.no_tie_break ? 2 : 0);
+  launch_classify_ids_as<true, false>(e, P.chunk_cap, classify_ids_blocks<true, false>(K, mode),
+                                      st, segs, src, ssk, ssi, op.fine_cnt, K, mode, false,
+                                      op.over);
 }
 
 void launch_map_ids(const LaunchEnv& e, const LevelParams& P, const DevState* st,
