@@ -413,6 +413,7 @@ constexpr int kMergeThreads = 512;
 constexpr int kMergeItems = 8;
 constexpr uint32_t kMergeRange = 1024;   // pairs a CTA is given on average
 constexpr uint32_t kMaxSampleChunks = 96;
+constexpr uint32_t kMinSplitSample = 5120;   // (larger samples are cut into chunks)
 static_assert(16u * 11 * kMaxK <= kMaxSampleChunks * kSampleChunk / 2, "a run per sample chunk");
 __global__ void __launch_bounds__(kMergeThreads, 2)
 k_sample_merge(const LevelSeg* segs, const uint64_t* samp_key, const uint32_t* samp_idx,
@@ -1693,8 +1694,15 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
     ps.S = (uint32_t)umin64(umin64(n_total, a * k_plain), P.samp_max);
     ps.local = e.local;
     plain_hist = (uint64_t)k_plain * ps.nch;
-    // (more chunks than one: half as long, on twice the SMs)
-    if (ps.S > (uint32_t)kSampleChunk) PS.sample_chunk = kSampleChunk / 2;
+    // Chunks sorted side by side and a merge take less than one CTA's sort of
+    // them all: 8192 float64 samples 41 -> 15 + 15 us, 6144 23 -> 11 + 11 (the
+    // merge's launch overlaps); at 4608 samples the two are even and below one
+    // CTA wins (partition of 2^20 keys, 2560 samples: 44.7 us, two chunks 49.7).
+    // 163,840 samples in chunks of 2048 instead of 4096: 23 + 17 -> 17 + 18 us, an
+    // overpartitioned step of 2^24 keys 349 -> 340.
+    if (ps.S > kMaxSampleChunks * 2048u) PS.sample_chunk = 4096;
+    else if (ps.S > (uint32_t)kSampleChunk) PS.sample_chunk = 2048;
+    else if (ps.S > kMinSplitSample) PS.sample_chunk = 1024;
     const uint64_t nsch = (ps.S + PS.sample_chunk - 1) / PS.sample_chunk;
     auto draw = [&](auto nt, auto it) {
       launch_sample_sort<decltype(nt)::value, decltype(it)::value, 1>(
