@@ -52,10 +52,10 @@ ALGO_BYTES_PER_KEY = {
 # grows in proportion to the keys; the capture and command are summarised in
 # profiles/).  Remove an entry whenever its kernel changes.
 MEASURED_TRAFFIC_PER_KEY = {
-    "L1.scatter": 23.64,       # 0.7696 + 0.8171 GB at 2^26 keys (k_scatter_units<512,12,0,0>)
-    "L1.classify": 9.50,       # 0.5473 + 0.0897 GB (k_classify_ids, ids included)
-    "L2.scatter": 25.35,       # 0.9512 + 0.7498 GB (k_scatter_units<512,12,1,0>)
-    "L2.classify": 9.39,       # 0.5517 + 0.0787 GB (k_classify_count<2>)
+    "L1.scatter": 23.65,       # 0.7686 + 0.8185 GB at 2^26 keys (k_scatter_units<512,12,0,0>)
+    "L1.classify": 9.56,       # 0.5509 + 0.0904 GB (k_classify_ids, ids included)
+    "L2.scatter": 25.30,       # 0.9494 + 0.7486 GB (k_scatter_units<256,12,1,0>)
+    "L2.classify": 10.02,      # 0.5832 + 0.0893 GB (k_classify_ids)
 }
 
 
