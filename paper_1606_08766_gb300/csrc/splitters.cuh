@@ -37,8 +37,13 @@ __device__ __forceinline__ uint32_t ceil_log2_dev(uint32_t k) {
   return l;
 }
 
+// An ordinary load: the sample's is in a call's first launch (k_sample_sort), which
+// may be set up while the launch before it still writes these keys (the last call's
+// output, sorted again), and a load through the read-only path is allowed only where
+// the data does not change while the kernel is resident.  The kernels that read keys
+// through that path start two launches later or more, when the keys are complete.
 __device__ __forceinline__ uint64_t load_key(const Src& s, uint64_t pos) {
-  const uint64_t k = __ldg(s.key + pos);
+  const uint64_t k = s.key[pos];
   return s.map_f64 ? f64_to_ordered(k) : k;
 }
 
