@@ -119,7 +119,6 @@ extern "C" rsort_status rsort_partition_noalloc(rsort_key_type type, const void*
   P.final_cap = 1;
   P.schunk_cap = samp / kSampleChunk + 2;
   P.bucket_cap = kk;
-  P.level1_oversample = 1;
   P.hinted = 1;
   P.classifier = 0;
   P.wide_scatter_k = 1 << 30;  // always the 2048-key sub-tile scatter

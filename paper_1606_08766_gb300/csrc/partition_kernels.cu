@@ -82,17 +82,9 @@ __global__ void k_init_plain(DevState* st, FinalItem* items, uint64_t n, uint64_
   push_final(st, items, final_cap, f, kErrFinalCap);
 }
 
-// Buckets and samples of a segment of m elements (in k: its bucket count).
-__device__ __forceinline__ uint32_t segment_samples(uint32_t m, uint32_t k, bool hinted,
-                                                    const LevelParams& P) {
-  const uint64_t a = hinted && P.level1_oversample ? 16ull * ceil_log2_dev(k)
-                                                   : (uint64_t)kDeepOversample;
-  return (uint32_t)umin64(umin64(m, a * k), P.samp_max);
-}
-
 __device__ __forceinline__ void fill_segment(LevelSeg& s, uint64_t start, uint32_t m, uint32_t k,
                                              uint32_t S, uint32_t nch, const LevelParams& P,
-                                             const KeyRange& range) {
+                                             uint32_t known, const KeyRange& range) {
   s.start = start;
   s.seed = P.level == 1 ? P.seed : splitmix64_at(P.seed, ((uint64_t)P.level << 40) ^ start);
   s.m = m;
@@ -103,7 +95,7 @@ __device__ __forceinline__ void fill_segment(LevelSeg& s, uint64_t start, uint32
   s.nunits = nch;
   // equal chunks inside the segment (the level's W bounds their size)
   s.W = nch ? (uint32_t)(((uint64_t)m + nch - 1) / nch) : P.W;
-  s.pad = 0;
+  s.known = known;
   s.range = range;
 }
 
@@ -125,17 +117,12 @@ __device__ __forceinline__ SegIn plan_shape(const SegIn* list_in, uint32_t g, ui
   for (int i = 0; i < 6; ++i) v[i] = 0;
   if (g >= G) return in;
   in = list_in[g];
-  uint32_t k;
-  if (in.k_hint >= 1) {
-    k = min(in.k_hint, kmax_level);
-  } else {
-    const uint32_t cls = ceil_log2_dev(in.m);
-    const uint32_t tb = (cls <= 32 && P.target_by_class[cls]) ? P.target_by_class[cls]
-                                                              : P.target_bucket;
-    const uint32_t want = in.m / tb + (in.m % tb ? 1u : 0u);
-    k = max(2u, min(want, kmax_level));
-  }
-  const uint32_t S = segment_samples(in.m, k, in.k_hint >= 1, P);
+  const uint32_t cls = ceil_log2_dev(in.m);
+  const uint32_t tb = (cls <= 32 && P.target_by_class[cls]) ? P.target_by_class[cls]
+                                                            : P.target_bucket;
+  const uint32_t want = in.m / tb + (in.m % tb ? 1u : 0u);
+  const uint32_t k = max(2u, min(want, kmax_level));
+  const uint32_t S = (uint32_t)umin64(umin64(in.m, (uint64_t)kDeepOversample * k), P.samp_max);
   const uint32_t nch = in.m / P.W + (in.m % P.W ? 1u : 0u);
   v[0] = S;
   v[1] = nch;
@@ -238,7 +225,8 @@ k_level_plan(DevState* st, const SegIn* list_in, LevelSeg* segs, LevelParams P, 
   if (tot[4] > P.bucket_cap) err |= kErrBucketCap;
   if (g < G) {
     LevelSeg s;
-    fill_segment(s, in.start, in.m, (uint32_t)v[4], (uint32_t)v[0], (uint32_t)v[1], P, in.range);
+    fill_segment(s, in.start, in.m, (uint32_t)v[4], (uint32_t)v[0], (uint32_t)v[1], P, in.known,
+                 in.range);
     s.samp_off = ex[0];
     s.chunk_off = ex[1];
     s.hist_off = ex[2];
@@ -349,7 +337,7 @@ k_sample_sort(DevState* st, LevelSeg* segs, Src src, uint64_t* samp_key, uint32_
   __shared__ uint64_t scan_sm[NT / 32];
   LevelSeg sg;
   if (ps.n) {
-    fill_segment(sg, 0, (uint32_t)ps.n, ps.k, ps.S, ps.nch, P, KeyRange{0, ~0ULL, 0, 0});
+    fill_segment(sg, 0, (uint32_t)ps.n, ps.k, ps.S, ps.nch, P, 0, KeyRange{0, ~0ULL});
     sg.samp_off = sg.chunk_off = sg.hist_off = sg.schunk_off = sg.bkt_off = sg.delta = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       reset_state(st, ps.local);
@@ -1076,20 +1064,21 @@ __device__ __forceinline__ void collect_buckets(DevState* st, const LevelSeg* se
     if (!emit_final || size == 0) continue;
     // its keys lie between its splitters (the segment's bounds at the ends)
     KeyRange kr = sg.range;
+    uint32_t known = sg.known;
     if (b >= 1) {
       kr.lo = ssk[sg.samp_off + ((uint64_t)b * sg.S) / sg.k];
-      kr.known |= 1u;
+      known |= 1u;
     }
     if (b + 1 < sg.k) {
       kr.hi = ssk[sg.samp_off + ((uint64_t)(b + 1) * sg.S) / sg.k];
-      kr.known |= 2u;
+      known |= 2u;
     }
     const bool eq = ordered && b >= 1 && b + 1 < sg.k && kr.lo == kr.hi;
     if (eq || size <= kBucketCap || last_level) {
       FinalItem it;
       it.start = start;
       it.aux = kr.lo;
-      it.bits = kr.known != 3u       ? kBitsUnknown
+      it.bits = known != 3u          ? kBitsUnknown
                 : kr.hi == kr.lo     ? (uint8_t)0
                                      : (uint8_t)(64 - __clzll((long long)(kr.hi - kr.lo)));
       it.size = size;
@@ -1106,7 +1095,7 @@ __device__ __forceinline__ void collect_buckets(DevState* st, const LevelSeg* se
       SegIn s;
       s.start = start;
       s.m = size;
-      s.k_hint = 0;
+      s.known = known;
       s.range = kr;
       const uint32_t slot = atomicAdd(&st->nseg[par_out], 1u);
       if (slot < P.seg_cap) list_out[slot] = s;
@@ -1625,8 +1614,8 @@ k_init_segments(DevState* st, const uint64_t* offsets, uint32_t nseg, uint64_t n
       SegIn in;
       in.start = a;
       in.m = (uint32_t)m;
-      in.k_hint = 0;
-      in.range = KeyRange{0, ~0ULL, 0, 0};
+      in.known = 0;
+      in.range = KeyRange{0, ~0ULL};
       const uint32_t slot = atomicAdd(&st->nseg[1], 1u);
       if (slot < seg_cap) list_l1[slot] = in;
       else atomicOr(&st->error, kErrSegCap);

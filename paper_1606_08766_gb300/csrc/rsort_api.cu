@@ -103,6 +103,7 @@ struct Plan {
   int direct = 0;           // n small enough for one in-SM sort
   uint32_t W1 = 0, Wd = 0;  // chunk sizes (level 1, deeper levels)
   uint64_t seg_cap = 0, samp_cap = 0, hist_cap = 0, chunk_cap = 0, schunk_cap = 0;
+  uint64_t samp_cap0 = 0;   // samples sorted in chunks (a one-segment level 1)
   uint64_t bucket_cap = 0, final_cap = 0;
   uint64_t samp_cap1 = 0, hist_cap1 = 0, chunk_cap1 = 0, schunk_cap1 = 0, bucket_cap1 = 0;
   bool need_tmp = false;
@@ -118,7 +119,7 @@ struct Plan {
   // arena offsets
   size_t off_tmp_key = 0, off_tmp_idx = 0, off_samp_key = 0, off_samp_idx = 0;
   size_t off_ssamp_key = 0, off_ssamp_idx = 0, off_hist = 0, off_sums = 0, off_segs = 0;
-  size_t off_plan = 0, off_chunk = 0, off_list0 = 0, off_list1 = 0, off_items = 0;
+  size_t off_list0 = 0, off_list1 = 0, off_items = 0;
   size_t off_state = 0, off_fine = 0, off_bid = 0;
   size_t total = 0;
 };
@@ -142,17 +143,19 @@ void layout(Plan& p) {
     p.off_tmp_key = take(p.n * 8);
     p.off_tmp_idx = take(p.n * 4);
   }
-  p.off_samp_key = take(p.samp_cap * 8);
-  p.off_samp_idx = take(p.samp_cap * 4);
+  // Two uses share the unsorted sample: samples that are sorted in chunks and
+  // merged (a one-segment level 1), and the segment of every chunk (the other
+  // levels, whose samples are one chunk a segment and sorted in registers).
+  p.off_samp_key = take(std::max(p.samp_cap0 * 8, p.chunk_cap * 4));
+  p.off_samp_idx = take(p.samp_cap0 * 4);
   p.off_ssamp_key = take((p.samp_cap + p.samp_extra) * 8);
   p.off_ssamp_idx = take((p.samp_cap + p.samp_extra) * 4);
   p.off_fine = take(p.fine_cap * 4);
   p.off_bid = take((p.n + 16) * 2);
-  p.off_hist = take(p.hist_cap * 4);
+  // (the plan's sums lie in the counters, which it precedes)
+  p.off_hist = take(std::max(p.hist_cap * 4, plan_sum_words(p.seg_cap) * 8));
   p.off_sums = take((p.hist_cap / kScanTile + 2) * 4);
   p.off_segs = take(p.seg_cap * sizeof(LevelSeg));
-  p.off_plan = take(plan_sum_words(p.seg_cap) * 8);
-  p.off_chunk = take(p.chunk_cap * 4);
   p.off_list0 = take(p.seg_cap * sizeof(SegIn));
   p.off_list1 = take(p.seg_cap * sizeof(SegIn));
   p.total = o;
@@ -214,7 +217,8 @@ void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int
     // bucket leave some beyond kBucketCap (at 2539 expected keys one in 150, at
     // 2730 keys and 64 samples still one in 10^4), which one CTA each then
     // merge-sorts; with 128, 1.5 times the mean is 5 deviations away
-    if (k1 < 2 && levels == 1 && n / p.k_plain > tb) p.oversample1 = 8 * kDeepOversample;
+    // (the plan of the least scratch keeps 16)
+    if (fine && k1 < 2 && levels == 1 && n / p.k_plain > tb) p.oversample1 = 8 * kDeepOversample;
   }
   // level 1 of one segment: 6 chunks per SM, so grids of 1, 2, 3 or 6 resident
   // CTAs per SM all get the same number of chunks
@@ -239,7 +243,11 @@ void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int
   }
   if (g1 > 1) p.W1 = p.Wd;
   const uint64_t segs_deep = n / (kBucketCap + 1) + 1;
-  p.seg_cap = std::max<uint64_t>(g1, segs_deep);
+  // a one-segment call's second level has at most its buckets
+  p.seg_cap = g1 > 1       ? std::max<uint64_t>(g1, segs_deep)
+              : levels < 2 ? 1
+              : levels < 3 ? std::min<uint64_t>(p.k_plain, segs_deep)
+                           : segs_deep;
   const uint32_t kmax1 = k1 >= 2 ? k1 : kMaxKDeep;
   // automatic fan-outs aim at the smallest target any segment class uses
   uint64_t tmin = p.target_bucket;
@@ -250,6 +258,7 @@ void plan_levels(Plan& p, uint64_t n, uint32_t k1, uint64_t g1, int num_sms, int
   p.bucket_cap1 = std::min<uint64_t>(p.bucket_cap1, (uint64_t)kmax1 * g1);
   const uint64_t a1 = k1 >= 2 ? 16ull * ceil_log2_host(k1) : (uint64_t)p.oversample1;
   p.samp_cap1 = std::min<uint64_t>(n, a1 * p.bucket_cap1);
+  p.samp_cap0 = g1 == 1 ? p.samp_cap1 : 0;
   p.chunk_cap1 = n / p.W1 + g1 + 1;
   p.hist_cap1 = (uint64_t)kmax1 * (n / p.W1) + p.bucket_cap1;
   p.schunk_cap1 = p.samp_cap1 / kSampleChunk + g1 + 1;
@@ -291,7 +300,6 @@ LevelParams level_params(const Plan& p, int level, uint64_t seed) {
   P.samp_max = level == 1 ? 0xffffffffu : p.samp_max;
   P.hinted = p.k1 >= 2;
   P.oversample = p.oversample1;
-  P.level1_oversample = 1;
   P.classifier = p.classifier;
   P.wide_scatter_k = p.wide_scatter_k;
   P.target_bucket = p.target_bucket;
@@ -366,7 +374,7 @@ void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const 
       src = Src{prev.key, prev.idx, 0};
     }
     src.bid = at<uint16_t>(ws, p.off_bid);
-    src.chunk_seg = at<uint32_t>(ws, p.off_chunk);
+    src.chunk_seg = at<uint32_t>(ws, p.off_samp_key);
     const Dst& dst = level_dst(L);
     const uint16_t where = &dst == &tmp ? kWhereTmp : kWhereOut;
     launch_level(e, P, st, lists[L & 1], lists[(L + 1) & 1], at<LevelSeg>(ws, p.off_segs), src,
@@ -374,7 +382,7 @@ void enqueue_levels_and_local(rsort_ctx* c, Workspace& ws, const Plan& p, const 
                  at<uint64_t>(ws, p.off_ssamp_key), at<uint32_t>(ws, p.off_ssamp_idx),
                  at<uint32_t>(ws, p.off_hist), at<uint32_t>(ws, p.off_sums), items, kmax,
                  L == p.levels, 1, nullptr, p.n, 0, nullptr,
-                 L == 1 && !segmented ? p.k_plain : 0u, at<uint64_t>(ws, p.off_plan));
+                 L == 1 && !segmented ? p.k_plain : 0u, at<uint64_t>(ws, p.off_hist));
   }
   launch_local_sort(e, st, items, p.final_cap, p.direct ? 1 : p.final_cap,
                     (const uint64_t*)d_keys_in, out, tmp, type == RSORT_KEY_F64, segmented);
@@ -545,7 +553,7 @@ void release_workspace(rsort_ctx* c, Workspace& ws, cudaStream_t s) {
 
 namespace {
 
-Plan plan_sort(rsort_ctx* c, uint64_t n, uint32_t p_virtual) {
+Plan plan_of(const rsort_ctx* c) {
   Plan p;
   p.classifier = c->classifier;
   p.wide_scatter_k = c->wide_scatter_k;
@@ -554,59 +562,81 @@ Plan plan_sort(rsort_ctx* c, uint64_t n, uint32_t p_virtual) {
   p.unit_scatter = c->unit_scatter;
   p.atomic_scatter = c->atomic_scatter;
   p.bulk_classify = c->bulk_classify;
-  const uint32_t k1 = p_virtual >= 2 ? p_virtual : 0;
+  return p;
+}
+
+// fine: see plan_levels (false: the plan of the least scratch).
+Plan plan_sort(const rsort_ctx* c, uint64_t n, uint32_t p_virtual, bool fine) {
+  Plan p = plan_of(c);
   if (n <= (uint64_t)kBucketCap) {
     p.n = n;
     p.direct = 1;
     p.final_cap = 2;
     p.seg_cap = 1;
-    p.need_tmp = false;
     p.levels = 0;
   } else {
-    const Plan q = p;
-    plan_levels(p, n, k1, 1, c->num_sms, c->max_levels, true);
-    p.need_tmp = true;
-    layout(p);
-    if (c->budget == 0 || p.total <= c->budget) return p;
-    // the budget counts: the plan that takes the least scratch
-    p = q;
-    plan_levels(p, n, k1, 1, c->num_sms, c->max_levels, false);
+    plan_levels(p, n, p_virtual >= 2 ? p_virtual : 0, 1, c->num_sms, c->max_levels, fine);
     p.need_tmp = true;
   }
   layout(p);
   return p;
 }
 
-Plan plan_segmented(rsort_ctx* c, uint64_t n, uint32_t num_segments) {
-  Plan p;
-  p.classifier = c->classifier;
-  p.wide_scatter_k = c->wide_scatter_k;
-  p.target_bucket = c->target_bucket;
-  for (int i = 0; i <= 32; ++i) p.target_by_class[i] = c->target_by_class[i];
-  p.unit_scatter = c->unit_scatter;
-  p.atomic_scatter = c->atomic_scatter;
-  p.bulk_classify = c->bulk_classify;
+Plan plan_segmented(const rsort_ctx* c, uint64_t n, uint32_t num_segments, bool fine) {
+  Plan p = plan_of(c);
   const uint64_t g1 = std::min<uint64_t>(num_segments, n / (kBucketCap + 1) + 1);
-  const Plan q = p;
-  for (const bool fine : {true, false}) {
-    p = q;
-    plan_levels(p, n, 0, std::max<uint64_t>(g1, 2), c->num_sms, c->max_levels, fine);
-    p.final_cap += num_segments;
-    p.need_tmp = true;
-    layout(p);
-    if (c->budget == 0 || p.total <= c->budget) break;
-  }
+  plan_levels(p, n, 0, std::max<uint64_t>(g1, 2), c->num_sms, c->max_levels, fine);
+  p.final_cap += num_segments;
+  p.need_tmp = true;
+  layout(p);
   return p;
+}
+
+Plan plan_partition(const rsort_ctx* c, uint64_t n, uint32_t k, uint32_t over, bool fine) {
+  Plan p = plan_of(c);
+  const uint32_t kk = k < 2 ? 2 : k;  // capacities as for two buckets when k = 1
+  plan_levels(p, n, kk, 1, c->num_sms, 1, fine);
+  p.final_cap = 1;
+  if (over > 1) {
+    p.samp_extra = (uint64_t)kk + 2;
+    p.fine_cap = 2 * (uint64_t)k * over + 16;  // counters, prefix sums, search state
+  }
+  layout(p);
+  return p;
+}
+
+// Reserves the scratch of a call in ws; make(fine) plans it.  The fine plan takes
+// more scratch (2^20 keys 16.9 MB, the other 15.5; 2^22 61.7, 61.2; above 2^25 the
+// two are one), which must not be what a budget refuses this call or a later one
+// for, so under a budget it is taken only where it is a small part of it.  A call
+// whose fine plan does not fit, in the budget or on the device, takes the other.
+// Under a budget what others hold changes from call to call, so scratch that fits
+// either plan is kept as it is (a captured call finds what the first one sized).
+constexpr uint64_t kFineBudgetShare = 16;
+template <typename MakePlan>
+rsort_status reserve_plan(rsort_ctx* c, Workspace& ws, cudaStream_t s, MakePlan make, Plan& p) {
+  p = make(true);
+  if (c->budget == 0 || p.total <= c->budget / kFineBudgetShare) {
+    if (p.total <= ws.bytes) return RSORT_OK;
+    const Plan least = make(false);
+    if ((c->budget == 0 || least.total > ws.bytes) &&
+        ensure_workspace(c, ws, p.total, s) == RSORT_OK)
+      return RSORT_OK;
+    p = least;
+  } else {
+    p = make(false);
+  }
+  return ensure_workspace(c, ws, p.total, s);
 }
 
 }  // namespace
 
 size_t sort_scratch_bytes(rsort_ctx* c, uint64_t n, uint32_t p_virtual) {
-  return n == 0 ? 0 : plan_sort(c, n, p_virtual).total;
+  return n == 0 ? 0 : plan_sort(c, n, p_virtual, false).total;
 }
 
 size_t segmented_scratch_bytes(rsort_ctx* c, uint64_t n, uint32_t num_segments) {
-  return (n == 0 || num_segments == 0) ? 0 : plan_segmented(c, n, num_segments).total;
+  return (n == 0 || num_segments == 0) ? 0 : plan_segmented(c, n, num_segments, false).total;
 }
 
 rsort_status enqueue_sort(rsort_ctx* c, Workspace& ws, const LaunchEnv& env, rsort_key_type type,
@@ -614,9 +644,10 @@ rsort_status enqueue_sort(rsort_ctx* c, Workspace& ws, const LaunchEnv& env, rso
                           uint64_t n, uint32_t p_virtual, uint64_t seed, DevState** st_out) {
   LaunchEnv e = env;
   e.overlap = n <= kOverlapMaxKeys;
-  Plan p = plan_sort(c, n, p_virtual);
+  Plan p;
   const uint32_t k1 = p_virtual >= 2 ? p_virtual : 0;
-  rsort_status rs = ensure_workspace(c, ws, p.total, e.stream);
+  rsort_status rs = reserve_plan(
+      c, ws, e.stream, [&](bool fine) { return plan_sort(c, n, p_virtual, fine); }, p);
   if (rs != RSORT_OK) return rs;
   DevState* st = at<DevState>(ws, p.off_state);
   FinalItem* items = at<FinalItem>(ws, p.off_items);
@@ -640,8 +671,9 @@ rsort_status enqueue_segmented(rsort_ctx* c, Workspace& ws, const LaunchEnv& env
                                uint32_t num_segments, uint64_t seed, DevState** st_out) {
   LaunchEnv e = env;
   e.overlap = n <= kOverlapMaxKeys;
-  Plan p = plan_segmented(c, n, num_segments);
-  rsort_status rs = ensure_workspace(c, ws, p.total, e.stream);
+  Plan p;
+  rsort_status rs = reserve_plan(
+      c, ws, e.stream, [&](bool fine) { return plan_segmented(c, n, num_segments, fine); }, p);
   if (rs != RSORT_OK) return rs;
   DevState* st = at<DevState>(ws, p.off_state);
   FinalItem* items = at<FinalItem>(ws, p.off_items);
@@ -803,32 +835,13 @@ rsort_status partition_impl(rsort_ctx* c, rsort_key_type type, const void* d_key
     return cuda_status(c);
   }
   Plan p;
-  p.classifier = c->classifier;
-  p.wide_scatter_k = c->wide_scatter_k;
-  p.target_bucket = c->target_bucket;
-  for (int i = 0; i <= 32; ++i) p.target_by_class[i] = c->target_by_class[i];
-  p.unit_scatter = c->unit_scatter;
-  p.atomic_scatter = c->atomic_scatter;
-  p.bulk_classify = c->bulk_classify;
-  const uint32_t kk = k < 2 ? 2 : k;  // capacities as for two buckets when k = 1
-  const Plan q = p;
-  for (const bool fine : {true, false}) {
-    p = q;
-    plan_levels(p, n, kk, 1, c->num_sms, 1, fine);
-    p.final_cap = 1;
-    p.need_tmp = false;
-    if (over > 1) {
-      p.samp_extra = (uint64_t)kk + 2;
-      p.fine_cap = 2 * (uint64_t)K + 16;  // counters, prefix sums, search state
-    }
-    layout(p);
-    if (c->budget == 0 || p.total <= c->budget) break;
-  }
   Workspace& ws = c->ws;
-  rsort_status rs = ensure_workspace(c, ws, p.total, s);
+  rsort_status rs = reserve_plan(
+      c, ws, s, [&](bool fine) { return plan_partition(c, n, k, over, fine); }, p);
   if (rs != RSORT_OK) return latch(c, rs);
   DevState* st = at<DevState>(ws, p.off_state);
   SegIn* list1 = at<SegIn>(ws, p.off_list1);
+  const uint32_t kk = k < 2 ? 2 : k;
   LevelParams P = level_params(p, 1, seed);
   P.no_tie_break = tie_break ? 0 : 1;
   Src src{(const uint64_t*)d_keys_in, nullptr, type == RSORT_KEY_F64};

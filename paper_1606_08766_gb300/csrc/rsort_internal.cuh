@@ -102,18 +102,17 @@ struct LocalPlan {
   uint8_t algo[3] = {kLocalBins, kLocalBins, kLocalBins};  // small, mid, medium
 };
 
-// Range of the keys of a segment or bucket, as far as splitters bound it.
+// Range of the keys of a segment or bucket, as far as splitters bound it (beside
+// it `known`: bit 0, lo is a bound; bit 1, hi is).
 struct KeyRange {
   uint64_t lo, hi;  // inclusive
-  uint32_t known;   // bit 0: lo is a bound, bit 1: hi is
-  uint32_t pad;
 };
 
 // A segment waiting to be partitioned (input of a level).
 struct SegIn {
   uint64_t start;   // absolute position (identical in every buffer)
   uint32_t m;       // elements
-  uint32_t k_hint;  // buckets requested (>= 1), or 0 to choose from m
+  uint32_t known;   // bounds of range
   KeyRange range;   // of its keys
 };
 
@@ -134,7 +133,7 @@ struct LevelSeg {
   uint32_t nschunks;
   uint32_t nunits;      // histogram units (one per chunk)
   uint32_t W;           // keys per chunk of this segment (all chunks equal but the last)
-  uint32_t pad;
+  uint32_t known;       // bounds of range
   KeyRange range;       // of the segment's keys
 };
 
@@ -221,7 +220,6 @@ struct LevelParams {
   // samples a bucket, the paper's rule), 0: it is automatic (oversample)
   int hinted = 0;
   uint32_t oversample = kDeepOversample;
-  int level1_oversample;  // 1: a = 16 ceil(log2 k) for hinted k (the paper's rule)
   int classifier;         // 0: splitter tree, 1: leading-bits table
   int wide_scatter_k;     // levels with at least this many buckets scatter 4096-key sub-tiles
   uint32_t target_bucket; // automatic fan-out aims at buckets of this many keys
