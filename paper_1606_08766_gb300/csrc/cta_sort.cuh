@@ -21,6 +21,8 @@
 //   still crowded       bitonic sort of the whole bucket (Appendix "Bitonic
 //                       Sort"), which needs no assumption on the keys
 //
+// (k_local_sort ranks a crowded bucket of at most a pair a thread instead.)
+//
 // A bucket whose keys are all equal and whose elements arrive in position
 // order (every bucket produced by the stable scatter) is already sorted; if
 // they arrive in another order, the bins are taken over the positions.
@@ -236,14 +238,22 @@ __device__ __noinline__ void cta_bitonic_regs(uint32_t m, CtaSortSmem s) {
 }
 
 // Bitonic sort of the m pairs in s.k / s.i (Appendix "Bitonic Sort"), ordered
-// by (key, position).  The register network always sorts NT*ITEMS pairs; a
-// bucket of at most an eighth of that is padded to its own power of two with
-// (UINT64_MAX, UINT32_MAX) and sorted in shared memory.
-template <int NT, int ITEMS>
+// by (key, position).  The register network sorts NT*ITEMS pairs; a bucket of at
+// most an eighth of that is padded to its own power of two with (UINT64_MAX,
+// UINT32_MAX) and sorted in shared memory.
+// SIZED: a half or a quarter of NT*ITEMS pairs where they hold the bucket (40,000
+// segments of 500 keys, half of them one value: 1485 us with 1024 pairs, 880 with
+// 512).  The kernels that rarely come here do without the code of three networks:
+// it cost a sort of 2^20 keys 1 us of 75.
+template <int NT, int ITEMS, bool SIZED>
 __device__ __forceinline__ void cta_bitonic_pairs(uint32_t m, const CtaSortSmem& s) {
-  if (m > (uint32_t)(NT * ITEMS / 8)) {
-    cta_bitonic_regs<NT, ITEMS>(m, s);
-    return;
+  constexpr uint32_t kCap = NT * ITEMS;
+  if (m > kCap / 8) {
+    if constexpr (SIZED) {
+      if (m <= kCap / 4) return cta_bitonic_regs<NT, ITEMS / 4>(m, s);
+      if (m <= kCap / 2) return cta_bitonic_regs<NT, ITEMS / 2>(m, s);
+    }
+    return cta_bitonic_regs<NT, ITEMS>(m, s);
   }
   const uint32_t P = next_pow2_u32(m);
   for (uint32_t e = m + threadIdx.x; e < P; e += NT) { s.k[e] = ~0ULL; s.i[e] = ~0u; }
@@ -380,7 +390,7 @@ __device__ __forceinline__ void order_bins(const CtaSortSmem& s, uint32_t nmulti
 //   One rsort_sort of 3001 normal float64 keys, by the bitonic network over
 //   shared memory and six launches: 90 us; with refined bins and one launch
 //   (k_direct_sort): 15 us.
-template <int NT, int ITEMS>
+template <int NT, int ITEMS, bool SIZED>
 __device__ __noinline__ int cta_sort_crowded(uint32_t m, uint64_t mn, int shift, CtaSortSmem s,
                                              uint32_t* s_sum, uint64_t* red) {
   using BS = BinSort<NT, ITEMS>;
@@ -426,7 +436,7 @@ __device__ __noinline__ int cta_sort_crowded(uint32_t m, uint64_t mn, int shift,
       return kAlgoBins;
     }
   }
-  cta_bitonic_pairs<NT, ITEMS>(m, s);
+  cta_bitonic_pairs<NT, ITEMS, SIZED>(m, s);
   return kAlgoBitonic;
 }
 
@@ -441,11 +451,12 @@ struct NoRelease {
 // m added to the counter of the branch taken (kAlgoRank, kAlgoInOrder,
 // kAlgoBitonic or kAlgoBins).  rank_max bounds rank-by-counting (at most NT
 // elements: one per thread); force_bitonic sorts every larger bucket by
-// bitonic sort instead of the bins.  released() is called once by every
+// bitonic sort instead of the bins; SIZED: see cta_bitonic_pairs.  released() is called once by every
 // thread of the CTA, together, as soon as key[] and idx[] are no longer read
 // (the pairs are in shared memory): the caller may then load the next
 // bucket into them while this one is finished.
-template <int NT, int ITEMS, typename InOrderFn, typename ReleaseFn = NoRelease>
+template <int NT, int ITEMS, bool SIZED = false, typename InOrderFn,
+          typename ReleaseFn = NoRelease>
 __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], uint32_t m,
                                InOrderFn in_position_order, const CtaSortSmem& s, uint64_t* red,
                                uint64_t* scan_sm, uint64_t* algo, uint32_t rank_max = kRankMax,
@@ -477,7 +488,7 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
       if (e < m) { s.k[e] = key[r]; s.i[e] = idx[r]; }
     }
     __syncthreads();
-    cta_bitonic_pairs<NT, ITEMS>(m, s);
+    cta_bitonic_pairs<NT, ITEMS, SIZED>(m, s);
 #pragma unroll
     for (int r = 0; r < ITEMS; ++r) {
       key[r] = 0;
@@ -548,7 +559,7 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
   }
   __syncthreads();
   if (crowd) {
-    const int how = cta_sort_crowded<NT, ITEMS>(m, mn, shift, s, s_sum, red);
+    const int how = cta_sort_crowded<NT, ITEMS, SIZED>(m, mn, shift, s, s_sum, red);
     // (no register of the pairs is kept across the call)
 #pragma unroll
     for (int r = 0; r < ITEMS; ++r) {

@@ -16,7 +16,8 @@
 //                  it: <= 1024 keys (128 threads, 8 CTAs per SM), <= 2048 keys
 //                  (128 threads, 5 per SM), <= 4096 keys (256 threads, 2 per
 //                  SM)
-//   k_local_rest   what the classes leave (crowded, copied and oversize
+//   k_local_crowded  a class's crowded buckets, of a large batch
+//   k_local_rest   what the classes leave (other crowded, copied and oversize
 //                  buckets), or every bucket of a call that has few
 // Buckets are taken from device work lists with atomic cursors by persistent
 // grids.  The final store restores float64 bit patterns.
@@ -175,10 +176,15 @@ __device__ __forceinline__ int64_t next_item(DevState* st, int cls, uint64_t cap
 // IT a thread; every pair takes its rank inside its bin from one shared-memory
 // atomic on the bin's 16-bit counter, the counters are scanned, the pairs go
 // to their slots, and the few bins that hold several are ordered by insertion.
-// A bucket with a crowded bin is handed to k_local_rest instead (a list of its
-// own), so that no register of this kernel serves that case: with the refined
-// bins and the bitonic network in this kernel the compiler spilled, and the
-// 1025..2048-key class of a 2^28-key sort took 2.63 to 3.40 ms.
+// A bucket with a crowded bin of more pairs than threads is handed on instead (a
+// list of its own), so that no register of this kernel serves that case: with the
+// refined bins and the bitonic network in this kernel the compiler spilled, and
+// the 1025..2048-key class of a 2^28-key sort took 2.63 to 3.40 ms.  Up to a pair a
+// thread it is ranked by counting here, and a bucket of one key alone needs no
+// other kernel either: it is in order, or its bins are taken over the positions.
+//   200,000 uint64 segments of 100 keys, all of a segment equal: 1980 us when such
+//   buckets were handed on, 386 here; half of them equal: 6550, 1313.  7*10^7 keys
+//   of 10,000 values, most of whose buckets hold one: 5055, 4436.
 //   2^28 uniform keys, before / after: 1025..2048 keys 2.12 / 1.50 ms (3.5
 //   TB/s of keys and positions read and written), 2049..4096 0.53 / 0.38,
 //   up to 1024 0.12 / 0.087.
@@ -203,7 +209,7 @@ __device__ __forceinline__ int64_t next_item(DevState* st, int cls, uint64_t cap
 //   9.0 ms with the bitonic network for such buckets, 3.3 ms with these.
 template <int NT, int IT, int CLS, int MINB, bool REFINE>
 __global__ void __launch_bounds__(NT, MINB)
-k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
+k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B, int crowd_list) {
   pdl_entry();
   using BS = BinSort<NT, IT>;
   constexpr int NW = NT / 32;
@@ -257,31 +263,10 @@ k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
     uint32_t claim = 0;
     if (tid == 0) claim = gridDim.x + atomicAdd(&st->cursor_c[kList], 1u);
     FinalItem fn{};
-    bool sorted = true;
-    if (m <= rank_max) {
-      // rank-by-counting (Appendix "Fast Work-Inefficient Ranking")
-      __syncthreads();  // the previous bucket has been written out
-      if (tid < m) {
-        sk[tid] = key[0];
-        si[tid] = idx[0];
-      }
-      if (tid == 0) {
-        if (claim < nitems) fn = items[item_slot(kList, claim, cap)];
-        s_f = fn;
-        count_algo(st->algo_elems, kAlgoRank, m);
-      }
-      __syncthreads();
-      uint32_t rank = 0;
-      if (tid < m)
-        for (uint32_t q = 0; q < m; ++q) rank += pair_less(sk[q], si[q], key[0], idx[0]) ? 1u : 0u;
-      __syncthreads();
-      if (tid < m) {
-        sk[rank] = key[0];
-        si[rank] = idx[0];
-      }
-      fn = s_f;
-      load(fn);
-    } else {
+    // all keys equal and in position order: sorted as they come
+    bool in_order = false;
+    bool sorted = m > rank_max;
+    if (m > rank_max) {
       // smallest key and width of the key range in bits
       uint64_t mn;
       int bits;
@@ -298,132 +283,188 @@ k_local_sort(DevState* st, FinalItem* items, uint64_t cap, Bufs B) {
         mn = f.aux;
         bits = f.bits;
       }
-      const int shift = bits > BS::kLogBins ? bits - BS::kLogBins : 0;
-      uint32_t hr[IT];  // counter halfword, then that << 16 | rank inside the bin
-      for_slots<NT, IT>(m, [&](int r) {
-        hr[r] = BS::half_of((uint32_t)((key[r] - mn) >> shift));
-      });
-      if (tid == 0) s_nmulti = 0;
+      in_order = bits == 0 && f.kind == kKindSort;
+      if (!in_order) {
+        const int shift = bits > BS::kLogBins ? bits - BS::kLogBins : 0;
+        uint32_t hr[IT];  // counter halfword, then that << 16 | rank inside the bin
+        if (bits == 0) {
+          // all keys equal, in no particular order: bins of their positions
+          uint64_t a = ~0ULL, b = 0;
+          for_slots<NT, IT>(m, [&](int r) {
+            a = idx[r] < a ? idx[r] : a;
+            b = idx[r] > b ? idx[r] : b;
+          });
+          __syncthreads();  // (s_red is written again)
+          block_minmax_u64<NT>(a, b, s_red);
+          const int pb = b != a ? 64 - __clzll((long long)(b - a)) : 0;
+          const int ps = pb > BS::kLogBins ? pb - BS::kLogBins : 0;
+          for_slots<NT, IT>(m, [&](int r) { hr[r] = BS::half_of((uint32_t)((idx[r] - a) >> ps)); });
+        } else {
+          for_slots<NT, IT>(m, [&](int r) {
+            hr[r] = BS::half_of((uint32_t)((key[r] - mn) >> shift));
+          });
+        }
+        if (tid == 0) s_nmulti = 0;
 #pragma unroll 1
-      for (int pass = 0;; ++pass) {
-        clear_bins<NT, IT>(hist);
-        uint4* run = (uint4*)(hist + tid * BS::kRun);
-        __syncthreads();  // (1) counters clear; the previous bucket written out
-        for_slots<NT, IT>(m, [&](int r) {
-          const uint32_t h = hr[r];
-          const uint32_t sh = (h & 1) << 4;
-          const uint32_t old = atomicAdd(&hist[h >> 1], 1u << sh);
-          hr[r] = (h << 16) | ((old >> sh) & 0xffffu);
-        });
-        if (tid == 0 && pass == 0 && claim < nitems) fn = items[item_slot(kList, claim, cap)];
-        __syncthreads();  // (2) counts complete
-        uint32_t sum = 0, any = 0;
-#pragma unroll
-        for (int q = 0; q < IT / 4; ++q) {
-          const uint4 v = run[q];
-          sum = __dp2a_lo(v.x, 0x0101u, sum);
-          sum = __dp2a_lo(v.y, 0x0101u, sum);
-          sum = __dp2a_lo(v.z, 0x0101u, sum);
-          sum = __dp2a_lo(v.w, 0x0101u, sum);
-          any |= v.x | v.y | v.z | v.w;
-        }
-        uint32_t inc = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-          if (lane >= o) inc += y;
-        }
-        // a bin of kBinLimit or more pairs sets one of the high bits
-        static_assert((kBinLimit & (kBinLimit - 1)) == 0, "the crowd test reads high bits");
-        constexpr uint32_t kHigh = 0xffffu & ~(uint32_t)(kBinLimit - 1);
-        const bool crowd = __any_sync(0xffffffffu, (any & (kHigh | (kHigh << 16))) != 0);
-        if (lane == 31) s_sum[warp] = inc | (crowd ? 0x80000000u : 0u);
-        __syncthreads();  // (3) warp sums
-        uint32_t pre = 0, all = 0;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-          const uint32_t v = s_sum[w];
-          pre += w < warp ? v : 0u;
-          all |= v;
-        }
-        sorted = (all >> 31) == 0;
-        const bool again = REFINE && pass == 0 && !sorted && shift > 0;
-        if (sorted || again) {
-          // (the crowd flags of the sums before, if any, shift out of at)
-          uint32_t at = (pre & 0xffffu) + inc - sum;
+        for (int pass = 0;; ++pass) {
+          clear_bins<NT, IT>(hist);
+          uint4* run = (uint4*)(hist + tid * BS::kRun);
+          __syncthreads();  // (1) counters clear; the previous bucket written out
+          for_slots<NT, IT>(m, [&](int r) {
+            const uint32_t h = hr[r];
+            const uint32_t sh = (h & 1) << 4;
+            const uint32_t old = atomicAdd(&hist[h >> 1], 1u << sh);
+            hr[r] = (h << 16) | ((old >> sh) & 0xffffu);
+          });
+          if (tid == 0 && pass == 0 && claim < nitems) fn = items[item_slot(kList, claim, cap)];
+          __syncthreads();  // (2) counts complete
+          uint32_t sum = 0, any = 0;
 #pragma unroll
           for (int q = 0; q < IT / 4; ++q) {
-            uint4 v = run[q];
-            auto step = [&](uint32_t& w) {
-              const uint32_t c = w;
-              w = at * 0x10001u + (c << 16);
-              at = __dp2a_lo(c, 0x0101u, at);
-            };
-            step(v.x);
-            step(v.y);
-            step(v.z);
-            step(v.w);
-            run[q] = v;
+            const uint4 v = run[q];
+            sum = __dp2a_lo(v.x, 0x0101u, sum);
+            sum = __dp2a_lo(v.y, 0x0101u, sum);
+            sum = __dp2a_lo(v.z, 0x0101u, sum);
+            sum = __dp2a_lo(v.w, 0x0101u, sum);
+            any |= v.x | v.y | v.z | v.w;
           }
-          if (tid == NT - 1) half[NT * BS::kRun * 2] = (uint16_t)m;
+          uint32_t inc = sum;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+          }
+          // a bin of kBinLimit or more pairs sets one of the high bits
+          static_assert((kBinLimit & (kBinLimit - 1)) == 0, "the crowd test reads high bits");
+          constexpr uint32_t kHigh = 0xffffu & ~(uint32_t)(kBinLimit - 1);
+          const bool crowd = __any_sync(0xffffffffu, (any & (kHigh | (kHigh << 16))) != 0);
+          if (lane == 31) s_sum[warp] = inc | (crowd ? 0x80000000u : 0u);
+          __syncthreads();  // (3) warp sums
+          uint32_t pre = 0, all = 0;
+#pragma unroll
+          for (int w = 0; w < NW; ++w) {
+            const uint32_t v = s_sum[w];
+            pre += w < warp ? v : 0u;
+            all |= v;
+          }
+          sorted = (all >> 31) == 0;
+          const bool again = REFINE && pass == 0 && !sorted && shift > 0;
+          if (sorted || again) {
+            // (the crowd flags of the sums before, if any, shift out of at)
+            uint32_t at = (pre & 0xffffu) + inc - sum;
+#pragma unroll
+            for (int q = 0; q < IT / 4; ++q) {
+              uint4 v = run[q];
+              auto step = [&](uint32_t& w) {
+                const uint32_t c = w;
+                w = at * 0x10001u + (c << 16);
+                at = __dp2a_lo(c, 0x0101u, at);
+              };
+              step(v.x);
+              step(v.y);
+              step(v.z);
+              step(v.w);
+              run[q] = v;
+            }
+            if (tid == NT - 1) half[NT * BS::kRun * 2] = (uint16_t)m;
+          }
+          if (!again) break;
+          __syncthreads();
+          // bin b, whose c pairs start at slot lo, becomes 2c parts from 2 lo
+          for_slots<NT, IT>(m, [&](int r) {
+            const uint32_t h = hr[r] >> 16;
+            const uint32_t lo = half[h], c = half[BS::next_half(h)] - lo;
+            const uint64_t off = (key[r] - mn) << (64 - shift);
+            hr[r] = BS::half_of(2 * lo + (uint32_t)__umul64hi(off, (uint64_t)(2 * c)));
+          });
+          __syncthreads();
         }
-        if (!again) break;
-        __syncthreads();
-        // bin b, whose c pairs start at slot lo, becomes 2c parts from 2 lo
+        if (tid == 0) s_f = fn;
+        if (!sorted && m > (uint32_t)NT) {
+          // crowded: the bucket goes to the call's list of such buckets
+          if (tid == 0) {
+            const uint32_t slot = atomicAdd(&st->nfinal_c[crowd_list], 1u);
+            const int a = crowd_array(crowd_list);
+            const int end = a == kClassCopy ? kClassBig : kListRefine + a - kClassSmall;
+            if ((uint64_t)slot + st->nfinal_c[a] + st->nfinal_c[end] < cap)
+              items[crowd_slot(st, crowd_list, slot, cap)] = f;
+            else
+              atomicOr(&st->error, kErrFinalCap);
+          }
+          __syncthreads();
+          f = s_f;
+          load(f);
+          continue;
+        }
+        if (sorted) {
+          __syncthreads();  // (4) bin starts in place
+          for_slots<NT, IT>(m, [&](int r) {
+            const uint32_t h = hr[r] >> 16, o = hr[r] & 0xffffu;
+            const uint32_t p = half[h] + o;
+            sk[p] = key[r];
+            si[p] = idx[r];
+            if (o == 1) multi[atomicAdd(&s_nmulti, 1u)] = (uint16_t)h;
+          });
+          if (tid == 0) count_algo(st->algo_elems, kAlgoBins, m);
+          __syncthreads();  // (5) pairs in place, the registers are free
+          fn = s_f;
+          load(fn);
+          // order every listed bin by insertion (an element alone in its bin is
+          // already in its final slot)
+          const uint32_t nmulti = s_nmulti;
+          for (uint32_t j = tid; j < nmulti; j += NT) {
+            const uint32_t h = multi[j];
+            const uint32_t lo = half[h], cnt = half[BS::next_half(h)] - lo;
+            uint64_t* bk = sk + lo;
+            uint32_t* bi = si + lo;
+            for (uint32_t a = 1; a < cnt; ++a) {
+              const uint64_t ka = bk[a];
+              const uint32_t ia = bi[a];
+              uint32_t q = a;
+              while (q > 0 && pair_less(ka, ia, bk[q - 1], bi[q - 1])) {
+                bk[q] = bk[q - 1];
+                bi[q] = bi[q - 1];
+                --q;
+              }
+              bk[q] = ka;
+              bi[q] = ia;
+            }
+          }
+        }
+      }
+    }
+    if (!sorted || in_order) {
+      // in order already, or (tiny buckets, and crowded ones that have a thread a
+      // pair) rank-by-counting (Appendix "Fast Work-Inefficient Ranking")
+      __syncthreads();  // the previous bucket has been written out
+      if (in_order) {
         for_slots<NT, IT>(m, [&](int r) {
-          const uint32_t h = hr[r] >> 16;
-          const uint32_t lo = half[h], c = half[BS::next_half(h)] - lo;
-          const uint64_t off = (key[r] - mn) << (64 - shift);
-          hr[r] = BS::half_of(2 * lo + (uint32_t)__umul64hi(off, (uint64_t)(2 * c)));
+          sk[r * NT + tid] = key[r];
+          si[r * NT + tid] = idx[r];
         });
-        __syncthreads();
+      } else if (tid < m) {
+        sk[tid] = key[0];
+        si[tid] = idx[0];
       }
-      if (tid == 0) s_f = fn;
-      if (!sorted) {
-        // crowded: the bucket goes to k_local_rest's list
-        if (tid == 0) {
-          const uint32_t slot = atomicAdd(&st->nfinal_c[kListCrowd], 1u);
-          if (slot < cap) items[item_slot(kListCrowd, slot, cap)] = f;
-          else atomicOr(&st->error, kErrFinalCap);
+      if (tid == 0) {
+        if (claim < nitems) fn = items[item_slot(kList, claim, cap)];
+        s_f = fn;
+        count_algo(st->algo_elems, in_order ? kAlgoInOrder : kAlgoRank, m);
+      }
+      __syncthreads();
+      if (!in_order) {
+        uint32_t rank = 0;
+        if (tid < m)
+          for (uint32_t q = 0; q < m; ++q)
+            rank += pair_less(sk[q], si[q], key[0], idx[0]) ? 1u : 0u;
+        __syncthreads();
+        if (tid < m) {
+          sk[rank] = key[0];
+          si[rank] = idx[0];
         }
-        __syncthreads();
-        f = s_f;
-        load(f);
-        continue;
       }
-      __syncthreads();  // (4) bin starts in place
-      for_slots<NT, IT>(m, [&](int r) {
-        const uint32_t h = hr[r] >> 16, o = hr[r] & 0xffffu;
-        const uint32_t p = half[h] + o;
-        sk[p] = key[r];
-        si[p] = idx[r];
-        if (o == 1) multi[atomicAdd(&s_nmulti, 1u)] = (uint16_t)h;
-      });
-      if (tid == 0) count_algo(st->algo_elems, kAlgoBins, m);
-      __syncthreads();  // (5) pairs in place, the registers are free
       fn = s_f;
       load(fn);
-      // order every listed bin by insertion (an element alone in its bin is
-      // already in its final slot)
-      const uint32_t nmulti = s_nmulti;
-      for (uint32_t j = tid; j < nmulti; j += NT) {
-        const uint32_t h = multi[j];
-        const uint32_t lo = half[h], cnt = half[BS::next_half(h)] - lo;
-        uint64_t* bk = sk + lo;
-        uint32_t* bi = si + lo;
-        for (uint32_t a = 1; a < cnt; ++a) {
-          const uint64_t ka = bk[a];
-          const uint32_t ia = bi[a];
-          uint32_t q = a;
-          while (q > 0 && pair_less(ka, ia, bk[q - 1], bi[q - 1])) {
-            bk[q] = bk[q - 1];
-            bi[q] = bi[q - 1];
-            --q;
-          }
-          bk[q] = ka;
-          bi[q] = ia;
-        }
-      }
     }
     __syncthreads();  // (6) sorted
     {
@@ -479,15 +520,57 @@ k_local_quicksort(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, ui
   }
 }
 
+// The crowded buckets of a class (cta_sort_pairs: refined bins, the bitonic
+// network), by CTAs of their size; with `own` the class's whole list, every bucket
+// by bitonic sort (tunables sort_small, sort_mid).
+//   k_local_rest takes them in sorts and small batches, which have few; in a large
+//   batch they can be all there is, and two CTAs of 512 threads an SM are too few
+//   for small ones: 20,000 segments of 1000 keys, half of them one value, 4058 us
+//   there, 846 here.  sort_mid on a sort of 8*10^6 keys: 1181 there, 672 here.
+template <int NT, int IT, int CLS, int MINB>
+__global__ void __launch_bounds__(NT, MINB)
+k_local_crowded(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, bool own) {
+  pdl_entry();
+  using BS = BinSort<NT, IT>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  CtaSortSmem s;
+  s.k = (uint64_t*)smem_raw;
+  s.i = (uint32_t*)(s.k + BS::kCap);
+  s.hist = s.i + BS::kCap;
+  __shared__ uint64_t red[2 * NT / 32];
+  __shared__ uint64_t scan_sm[NT / 32];
+  __shared__ uint32_t s_next;
+  constexpr int kCrowd = CLS == kClassSmall ? kListCrowdSmall : kListCrowdMid;
+  const int list = own ? CLS : kCrowd;
+  const uint32_t total = (uint32_t)umin64(st->nfinal_c[list], cap);
+  const uint32_t rank_max = own ? st->local.rank_max : 0u;  // (small crowded ones are done)
+  for (uint32_t at = blockIdx.x; at < total;) {
+    const FinalItem f = items[own ? item_slot(CLS, at, cap) : crowd_slot(st, kCrowd, at, cap)];
+    if (threadIdx.x == 0) s_next = gridDim.x + atomicAdd(&st->cursor_c[list], 1u);
+    uint64_t key[IT];
+    uint32_t idx[IT];
+    load_bucket<NT, IT>(B, f, key, idx);
+    cta_sort_pairs<NT, IT, true>(key, idx, f.size, [&] { return f.kind == kKindSort; }, s, red,
+                                 scan_sm, st->algo_elems, rank_max, own);
+    for (uint32_t t = threadIdx.x; t < f.size; t += NT)
+      store_out(B, f.start + t, s.k[t], s.i[t]);
+    __syncthreads();
+    at = s_next;
+    __syncthreads();
+  }
+}
+
 // Everything the class kernels leave, by 512-thread CTAs of 8 slots: the
 // copy-through buckets (size 1, or equality buckets already in position order:
 // a coalesced copy that restores float64 bit patterns), the buckets with
 // crowded bins (cta_sort_pairs: refined bins, the bitonic network), and the
-// oversize ones (after the last partition level; rare).  With `classes` the
-// size classes' own lists too (bit c: list c): a call of few buckets finishes
-// in this one launch, whose slowest bucket bounds it, instead of one launch
-// per class, each as long as its slowest bucket.  bitonic: bit c sorts class
-// c's buckets by bitonic sort.
+// oversize ones (after the last partition level; rare).  lists: bit l takes list
+// l; with the size classes' own lists a call of few buckets finishes in this one
+// launch, whose slowest bucket bounds it, instead of one launch per class, each as
+// long as its slowest bucket.  bitonic: bit c sorts class c's buckets by bitonic
+// sort.  BATCH: networks fitted to a bucket (SIZED); 1000 segments of 1000 keys
+// spread over 63 octaves 243 us without, 99 with.
+template <bool BATCH>
 __global__ void __launch_bounds__(kRestThreads, 2)
 k_local_rest(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, uint32_t lists,
              uint32_t bitonic) {
@@ -504,15 +587,16 @@ k_local_rest(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, uint32_
   const uint32_t rank_max = st->local.rank_max;
   // lists in turn, the longest work first (an oversize bucket's merges run
   // longest)
+  constexpr int kLists = kListCrowd + 1;
   auto list_of = [](int q) {
-    constexpr int order[kNumLists] = {kClassBig,       kListCrowd,      kListRefine + 2,
-                                      kClassMedium,    kListRefine + 1, kClassMid,
-                                      kListRefine + 0, kClassSmall,     kClassCopy};
+    constexpr int order[kLists] = {kClassBig,       kListCrowd,      kListRefine + 2,
+                                   kClassMedium,    kListRefine + 1, kClassMid,
+                                   kListRefine + 0, kClassSmall,     kClassCopy};
     return order[q];
   };
-  uint32_t end[kNumLists], total = 0;
+  uint32_t end[kLists], total = 0;
 #pragma unroll
-  for (int q = 0; q < kNumLists; ++q) {
+  for (int q = 0; q < kLists; ++q) {
     const int l = list_of(q);
     total += (lists >> l) & 1u ? (uint32_t)umin64(st->nfinal_c[l], cap) : 0u;
     end[q] = total;
@@ -522,13 +606,14 @@ k_local_rest(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, uint32_
     int l = list_of(0);
     uint32_t from = 0;
 #pragma unroll
-    for (int q = 0; q + 1 < kNumLists; ++q) {
+    for (int q = 0; q + 1 < kLists; ++q) {
       if (at >= end[q]) {
         l = list_of(q + 1);
         from = end[q];
       }
     }
-    const FinalItem f = items[item_slot(l, at - from, cap)];
+    const FinalItem f = items[l == kListCrowd ? crowd_slot(st, l, at - from, cap)
+                                              : item_slot(l, at - from, cap)];
     if (threadIdx.x == 0) s_next = gridDim.x + atomicAdd(&st->cursor_rest, 1u);
     if (l == kClassCopy) {
       if (f.where != kWhereOut || B.f64) {  // else already in place
@@ -546,9 +631,8 @@ k_local_rest(DevState* st, const FinalItem* items, uint64_t cap, Bufs B, uint32_
       uint64_t key[IT];
       uint32_t idx[IT];
       load_bucket<NT, IT>(B, f, key, idx);
-      cta_sort_pairs<NT, IT>(key, idx, f.size, [&] { return f.kind == kKindSort; }, s, red,
-                             scan_sm, st->algo_elems, rank_max,
-                             (bitonic >> l) & 1u);
+      cta_sort_pairs<NT, IT, BATCH>(key, idx, f.size, [&] { return f.kind == kKindSort; }, s, red,
+                                    scan_sm, st->algo_elems, rank_max, (bitonic >> l) & 1u);
       for (uint32_t t = threadIdx.x; t < f.size; t += NT)
         store_out(B, f.start + t, s.k[t], s.i[t]);
     }
@@ -619,6 +703,12 @@ constexpr int kMidItems = (int)kMidCap / kMidThreads;  // 16
 constexpr int kMidPerSm = 5;
 constexpr int kMidRefinePerSm = 4;
 static_assert(kMidThreads * kMidItems == (int)kMidCap, "mid class fits one CTA");
+// Their crowded buckets: the network's registers (three words a pair) set the
+// shape.
+constexpr int kSmallCrowdPerSm = 8;
+constexpr int kMidCrowdThreads = 256;
+constexpr int kMidCrowdItems = (int)kMidCap / kMidCrowdThreads;  // 8
+constexpr int kMidCrowdPerSm = 4;
 // The medium class (2049..4096 keys): 256 threads of 16 slots, two CTAs per
 // SM (with the next bucket claimed and loaded early, this measured 2 %
 // faster than 512 threads of 8 slots, which had spread every bucket's fixed
@@ -637,13 +727,25 @@ constexpr size_t kRestSmem = BinSort<kRestThreads, kBucketCap / kRestThreads>::k
 // 43 -> 29 us against a launch per class; the class kernels sort a bucket in
 // less SM time and win above.
 constexpr uint64_t kOneLaunchPerSm = 8;
+// Batches that may have more buckets than this per SM launch k_local_crowded for
+// the small and the mid class: the two launches cost 3 us, against 38 of 1000
+// uniform segments of 1000 keys and 147 of 10,000 of 1100.
+constexpr uint64_t kCrowdLaunchPerSm = 54;
 
 template <int NT, int IT, int CLS, int MINB, bool REFINE>
 void launch_class(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t cap, const Bufs& B,
-                  const char* name) {
+                  int crowd_list, const char* name) {
   Scope sc(e, name);
   launch_kernel(e, k_local_sort<NT, IT, CLS, MINB, REFINE>, e.num_sms * MINB, NT,
-                BinSort<NT, IT>::kSmem, st, items, cap, B);
+                BinSort<NT, IT>::kSmem, st, items, cap, B, crowd_list);
+}
+
+template <int NT, int IT, int CLS, int MINB>
+void launch_crowded(const LaunchEnv& e, DevState* st, const FinalItem* items, uint64_t cap,
+                    const Bufs& B, bool own, const char* name) {
+  Scope sc(e, name);
+  launch_kernel(e, k_local_crowded<NT, IT, CLS, MINB>, e.num_sms * MINB, NT,
+                BinSort<NT, IT>::kSmem, st, items, cap, B, own);
 }
 
 template <int NT, int IT, int CLS, int MINB, int MINBR>
@@ -667,7 +769,16 @@ void set_local_kernel_attributes() {
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs_smem_bytes(kMidCap));
   cudaFuncSetAttribute(k_local_quicksort<kLocalThreads, kBucketCap, kClassMedium>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs_smem_bytes(kBucketCap));
-  cudaFuncSetAttribute(k_local_rest, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_local_crowded<kSmallThreads, kSmallItems, kClassSmall, kSmallCrowdPerSm>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)BinSort<kSmallThreads, kSmallItems>::kSmem);
+  cudaFuncSetAttribute(
+      k_local_crowded<kMidCrowdThreads, kMidCrowdItems, kClassMid, kMidCrowdPerSm>,
+      cudaFuncAttributeMaxDynamicSharedMemorySize,
+      (int)BinSort<kMidCrowdThreads, kMidCrowdItems>::kSmem);
+  cudaFuncSetAttribute(k_local_rest<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)kRestSmem);
+  cudaFuncSetAttribute(k_local_rest<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)kRestSmem);
 }
 
@@ -695,8 +806,8 @@ void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint6
   B.out = out;
   B.tmp = tmp;
   B.f64 = f64;
-  // k_local_rest takes a class whose algorithm is bitonic, and every class of
-  // a call with few buckets
+  // k_local_rest takes every class of a call with few buckets, the medium class
+  // when its algorithm is bitonic, and what the class kernels note as crowded
   const uint8_t* algo = e.local.algo;
   const bool one = max_items <= kOneLaunchPerSm * (uint64_t)e.num_sms;
   const bool refine = segmented && f64;
@@ -704,16 +815,24 @@ void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint6
   for (int c = kClassSmall; c <= kClassMedium; ++c) {
     const uint8_t a = algo[c - kClassSmall];
     if (a == kLocalBitonic) bitonic |= 1u << c;
-    if (a == kLocalBitonic || (one && a == kLocalBins)) lists |= 1u << c;
+    if ((a == kLocalBitonic && (one || c == kClassMedium)) || (one && a == kLocalBins))
+      lists |= 1u << c;
     if (one && a == kLocalBins) lists |= 1u << (kListRefine + c - kClassSmall);
   }
   auto own = [&](int c) { return algo[c - kClassSmall] == kLocalBins && !((lists >> c) & 1u); };
+  // the small and the mid class's crowded buckets in kernels of their shape
+  const bool split = segmented && max_items > kCrowdLaunchPerSm * (uint64_t)e.num_sms;
+  const int crowd_small = split ? kListCrowdSmall : kListCrowd;
+  const int crowd_mid = split ? kListCrowdMid : kListCrowd;
+  auto crowded = [&](int c) {
+    return own(c) ? split : algo[c - kClassSmall] == kLocalBitonic && !one;
+  };
   if (own(kClassSmall)) {
     launch_class<kSmallThreads, kSmallItems, kClassSmall, kSmallPerSm, false>(
-        e, st, items, item_cap, B, "local_sort");
+        e, st, items, item_cap, B, crowd_small, "local_sort");
     if (refine)
       launch_class<kSmallThreads, kSmallItems, kClassSmall, kSmallRefinePerSm, true>(
-          e, st, items, item_cap, B, "local_sort_refine");
+          e, st, items, item_cap, B, crowd_small, "local_sort_refine");
   }
   if (algo[kClassMid - kClassSmall] == kLocalQuick) {
     Scope sc(e, "local_sort_mid");
@@ -721,11 +840,11 @@ void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint6
                   kLocalThreads, qs_smem_bytes(kMidCap), st, items, item_cap, B,
                   0x243f6a8885a308d3ULL);
   } else if (own(kClassMid)) {
-    launch_class<kMidThreads, kMidItems, kClassMid, kMidPerSm, false>(e, st, items, item_cap, B,
-                                                                      "local_sort_mid");
+    launch_class<kMidThreads, kMidItems, kClassMid, kMidPerSm, false>(
+        e, st, items, item_cap, B, crowd_mid, "local_sort_mid");
     if (refine)
       launch_class<kMidThreads, kMidItems, kClassMid, kMidRefinePerSm, true>(
-          e, st, items, item_cap, B, "local_sort_mid_refine");
+          e, st, items, item_cap, B, crowd_mid, "local_sort_mid_refine");
   }
   if (algo[kClassMedium - kClassSmall] == kLocalQuick) {
     Scope sc(e, "local_sort_medium");
@@ -734,16 +853,26 @@ void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint6
                   0x9e3779b97f4a7c15ULL);
   } else if (own(kClassMedium)) {
     launch_class<kMediumThreads, kMediumItems, kClassMedium, kMediumPerSm, false>(
-        e, st, items, item_cap, B, "local_sort_medium");
+        e, st, items, item_cap, B, kListCrowd, "local_sort_medium");
     if (refine)
       launch_class<kMediumThreads, kMediumItems, kClassMedium, kMediumPerSm, true>(
-          e, st, items, item_cap, B, "local_sort_medium_refine");
+          e, st, items, item_cap, B, kListCrowd, "local_sort_medium_refine");
   }
+  if (crowded(kClassSmall))
+    launch_crowded<kSmallThreads, kSmallItems, kClassSmall, kSmallCrowdPerSm>(
+        e, st, items, item_cap, B, !own(kClassSmall), "local_sort_crowded");
+  if (crowded(kClassMid))
+    launch_crowded<kMidCrowdThreads, kMidCrowdItems, kClassMid, kMidCrowdPerSm>(
+        e, st, items, item_cap, B, !own(kClassMid), "local_sort_mid_crowded");
   {
     Scope sc(e, "local_rest");
     const uint64_t grid = umin64(umax64(max_items, 1), (uint64_t)e.num_sms * 2);
-    launch_kernel(e, k_local_rest, (int)grid, kRestThreads, kRestSmem, st, items, item_cap, B,
-                  lists, bitonic);
+    if (segmented)
+      launch_kernel(e, k_local_rest<true>, (int)grid, kRestThreads, kRestSmem, st, items, item_cap,
+                    B, lists, bitonic);
+    else
+      launch_kernel(e, k_local_rest<false>, (int)grid, kRestThreads, kRestSmem, st, items, item_cap,
+                    B, lists, bitonic);
   }
 }
 

@@ -951,7 +951,7 @@ rsort_status rsort_sort(rsort_ctx* c, rsort_key_type type, const void* d_keys_in
     const double mean = opt_stats->p ? (double)n / opt_stats->p : (double)n;
     opt_stats->max_over_mean = mean > 0 ? opt_stats->max_bucket / mean : 0.0;
     opt_stats->final_buckets = 0;
-    // (kListCrowd's buckets are on their class's list too)
+    // (crowded buckets are on their class's list too)
     for (int i = 0; i < kListCrowd; ++i) opt_stats->final_buckets += h.nfinal_c[i];
     // per key: level 1's classify reads 8 B and writes a 2-byte bucket id,
     // its scatter reads 8 + 2 and writes 12; a deeper level reads 8 and

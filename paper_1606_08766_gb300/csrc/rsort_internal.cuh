@@ -57,21 +57,29 @@ enum : int {
   // sorted with bins refined to the keys' density (their bit patterns crowd a
   // few octaves, so equal-width bins would not do)
   kListRefine = 5,   // + (class - kClassSmall)
-  // buckets in which a class kernel found crowded bins
+  // buckets in which a class kernel found crowded bins: those for k_local_rest,
+  // and in large batches the small and the mid class's for k_local_crowded
   kListCrowd = 8,
-  kNumLists = 9,
-  kNumItemArrays = 5
+  kListCrowdSmall = 9,
+  kListCrowdMid = 10,
+  kNumLists = 11,
+  kNumItemArrays = 4
 };
 
 // Slot of a list's item i among kNumItemArrays arrays of cap items.  A bucket
-// is on one list only, except that a class's may be on kListCrowd as well; so
-// two lists share an array, one from its start and one from its end:
-// copies | oversize, each class | its refine list, and the crowded ones alone.
+// is on one of these lists only, so two share an array, one from its start and
+// one from its end: copies | oversize, each class | its refine list.
 __host__ __device__ __forceinline__ uint64_t item_slot(int list, uint64_t i, uint64_t cap) {
-  if (list == kListCrowd) return 4 * cap + i;
   if (list == kClassBig) return cap - 1 - i;
   if (list >= kListRefine) return (uint64_t)(list - kListRefine + 2) * cap - 1 - i;
   return (uint64_t)list * cap + i;
+}
+// The array of a list of crowded buckets.  Such a bucket is noted while its own
+// class's list is still being read, so in another array: the two lists there, which
+// are complete by then, and the crowded ones are different buckets, and fit
+// together.
+__host__ __device__ __forceinline__ constexpr int crowd_array(int list) {
+  return list == kListCrowd ? kClassCopy : list == kListCrowdSmall ? kClassMid : kClassMedium;
 }
 // Which in-SM algorithm finished a bucket (rsort_stats.algo_elems counts the
 // elements each one handled):
@@ -180,6 +188,13 @@ struct alignas(16) DevState {
   uint32_t l1_nb;
   uint32_t l1_ordered;
 };
+
+// Slot of crowded bucket i of a list: after the first list of its array.
+__device__ __forceinline__ uint64_t crowd_slot(const DevState* st, int list, uint64_t i,
+                                               uint64_t cap) {
+  const int a = crowd_array(list);
+  return (uint64_t)a * cap + st->nfinal_c[a] + i;
+}
 
 // LevelParams::stable / in_order value: decided on the device.  Level 1
 // keeps input order when at least 1/kAutoOrderShare of its buckets are
