@@ -30,6 +30,12 @@ namespace {
 constexpr size_t kNoAllocBytes = 8u << 20;      // 8 MiB
 constexpr uint32_t kNoAllocMaxK = 1024;          // buckets per call
 constexpr uint64_t kNoAllocMaxChunks = 512;      // chunks of the classify/scatter grid
+// Calls of more keys than this launch in the ordinary way.  Set up early, the next
+// kernels' CTAs lie on the SMs beside the two of the staged scatter for all of its
+// long pass (overlapped, ordinary, us: 5*10^6 keys, 64 buckets 132, 140, 1000
+// buckets 211, 206; 1.6*10^7 keys 315, 303 and 492, 462; 1.3*10^8 2273, 2069 and
+// 3880, 3543).
+constexpr uint64_t kNoAllocOverlapMax = 1ull << 23;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
@@ -148,7 +154,7 @@ extern "C" rsort_status rsort_partition_noalloc(rsort_key_type type, const void*
   e.num_sms = sms;
   e.timer = nullptr;
   e.launches = nullptr;
-  e.overlap = n <= kOverlapMaxKeys;
+  e.overlap = n <= kNoAllocOverlapMax;
   // The control block is reset by the first kernel; every other scratch word
   // read later is written earlier in the same call.
   Src src{(const uint64_t*)d_keys_in, nullptr, type == RSORT_KEY_F64};

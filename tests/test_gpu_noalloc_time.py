@@ -1,0 +1,34 @@
+"""The allocation-free partition step takes no longer a key up to 2^27 keys, where
+other calls overlap their launches, than above."""
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _ms(n, k, keys):
+    from paper_1606_08766_gb300.binding import partition_noalloc
+    keys = keys[:n]
+    ko, po = torch.empty_like(keys), torch.empty(n, dtype=torch.int32, device="cuda")
+    off = torch.empty(k + 1, dtype=torch.int64, device="cuda")
+    a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    ts = []
+    for _ in range(4):
+        a.record()
+        for _ in range(4):
+            partition_noalloc(keys, k, 3, ko, po, off)
+        b.record()
+        b.synchronize()
+        ts.append(a.elapsed_time(b))
+    return sorted(ts)[1] / n
+
+
+@pytest.mark.parametrize("k", [64, 1000])
+def test_time_a_key_at_the_overlap_bound(k):
+    n = 1 << 27
+    g = torch.Generator(device="cuda").manual_seed(1)
+    keys = torch.randint(-(1 << 63), (1 << 63) - 1, (n + 4096,), dtype=torch.int64, device="cuda",
+                         generator=g)
+    # (launches overlapped at 2^27 keys: 1.10)
+    assert _ms(n, k, keys) < 1.04 * _ms(n + 4096, k, keys)
