@@ -165,7 +165,7 @@ rsort_status rsort_partition_ex(rsort_ctx *ctx, rsort_key_type type, const void 
  *     IEEE bit pattern.
  * d_keys [n] (1 <= n <= 2^24, device); k in {2, 4, 8, 16, 32}; *d_pos_out
  * (device u64) receives the position of the chosen element.  CTAs reduce
- * subtrees of 4096 leaves; their windows pass through the context's scratch
+ * subtrees of 2048 leaves; their windows pass through the context's scratch
  * (less than 1 byte per leaf).
  * Errors: EINVAL, ENOMEM, ECUDA. */
 rsort_status rsort_approx_median(rsort_ctx *ctx, rsort_key_type type, const void *d_keys,
