@@ -440,27 +440,18 @@ __device__ __noinline__ int cta_sort_crowded(uint32_t m, uint64_t mn, int shift,
   return kAlgoBitonic;
 }
 
-// No-op for cta_sort_pairs' released callback.
-struct NoRelease {
-  __device__ void operator()() const {}
-};
-
 // Sorts the m pairs; on return s.k[0..m) / s.i[0..m) hold them in order.
 // in_position_order() says whether the elements arrive with increasing
 // positions; it is asked only when all keys are equal.  algo (nullable) gets
 // m added to the counter of the branch taken (kAlgoRank, kAlgoInOrder,
 // kAlgoBitonic or kAlgoBins).  rank_max bounds rank-by-counting (at most NT
 // elements: one per thread); force_bitonic sorts every larger bucket by
-// bitonic sort instead of the bins; SIZED: see cta_bitonic_pairs.  released() is called once by every
-// thread of the CTA, together, as soon as key[] and idx[] are no longer read
-// (the pairs are in shared memory): the caller may then load the next
-// bucket into them while this one is finished.
-template <int NT, int ITEMS, bool SIZED = false, typename InOrderFn,
-          typename ReleaseFn = NoRelease>
+// bitonic sort instead of the bins; SIZED: see cta_bitonic_pairs.
+template <int NT, int ITEMS, bool SIZED = false, typename InOrderFn>
 __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], uint32_t m,
                                InOrderFn in_position_order, const CtaSortSmem& s, uint64_t* red,
                                uint64_t* scan_sm, uint64_t* algo, uint32_t rank_max = kRankMax,
-                               bool force_bitonic = false, ReleaseFn released = ReleaseFn()) {
+                               bool force_bitonic = false) {
   const uint32_t tid = threadIdx.x;
   if (m <= rank_max && m <= (uint32_t)NT) {
     count_algo(algo, kAlgoRank, m);
@@ -477,7 +468,6 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
     __syncthreads();
     if (tid < m) { s.k[rank] = key[0]; s.i[rank] = idx[0]; }
     __syncthreads();
-    released();
     return;
   }
   if (force_bitonic) {
@@ -494,7 +484,6 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
       key[r] = 0;
       idx[r] = 0;
     }
-    released();
     return;
   }
   uint64_t mn = ~0ULL, mx = 0;
@@ -511,7 +500,6 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
       if (e < m) { s.k[e] = key[r]; s.i[e] = idx[r]; }
     }
     __syncthreads();
-    released();
     return;
   }
   // all keys equal, in no particular order: (key, position) order is the
@@ -560,7 +548,8 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
   __syncthreads();
   if (crowd) {
     const int how = cta_sort_crowded<NT, ITEMS, SIZED>(m, mn, shift, s, s_sum, red);
-    // (no register of the pairs is kept across the call)
+    // (so that no register of the pairs is kept across the call: a caller's loop
+    // would keep those of slots it does not load, 32 bytes spilled or 124)
 #pragma unroll
     for (int r = 0; r < ITEMS; ++r) {
       key[r] = 0;
@@ -568,13 +557,11 @@ __device__ void cta_sort_pairs(uint64_t (&key)[ITEMS], uint32_t (&idx)[ITEMS], u
     }
     count_algo(algo, how, m);
     restore_common_key<NT>(s, m, s_by_pos, s_key_all);
-    released();
     return;
   }
   count_algo(algo, kAlgoBins, m);
   place_in_bins<NT, ITEMS>(key, idx, hr, m, s, &s_nmulti);
   __syncthreads();
-  released();
   order_bins<NT, ITEMS>(s, s_nmulti);
   __syncthreads();
   restore_common_key<NT>(s, m, s_by_pos, s_key_all);

@@ -505,9 +505,6 @@ constexpr int kCT = 2048;                       // keys per classify pipeline st
 constexpr int kCStages = 3;                     // classify stages at level 1 (2 in flight)
 constexpr int kCStagesDeep = 2;                 // deeper levels: fewer stages, more CTAs per SM
 constexpr int kCItems = kCT / kPartThreads;     // 8 keys per lane per stage
-constexpr int kST = 2048;                       // keys per scatter sub-tile
-constexpr int kSItems = kST / kPartThreads;     // 8 keys per lane per sub-tile
-static_assert(kSItems * 32 * kPartWarps == kST, "warp w owns kSItems*32 consecutive keys");
 
 struct PartSmem {
   Splitters sp;
@@ -518,10 +515,6 @@ struct PartSmem {
   uint8_t* wwin;       // [kPartWarps][K] scatter: per-warp winner lane of each bucket
   unsigned char* buf;  // classify: kCStages key stages; scatter: two sub-tile buffers
 };
-
-
-// one scatter sub-tile buffer: keys, positions, bucket ids
-constexpr size_t kSBufBytes = (size_t)kST * (8 + 4 + 2);
 
 // mode: bit 0 the classifier (0 tree, 1 table), bit 1 no tie-breaking.
 __host__ __device__ inline size_t part_common_bytes(uint32_t kmax, int mode) {
@@ -535,20 +528,7 @@ __host__ __device__ inline size_t classify_smem_bytes(uint32_t kmax, int mode, i
   return part_common_bytes(kmax, mode) + (size_t)stages * kCT * 8;
 }
 
-__host__ __device__ inline size_t part_smem_bytes(uint32_t kmax, bool scatter, int mode) {
-  size_t b = part_common_bytes(kmax, mode);
-  if (scatter) {
-    b += (size_t)(kmax + 1) * 4 + 4;
-    b += (size_t)kPartWarps * cnt_stride(kmax) * 2;
-    b = (b + 15) & ~(size_t)15;
-    b += 2 * kSBufBytes;
-  } else {
-    b += (size_t)kCStages * kCT * 8;
-  }
-  return b;
-}
-
-__device__ inline PartSmem carve(unsigned char* base, uint32_t kmax, bool scatter, int mode) {
+__device__ inline PartSmem carve(unsigned char* base, uint32_t kmax, int mode) {
   PartSmem s;
   const size_t Kp = next_pow2_u32(kmax);
   unsigned char* p = base;
@@ -572,11 +552,6 @@ __device__ inline PartSmem carve(unsigned char* base, uint32_t kmax, bool scatte
   s.wcnt = nullptr;
   s.dlt = nullptr;
   s.wwin = nullptr;
-  if (scatter) {
-    s.sbase = (uint32_t*)p; p += (size_t)(kmax + 1) * 4 + 4;
-    s.wcnt = (uint16_t*)p; p += (size_t)kPartWarps * cnt_stride(kmax) * 2;
-    p = (unsigned char*)(((uintptr_t)p + 15) & ~(uintptr_t)15);
-  }
   s.buf = p;
   return s;
 }
@@ -603,7 +578,7 @@ __host__ __device__ inline size_t scatter_smem_bytes(uint32_t kmax, int mode, in
 
 __device__ inline PartSmem carve_scatter(unsigned char* base, uint32_t kmax, int mode, int nw,
                                          bool stable = true) {
-  PartSmem s = carve(base, kmax, false, mode);
+  PartSmem s = carve(base, kmax, mode);
   unsigned char* p = base + part_common_bytes(kmax, mode);
   s.sbase = (uint32_t*)p;
   p += (size_t)(kmax + 1) * 4 + 4;
@@ -630,7 +605,7 @@ k_classify_count(const DevState* st, const LevelSeg* segs, Src src, const uint64
                  const uint32_t* ssi, uint32_t* hist, uint32_t W, uint32_t kmax, int mode) {
   pdl_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  PartSmem sm = carve(smem_raw, kmax, false, mode);
+  PartSmem sm = carve(smem_raw, kmax, mode);
   uint64_t* stage = (uint64_t*)sm.buf;
   const uint64_t pol = l2_evict_first_policy();
   const uint64_t total = st->total_chunks;
@@ -1501,15 +1476,14 @@ void set_partition_kernel_attributes() {
   set_sample_sort_attributes<1024, 8, 1>();
   cudaFuncSetAttribute(k_sample_merge, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)BinSort<kMergeThreads, kMergeItems>::kSmem);
-  const size_t c = umax64(part_smem_bytes(kMaxK, false, 0), part_smem_bytes(kMaxK, false, 1));
-  const size_t s = umax64(part_smem_bytes(kMaxK, true, 0), part_smem_bytes(kMaxK, true, 1));
+  const size_t c = umax64(classify_smem_bytes(kMaxK, 0, kCStages),
+                          classify_smem_bytes(kMaxK, 1, kCStages));
   cudaFuncSetAttribute(k_classify_count<kCStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)c);
   cudaFuncSetAttribute(k_classify_count<kCStagesDeep>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)umax64(classify_smem_bytes(kMaxKDeep, 0, kCStagesDeep),
                                    classify_smem_bytes(kMaxKDeep, 1, kCStagesDeep)));
-  (void)s;
   cudaFuncSetAttribute(k_scatter<kPartThreads, 2048, true>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)umax64(scatter_smem_bytes(kMaxK, 0, kPartWarps, 2048),
@@ -1546,21 +1520,24 @@ void set_partition_kernel_attributes() {
   cudaGetLastError();  // a refused attribute only disables the variant
 }
 
-// Resident CTAs per SM of the classify / scatter kernels for a bucket bound.
-int part_blocks_per_sm(uint32_t kmax, bool scatter, int mode, bool stable = true) {
+// Resident CTAs per SM of the classify and of the 2048-key scatter for a bucket
+// bound.
+int classify_blocks_per_sm(uint32_t kmax, int mode) {
   int nb = 0;
-  const size_t smem = part_smem_bytes(kmax, scatter, mode);
-  if (scatter && stable)
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_classify_count<kCStages>, kPartThreads,
+                                                classify_smem_bytes(kmax, mode, kCStages));
+  return nb > 0 ? nb : 1;
+}
+
+int scatter_blocks_per_sm(uint32_t kmax, int mode, bool stable) {
+  int nb = 0;
+  const size_t smem = scatter_smem_bytes(kmax, mode, kPartWarps, 2048, stable);
+  if (stable)
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_scatter<kPartThreads, 2048, true>,
-                                                  kPartThreads,
-                                                  scatter_smem_bytes(kmax, mode, kPartWarps, 2048));
-  else if (scatter)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &nb, k_scatter<kPartThreads, 2048, false>, kPartThreads,
-        scatter_smem_bytes(kmax, mode, kPartWarps, 2048, false));
+                                                  kPartThreads, smem);
   else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_classify_count<kCStages>, kPartThreads,
-                                                  smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_scatter<kPartThreads, 2048, false>,
+                                                  kPartThreads, smem);
   return nb > 0 ? nb : 1;
 }
 
@@ -1740,18 +1717,17 @@ void launch_level(const LaunchEnv& e, const LevelParams& P, DevState* st, const 
     }
   }
   const int mode = P.classifier | (P.no_tie_break ? 2 : 0);
-  const size_t smem_c = part_smem_bytes((uint32_t)kmax_level, false, mode);
-  const size_t smem_s = part_smem_bytes((uint32_t)kmax_level, true, mode);
+  const size_t smem_c = classify_smem_bytes((uint32_t)kmax_level, mode, kCStages);
   // deeper levels take the 2-stage classify when their buckets fit its shared memory
   const bool deep_c = P.level > 1 && (uint32_t)kmax_level <= (uint32_t)kMaxKDeep;
   const size_t smem_cd = classify_smem_bytes((uint32_t)kmax_level, mode, kCStagesDeep);
   const int grid_c = grid_for(
       P.chunk_cap, 1,
       sms * (deep_c ? classify_deep_blocks_per_sm((uint32_t)kmax_level, mode)
-                    : part_blocks_per_sm((uint32_t)kmax_level, false, mode)));
+                    : classify_blocks_per_sm((uint32_t)kmax_level, mode)));
   const bool stable = P.stable == 1;
   const int grid_s = grid_for(P.chunk_cap, 1,
-                              sms * part_blocks_per_sm((uint32_t)kmax_level, true, mode, stable));
+                              sms * scatter_blocks_per_sm((uint32_t)kmax_level, mode, stable));
   const bool wide = kmax_level >= P.wide_scatter_k &&
                     scatter_smem_bytes((uint32_t)kmax_level, mode, 16, 4096, stable) <=
                         g_wide_scatter_smem_max;

@@ -15,7 +15,6 @@ namespace rsort {
 constexpr int kPartThreads = 256;                 // classify / scatter CTA
 constexpr int kPartWarps = kPartThreads / 32;
 constexpr int kItems = 16;                        // keys per lane per sub-tile
-constexpr int kWarpSpan = 32 * kItems;            // 512 consecutive keys per warp
 constexpr int kSubTile = kPartThreads * kItems;   // 4096 keys staged per sub-tile
 constexpr int kMinChunk = 1024;                   // smallest level-1 chunk of a small call
 constexpr int kFineTile = 6144;                   // keys of an unordered scatter sub-tile
@@ -27,7 +26,6 @@ constexpr int kBucketCap = 4096;                  // T_s: largest bucket one CTA
 constexpr int kTargetBucket = 1536;               // aim for this final bucket size
                                                   // (mostly below the 1024-key class)
 constexpr int kSampleChunk = 8192;                // sample sort: pairs per CTA chunk
-constexpr int kSampleThreads = 512;               // sample sort CTA
 constexpr int kDeepOversample = 16;               // samples per bucket at levels >= 2
 constexpr int kMaxLevels = 3;                     // partition levels before fallback
 constexpr int kLocalThreads = 256;                // in-SM quicksort CTA
