@@ -743,6 +743,7 @@ void launch_class(const LaunchEnv& e, DevState* st, FinalItem* items, uint64_t c
 template <int NT, int IT, int CLS, int MINB>
 void launch_crowded(const LaunchEnv& e, DevState* st, const FinalItem* items, uint64_t cap,
                     const Bufs& B, bool own, const char* name) {
+  static_assert(BinSort<NT, IT>::kSmem <= 44 * 1024, "within the default limit (with statics)");
   Scope sc(e, name);
   launch_kernel(e, k_local_crowded<NT, IT, CLS, MINB>, e.num_sms * MINB, NT,
                 BinSort<NT, IT>::kSmem, st, items, cap, B, own);
@@ -769,17 +770,12 @@ void set_local_kernel_attributes() {
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs_smem_bytes(kMidCap));
   cudaFuncSetAttribute(k_local_quicksort<kLocalThreads, kBucketCap, kClassMedium>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs_smem_bytes(kBucketCap));
-  cudaFuncSetAttribute(k_local_crowded<kSmallThreads, kSmallItems, kClassSmall, kSmallCrowdPerSm>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)BinSort<kSmallThreads, kSmallItems>::kSmem);
-  cudaFuncSetAttribute(
-      k_local_crowded<kMidCrowdThreads, kMidCrowdItems, kClassMid, kMidCrowdPerSm>,
-      cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)BinSort<kMidCrowdThreads, kMidCrowdItems>::kSmem);
   cudaFuncSetAttribute(k_local_rest<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)kRestSmem);
-  cudaFuncSetAttribute(k_local_rest<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)kRestSmem);
+  // (k_local_crowded needs no attribute, k_local_rest<true> gets it where it is
+  // launched: the kernels of batches alone are not loaded before the first one.
+  // Loaded with the others they move the others' code, and a sort of 5000 keys or
+  // a partition of 4096 took 1 us of 30 longer.)
 }
 
 bool direct_sort_takes(const LocalPlan& local, uint64_t n) {
@@ -867,12 +863,15 @@ void launch_local_sort(const LaunchEnv& e, DevState* st, FinalItem* items, uint6
   {
     Scope sc(e, "local_rest");
     const uint64_t grid = umin64(umax64(max_items, 1), (uint64_t)e.num_sms * 2);
-    if (segmented)
+    if (segmented) {
+      cudaFuncSetAttribute(k_local_rest<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kRestSmem);
       launch_kernel(e, k_local_rest<true>, (int)grid, kRestThreads, kRestSmem, st, items, item_cap,
                     B, lists, bitonic);
-    else
+    } else {
       launch_kernel(e, k_local_rest<false>, (int)grid, kRestThreads, kRestSmem, st, items, item_cap,
                     B, lists, bitonic);
+    }
   }
 }
 
