@@ -186,7 +186,7 @@ __device__ __forceinline__ int64_t next_item(DevState* st, int cls, uint64_t cap
 //   buckets were handed on, 386 here; half of them equal: 6550, 1313.  7*10^7 keys
 //   of 10,000 values, most of whose buckets hold one: 5055, 4436.
 //   2^28 uniform keys, before / after: 1025..2048 keys 2.12 / 1.50 ms (3.5
-//   TB/s of keys and positions read and written), 2049..4096 0.53 / 0.38,
+//   TB/s of keys and positions read and written), 2049..4096 0.53 / 0.33,
 //   up to 1024 0.12 / 0.087.
 //
 // The kernel is bound by its instructions and by the latency between its
