@@ -197,7 +197,8 @@ rsort_status rsort_sort(rsort_ctx *ctx, rsort_key_type type, const void *d_keys_
  * d_offsets: device array of num_segments + 1 nondecreasing u64 values with
  * d_offsets[num_segments] <= n; keys outside the segments are left untouched.
  * Offsets are checked on the device: a violation skips that segment and is
- * reported as RSORT_EDEVICE by rsort_check.  d_keys_in must not alias
+ * reported as RSORT_EDEVICE by rsort_check; where offsets decrease, segments
+ * may overlap, and those above 4096 keys are skipped too.  d_keys_in must not alias
  * d_keys_out.  No host synchronisation: once the context's scratch has been
  * sized by a first call of the same n, the call can be captured in a CUDA
  * graph.  Errors: EINVAL, ENOMEM, ECUDA (EDEVICE via rsort_check). */

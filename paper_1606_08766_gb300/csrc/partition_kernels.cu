@@ -177,7 +177,9 @@ k_level_plan(DevState* st, const SegIn* list_in, LevelSeg* segs, LevelParams P, 
   pdl_entry();
   __shared__ uint64_t sm[kPlanThreads / 32];
   const uint32_t G0 = st->nseg[par_in];
-  const bool over = G0 > P.seg_cap;
+  // (segments that may overlap are not partitioned: the ids and outputs of one
+  // would be overwritten by another's while its counts are its own)
+  const bool over = G0 > P.seg_cap || (st->error & kErrUnordered) != 0;
   const uint32_t G = over ? 0u : G0;
   const uint32_t ncta = max(1u, (G + kPlanThreads - 1) / kPlanThreads);
   const uint32_t t = blockIdx.x;
@@ -253,7 +255,8 @@ k_level_plan(DevState* st, const SegIn* list_in, LevelSeg* segs, LevelParams P, 
   }
   if (threadIdx.x != 0 || t + 1 != ncta) return;
   st->nseg[par_in ^ 1] = 0;
-  if (over) err |= kErrSegCap;
+  if (G0 > P.seg_cap) err |= kErrSegCap;
+  if (over && err == 0) err = kErrUnordered;
   if (err) {
     atomicOr(&st->error, err);
     st->cur_nseg = 0;
@@ -1563,7 +1566,9 @@ int wide_scatter_blocks_per_sm(uint32_t kmax, int mode, bool stable) {
 // routed by size: empty ones are skipped, those that fit one CTA go straight
 // to the in-SM sort (original positions relative to the segment start), the
 // rest become level-1 segments of the sample sort.  Bad offsets raise a
-// device error flag instead of being followed.
+// device error flag instead of being followed; where they decrease, segments may
+// overlap, and the plan leaves the level-1 segments out (the others are read from
+// the input and written in their own range).
 __global__ void __launch_bounds__(256)
 k_init_segments(DevState* st, const uint64_t* offsets, uint32_t nseg, uint64_t n,
                 SegIn* list_l1, FinalItem* items, uint64_t seg_cap, uint64_t final_cap,
@@ -1573,7 +1578,7 @@ k_init_segments(DevState* st, const uint64_t* offsets, uint32_t nseg, uint64_t n
        s += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t a = offsets[s], b = offsets[s + 1];
     if (b < a || b > n || (b - a) > 0xFFFFFFFFull) {
-      atomicOr(&st->error, kErrBadOffsets);
+      atomicOr(&st->error, kErrBadOffsets | (b < a ? kErrUnordered : 0u));
       continue;
     }
     const uint64_t m = b - a;

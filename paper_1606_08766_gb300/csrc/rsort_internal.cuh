@@ -216,6 +216,7 @@ enum : uint32_t {
   kErrBucketCap = 1u << 6,
   kErrBadOffsets = 1u << 7,
   kErrWait = 1u << 8,         // a bounded wait on a bulk copy gave up
+  kErrUnordered = 1u << 9,    // decreasing offsets: segments may overlap
 };
 
 // Parameters of one level, fixed on the host.
