@@ -14,14 +14,14 @@ def _ms(n, k, keys):
     off = torch.empty(k + 1, dtype=torch.int64, device="cuda")
     a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
     ts = []
-    for _ in range(4):
+    for _ in range(6):
         a.record()
         for _ in range(4):
             partition_noalloc(keys, k, 3, ko, po, off)
         b.record()
         b.synchronize()
         ts.append(a.elapsed_time(b))
-    return sorted(ts)[1] / n
+    return min(ts) / n
 
 
 @pytest.mark.parametrize("k", [64, 1000])
@@ -30,5 +30,5 @@ def test_time_a_key_at_the_overlap_bound(k):
     g = torch.Generator(device="cuda").manual_seed(1)
     keys = torch.randint(-(1 << 63), (1 << 63) - 1, (n + 4096,), dtype=torch.int64, device="cuda",
                          generator=g)
-    # (launches overlapped at 2^27 keys: 1.10)
-    assert _ms(n, k, keys) < 1.04 * _ms(n + 4096, k, keys)
+    # (launches overlapped at 2^27 keys: 1.10; ordinary 1.00)
+    assert _ms(n, k, keys) < 1.06 * _ms(n + 4096, k, keys)
